@@ -59,6 +59,9 @@ VARIANT_KERNELS = {
                    "k_x_product_pr_pipe (pruned, pipelined, twiddles in shared memory)"],
     "energy_inv": ["k_inv_energy", "k_inv_energy_tma", "k_inv_energy_warp"],
 }
+# kernels of the even form in the same pass slots
+EVEN_KERNELS = {"energy_fwd": "k_ev_gen_y", "py_fwd": "k_ev_x", "px_product": "k_ev_corr", "py_inv": "k_ev_inv_x",
+                "energy_inv": "k_ev_inv_y"}
 KERNEL_NAMES = {"batch": "all passes of all instances (graph)", "energy_fwd": "k_fwd_energy", "py_fwd": "k_fwd_y", "px_product": "k_x_product",
                 "py_inv": "k_inv_y", "energy_inv": "k_inv_energy", "tables": "k_setup", "mu_solve": "k_mu_sect, k_mu_halley"}
 
@@ -112,6 +115,28 @@ def pass_bytes(s):
     out = Q * Q * n_omega
     return {"energy_fwd": 8 * W1, "py_fwd": 8 * (W1 + W2), "px_product": 8 * (W2 + W3),
             "py_inv": 8 * (W3 + W4), "energy_inv": 8 * W4 + 4 * out}
+
+
+def even_pass_bytes(s, grid, band, precision, fp32=0):
+    """The same for the even form (csrc/even.cuh), which a generated A takes on
+    FP32 Im chi grids of several zones whose edge rows weigh below 2^-24 (real
+    buffers over one quadrant, k_x <= k_y between the momentum passes), or None
+    when the call does not take it."""
+    if precision != fp32 or grid["zones"] == 1 or grid.get("quantity", 0) != 0:
+        return None
+    if (math.pi * grid["zones"] * band["ff_a"]) ** 2 < 8 * 24 * math.log(2.0):
+        return None
+    lens = [16 << i for i in range(8)] + [24 << i for i in range(7)]
+    need = [m for m in lens if m >= (s.N + s.q_extent // 2 + 1) // 2]
+    J0 = s.n_eps // 2
+    ne = min(s.n_eps, J0 + s.n_omega) - max(0, J0 - s.n_omega)
+    if not need or ne > 768 or s.N < 4:
+        return None
+    M, Nh, nl = min(need), s.N // 2, s.q_extent // 2 + 1
+    B1, B2, B3, B4 = Nh * M * ne, M * (M + 1) // 2 * ne, M * (M + 1) // 2 * s.n_omega, nl * M * s.n_omega
+    out = s.q_extent * s.q_extent * s.n_omega
+    return {"energy_fwd": 4 * B1, "py_fwd": 4 * (B1 + B2), "px_product": 4 * (B2 + B3),
+            "py_inv": 4 * (B3 + B4), "energy_inv": 4 * (B4 + out)}
 
 
 def measured_peaks():
@@ -658,7 +683,8 @@ def main():
             step()
         ptimes = plan.pass_times()
         plan.profile(False)
-        pb0 = pass_bytes(s)
+        even = even_pass_bytes(s, grid, bands[0], prec)
+        pb0 = even or pass_bytes(s)
         dom_pass = max((k for k in ptimes if k in pb0 and ptimes[k][1] > 0), key=lambda k: ptimes[k][0])
 
     # --- device-timed region: inputs resident; the dominant pass's events are
@@ -740,20 +766,23 @@ def main():
                     for i in range(len(grids))) + (1 if batched and persistent else 0)) * args.steps
     if batched:
         # concurrent instances: no per-pass split, the batch as one unit
-        pipeline_bytes = sum(sum(pass_bytes(plan.sizes[i]).values()) for i in range(len(grids)))
+        # the persistent launch and the tensor-core form run the general passes
+        general = persistent or prec != lh.FP32
+        pipeline_bytes = sum(sum(((None if general else even_pass_bytes(plan.sizes[i], grids[i], bands[i], prec))
+                                  or pass_bytes(plan.sizes[i])).values()) for i in range(len(grids)))
         dom, pb, dom_ms, traffic = "batch", {"batch": pipeline_bytes}, step_ms, None
         achieved = pipeline_bytes / (step_ms * 1e-3) / 1e9
     else:
         # roofline of the dominant kernel (largest share of device time in the
         # profiled run), its duration from the events of the timed region
-        pb = pass_bytes(s)
+        pb = pb0
         dom = dom_pass
         dom_ms = dom_live[dom][0] / dom_live[dom][1]
         achieved = pb[dom] / (dom_ms * 1e-3) / 1e9
         pipeline_bytes = sum(pb.values())
     variants = plan.variants(0) if not batched else {}
     if not batched:
-        traffic = None if args.grid else recorded_traffic(dom, args.workload, variants.get(dom, 0))
+        traffic = None if args.grid or even else recorded_traffic(dom, args.workload, variants.get(dom, 0))
     plain = None
     if batched:
         # the same instances one after another on one stream, no graph: the
@@ -803,7 +832,8 @@ def main():
                                          "speedup_persistent": cg_ms / step_ms}
             cg.close()
             del cg_out
-    dom_kernel = (VARIANT_KERNELS[dom][variants[dom]] if dom in VARIANT_KERNELS else KERNEL_NAMES[dom])
+    dom_kernel = (EVEN_KERNELS[dom] if not batched and even else
+                  VARIANT_KERNELS[dom][variants[dom]] if dom in VARIANT_KERNELS else KERNEL_NAMES[dom])
     tc = None
     kk = None
     thermal = None
@@ -822,7 +852,7 @@ def main():
         except Exception as exc:   # an extra object: never the main line's failure
             batch = {"unavailable": str(exc)}
         tc = tensor_core_form(lh, grids, bands, out, args.steps, not args.no_autotune, mu, stream)
-        if "py_inv_ms" in tc:
+        if "py_inv_ms" in tc and not even:   # the even form has no p_y inverse of that shape
             tc["py_inv_ms_fp32"] = round(ptimes["py_inv"][0] / max(ptimes["py_inv"][1], 1), 5)
             tc["py_inv_roofline_frac"] = pb["py_inv"] / (tc["py_inv_ms"] * 1e-3) / 1e9 / peak
 
@@ -841,6 +871,7 @@ def main():
                              "far above the 129 MB L2".format(pipeline_bytes / 1e9),
                        "autotune": not args.no_autotune,
                        "precision": args.precision,
+                       "form": "even (cosine transforms)" if not batched and even else "3D complex",
                        "variants": variants,
                        "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
             "roofline": {"bound": "hbm", "kernel": dom_kernel, "achieved": achieved, "peak": peak,

@@ -113,6 +113,7 @@ struct Work {
     const void *tc;        // tensor-core DFT matrices (k_tc.cu), or null
     const void *ptw = nullptr;   // per-stage twiddle tables of the pruned engine (FP32), or null
     const void *etw = nullptr;   // per-stage twiddle tables of the lines-across-lanes energy pass, or null
+    const void *evt = nullptr;   // tables of the even form's cosine transforms (FP32), or null
     InstState *state;      // [1]
     unsigned *status;      // plan-wide device status word
     double *mu_acc;        // scratch for the chemical potential solve

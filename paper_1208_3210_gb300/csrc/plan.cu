@@ -17,6 +17,7 @@
 #include <string>
 #include <vector>
 
+#include "even.cuh"
 #include "kernels.cuh"
 
 namespace lh {
@@ -56,6 +57,14 @@ size_t pr_twiddle_bytes();
 size_t et_twiddle_bytes();
 cudaError_t launch_et_twiddles(float2 *out, cudaStream_t s);
 cudaError_t launch_pr_twiddles(float2 *out, cudaStream_t s);
+size_t ev_table_bytes();
+cudaError_t launch_ev_tables(float2 *out, cudaStream_t s);
+cudaError_t launch_ev_gen_y(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, cudaStream_t s);
+cudaError_t launch_ev_x(const EvGeom &v, const Work<float> &w, cudaStream_t s);
+cudaError_t launch_ev_corr(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, int sms,
+                           cudaStream_t s);
+cudaError_t launch_ev_inv_x(const EvGeom &v, const Work<float> &w, cudaStream_t s);
+cudaError_t launch_ev_inv_y(const Geom &g, const EvGeom &v, const Work<float> &w, float *out, cudaStream_t s);
 bool pr_fwd_applies(const Geom &g);
 bool pr_inv_applies(const Geom &g);
 bool et_inv_applies(const Geom &g);
@@ -147,7 +156,9 @@ struct lindhard_plan {
         size_t X = 0, Y = 0, Z = 0, partial = 0, axis = 0, eps32 = 0, eps64 = 0, state = 0, acc = 0, bar = 0;
     };
     std::vector<Slot> slots;
-    size_t off_tw32 = 0, off_tw64 = 0, off_status = 0, off_tc = 0, off_dmu = 0, off_prtw = 0, off_etw = 0;
+    size_t off_tw32 = 0, off_tw64 = 0, off_status = 0, off_tc = 0, off_dmu = 0, off_prtw = 0, off_etw = 0, off_evt = 0;
+    // the even form's geometry of each instance (even.cuh); M = 0: not taken
+    std::vector<EvGeom> even;
     std::vector<size_t> off_kk;   // Kramers-Kronig weight tables per instance (FP32 grids)
     int tw_len = 0;
     bool backward = false;       // LINDHARD_PLAN_BACKWARD
@@ -523,6 +534,12 @@ extern "C" lindhard_status lindhard_plan_create(const lindhard_grid *grids, int 
     p->mu_G = mu_grid_size(p->num_sms, maxNpts);
     p->tw_len = maxLen;
 
+    p->even.assign(batch, EvGeom{});
+    for (int i = 0; i < batch; ++i) {
+        EvGeom v;
+        if (p->precision[i] == LINDHARD_FP32 && !p->direct && ev_geom(p->geoms[i], v)) p->even[i] = v;
+    }
+
     // bytes of each workspace part for instance i
     struct Need { size_t X, Y, Z, partial, axis, eps32, eps64; };
     auto need_of = [&](int i) {
@@ -540,6 +557,10 @@ extern "C" lindhard_status lindhard_plan_create(const lindhard_grid *grids, int 
             n.Y = std::max({(size_t)g.N * (size_t)d.t.xs2, (size_t)g.P * (size_t)d.cs,
                             (size_t)g.Q * g.Q * d.o.SP}) * cb;
         }
+        if (p->even[i].M) {
+            n.X = std::max(n.X, sizeof(float) * (size_t)ev_x_floats(p->even[i]));
+            n.Y = std::max(n.Y, sizeof(float) * (size_t)ev_y_floats(p->even[i]));
+        }
         n.Z = p->backward ? (size_t)g.Q * (size_t)g.xs3 * cb : 0;
         // the last pass's per-CTA sums, then the first reduction level's
         n.partial = p->backward ? (size_t)(bw_energy_blocks(g) + bw_partial_extra_rows()) * 5 * sizeof(double) : 0;
@@ -554,6 +575,7 @@ extern "C" lindhard_status lindhard_plan_create(const lindhard_grid *grids, int 
     p->off_status = o; o = align_up(o + sizeof(unsigned));
     p->off_prtw = o; o = align_up(o + pr_twiddle_bytes());   // pruned engine's per-stage twiddles
     p->off_etw = o; o = align_up(o + et_twiddle_bytes());     // energy pass's per-stage twiddles
+    p->off_evt = o; o = align_up(o + ev_table_bytes());       // the even form's tables
     p->off_dmu = o; o = align_up(o + sizeof(double) * 5 * kDmuBlocks);
     // tensor-core DFT matrices of every supported length (plans with a
     // LINDHARD_SPLITBF16_TC grid only)
@@ -611,6 +633,7 @@ extern "C" lindhard_status lindhard_plan_create(const lindhard_grid *grids, int 
         e = launch_twiddles(p->tw_len, (float2 *)(p->ws + p->off_tw32), (double2 *)(p->ws + p->off_tw64), 0);
     if (e == cudaSuccess) e = launch_pr_twiddles((float2 *)(p->ws + p->off_prtw), 0);
     if (e == cudaSuccess) e = launch_et_twiddles((float2 *)(p->ws + p->off_etw), 0);
+    if (e == cudaSuccess) e = launch_ev_tables((float2 *)(p->ws + p->off_evt), 0);
     if (e == cudaSuccess && p->off_tc) e = launch_tc_mats(p->ws + p->off_tc, 0);
     for (int i = 0; i < batch && e == cudaSuccess; ++i)
         if (p->off_kk[i]) e = launch_kk_tables(p->geoms[i].n_omega, p->ws + p->off_kk[i], 0);
@@ -807,6 +830,7 @@ static Work<Real> work_of(lindhard_plan *p, int i)
     w.tc = p->off_tc ? (const void *)(p->ws + p->off_tc) : nullptr;
     w.ptw = sizeof(Real) == 4 ? (const void *)(p->ws + p->off_prtw) : nullptr;
     w.etw = sizeof(Real) == 4 ? (const void *)(p->ws + p->off_etw) : nullptr;
+    w.evt = sizeof(Real) == 4 ? (const void *)(p->ws + p->off_evt) : nullptr;
     w.state = (InstState *)(p->ws + sl.state);
     w.status = (unsigned *)(p->ws + p->off_status);
     w.mu_acc = (double *)(p->ws + sl.acc);
@@ -929,6 +953,16 @@ static cudaError_t enqueue_forward(lindhard_plan *p, const std::vector<Band> &bs
                 for (int k = 0; k < 5 && e == cudaSuccess; ++k)
                     e = timed(p, 2 + k, s, [&] { return launch_direct_stage(k, g, b, w, a_i, o_i, s); });
                 a_off += (size_t)g.N * g.N * g.n_eps;
+                o_off += (size_t)g.Q * g.Q * g.n_omega;
+                continue;
+            }
+            if (const EvGeom &v = p->even[i]; A_in == nullptr && v.M && ev_band_applies(g, b)) {
+                // generated A, even in p_x and p_y: the cosine-transform form
+                if (e == cudaSuccess) e = timed(p, 2, s, [&] { return launch_ev_gen_y(g, v, b, w, s); });
+                if (e == cudaSuccess) e = timed(p, 3, s, [&] { return launch_ev_x(v, w, s); });
+                if (e == cudaSuccess) e = timed(p, 4, s, [&] { return launch_ev_corr(g, v, b, w, p->num_sms, s); });
+                if (e == cudaSuccess) e = timed(p, 5, s, [&] { return launch_ev_inv_x(v, w, s); });
+                if (e == cudaSuccess) e = timed(p, 6, s, [&] { return launch_ev_inv_y(g, v, w, o_i, s); });
                 o_off += (size_t)g.Q * g.Q * g.n_omega;
                 continue;
             }

@@ -131,6 +131,143 @@ inline bool ev_band_applies(const Geom &g, const Band &b)
 }
 
 // ---------------------------------------------------------------------------
+// Packed arithmetic.  A thread carries two complex columns at once, one in each
+// half of every register pair: four neighbouring floats x0..x3 of a row are the
+// columns x0 + i x2 and x1 + i x3, so a row's 16 bytes are (re, im) as they
+// lie, every complex operation is the same FP32x2 instruction for both columns
+// with no swap of register halves, and every twiddle, address and predicate
+// serves both.  Against one complex column a thread (75 instructions a point,
+// issue slots 70% busy) this issues half the instructions; what bounds the
+// passes now is the L1 data pipe (60-65%, the two exchanges) and the wait for
+// loads.  1024^2 x 512, us, one column -> two: generation 338 -> 289, p_x 440
+// -> 396, inverse k_x 250 -> 244, inverse k_y 280 -> 267 (5.5 TB/s).
+struct Cx2 { float2 re, im; };
+
+__device__ __forceinline__ float2 dup2(float c) { return make_float2(c, c); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return psub<true>(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ Cx2 add(Cx2 a, Cx2 b) { return {add2(a.re, b.re), add2(a.im, b.im)}; }
+__device__ __forceinline__ Cx2 sub(Cx2 a, Cx2 b) { return {sub2(a.re, b.re), sub2(a.im, b.im)}; }
+// a + i b and a - i b
+__device__ __forceinline__ Cx2 add_i(Cx2 a, Cx2 b) { return {sub2(a.re, b.im), add2(a.im, b.re)}; }
+__device__ __forceinline__ Cx2 sub_i(Cx2 a, Cx2 b) { return {add2(a.re, b.im), sub2(a.im, b.re)}; }
+// a times w or conj(w)
+template <bool CONJ>
+__device__ __forceinline__ Cx2 mul_w(Cx2 a, float2 w)
+{
+    const float2 wr = dup2(w.x), wi = dup2(w.y);
+    if constexpr (CONJ) return {fma2(a.re, wr, mul2(a.im, wi)), fma2(a.im, wr, neg2(mul2(a.re, wi)))};
+    else return {fma2(a.re, wr, neg2(mul2(a.im, wi))), fma2(a.im, wr, mul2(a.re, wi))};
+}
+
+// Small DFTs, positive exponent with INV.  The multiplications by sqrt(1/2)
+// and sqrt(3/4) ride on the sums that follow as fused multiply-adds; 12 = 3 x 4
+// by the prime-factor map (Good 1958), which needs no twiddles.
+template <bool INV>
+__device__ __forceinline__ void dft3(Cx2 &a, Cx2 &b, Cx2 &c)
+{
+    const float2 h = dup2(-0.5f), s = dup2(INV ? -0.86602540378443864676f : 0.86602540378443864676f), n = neg2(s);
+    const Cx2 t = add(b, c), d = sub(b, c), m = {fma2(t.re, h, a.re), fma2(t.im, h, a.im)};
+    a = add(a, t);
+    b = {fma2(d.im, s, m.re), fma2(d.re, n, m.im)};   // m - i s d
+    c = {fma2(d.im, n, m.re), fma2(d.re, s, m.im)};   // m + i s d
+}
+template <bool INV>
+__device__ __forceinline__ void dft4(Cx2 &a, Cx2 &b, Cx2 &c, Cx2 &d)
+{
+    const Cx2 p = add(a, c), m = sub(a, c), q = add(b, d), r = sub(b, d);
+    a = add(p, q);
+    c = sub(p, q);
+    b = INV ? add_i(m, r) : sub_i(m, r);
+    d = INV ? sub_i(m, r) : add_i(m, r);
+}
+// (e + w o, e - w o) for w = e^{-+ i pi/4} (K = 1) or e^{-+ 3 i pi/4} (K = 3)
+template <bool INV, int K>
+__device__ __forceinline__ void combine45(Cx2 e, Cx2 o, Cx2 &lo, Cx2 &hi)
+{
+    const float2 c = dup2(0.70710678118654752440f), n = dup2(-0.70710678118654752440f);
+    const float2 s = add2(o.re, o.im), d = sub2(o.im, o.re);
+    // forward: w1 o = c (s + i d), w3 o = c (d - i s); inverse: w1 o = c (-d + i s), w3 o = c (-s - i d)
+    if constexpr (K == 1 && !INV) {
+        lo = {fma2(s, c, e.re), fma2(d, c, e.im)};
+        hi = {fma2(s, n, e.re), fma2(d, n, e.im)};
+    } else if constexpr (K == 3 && !INV) {
+        lo = {fma2(d, c, e.re), fma2(s, n, e.im)};
+        hi = {fma2(d, n, e.re), fma2(s, c, e.im)};
+    } else if constexpr (K == 1) {
+        lo = {fma2(d, n, e.re), fma2(s, c, e.im)};
+        hi = {fma2(d, c, e.re), fma2(s, n, e.im)};
+    } else {
+        lo = {fma2(s, n, e.re), fma2(d, n, e.im)};
+        hi = {fma2(s, c, e.re), fma2(d, c, e.im)};
+    }
+}
+template <bool INV>
+__device__ __forceinline__ void dft8(Cx2 *v)
+{
+    Cx2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
+    dft4<INV>(e0, e1, e2, e3);
+    dft4<INV>(o0, o1, o2, o3);
+    v[0] = add(e0, o0);
+    v[4] = sub(e0, o0);
+    v[2] = INV ? add_i(e2, o2) : sub_i(e2, o2);
+    v[6] = INV ? sub_i(e2, o2) : add_i(e2, o2);
+    combine45<INV, 1>(e1, o1, v[1], v[5]);
+    combine45<INV, 3>(e3, o3, v[3], v[7]);
+}
+template <int R, bool INV>
+__device__ __forceinline__ void dft(Cx2 *v)
+{
+    if constexpr (R == 2) {
+        const Cx2 a = v[0], b = v[1];
+        v[0] = add(a, b);
+        v[1] = sub(a, b);
+    } else if constexpr (R == 4) {
+        dft4<INV>(v[0], v[1], v[2], v[3]);
+    } else if constexpr (R == 8) {
+        dft8<INV>(v);
+    } else if constexpr (R == 12) {
+        // inputs n = 3 i + 4 j, outputs k = 9 k4 + 4 k3 (mod 12)
+        Cx2 t[3][4];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) t[j][i] = v[(3 * i + 4 * j) % 12];
+            dft4<INV>(t[j][0], t[j][1], t[j][2], t[j][3]);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            dft3<INV>(t[0][k], t[1][k], t[2][k]);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) v[(9 * k + 4 * q) % 12] = t[q][k];
+        }
+    } else {
+        static_assert(R == 16, "radices of the schedules");
+        Cx2 e[8], o[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { e[i] = v[2 * i]; o[i] = v[2 * i + 1]; }
+        dft8<INV>(e);
+        dft8<INV>(o);
+        v[0] = add(e[0], o[0]);
+        v[8] = sub(e[0], o[0]);
+        v[4] = INV ? add_i(e[4], o[4]) : sub_i(e[4], o[4]);
+        v[12] = INV ? sub_i(e[4], o[4]) : add_i(e[4], o[4]);
+        combine45<INV, 1>(e[2], o[2], v[2], v[10]);
+        combine45<INV, 3>(e[6], o[6], v[6], v[14]);
+#pragma unroll
+        for (int k = 1; k < 8; k += 2) {
+            const float c = (float)cos48(3 * k), s = (float)sin48(3 * k);
+            const Cx2 w = mul_w<!INV>(o[k], make_float2(c, s));
+            v[k] = add(e[k], w);
+            v[k + 8] = sub(e[k], w);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Radix schedules of the cosine transform's FFT (DCT-III order; DCT-II runs
 // them reversed).  The first radix R0 is half of the values per thread, so
 // that a thread owns butterflies j and M/R0 - j and with them rows n and M - n.
@@ -159,8 +296,14 @@ __host__ __device__ constexpr int ev_ns(int M, int s, bool rev)
 {
     return s == 0 ? 1 : ev_ns(M, s - 1, rev) * ev_radix(M, s - 1, rev);
 }
-// Tables (float2 units): per length M the M values w_j = e^{i pi j / 2M}, then
-// per direction and stage s >= 1 rows k < Ns of (w, w^2), w = e^{-2 pi i k / (Ns Rs)}.
+// Tables (float2): per length M the values w_j = e^{i pi j / 2M}, j < M, then
+// per direction and stage s >= 1 rows k < Ns of w, w^2 (and for radices above 4
+// w^3, w^4), w = e^{-2 pi i k / (Ns Rs)}; the higher powers are products of
+// these, one rounding deep up to w^8.  (All powers from a table, as register
+// pairs ready for the packed products, loaded no slower per value but took a
+// third of the L1 data pipe: a 16-byte load costs four wavefronts however many
+// lanes share its address.)
+__host__ __device__ constexpr int ev_row(int R) { return R > 4 ? 4 : 2; }
 __host__ __device__ constexpr int ev_table_offset(int M, int s, bool rev)   // s = 0: the w_j
 {
     int o = 0;
@@ -171,53 +314,65 @@ __host__ __device__ constexpr int ev_table_offset(int M, int s, bool rev)   // s
         for (int d = 0; d < 2; ++d)
             for (int st = 1; st < ev_nstages(L); ++st) {
                 if (L == M && s == st && rev == (d != 0)) return o;
-                o += 2 * ev_ns(L, st, d != 0);
+                o += ev_ns(L, st, d != 0) * ev_row(ev_radix(L, st, d != 0));
             }
     }
     return o;
 }
 __host__ __device__ constexpr int ev_table_entries() { return ev_table_offset(0, 0, false); }
-
-// Tiles: C complex columns (2C floats of a row), about 768 threads per SM (up
-// to 85 registers each): the loads of one CTA's tile overlap the butterflies
-// of another's.
-template <int M> struct EvCfg {
-    static constexpr int C = M <= 24 ? 64 : M <= 96 ? 32 : M <= 384 ? 16 : M <= 1536 ? 8 : 4;
-    static constexpr int T = C * M / ev_vpt(M);
-    static constexpr int MINB = M >= 1024 ? 1 : 768 / T;
-};
-
-// v[1..R) times the powers of (w, w^2) (conjugated with CONJ).
-template <int R, bool CONJ>
-__device__ __forceinline__ void ev_twiddle(float2 *v, const float4 *row)
+// w^1..w^(R-1) from a table row
+template <int R>
+__device__ __forceinline__ void ev_powers(float2 *w, const float2 *__restrict__ row)
 {
-    const float4 q = __ldg(row);
-    float2 w[R];
+    const float4 q = __ldg(reinterpret_cast<const float4 *>(row));
     w[1] = make_float2(q.x, q.y);
     if constexpr (R > 2) w[2] = make_float2(q.z, q.w);
+    if constexpr (R == 4) w[3] = cmul(w[1], w[2]);
+    if constexpr (R > 4) {
+        const float4 p = __ldg(reinterpret_cast<const float4 *>(row) + 1);
+        w[3] = make_float2(p.x, p.y);
+        w[4] = make_float2(p.z, p.w);
 #pragma unroll
-    for (int r = 3; r < R; ++r) w[r] = cmul(w[r / 2], w[r - r / 2]);
-#pragma unroll
-    for (int r = 1; r < R; ++r) v[r] = CONJ ? cmulc(v[r], w[r]) : cmul(v[r], w[r]);
+        for (int r = 5; r < R; ++r) w[r] = r <= 8 ? cmul(w[4], w[r - 4]) : cmul(w[8], w[r - 8]);
+    }
 }
 
-// One tile of C complex columns, VPT values per thread.  REV = false: DCT-III
-// (positive exponent), the first stage on the butterfly pairs; REV = true:
-// DCT-II (negative exponent), the last stage on the pairs.  Thread: column
-// tid % C, unit u = tid / C.
+// Tiles: C packs of two complex columns (4C floats, 64 to 512 bytes of a row).
+// Per SM 512 threads at 16 values each and 384 at 24: a load in flight holds its
+// place in L1, and a fourth tile of 53 KB per SM left so little of it that the
+// passes that load slowed down (k_ev_x at 1024^2 x 512 0.40 -> 0.52 ms); the
+// generating pass, which loads nothing, runs four (0.31 -> 0.29 ms).
+template <int M> struct EvCfg {
+    static constexpr int C = M <= 24 ? 32 : M <= 48 ? 16 : M <= 256 ? 8 : M <= 1536 ? 4 : 2;
+    static constexpr int T = C * M / ev_vpt(M);
+    static constexpr int MINB_GEN = 512 / T;
+    static constexpr int MINB = ev_vpt(M) == 16 ? 512 / T : 384 / T > 0 ? 384 / T : 1;
+};
+
+// One tile of C packs, VPT values per thread.  REV = false: DCT-III (positive
+// exponent), the first stage on the butterfly pairs; REV = true: DCT-II
+// (negative exponent), the last stage on the pairs.  Thread: pack tid % C,
+// unit u = tid / C.
 template <int M, bool REV>
 struct EvFft {
     static constexpr int C = EvCfg<M>::C, T = EvCfg<M>::T, VPT = ev_vpt(M), TPC = M / VPT, NS = ev_nstages(M);
     static constexpr int RF = ev_radix(M, 0, REV), RP = ev_vpt(M) / 2, NBP = M / RP;   // RP, NBP: the paired stage
-    // rows of C values; narrow rows get one empty row after every RF rows, so
-    // that the first exchange's writes (rows RF apart) fall into different banks
-    static constexpr bool PAD = C < 16;
-    static constexpr int SMEM_ELEMS = (PAD ? M + M / RF : M) * C;
+    // rows of C packs (16 bytes each); rows narrower than 128 bytes get one
+    // empty row after every RF rows, so that the first exchange's writes (rows
+    // RF apart) fall into different banks
+    static constexpr bool PAD = C < 8;
+    static constexpr int SMEM_ELEMS = (PAD ? M + M / RF : M) * C;   // packs
     static_assert(NBP == 2 * TPC, "a thread owns one butterfly pair");
 
     __device__ __forceinline__ static int srow(int row) { return (PAD ? row + row / RF : row) * C; }
     // offset of `step` further rows (a multiple of RF, or inside a block of RF)
     __host__ __device__ static constexpr int soff(int step) { return (PAD ? step + step / RF : step) * C; }
+    __device__ __forceinline__ static void st(float4 *p, Cx2 v) { *p = make_float4(v.re.x, v.re.y, v.im.x, v.im.y); }
+    __device__ __forceinline__ static Cx2 ld(const float4 *p)
+    {
+        const float4 q = *p;
+        return {make_float2(q.x, q.y), make_float2(q.z, q.w)};
+    }
     template <int S>
     __device__ __forceinline__ static int butterfly(int b, int u)
     {
@@ -226,7 +381,7 @@ struct EvFft {
         else return u + b * TPC;
     }
     template <int S>
-    __device__ __forceinline__ static void rest(float2 *v, float2 *sm, int u, const float2 *__restrict__ tab)
+    __device__ __forceinline__ static void rest(Cx2 *v, float4 *sm, int u, const float2 *__restrict__ tab)
     {
         if constexpr (S < NS) {
             constexpr int Rp = ev_radix(M, S - 1, REV), Nsp = ev_ns(M, S - 1, REV);
@@ -237,38 +392,50 @@ struct EvFft {
 #pragma unroll
             for (int b = 0; b < VPT / Rp; ++b) {
                 const int j = butterfly<S - 1>(b, u);
-                float2 *p = sm + srow((j / Nsp) * (Nsp * Rp) + j % Nsp);
+                float4 *p = sm + srow((j / Nsp) * (Nsp * Rp) + j % Nsp);
 #pragma unroll
-                for (int r = 0; r < Rp; ++r) p[soff(r * Nsp)] = v[b * Rp + r];
+                for (int r = 0; r < Rp; ++r) st(p + soff(r * Nsp), v[b * Rp + r]);
             }
             __syncthreads();
 #pragma unroll
             for (int b = 0; b < VPT / Rs; ++b) {
                 const int j = butterfly<S>(b, u);
-                const float2 *p = sm + srow(j);
+                const float4 *p = sm + srow(j);
+                float2 w[Rs];
+                ev_powers<Rs>(w, tab + ev_table_offset(M, S, REV) + j % Ns * ev_row(Rs));
+                v[b * Rs] = ld(p);
 #pragma unroll
-                for (int r = 0; r < Rs; ++r) v[b * Rs + r] = p[soff(r * (M / Rs))];
-                ev_twiddle<Rs, !REV>(v + b * Rs, reinterpret_cast<const float4 *>(tab + ev_table_offset(M, S, REV)) + j % Ns);
-                Dft<Rs, !REV, float2>::run(v + b * Rs);
+                for (int r = 1; r < Rs; ++r) v[b * Rs + r] = mul_w<!REV>(ld(p + soff(r * (M / Rs))), w[r]);
+                dft<Rs, !REV>(v + b * Rs);
             }
             rest<S + 1>(v, sm, u, tab);
         }
     }
-    // sm: this thread's column of the tile's exchange buffer (base + tid % C);
+    // sm: this thread's pack of the tile's exchange buffer (base + tid % C);
     // v: first-stage inputs on entry, last-stage outputs on exit
-    __device__ __forceinline__ static void run(float2 *v, float2 *sm, int u, const float2 *__restrict__ tab)
+    __device__ __forceinline__ static void run(Cx2 *v, float4 *sm, int u, const float2 *__restrict__ tab)
     {
 #pragma unroll
-        for (int b = 0; b < VPT / RF; ++b) Dft<RF, !REV, float2>::run(v + b * RF);
+        for (int b = 0; b < VPT / RF; ++b) dft<RF, !REV>(v + b * RF);
         rest<1>(v, sm, u, tab);
     }
 };
+
+// A pack from global memory, read once: not kept in L1, whose few KB beside the
+// exchange buffers hold the tables.
+__device__ __forceinline__ Cx2 ev_load(const float *p)
+{
+    float4 q;
+    asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+        : "=f"(q.x), "=f"(q.y), "=f"(q.z), "=f"(q.w) : "l"(p));
+    return {make_float2(q.x, q.y), make_float2(q.z, q.w)};
+}
 
 // The pairs (n, M - n) of a thread's two paired butterflies (rows j + r NBP in
 // v[b RP + r]): f(row n, value at n, value at M - n) for every pair, with
 // M - 0 taken as row 0 itself.
 template <int RP, int NBP, int TPC, typename F>
-__device__ __forceinline__ void ev_pairs(float2 *v, int u, F &&f)
+__device__ __forceinline__ void ev_pairs(Cx2 *v, int u, F &&f)
 {
     if (u != 0) {
 #pragma unroll
@@ -286,40 +453,40 @@ __device__ __forceinline__ void ev_pairs(float2 *v, int u, F &&f)
 // z -> V of the DCT-III, in place: V_n = w (a - i b), V_{M-n} = conj(w) (a + i b)
 // for a = z_n, b = z_{M-n} (row 0: V_0 = z_0).
 template <int M>
-__device__ __forceinline__ void ev_pre(float2 *v, int u, const float2 *__restrict__ tab)
+__device__ __forceinline__ void ev_pre(Cx2 *v, int u, const float2 *__restrict__ tab)
 {
     constexpr int RP = ev_vpt(M) / 2, NBP = M / RP, TPC = M / ev_vpt(M);
     const float2 *wt = tab + ev_table_offset(M, 0, false);
-    ev_pairs<RP, NBP, TPC>(v, u, [&](int n, float2 &a, float2 &b) {
-        if (&a == &b) {
-            // n = 0: unchanged; n = M/2: w (1 - i) a = sqrt(2) a
-            if (n != 0) a = make_float2(1.41421356237309505f * a.x, 1.41421356237309505f * a.y);
+    ev_pairs<RP, NBP, TPC>(v, u, [&](int n, Cx2 &a, Cx2 &b) {
+        if (&a == &b) {   // n = 0: unchanged; n = M/2: w (1 - i) a = sqrt(2) a
+            const float2 c = dup2(1.41421356237309505f);
+            if (n != 0) a = {mul2(a.re, c), mul2(a.im, c)};
             return;
         }
         const float2 w = __ldg(wt + n);
-        const float2 s = make_float2(a.x + b.y, a.y - b.x), d = make_float2(a.x - b.y, a.y + b.x);
-        a = cmul(s, w);
-        b = cmulc(d, w);
+        const Cx2 s = sub_i(a, b), d = add_i(a, b);
+        a = mul_w<false>(s, w);
+        b = mul_w<true>(d, w);
     });
 }
 
 // V -> 2 z of the DCT-II, in place: 2 z_n = conj(w) V_n + w V_{M-n},
 // 2 z_{M-n} = -i (w V_{M-n} - conj(w) V_n).
 template <int M>
-__device__ __forceinline__ void ev_post(float2 *v, int u, const float2 *__restrict__ tab)
+__device__ __forceinline__ void ev_post(Cx2 *v, int u, const float2 *__restrict__ tab)
 {
     constexpr int RP = ev_vpt(M) / 2, NBP = M / RP, TPC = M / ev_vpt(M);
     const float2 *wt = tab + ev_table_offset(M, 0, false);
-    ev_pairs<RP, NBP, TPC>(v, u, [&](int n, float2 &a, float2 &b) {
+    ev_pairs<RP, NBP, TPC>(v, u, [&](int n, Cx2 &a, Cx2 &b) {
         if (&a == &b) {
-            const float c = n == 0 ? 2.0f : 1.41421356237309505f;
-            a = make_float2(c * a.x, c * a.y);
+            const float2 c = dup2(n == 0 ? 2.0f : 1.41421356237309505f);
+            a = {mul2(a.re, c), mul2(a.im, c)};
             return;
         }
         const float2 w = __ldg(wt + n);
-        const float2 s = cmulc(a, w), t = cmul(b, w);
-        a = cadd(s, t);
-        b = make_float2(t.y - s.y, s.x - t.x);
+        const Cx2 s = mul_w<true>(a, w), t = mul_w<false>(b, w);
+        a = add(s, t);
+        b = {sub2(t.im, s.im), sub2(s.re, t.re)};
     });
 }
 

@@ -11,18 +11,28 @@
 
 namespace lh {
 
+// 1/x as the hardware approximation (relative error about 2^-23; x lies in
+// [gamma^2, 4 e_max^2 + gamma^2], away from zero, subnormals and overflow)
+__device__ __forceinline__ float ev_rcp(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // One block per table and slice: the tables' places and periods come as an
 // argument (evaluating ev_table_offset per entry on the device took 0.5 ms).
 struct EvTabs {
-    struct { int off, count, period; } t[64];   // period 0: the w_j of length `count`
+    struct { int off, count, row, period; } t[64];   // row 0: the w_j, j < period
 };
 __global__ void k_ev_tables(float2 *out, EvTabs tabs)
 {
-    const int off = tabs.t[blockIdx.x].off, count = tabs.t[blockIdx.x].count, period = tabs.t[blockIdx.x].period;
+    const int off = tabs.t[blockIdx.x].off, count = tabs.t[blockIdx.x].count, row = tabs.t[blockIdx.x].row,
+              period = tabs.t[blockIdx.x].period;
     for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < count; i += gridDim.y * blockDim.x) {
         double s, c;
-        if (period == 0) sincospi(0.5 * (double)i / (double)count, &s, &c);
-        else sincospi(-2.0 * (double)((i / 2) * (i % 2 + 1)) / (double)period, &s, &c);
+        if (row == 0) sincospi(0.5 * (double)i / (double)period, &s, &c);
+        else sincospi(-2.0 * (double)((i / row) * (i % row + 1)) / (double)period, &s, &c);
         out[off + i] = make_float2((float)c, (float)s);
     }
 }
@@ -32,13 +42,13 @@ cudaError_t launch_ev_tables(float2 *out, cudaStream_t s)
     int n = 0, o = 0;
     for (int i = 0; ev_len(i) != 0; ++i) {   // the order of ev_table_offset
         const int M = ev_len(i);
-        tabs.t[n++] = {o, M, 0};
+        tabs.t[n++] = {o, M, 0, M};
         o += M;
         for (int d = 0; d < 2; ++d)
             for (int st = 1; st < ev_nstages(M); ++st) {
-                const int Ns = ev_ns(M, st, d != 0);
-                tabs.t[n++] = {o, 2 * Ns, Ns * ev_radix(M, st, d != 0)};
-                o += 2 * Ns;
+                const int Ns = ev_ns(M, st, d != 0), R = ev_radix(M, st, d != 0);
+                tabs.t[n++] = {o, Ns * ev_row(R), ev_row(R), Ns * R};
+                o += Ns * ev_row(R);
             }
     }
     k_ev_tables<<<dim3(n, 4), 128, 0, s>>>(out, tabs);
@@ -48,47 +58,59 @@ size_t ev_table_bytes() { return (size_t)ev_table_entries() * sizeof(float2); }
 
 // Grid: Nh x (column tiles), the tiles of one p_x neighbours.
 template <int M>
-__global__ void __launch_bounds__(EvCfg<M>::T, EvCfg<M>::MINB)
+__global__ void __launch_bounds__(EvCfg<M>::T, EvCfg<M>::MINB_GEN)
 k_ev_gen_y(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const float2 *__restrict__ eps,
            const InstState *__restrict__ st, float *__restrict__ B1, const float2 *__restrict__ tab, int ntile)
 {
     using F = EvFft<M, false>;
     constexpr int C = F::C, T = F::T, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    LH_REQUIRE_SMEM(F::SMEM_ELEMS, float2)
-    float2 *sm = reinterpret_cast<float2 *>(smem_raw);
+    LH_REQUIRE_SMEM(F::SMEM_ELEMS, float4)
+    float4 *sm = reinterpret_cast<float4 *>(smem_raw);
     const int jx = blockIdx.x / ntile, ct = blockIdx.x % ntile;
     const int col = threadIdx.x % C, u = threadIdx.x / C;
 
-    // band energy and amplitude of every row, once per tile (3 Nh floats in
-    // the exchange buffer: Nh <= M and at least 4 columns of 8 bytes)
-    float *bx = reinterpret_cast<float *>(smem_raw), *bl = bx + v.Nh, *ba = bl + v.Nh;
+    // band energy and amplitude of every row, once per tile (16 Nh bytes in the
+    // exchange buffer, which has M > Nh rows of at least two packs)
+    float4 *rows = sm;
     const AxisTab ax = axis[g.N / 2 + jx];
-    for (int i = threadIdx.x; i < v.Nh; i += T)
-        band_point_f32(band, ax, axis[g.N / 2 + i], st, bx[i], bl[i], ba[i]);
+    for (int i = threadIdx.x; i < v.Nh; i += T) {
+        float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+        band_point_f32(band, ax, axis[g.N / 2 + i], st, q.x, q.y, q.z);
+        rows[i] = q;
+    }
     __syncthreads();
 
-    // energies 2c, 2c + 1 of the window; columns past its end hold zeros
-    const int e = 2 * (ct * C + col);
-    const float2 e0 = e < v.ne ? __ldg(&eps[v.e0 + e]) : make_float2(0.f, 0.f);
-    const float2 e1 = e + 1 < v.ne ? __ldg(&eps[v.e0 + e + 1]) : make_float2(0.f, 0.f);
-    const float on0 = e < v.ne ? 1.f : 0.f, on1 = e + 1 < v.ne ? 1.f : 0.f;
-    const float g2 = band.gam2;
-    float2 z[VPT];
+    // energies e..e+3 of the window, as (hi, lo); past its end amplitude 0
+    const int e = 4 * (ct * C + col);
+    float2 eh[2], el[2], on[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int k = e + 2 * h;
+        const float2 a = __ldg(&eps[v.e0 + min(k, v.ne - 1)]), b = __ldg(&eps[v.e0 + min(k + 1, v.ne - 1)]);
+        eh[h] = make_float2(a.x, b.x);
+        el[h] = make_float2(a.y, b.y);
+        on[h] = make_float2(k < v.ne ? 1.f : 0.f, k + 1 < v.ne ? 1.f : 0.f);
+    }
+    const float2 g2 = dup2(band.gam2);
+    Cx2 z[VPT];
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
         const int j = F::template butterfly<0>(b, u);
 #pragma unroll
         for (int r = 0; r < RP; ++r) {
             const int n = j + r * NBP;
-            float2 a = make_float2(0.f, 0.f);
+            float2 a[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
             if (n < v.Nh) {
-                const float xhi = bx[n], xlo = bl[n], amp = ba[n];
-                const float d0 = (e0.x - xhi) + (e0.y - xlo), d1 = (e1.x - xhi) + (e1.y - xlo);
-                a = make_float2(on0 * amp * __fdividef(1.0f, fmaf(d0, d0, g2)),
-                                on1 * amp * __fdividef(1.0f, fmaf(d1, d1, g2)));
+                const float4 q = rows[n];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float2 d = add2(sub2(eh[h], dup2(q.x)), sub2(el[h], dup2(q.y)));
+                    const float2 x = fma2(d, d, g2);
+                    a[h] = mul2(mul2(on[h], dup2(q.z)), make_float2(ev_rcp(x.x), ev_rcp(x.y)));
+                }
             }
-            z[b * RP + r] = a;
+            z[b * RP + r] = {a[0], a[1]};
         }
     }
     ev_pre<M>(z, u, tab);
@@ -101,7 +123,7 @@ k_ev_gen_y(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const 
         for (int b = 0; b < VPT / RL; ++b)
 #pragma unroll
             for (int r = 0; r < RL; ++r)
-                *reinterpret_cast<float2 *>(o + (long long)(u + b * TPC + r * (M / RL)) * v.ES) = z[b * RL + r];
+                F::st(reinterpret_cast<float4 *>(o + (u + b * TPC + r * (M / RL)) * v.ES), z[b * RL + r]);
     }
 }
 
@@ -113,22 +135,21 @@ k_ev_x(EvGeom v, const float *__restrict__ B1, float *__restrict__ B2, const flo
     using F = EvFft<M, false>;
     constexpr int C = F::C, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    LH_REQUIRE_SMEM(F::SMEM_ELEMS, float2)
-    float2 *sm = reinterpret_cast<float2 *>(smem_raw);
+    LH_REQUIRE_SMEM(F::SMEM_ELEMS, float4)
+    float4 *sm = reinterpret_cast<float4 *>(smem_raw);
     const int ky = blockIdx.x / ntile, ct = blockIdx.x % ntile;
     const int col = threadIdx.x % C, u = threadIdx.x / C;
-    const int e = 2 * (ct * C + col);
+    const int e = 4 * (ct * C + col);
     const bool on = e < v.ES;
     const float *in = B1 + (long long)ky * v.ES + e;
-    float2 z[VPT];
+    Cx2 z[VPT];
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
         const int j = F::template butterfly<0>(b, u);
 #pragma unroll
         for (int r = 0; r < RP; ++r) {
             const int n = j + r * NBP;
-            z[b * RP + r] = on && n < v.Nh ? __ldcs(reinterpret_cast<const float2 *>(in + n * v.s1))
-                                           : make_float2(0.f, 0.f);
+            z[b * RP + r] = on && n < v.Nh ? ev_load(in + n * v.s1) : Cx2{dup2(0.f), dup2(0.f)};
         }
     }
     ev_pre<M>(z, u, tab);
@@ -141,7 +162,7 @@ k_ev_x(EvGeom v, const float *__restrict__ B1, float *__restrict__ B2, const flo
 #pragma unroll
             for (int r = 0; r < RL; ++r) {
                 const int kx = u + b * TPC + r * (M / RL);
-                if (kx <= ky) *reinterpret_cast<float2 *>(o + kx * v.s2) = z[b * RL + r];
+                if (kx <= ky) F::st(reinterpret_cast<float4 *>(o + kx * v.s2), z[b * RL + r]);
             }
     }
 }
@@ -149,10 +170,10 @@ k_ev_x(EvGeom v, const float *__restrict__ B1, float *__restrict__ B2, const flo
 template <int M>
 cudaError_t launch_ev_gen_y_t(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, cudaStream_t s)
 {
-    const size_t smem = sizeof(float2) * EvFft<M, false>::SMEM_ELEMS;
+    const size_t smem = sizeof(float4) * EvFft<M, false>::SMEM_ELEMS;
     static const cudaError_t e = smem_attrs(k_ev_gen_y<M>, smem);
     if (e != cudaSuccess) return e;
-    const int ntile = (v.ES + 2 * EvCfg<M>::C - 1) / (2 * EvCfg<M>::C);
+    const int ntile = (v.ES + 4 * EvCfg<M>::C - 1) / (4 * EvCfg<M>::C);
     k_ev_gen_y<M><<<v.Nh * ntile, EvCfg<M>::T, smem, s>>>(g, v, band, w.axis, (const float2 *)w.eps, w.state,
                                                           (float *)w.X, (const float2 *)w.evt, ntile);
     return cudaGetLastError();
@@ -160,10 +181,10 @@ cudaError_t launch_ev_gen_y_t(const Geom &g, const EvGeom &v, const Band &band, 
 template <int M>
 cudaError_t launch_ev_x_t(const EvGeom &v, const Work<float> &w, cudaStream_t s)
 {
-    const size_t smem = sizeof(float2) * EvFft<M, false>::SMEM_ELEMS;
+    const size_t smem = sizeof(float4) * EvFft<M, false>::SMEM_ELEMS;
     static const cudaError_t e = smem_attrs(k_ev_x<M>, smem);
     if (e != cudaSuccess) return e;
-    const int ntile = (v.ES + 2 * EvCfg<M>::C - 1) / (2 * EvCfg<M>::C);
+    const int ntile = (v.ES + 4 * EvCfg<M>::C - 1) / (4 * EvCfg<M>::C);
     k_ev_x<M><<<M * ntile, EvCfg<M>::T, smem, s>>>(v, (const float *)w.X, (float *)w.Y, (const float2 *)w.evt, ntile);
     return cudaGetLastError();
 }

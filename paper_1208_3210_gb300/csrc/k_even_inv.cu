@@ -17,20 +17,19 @@ k_ev_inv_x(EvGeom v, const float *__restrict__ B3, float *__restrict__ B4, const
     using F = EvFft<M, true>;
     constexpr int C = F::C, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP, RF = F::RF;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    LH_REQUIRE_SMEM(F::SMEM_ELEMS, float2)
-    float2 *sm = reinterpret_cast<float2 *>(smem_raw);
+    LH_REQUIRE_SMEM(F::SMEM_ELEMS, float4)
+    float4 *sm = reinterpret_cast<float4 *>(smem_raw);
     const int ky = blockIdx.x / ntile, ct = blockIdx.x % ntile;
     const int col = threadIdx.x % C, u = threadIdx.x / C;
-    const int m = 2 * (ct * C + col);
+    const int m = 4 * (ct * C + col);
     const bool on = m < v.WS;
-    float2 z[VPT];
+    Cx2 z[VPT];
 #pragma unroll
     for (int b = 0; b < VPT / RF; ++b)
 #pragma unroll
         for (int r = 0; r < RF; ++r) {
             const int kx = u + b * TPC + r * (M / RF), lo = min(kx, ky), hi = max(kx, ky);
-            z[b * RF + r] = on ? __ldg(reinterpret_cast<const float2 *>(B3 + lo * v.s3 + (long long)hi * v.WS + m))
-                               : make_float2(0.f, 0.f);
+            z[b * RF + r] = on ? ev_load(B3 + lo * v.s3 + hi * v.WS + m) : Cx2{dup2(0.f), dup2(0.f)};
         }
     F::run(z, sm + col, u, tab);
     ev_post<M>(z, u, tab);
@@ -42,16 +41,16 @@ k_ev_inv_x(EvGeom v, const float *__restrict__ B3, float *__restrict__ B4, const
 #pragma unroll
             for (int r = 0; r < RP; ++r) {
                 const int l = j + r * NBP;
-                if (l < v.nl) *reinterpret_cast<float2 *>(o + l * v.s4) = z[b * RP + r];
+                if (l < v.nl) F::st(reinterpret_cast<float4 *>(o + l * v.s4), z[b * RP + r]);
             }
-            // lag M of grids that keep it (Q = 2N = 2M): no pair of points is that far apart
-            if (b == 0 && u == 0 && v.nl > M) *reinterpret_cast<float2 *>(o + M * v.s4) = make_float2(0.f, 0.f);
         }
+        // lag M of grids that keep it (Q = 2N = 2M): no pair of points is that far apart
+        if (u == 0 && v.nl > M) *reinterpret_cast<float4 *>(o + M * v.s4) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
 
-// Grid: nl x (column tiles), the tiles of one s_x neighbours.  VEC: both
-// transfers of a column in one 8-byte store (n_omega even, out 8-byte aligned).
+// Grid: nl x (column tiles), the tiles of one s_x neighbours.  VEC: the four
+// transfers of a pack in one 16-byte store (n_omega % 4 == 0, out aligned).
 template <int M, bool VEC>
 __global__ void __launch_bounds__(EvCfg<M>::T, EvCfg<M>::MINB)
 k_ev_inv_y(EvGeom v, int Q, int n_omega, const float *__restrict__ B4, float *__restrict__ out,
@@ -60,20 +59,20 @@ k_ev_inv_y(EvGeom v, int Q, int n_omega, const float *__restrict__ B4, float *__
     using F = EvFft<M, true>;
     constexpr int C = F::C, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP, RF = F::RF;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    LH_REQUIRE_SMEM(F::SMEM_ELEMS, float2)
-    float2 *sm = reinterpret_cast<float2 *>(smem_raw);
+    LH_REQUIRE_SMEM(F::SMEM_ELEMS, float4)
+    float4 *sm = reinterpret_cast<float4 *>(smem_raw);
     const int sx = blockIdx.x / ntile, ct = blockIdx.x % ntile;
     const int col = threadIdx.x % C, u = threadIdx.x / C;
-    const int m = 2 * (ct * C + col);
+    const int m = 4 * (ct * C + col);
     const bool on = m < v.WS;
     const float *in = B4 + (long long)sx * v.s4 + m;
-    float2 z[VPT];
+    Cx2 z[VPT];
 #pragma unroll
     for (int b = 0; b < VPT / RF; ++b)
 #pragma unroll
-        for (int r = 0; r < RF; ++r)
-            z[b * RF + r] = on ? __ldcs(reinterpret_cast<const float2 *>(in + (long long)(u + b * TPC + r * (M / RF)) * v.WS))
-                               : make_float2(0.f, 0.f);
+        for (int r = 0; r < RF; ++r) {
+            z[b * RF + r] = on ? ev_load(in + (u + b * TPC + r * (M / RF)) * v.WS) : Cx2{dup2(0.f), dup2(0.f)};
+        }
     F::run(z, sm + col, u, tab);
     ev_post<M>(z, u, tab);
     if (m >= n_omega) return;
@@ -81,15 +80,17 @@ k_ev_inv_y(EvGeom v, int Q, int n_omega, const float *__restrict__ B4, float *__
     const bool two_x = sx > 0 && sx < Q / 2;
     float *ox = out + (long long)(Q / 2 - sx) * Q * n_omega + m;
     const long long mx = 2LL * sx * Q * n_omega;
-    auto put = [&](float *o, float2 c) {
+    auto put = [&](float *o, float4 c) {
         if constexpr (VEC) {
-            *reinterpret_cast<float2 *>(o) = c;
+            *reinterpret_cast<float4 *>(o) = c;
         } else {
             o[0] = c.x;
             if (m + 1 < n_omega) o[1] = c.y;
+            if (m + 2 < n_omega) o[2] = c.z;
+            if (m + 3 < n_omega) o[3] = c.w;
         }
     };
-    auto put_lag = [&](int sy, float2 c) {
+    auto put_lag = [&](int sy, float4 c) {
         if (sy > Q / 2) return;
         float *o = ox + (long long)(Q / 2 - sy) * n_omega;
         put(o, c);
@@ -100,36 +101,39 @@ k_ev_inv_y(EvGeom v, int Q, int n_omega, const float *__restrict__ B4, float *__
             if (two_x) put(o + mx, c);
         }
     };
+    const float2 sc = dup2(v.scale);
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
         const int j = F::template butterfly<F::NS - 1>(b, u);
 #pragma unroll
-        for (int r = 0; r < RP; ++r)
-            put_lag(j + r * NBP, make_float2(v.scale * z[b * RP + r].x, v.scale * z[b * RP + r].y));
+        for (int r = 0; r < RP; ++r) {
+            const float2 a = mul2(z[b * RP + r].re, sc), c = mul2(z[b * RP + r].im, sc);
+            put_lag(j + r * NBP, make_float4(a.x, a.y, c.x, c.y));
+        }
     }
-    if (u == 0 && v.nl > M) put_lag(M, make_float2(0.f, 0.f));
+    if (u == 0 && v.nl > M) put_lag(M, make_float4(0.f, 0.f, 0.f, 0.f));
 }
 
 template <int M>
 cudaError_t launch_ev_inv_x_t(const EvGeom &v, const Work<float> &w, cudaStream_t s)
 {
-    const size_t smem = sizeof(float2) * EvFft<M, true>::SMEM_ELEMS;
+    const size_t smem = sizeof(float4) * EvFft<M, true>::SMEM_ELEMS;
     static const cudaError_t e = smem_attrs(k_ev_inv_x<M>, smem);
     if (e != cudaSuccess) return e;
-    const int ntile = (v.WS + 2 * EvCfg<M>::C - 1) / (2 * EvCfg<M>::C);
+    const int ntile = (v.WS + 4 * EvCfg<M>::C - 1) / (4 * EvCfg<M>::C);
     k_ev_inv_x<M><<<M * ntile, EvCfg<M>::T, smem, s>>>(v, (const float *)w.X, (float *)w.Y, (const float2 *)w.evt, ntile);
     return cudaGetLastError();
 }
 template <int M>
 cudaError_t launch_ev_inv_y_t(const Geom &g, const EvGeom &v, const Work<float> &w, float *out, cudaStream_t s)
 {
-    const size_t smem = sizeof(float2) * EvFft<M, true>::SMEM_ELEMS;
+    const size_t smem = sizeof(float4) * EvFft<M, true>::SMEM_ELEMS;
     static const cudaError_t e0 = smem_attrs(k_ev_inv_y<M, true>, smem);
     static const cudaError_t e1 = smem_attrs(k_ev_inv_y<M, false>, smem);
     if (e0 != cudaSuccess) return e0;
     if (e1 != cudaSuccess) return e1;
-    const int ntile = (v.WS + 2 * EvCfg<M>::C - 1) / (2 * EvCfg<M>::C);
-    auto k = g.n_omega % 2 == 0 && reinterpret_cast<uintptr_t>(out) % 8 == 0 ? k_ev_inv_y<M, true> : k_ev_inv_y<M, false>;
+    const int ntile = (v.WS + 4 * EvCfg<M>::C - 1) / (4 * EvCfg<M>::C);
+    auto k = g.n_omega % 4 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0 ? k_ev_inv_y<M, true> : k_ev_inv_y<M, false>;
     k<<<v.nl * ntile, EvCfg<M>::T, smem, s>>>(v, g.Q, g.n_omega, (const float *)w.Y, out, (const float2 *)w.evt, ntile);
     return cudaGetLastError();
 }

@@ -4,14 +4,15 @@
 // Appendix A: the split at e = 0, or at temperature kT the Fermi weights of
 // Eq. A1), by FFT along the energy axis.
 //
-// One warp per pair of lines (the schedules and exchanges of et_tiles.cuh):
-// each line's z = a + i b is transformed, a^ and b^ are separated and
-// conj(a^) b^ formed in registers, then the two lines' products share one
-// inverse transform (W = P1 + i P2).  The forward's last stage and the
-// inverse's first own the same frequencies in the same threads, so nothing
-// between the transforms leaves the registers.  1.5 transforms a line.
-#include "et_tiles.cuh"
+// A pair of lines per TPL lanes: each line's z = a + i b is transformed, a^ and
+// b^ are separated and conj(a^) b^ formed in registers, then the two lines'
+// products share one inverse transform (W = P1 + i P2).  The forward's last
+// stage and the inverse's first own the same frequencies in the same threads,
+// so nothing between the transforms leaves the registers.  1.5 transforms a
+// line, of two stages and one exchange each (even_line.cuh).
 #include "even.cuh"
+#include "even_line.cuh"
+#include "et_tiles.cuh"
 
 namespace lh {
 
@@ -31,11 +32,119 @@ __device__ __forceinline__ void ev_tri(int t, int M, int &kx, int &ky)
     }
 }
 
+
+// FULL: ne == L with the split at L/2.  THERMAL: Fermi weights (odd: the odd
+// part, Im chi_T).  HALF: WS <= L/2, the upper half of the lags is not formed.
+template <int L, bool FULL, bool THERMAL, bool HALF>
+__global__ void __launch_bounds__(32 * EVC_WARPS, EvLine<L>::MINB)
+k_ev_corr(Geom g, EvGeom v, Band band, const float *__restrict__ B2, float *__restrict__ B3,
+          const float2 *__restrict__ tab, int iters, int odd)
+{
+    using E = EvLine<L>;
+    constexpr int VPT = E::VPT, TPL = E::TPL, R0 = E::R0, R1 = E::R1;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    LH_REQUIRE_SMEM(EVC_WARPS * E::WARP_ELEMS + (THERMAL ? L : 0), float2)
+    const int lane = (int)threadIdx.x % 32, warp = (int)threadIdx.x / 32;
+    const int sl = lane / TPL, u = lane % TPL;
+    float2 *sm = reinterpret_cast<float2 *>(smem_raw) + warp * E::WARP_ELEMS + sl * E::LP;
+    float2 *wf = reinterpret_cast<float2 *>(smem_raw) + EVC_WARPS * E::WARP_ELEMS;
+    if constexpr (THERMAL) {
+        et_fermi_weights<L>(g, band, wf, (int)threadIdx.x, 32 * EVC_WARPS);
+        __syncthreads();
+    }
+    const int npairs = v.M / 2 * (v.M + 1) / 2;
+    const bool u0 = u == 0;
+
+    for (int it = 0; it < iters; ++it) {
+        const int f = ((blockIdx.x * EVC_WARPS + warp) * iters + it) * E::LPI + sl;
+        const bool live = f < npairs;
+        float2 pa[2][R1 / 2], pb[2][R1 / 2], ph[2], x[VPT];
+#pragma unroll
+        for (int r = 0; r < R1 / 2; ++r) pa[1][r] = pb[1][r] = make_float2(0.f, 0.f);
+        ph[1] = make_float2(0.f, 0.f);
+        float raw[VPT];
+        int kx, ky;
+        ev_tri(live ? 2 * f : 0, v.M, kx, ky);
+        auto load = [&] {
+            const float *p = B2 + (kx * v.s2 + (long long)ky * v.ES + u);
+#pragma unroll
+            for (int i = 0; i < VPT; ++i)
+                raw[i] = live && (FULL || u + E::first(i) < v.ne) ? __ldcs(p + E::first(i)) : 0.f;
+        };
+        load();
+        // one copy of the forward code for both lines (the body unrolled twice
+        // spent a tenth of its time waiting for instructions)
+#pragma unroll 1
+        for (int q = 0; q < 2; ++q) {
+#pragma unroll
+            for (int r = 0; r < R1 / 2; ++r) {
+                pa[0][r] = pa[1][r];
+                pb[0][r] = pb[1][r];
+            }
+            ph[0] = ph[1];
+            E::template first_stage<FULL, THERMAL>(x, raw, u, v.J0, wf);
+            if (q == 0) {   // the second line's values travel during the first one's transform
+                ev_tri(live ? 2 * f + 1 : 0, v.M, kx, ky);
+                load();
+            }
+            E::forward_rest(x, sm, u, tab);
+            // conj(a^) b^ with a^ = Z(k) + conj Z(-k), b^ = (Z(k) - conj Z(-k)) / i
+            // (halved in the input), k <= L/2
+            auto prod = [&](float2 zk, float2 zm) {
+                const float2 p = cmulc(make_float2(zk.y + zm.y, zm.x - zk.x), make_float2(zk.x + zm.x, zk.y - zm.y));
+                return THERMAL ? odd_part(p, odd != 0) : p;
+            };
+#pragma unroll
+            for (int r = 0; r < R1 / 2; ++r) {
+                pa[1][r] = prod(x[r], u0 ? x[(R1 - r) % R1] : x[R1 + R1 - 1 - r]);
+                pb[1][r] = prod(x[R1 + r], u0 ? x[R1 + R1 - 1 - r] : x[R1 - 1 - r]);
+            }
+            ph[1] = prod(x[R1 / 2], x[R1 / 2]);   // k = L/2, used where u = 0
+        }
+        // W(k) = P1 + i P2 and W(L - k) = conj P1 + i conj P2 in the inverse's
+        // first-stage order (rows j2[b] + r R0)
+        auto w_of = [](float2 x1, float2 x2) { return make_float2(x1.x - x2.y, x1.y + x2.x); };
+        auto w_conj = [](float2 x1, float2 x2) { return make_float2(x1.x + x2.y, x2.x - x1.y); };
+#pragma unroll
+        for (int r = 0; r < R1 / 2; ++r) {
+            x[r] = w_of(pa[0][r], pa[1][r]);
+            x[R1 + r] = w_of(pb[0][r], pb[1][r]);
+            x[R1 + R1 - 1 - r] = u0 ? w_conj(pb[0][r], pb[1][r]) : w_conj(pa[0][r], pa[1][r]);
+        }
+        // u > 0: row R1 - 1 - r mirrors pb[r]; u = 0: row R1 - r mirrors pa[r], row R1/2 is k = L/2
+#pragma unroll
+        for (int r = R1 / 2; r < R1; ++r) {
+            const float2 hi = w_conj(pb[0][R1 - 1 - r], pb[1][R1 - 1 - r]);
+            const float2 lo = r == R1 / 2 ? w_of(ph[0], ph[1]) : w_conj(pa[0][(R1 - r) % (R1 / 2)], pa[1][(R1 - r) % (R1 / 2)]);
+            x[r] = u0 ? lo : hi;
+        }
+        E::template inverse<HALF>(x, sm, u, tab);
+        if (live) {
+            long long ob[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                ev_tri(2 * f + q, v.M, kx, ky);
+                ob[q] = kx * v.s3 + (long long)ky * v.WS + u;
+            }
+#pragma unroll
+            for (int i = 0; i < VPT; ++i) {
+                const int m = E::last(i);
+                if ((!HALF || i % R0 < R0 / 2) && u + m < v.WS) {   // the row's padding too: finite values (WS <= L)
+                    B3[ob[0] + m] = x[i].x;
+                    B3[ob[1] + m] = x[i].y;
+                }
+            }
+        }
+    }
+}
+
+// The same at 768 energies, which has no two-stage schedule at these register
+// counts: three stages on the schedules and tables of et_tiles.cuh.
 // FULL: ne == L with the split at L/2.  THERMAL: Fermi weights; ODD: the odd
 // part (Im chi_T).
 template <int L, bool FULL, bool THERMAL>
 __global__ void __launch_bounds__(32 * EVC_WARPS)
-k_ev_corr(Geom g, EvGeom v, Band band, const float *__restrict__ B2, float *__restrict__ B3,
+k_ev_corr3(Geom g, EvGeom v, Band band, const float *__restrict__ B2, float *__restrict__ B3,
           const float2 *__restrict__ etw, int iters, int odd)
 {
     using G = EtGeo<L>;
@@ -213,30 +322,53 @@ k_ev_corr(Geom g, EvGeom v, Band band, const float *__restrict__ B2, float *__re
     }
 }
 
-template <int L, bool FULL, bool THERMAL>
+
+static int ev_corr_iters(int npairs, int lpi, int sms)
+{
+    // pairs per warp: up to 8 rounds while every SM still gets 48 warps' worth
+    const int rounds = (npairs + lpi - 1) / lpi, it = rounds / (sms * 48);
+    return it < 1 ? 1 : it > 8 ? 8 : it;
+}
+template <int L, bool FULL, bool THERMAL, bool HALF>
 cudaError_t launch_ev_corr_t(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, int sms,
                              cudaStream_t s)
 {
-    constexpr int LPI = EtGeo<L>::LPI;
-    const size_t smem = sizeof(float2) * (EVC_WARPS * LPI * EtGeo<L>::LP + (THERMAL ? L : 0));
-    static const cudaError_t e = smem_attrs(k_ev_corr<L, FULL, THERMAL>, smem);
+    using E = EvLine<L>;
+    const size_t smem = sizeof(float2) * (EVC_WARPS * E::WARP_ELEMS + (THERMAL ? L : 0));
+    static const cudaError_t e = smem_attrs(k_ev_corr<L, FULL, THERMAL, HALF>, smem);
     if (e != cudaSuccess) return e;
-    const int npairs = v.M / 2 * (v.M + 1) / 2;
-    // pairs per warp: up to 8 rounds while every SM still gets 48 warps' worth
-    const int rounds = (npairs + LPI - 1) / LPI;
-    const int iters = rounds / (sms * 48) < 1 ? 1 : rounds / (sms * 48) > 8 ? 8 : rounds / (sms * 48);
-    const int per = EVC_WARPS * iters;
-    k_ev_corr<L, FULL, THERMAL><<<(rounds + per - 1) / per, 32 * EVC_WARPS, smem, s>>>(
-        g, v, band, (const float *)w.Y, (float *)w.X, (const float2 *)w.etw, iters, g.quantity == LINDHARD_IMCHI_T);
+    const int npairs = v.M / 2 * (v.M + 1) / 2, iters = ev_corr_iters(npairs, E::LPI, sms);
+    const int per = EVC_WARPS * iters * E::LPI;
+    k_ev_corr<L, FULL, THERMAL, HALF><<<(npairs + per - 1) / per, 32 * EVC_WARPS, smem, s>>>(
+        g, v, band, (const float *)w.Y, (float *)w.X, (const float2 *)w.evt + ev_line_table<L>(), iters,
+        g.quantity == LINDHARD_IMCHI_T);
     return cudaGetLastError();
 }
 template <int L>
 cudaError_t launch_ev_corr_l(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, int sms,
                              cudaStream_t s)
 {
-    if (g.quantity != LINDHARD_IMCHI) return launch_ev_corr_t<L, false, true>(g, v, band, w, sms, s);
-    if (v.ne == L && v.J0 == L / 2) return launch_ev_corr_t<L, true, false>(g, v, band, w, sms, s);
-    return launch_ev_corr_t<L, false, false>(g, v, band, w, sms, s);
+    const bool half = v.WS <= L / 2;
+    if (g.quantity != LINDHARD_IMCHI)
+        return half ? launch_ev_corr_t<L, false, true, true>(g, v, band, w, sms, s)
+                    : launch_ev_corr_t<L, false, true, false>(g, v, band, w, sms, s);
+    if (v.ne == L && v.J0 == L / 2 && half) return launch_ev_corr_t<L, true, false, true>(g, v, band, w, sms, s);
+    return half ? launch_ev_corr_t<L, false, false, true>(g, v, band, w, sms, s)
+                : launch_ev_corr_t<L, false, false, false>(g, v, band, w, sms, s);
+}
+template <bool THERMAL>
+cudaError_t launch_ev_corr3(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, int sms,
+                            cudaStream_t s)
+{
+    constexpr int L = 768, LPI = EtGeo<L>::LPI;
+    const size_t smem = sizeof(float2) * (EVC_WARPS * LPI * EtGeo<L>::LP + (THERMAL ? L : 0));
+    static const cudaError_t e = smem_attrs(k_ev_corr3<L, false, THERMAL>, smem);
+    if (e != cudaSuccess) return e;
+    const int npairs = v.M / 2 * (v.M + 1) / 2, iters = ev_corr_iters(npairs, LPI, sms);
+    const int per = EVC_WARPS * iters * LPI;
+    k_ev_corr3<L, false, THERMAL><<<(npairs + per - 1) / per, 32 * EVC_WARPS, smem, s>>>(
+        g, v, band, (const float *)w.Y, (float *)w.X, (const float2 *)w.etw, iters, g.quantity == LINDHARD_IMCHI_T);
+    return cudaGetLastError();
 }
 cudaError_t launch_ev_corr(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, int sms,
                            cudaStream_t s)
@@ -246,7 +378,9 @@ cudaError_t launch_ev_corr(const Geom &g, const EvGeom &v, const Band &band, con
     case 256: return launch_ev_corr_l<256>(g, v, band, w, sms, s);
     case 384: return launch_ev_corr_l<384>(g, v, band, w, sms, s);
     case 512: return launch_ev_corr_l<512>(g, v, band, w, sms, s);
-    case 768: return launch_ev_corr_l<768>(g, v, band, w, sms, s);
+    case 768:
+        return g.quantity != LINDHARD_IMCHI ? launch_ev_corr3<true>(g, v, band, w, sms, s)
+                                            : launch_ev_corr3<false>(g, v, band, w, sms, s);
     default: return cudaErrorInvalidValue;
     }
 }

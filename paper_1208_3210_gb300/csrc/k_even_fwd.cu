@@ -8,6 +8,7 @@
 //                k_x <= k_y is written (A is symmetric under p_x <-> p_y and
 //                both axes list their frequencies in the same order)
 #include "even.cuh"
+#include "even_line.cuh"
 
 namespace lh {
 
@@ -23,7 +24,7 @@ __device__ __forceinline__ float ev_rcp(float x)
 // One block per table and slice: the tables' places and periods come as an
 // argument (evaluating ev_table_offset per entry on the device took 0.5 ms).
 struct EvTabs {
-    struct { int off, count, row, period; } t[64];   // row 0: the w_j, j < period
+    struct { int off, count, row, period; } t[68];   // row 0: the w_j, j < period; row -1: even_line.cuh
 };
 __global__ void k_ev_tables(float2 *out, EvTabs tabs)
 {
@@ -32,7 +33,8 @@ __global__ void k_ev_tables(float2 *out, EvTabs tabs)
     for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < count; i += gridDim.y * blockDim.x) {
         double s, c;
         if (row == 0) sincospi(0.5 * (double)i / (double)period, &s, &c);
-        else sincospi(-2.0 * (double)((i / row) * (i % row + 1)) / (double)period, &s, &c);
+        else if (row > 0) sincospi(-2.0 * (double)((i / row) * (i % row + 1)) / (double)period, &s, &c);
+        else sincospi(-2.0 * (double)((i % 64 / 2) * (i / 64 * 2 + i % 2 + 1)) / (double)period, &s, &c);
         out[off + i] = make_float2((float)c, (float)s);
     }
 }
@@ -51,10 +53,11 @@ cudaError_t launch_ev_tables(float2 *out, cudaStream_t s)
                 o += Ns * ev_row(R);
             }
     }
+    for (int i = 0; ev_line_len(i) != 0; ++i) tabs.t[n++] = {(o + 1) / 2 * 2 + 128 * i, 128, -1, ev_line_len(i)};
     k_ev_tables<<<dim3(n, 4), 128, 0, s>>>(out, tabs);
     return cudaGetLastError();
 }
-size_t ev_table_bytes() { return (size_t)ev_table_entries() * sizeof(float2); }
+size_t ev_table_bytes() { return (size_t)ev_all_tables() * sizeof(float2); }
 
 // Grid: Nh x (column tiles), the tiles of one p_x neighbours.
 template <int M>

@@ -434,8 +434,8 @@ __device__ __forceinline__ Cx2 ev_load(const float *p)
 // The pairs (n, M - n) of a thread's two paired butterflies (rows j + r NBP in
 // v[b RP + r]): f(row n, value at n, value at M - n) for every pair, with
 // M - 0 taken as row 0 itself.
-template <int RP, int NBP, int TPC, typename F>
-__device__ __forceinline__ void ev_pairs(Cx2 *v, int u, F &&f)
+template <int RP, int NBP, int TPC, typename V, typename F>
+__device__ __forceinline__ void ev_pairs(V *v, int u, F &&f)
 {
     if (u != 0) {
 #pragma unroll

@@ -80,6 +80,30 @@ __host__ __device__ constexpr int ev_line_table()
 }
 __host__ __device__ constexpr int ev_all_tables() { return (ev_table_entries() + 1) / 2 * 2 + 4 * 128; }
 
+constexpr int EVC_WARPS = 4;
+
+// Line t of the triangle k_x <= k_y, rows k_x and M - 1 - k_x folded to M + 1
+// entries: t = f (M + 1) + c.
+__device__ __forceinline__ void ev_tri(int t, int M, int &kx, int &ky)
+{
+    const int f = t / (M + 1), c = t - f * (M + 1);
+    if (c < M - f) {
+        kx = f;
+        ky = f + c;
+    } else {
+        kx = M - 1 - f;
+        ky = c - 1;   // kx + (c - (M - f))
+    }
+}
+
+
+// Rounds per warp: up to 8 while every SM still gets 48 warps' worth.
+inline int ev_corr_iters(int npairs, int lpi, int sms)
+{
+    const int rounds = (npairs + lpi - 1) / lpi, it = rounds / (sms * 48);
+    return it < 1 ? 1 : it > 8 ? 8 : it;
+}
+
 template <int L>
 struct EvLine {
     static constexpr int R0 = L == 512 ? 32 : 16, R1 = L / R0, VPT = 2 * R1, TPL = L / VPT, LPI = 32 / TPL;

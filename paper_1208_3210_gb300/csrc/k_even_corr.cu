@@ -16,23 +16,6 @@
 
 namespace lh {
 
-constexpr int EVC_WARPS = 4;
-
-// Line t of the triangle k_x <= k_y, rows k_x and M - 1 - k_x folded to M + 1
-// entries: t = f (M + 1) + c.
-__device__ __forceinline__ void ev_tri(int t, int M, int &kx, int &ky)
-{
-    const int f = t / (M + 1), c = t - f * (M + 1);
-    if (c < M - f) {
-        kx = f;
-        ky = f + c;
-    } else {
-        kx = M - 1 - f;
-        ky = c - 1;   // kx + (c - (M - f))
-    }
-}
-
-
 // FULL: ne == L with the split at L/2.  THERMAL: Fermi weights (odd: the odd
 // part, Im chi_T).  HALF: WS <= L/2, the upper half of the lags is not formed.
 template <int L, bool FULL, bool THERMAL, bool HALF>
@@ -323,12 +306,6 @@ k_ev_corr3(Geom g, EvGeom v, Band band, const float *__restrict__ B2, float *__r
 }
 
 
-static int ev_corr_iters(int npairs, int lpi, int sms)
-{
-    // pairs per warp: up to 8 rounds while every SM still gets 48 warps' worth
-    const int rounds = (npairs + lpi - 1) / lpi, it = rounds / (sms * 48);
-    return it < 1 ? 1 : it > 8 ? 8 : it;
-}
 template <int L, bool FULL, bool THERMAL, bool HALF>
 cudaError_t launch_ev_corr_t(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, int sms,
                              cudaStream_t s)

@@ -6,7 +6,8 @@
 //                tile of energies, transformed along p_y
 //   k_ev_x     : B2 [M][M][ES]: B1 transformed along p_x for each k_y; only
 //                k_x <= k_y is written (A is symmetric under p_x <-> p_y and
-//                both axes list their frequencies in the same order)
+//                both axes list their frequencies in the same order).  The
+//                adjoint's weights take it too (k_even_bw.cu), with every k_x.
 #include "even.cuh"
 #include "even_line.cuh"
 
@@ -130,10 +131,12 @@ k_ev_gen_y(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const 
     }
 }
 
-// Grid: M x (column tiles), the tiles of one k_y neighbours.
-template <int M>
+// Grid: M x (column tiles), the tiles of one k_y neighbours.  Rows [0, rows) of
+// planes of RS-float rows, sp floats apart in B1 and dp in B2.  TRI: k_x <= k_y.
+template <int M, bool TRI>
 __global__ void __launch_bounds__(EvCfg<M>::T, EvCfg<M>::MINB)
-k_ev_x(EvGeom v, const float *__restrict__ B1, float *__restrict__ B2, const float2 *__restrict__ tab, int ntile)
+k_ev_x(int rows, int RS, long long sp, long long dp, const float *__restrict__ B1, float *__restrict__ B2,
+       const float2 *__restrict__ tab, int ntile)
 {
     using F = EvFft<M, false>;
     constexpr int C = F::C, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP;
@@ -143,8 +146,8 @@ k_ev_x(EvGeom v, const float *__restrict__ B1, float *__restrict__ B2, const flo
     const int ky = blockIdx.x / ntile, ct = blockIdx.x % ntile;
     const int col = threadIdx.x % C, u = threadIdx.x / C;
     const int e = 4 * (ct * C + col);
-    const bool on = e < v.ES;
-    const float *in = B1 + (long long)ky * v.ES + e;
+    const bool on = e < RS;
+    const float *in = B1 + (long long)ky * RS + e;
     Cx2 z[VPT];
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
@@ -152,20 +155,20 @@ k_ev_x(EvGeom v, const float *__restrict__ B1, float *__restrict__ B2, const flo
 #pragma unroll
         for (int r = 0; r < RP; ++r) {
             const int n = j + r * NBP;
-            z[b * RP + r] = on && n < v.Nh ? ev_load(in + n * v.s1) : Cx2{dup2(0.f), dup2(0.f)};
+            z[b * RP + r] = on && n < rows ? ev_load(in + n * sp) : Cx2{dup2(0.f), dup2(0.f)};
         }
     }
     ev_pre<M>(z, u, tab);
     F::run(z, sm + col, u, tab);
     if (on) {
-        float *o = B2 + (long long)ky * v.ES + e;
+        float *o = B2 + (long long)ky * RS + e;
         constexpr int RL = ev_radix(M, F::NS - 1, false);
 #pragma unroll
         for (int b = 0; b < VPT / RL; ++b)
 #pragma unroll
             for (int r = 0; r < RL; ++r) {
                 const int kx = u + b * TPC + r * (M / RL);
-                if (kx <= ky) F::st(reinterpret_cast<float4 *>(o + kx * v.s2), z[b * RL + r]);
+                if (!TRI || kx <= ky) F::st(reinterpret_cast<float4 *>(o + kx * dp), z[b * RL + r]);
             }
     }
 }
@@ -181,14 +184,15 @@ cudaError_t launch_ev_gen_y_t(const Geom &g, const EvGeom &v, const Band &band, 
                                                           (float *)w.X, (const float2 *)w.evt, ntile);
     return cudaGetLastError();
 }
-template <int M>
-cudaError_t launch_ev_x_t(const EvGeom &v, const Work<float> &w, cudaStream_t s)
+template <int M, bool TRI>
+cudaError_t launch_ev_x_t(int rows, int RS, long long sp, long long dp, const float *src, float *dst,
+                          const Work<float> &w, cudaStream_t s)
 {
     const size_t smem = sizeof(float4) * EvFft<M, false>::SMEM_ELEMS;
-    static const cudaError_t e = smem_attrs(k_ev_x<M>, smem);
+    static const cudaError_t e = smem_attrs(k_ev_x<M, TRI>, smem);
     if (e != cudaSuccess) return e;
-    const int ntile = (v.ES + 4 * EvCfg<M>::C - 1) / (4 * EvCfg<M>::C);
-    k_ev_x<M><<<M * ntile, EvCfg<M>::T, smem, s>>>(v, (const float *)w.X, (float *)w.Y, (const float2 *)w.evt, ntile);
+    const int ntile = (RS + 4 * EvCfg<M>::C - 1) / (4 * EvCfg<M>::C);
+    k_ev_x<M, TRI><<<M * ntile, EvCfg<M>::T, smem, s>>>(rows, RS, sp, dp, src, dst, (const float2 *)w.evt, ntile);
     return cudaGetLastError();
 }
 cudaError_t launch_ev_gen_y(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, cudaStream_t s)
@@ -199,7 +203,13 @@ cudaError_t launch_ev_gen_y(const Geom &g, const EvGeom &v, const Band &band, co
 }
 cudaError_t launch_ev_x(const EvGeom &v, const Work<float> &w, cudaStream_t s)
 {
-#define CALL(M_) launch_ev_x_t<M_>(v, w, s)
+#define CALL(M_) launch_ev_x_t<M_, true>(v.Nh, v.ES, v.s1, v.s2, (const float *)w.X, (float *)w.Y, w, s)
+    LH_EV_SWITCH(v.M, CALL)
+#undef CALL
+}
+cudaError_t launch_ev_x_all(const EvGeom &v, const Work<float> &w, const float *src, float *dst, cudaStream_t s)
+{
+#define CALL(M_) launch_ev_x_t<M_, false>(v.nl < v.M ? v.nl : v.M, v.WS, v.s4, v.s3, src, dst, w, s)
     LH_EV_SWITCH(v.M, CALL)
 #undef CALL
 }

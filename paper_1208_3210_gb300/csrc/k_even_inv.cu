@@ -2,17 +2,20 @@
 // C(k_x, k_y, w_m) back to the lags (Sec. 3's inverse transform).
 //
 //   k_ev_inv_x : B3 [M][M][WS] (k_x <= k_y, symmetric) -> B4 [nl][M][WS],
-//                lags s_x >= 0 for each k_y
+//                lags s_x >= 0 for each k_y (and the adjoint's spectra to
+//                p_x >= 0)
 //   k_ev_inv_y : B4 -> Im chi at the four lags (+-s_x, +-s_y), times the Eq. 9
 //                prefactor, out [Q][Q][n_omega]
 #include "even.cuh"
 
 namespace lh {
 
-// Grid: M x (column tiles), the tiles of one k_y neighbours.
+// Grid: M x (column tiles), the tiles of one k_y neighbours.  `rows` outputs;
+// planes of RS-float rows, sp floats apart in B3 and dp in B4.
 template <int M>
 __global__ void __launch_bounds__(EvCfg<M>::T, EvCfg<M>::MINB)
-k_ev_inv_x(EvGeom v, const float *__restrict__ B3, float *__restrict__ B4, const float2 *__restrict__ tab, int ntile)
+k_ev_inv_x(int rows, int RS, long long sp, long long dp, const float *__restrict__ B3, float *__restrict__ B4,
+           const float2 *__restrict__ tab, int ntile)
 {
     using F = EvFft<M, true>;
     constexpr int C = F::C, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP, RF = F::RF;
@@ -22,30 +25,30 @@ k_ev_inv_x(EvGeom v, const float *__restrict__ B3, float *__restrict__ B4, const
     const int ky = blockIdx.x / ntile, ct = blockIdx.x % ntile;
     const int col = threadIdx.x % C, u = threadIdx.x / C;
     const int m = 4 * (ct * C + col);
-    const bool on = m < v.WS;
+    const bool on = m < RS;
     Cx2 z[VPT];
 #pragma unroll
     for (int b = 0; b < VPT / RF; ++b)
 #pragma unroll
         for (int r = 0; r < RF; ++r) {
             const int kx = u + b * TPC + r * (M / RF), lo = min(kx, ky), hi = max(kx, ky);
-            z[b * RF + r] = on ? ev_load(B3 + lo * v.s3 + hi * v.WS + m) : Cx2{dup2(0.f), dup2(0.f)};
+            z[b * RF + r] = on ? ev_load(B3 + lo * sp + hi * RS + m) : Cx2{dup2(0.f), dup2(0.f)};
         }
     F::run(z, sm + col, u, tab);
     ev_post<M>(z, u, tab);
     if (on) {
-        float *o = B4 + (long long)ky * v.WS + m;
+        float *o = B4 + (long long)ky * RS + m;
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
             const int j = F::template butterfly<F::NS - 1>(b, u);
 #pragma unroll
             for (int r = 0; r < RP; ++r) {
                 const int l = j + r * NBP;
-                if (l < v.nl) F::st(reinterpret_cast<float4 *>(o + l * v.s4), z[b * RP + r]);
+                if (l < rows) F::st(reinterpret_cast<float4 *>(o + l * dp), z[b * RP + r]);
             }
         }
         // lag M of grids that keep it (Q = 2N = 2M): no pair of points is that far apart
-        if (u == 0 && v.nl > M) *reinterpret_cast<float4 *>(o + M * v.s4) = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (u == 0 && rows > M) *reinterpret_cast<float4 *>(o + M * dp) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
 
@@ -115,13 +118,14 @@ k_ev_inv_y(EvGeom v, int Q, int n_omega, const float *__restrict__ B4, float *__
 }
 
 template <int M>
-cudaError_t launch_ev_inv_x_t(const EvGeom &v, const Work<float> &w, cudaStream_t s)
+cudaError_t launch_ev_inv_x_t(int rows, int RS, long long sp, long long dp, const Work<float> &w, cudaStream_t s)
 {
     const size_t smem = sizeof(float4) * EvFft<M, true>::SMEM_ELEMS;
     static const cudaError_t e = smem_attrs(k_ev_inv_x<M>, smem);
     if (e != cudaSuccess) return e;
-    const int ntile = (v.WS + 4 * EvCfg<M>::C - 1) / (4 * EvCfg<M>::C);
-    k_ev_inv_x<M><<<M * ntile, EvCfg<M>::T, smem, s>>>(v, (const float *)w.X, (float *)w.Y, (const float2 *)w.evt, ntile);
+    const int ntile = (RS + 4 * EvCfg<M>::C - 1) / (4 * EvCfg<M>::C);
+    k_ev_inv_x<M><<<M * ntile, EvCfg<M>::T, smem, s>>>(rows, RS, sp, dp, (const float *)w.X, (float *)w.Y,
+                                                       (const float2 *)w.evt, ntile);
     return cudaGetLastError();
 }
 template <int M>
@@ -139,7 +143,14 @@ cudaError_t launch_ev_inv_y_t(const Geom &g, const EvGeom &v, const Work<float> 
 }
 cudaError_t launch_ev_inv_x(const EvGeom &v, const Work<float> &w, cudaStream_t s)
 {
-#define CALL(M_) launch_ev_inv_x_t<M_>(v, w, s)
+#define CALL(M_) launch_ev_inv_x_t<M_>(v.nl, v.WS, v.s3, v.s4, w, s)
+    LH_EV_SWITCH(v.M, CALL)
+#undef CALL
+}
+// The adjoint's: X [M][M][ES] (k_x <= k_y) -> Y [Nh][M][ES].
+cudaError_t launch_ev_inv_x_bw(const EvGeom &v, const Work<float> &w, cudaStream_t s)
+{
+#define CALL(M_) launch_ev_inv_x_t<M_>(v.Nh, v.ES, v.s2, v.s1, w, s)
     LH_EV_SWITCH(v.M, CALL)
 #undef CALL
 }

@@ -65,6 +65,15 @@ cudaError_t launch_ev_corr(const Geom &g, const EvGeom &v, const Band &band, con
                            cudaStream_t s);
 cudaError_t launch_ev_inv_x(const EvGeom &v, const Work<float> &w, cudaStream_t s);
 cudaError_t launch_ev_inv_y(const Geom &g, const EvGeom &v, const Work<float> &w, float *out, cudaStream_t s);
+bool ev_bw_applies(const EvGeom &v);
+int ev_chain_blocks(const EvGeom &v);
+cudaError_t launch_ev_w_y(const Geom &g, const EvGeom &v, const float *wts, const Work<float> &w, cudaStream_t s);
+cudaError_t launch_ev_x_all(const EvGeom &v, const Work<float> &w, const float *src, float *dst, cudaStream_t s);
+cudaError_t launch_ev_bw(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, const float *W2,
+                         int sms, cudaStream_t s);
+cudaError_t launch_ev_inv_x_bw(const EvGeom &v, const Work<float> &w, cudaStream_t s);
+cudaError_t launch_ev_chain(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, double *partial,
+                            cudaStream_t s);
 bool pr_fwd_applies(const Geom &g);
 bool pr_inv_applies(const Geom &g);
 bool et_inv_applies(const Geom &g);
@@ -564,6 +573,13 @@ extern "C" lindhard_status lindhard_plan_create(const lindhard_grid *grids, int 
         n.Z = p->backward ? (size_t)g.Q * (size_t)g.xs3 * cb : 0;
         // the last pass's per-CTA sums, then the first reduction level's
         n.partial = p->backward ? (size_t)(bw_energy_blocks(g) + bw_partial_extra_rows()) * 5 * sizeof(double) : 0;
+        if (p->backward && ev_bw_applies(p->even[i])) {
+            // the adjoint's even form: X also holds G [M][M][ES], Z the weights' spectra [M][M][WS]
+            const EvGeom &v = p->even[i];
+            n.X = std::max(n.X, sizeof(float) * (size_t)(v.M * v.s2));
+            n.Z = std::max(n.Z, sizeof(float) * (size_t)(v.M * v.s3));
+            n.partial = std::max(n.partial, (size_t)(ev_chain_blocks(v) + bw_partial_extra_rows()) * 5 * sizeof(double));
+        }
         n.axis = (size_t)g.N * sizeof(AxisTab);
         n.eps32 = (size_t)g.n_eps * sizeof(float2);
         n.eps64 = (size_t)g.n_eps * sizeof(double);
@@ -1093,6 +1109,21 @@ extern "C" lindhard_status lindhard_imchi_backward(lindhard_plan *p, const lindh
                              nullptr, p->mu_G, s);
             if (e == cudaSuccess)
                 e = launch_solve_mu(g, b, wk.axis, wk.state, wk.mu_acc, wk.barrier, wk.status, nullptr, p->mu_G, s);
+        }
+        if (const EvGeom &v = p->even[i]; A_in == nullptr && !dA && ev_bw_applies(v) && ev_band_applies(g, b)) {
+            // parameter gradient of a generated A: the even form (k_even_bw.cu)
+            if (e == cudaSuccess) e = launch_ev_gen_y(g, v, b, wk, s);
+            if (e == cudaSuccess) e = launch_ev_x(v, wk, s);                                         // Y = A^
+            if (e == cudaSuccess) e = launch_ev_w_y(g, v, w + o_off, wk, s);                          // X
+            if (e == cudaSuccess) e = launch_ev_x_all(v, wk, (const float *)X, (float *)Z, s);       // Z = W^
+            if (e == cudaSuccess) e = launch_ev_bw(g, v, b, wk, (const float *)Z, p->num_sms, s);     // X = G
+            if (e == cudaSuccess) e = launch_ev_inv_x_bw(v, wk, s);                                   // Y
+            if (e == cudaSuccess) e = launch_ev_chain(g, v, b, wk, partial, s);
+            if (e == cudaSuccess) e = launch_reduce_params(partial, ev_chain_blocks(v), dparams + 5 * i, s);
+            if (e != cudaSuccess) return cuda_fail(e, "backward launch");
+            a_off += (size_t)g.N * g.N * g.n_eps;
+            o_off += (size_t)g.Q * g.Q * g.n_omega;
+            continue;
         }
         if (e == cudaSuccess) e = launch_fwd_energy(g, b, wk, A_in ? A_in + a_off : nullptr, s);   // X = U1
         if (e == cudaSuccess) e = launch_fwd_y(g, wk, s, p->yvar_fwd[i]);                           // Y = U2

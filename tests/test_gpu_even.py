@@ -108,3 +108,47 @@ def test_unaligned_output(lh):
     plan.status()
     assert torch.equal(buf[1:], ref)
     plan.close()
+
+
+# Adjoint: the parameter gradient alone takes the even form, with dL/dA asked
+# for too the general one.  Both sum dL/dA dA/dtheta with dL/dA within 5e-7 of
+# its maximum (the measured error of either form on every cell), so each
+# component agrees within 1e-6 max|dL/dA| sum|dA/dtheta|.
+@pytest.mark.parametrize("zones,npz,n_eps,n_omega,q,quantity", [
+    (4, 4, 3, 2, 16, 0), (4, 10, 34, 17, 40, 0), (5, 24, 37, 30, 118, 0), (4, 32, 128, 64, 128, 0),
+    (4, 16, 201, 90, 128, 0), (6, 32, 20, 10, 2, 0), (4, 16, 300, 150, 64, 0), (4, 12, 512, 256, 48, 0),
+    (4, 20, 401, 33, 60, 0), (4, 12, 40, 25, 48, 1), (4, 12, 150, 75, 48, 2), (4, 12, 200, 150, 60, 1),
+    (4, 12, 300, 200, 48, 2)])
+def test_parameter_gradient(lh, zones, npz, n_eps, n_omega, q, quantity):
+    import torch
+    grid = wl.grid_params(zones, npz, n_eps, 2.0, n_omega=n_omega, q_extent=q, quantity=quantity)
+    band = wl.band_params(filling=1.1, gamma=0.1, ff_a=1.1, **({"kT": 0.06} if quantity else {}))
+    w = torch.from_numpy(wl.loss_weights(grid, seed=3)).cuda().reshape(-1) - 0.3
+    plan = lh.Plan([grid], backward=True)
+    dp = torch.zeros(5, dtype=torch.float64, device="cuda")
+    ref = torch.zeros(5, dtype=torch.float64, device="cuda")
+    dA = torch.empty(plan.a_elems(), device="cuda")
+    plan.backward(w, bands=[band], dparams=dp)
+    plan.backward(w, bands=[band], dA=dA, dparams=ref)
+    plan.status()
+    plan.close()
+    b = dict(band, mu=oracle.solve_mu(0, band["t"], band["tp"], band["tpp"], band["gamma"], npz, 1.1))
+    scale = float(dA.abs().max()) * np.abs(oracle.spectral_dtheta(b, grid)).reshape(5, -1).sum(1)
+    assert np.all(np.abs((dp - ref).cpu().numpy()) <= 1e-6 * scale), ((dp - ref).cpu().numpy() / scale)
+
+
+def test_parameter_gradient_free_electrons(lh):
+    import torch
+    grid = wl.grid_params(4, 16, 40, 2.0)
+    band = wl.band_params(kind=1, mu=0.7, filling=float("nan"), gamma=0.1, ff_a=1.0)
+    w = torch.from_numpy(wl.loss_weights(grid, seed=3)).cuda().reshape(-1)
+    plan = lh.Plan([grid], backward=True)
+    dp, ref = (torch.zeros(5, dtype=torch.float64, device="cuda") for _ in range(2))
+    dA = torch.empty(plan.a_elems(), device="cuda")
+    plan.backward(w, bands=[band], dparams=dp)
+    plan.backward(w, bands=[band], dA=dA, dparams=ref)
+    plan.status()
+    plan.close()
+    scale = float(dA.abs().max()) * np.abs(oracle.spectral_dtheta(band, grid)).reshape(5, -1).sum(1)
+    assert dp[:3].abs().max().item() == 0.0
+    assert np.all(np.abs((dp - ref).cpu().numpy())[3:] <= 1e-6 * scale[3:])

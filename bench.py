@@ -411,7 +411,7 @@ def kk_rpa_form(plan, out, steps, stream, peak, v0=0.05):
     nbytes = 16 * s.q_extent * s.q_extent * s.n_omega
     res = {"v0_ev": v0, "bytes_per_call": nbytes}
     outs = {}
-    for v, name in ((0, "tensor_core"), (1, "fp32_simt")):
+    for v, name in ((0, "fft"), (1, "fp32_sum")):
         try:
             plan.kk_rpa(out, v0=v0, variant=v)
         except Exception as exc:
@@ -431,7 +431,7 @@ def kk_rpa_form(plan, out, steps, stream, peak, v0=0.05):
         res[name] = {"ms": ms, "gbs": nbytes / (ms * 1e-3) / 1e9, "frac_of_hbm_peak": nbytes / (ms * 1e-3) / 1e9 / peak,
                      "calls": n}
     if 0 in outs and 1 in outs:
-        res["max_rel_diff_tc_vs_fp32"] = float((outs[0] - outs[1]).abs().max() / outs[1].abs().max().clamp_min(1e-30))
+        res["max_rel_diff_fft_vs_sum"] = float((outs[0] - outs[1]).abs().max() / outs[1].abs().max().clamp_min(1e-30))
     return res
 
 

@@ -355,9 +355,8 @@ lindhard_status lindhard_envelope_k0(lindhard_plan *plan, int index, const float
  * q = 0 chi_RPA is 0 (its limit), unless v0 = 0 (then chi_RPA = chi).
  * imchi: device, the instance's [Q][Q][n_omega] block as lindhard_imchi wrote
  * it.  re_out: device [Q][Q][n_omega].  rpa_out: device [Q][Q][n_omega][2]
- * (re, im; 8-byte aligned), or NULL.  variant 0: the far field |k - m| >= 8
- * on the tensor cores (BF16 hi/lo, three products, FP32 accumulation) and the
- * near band in FP32, n_omega <= 256; variant 1: FP32 SIMT throughout,
+ * (re, im; 8-byte aligned), or NULL.  variant 0: the sum as a discrete Hilbert
+ * transform by FP32 FFT, n_omega <= 256; variant 1: the sum itself in FP32,
  * n_omega <= 1536 (otherwise LINDHARD_EUNSUPPORTED).  Plans whose grid is
  * LINDHARD_FP64 are rejected (LINDHARD_EINVAL), and so are LINDHARD_SQW
  * grids (the relation reads Im chi; LINDHARD_IMCHI_T is accepted).  Enqueued

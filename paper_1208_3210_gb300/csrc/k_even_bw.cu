@@ -175,7 +175,7 @@ k_ev_bw(Geom g, EvGeom v, Band band, const float *__restrict__ B2, const float *
                 if (!self) zm = make_float2(gk.x + hk.y, hk.x - gk.y);    // conj g^ + i conj h^
             };
             ev_pairs<R1, R0, TPL>(x, u, turn);
-            E::template inverse<false>(x, sm, u, tab);
+            E::inverse(x, sm, u, tab);
             if (live) {
                 float *o = G3 + (kx * v.s2 + (long long)ky * v.ES + u);
 #pragma unroll

@@ -101,7 +101,7 @@ k_ev_corr(Geom g, EvGeom v, Band band, const float *__restrict__ B2, float *__re
             const float2 lo = r == R1 / 2 ? w_of(ph[0], ph[1]) : w_conj(pa[0][(R1 - r) % (R1 / 2)], pa[1][(R1 - r) % (R1 / 2)]);
             x[r] = u0 ? lo : hi;
         }
-        E::template inverse<HALF>(x, sm, u, tab);
+        E::inverse(x, sm, u, tab);
         if (live) {
             long long ob[2];
 #pragma unroll

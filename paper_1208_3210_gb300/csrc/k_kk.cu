@@ -11,42 +11,31 @@
 //   Re chi_m = sum_k W(m, k) Im chi_k,  W(m, k) = (4/pi) k / (k^2 - m^2)
 //              for k >= 1 with k - m odd, 0 otherwise.
 //
-// Split by parity, the even outputs take the odd inputs and the odd outputs
-// the even inputs: two products [lines x n_omega/2] . [n_omega/2 x n_omega/2]^T.
-//
-//   k_kk_tc   : the far field |k - m| >= 8 on the tensor cores (tcgen05,
-//               BF16 hi + lo operands, three products, FP32 accumulation in
-//               tensor memory, 128 lines per block), the near band
-//               |k - m| < 8 (the largest weights, where a BF16 split would
-//               cost most of the accuracy) in FP32 in the epilogue, then
-//               chi_RPA.  n_omega <= 256.
+//   k_kk_fft  : the sum as a Hilbert transform by FFT (below), two lines per
+//               8 or 16 lanes, then chi_RPA.  n_omega <= 256.
 //   k_kk_simt : the whole sum in FP32 SIMT (every weight from an FP32 table),
 //               then chi_RPA.  n_omega <= 1536.
 //
 // V_q = v0 / |q|^2 at q = ((l_x - Q/2) dp, (l_y - Q/2) dp); at q = 0 chi_RPA
 // takes its limit 0 (v0 = 0: chi_RPA = chi everywhere).  The weight tables
 // are built once per plan in FP64 (k_kk_tables).
+#include <algorithm>
+
+#include "even_line.cuh"
 #include "kernels.cuh"
-#include "tc.cuh"
-#include "tma.cuh"
 
 namespace lh {
 
-constexpr int KK_BAND = 8;        // |k - m| < KK_BAND: near band, FP32
-constexpr int KK_MAX_TC = 256;    // longest n_omega of the tensor-core form
+constexpr int KK_MAX_FFT = 256;   // longest n_omega of the FFT form
 constexpr int KK_MAX_SIMT = 1536;
 
-// padded half width of the tensor-core operands (a multiple of the MMA's K = 16)
-__host__ __device__ constexpr int kk_kp(int nw)
-{
-    return (nw + 1) / 2 <= 16 ? 16 : (nw + 1) / 2 <= 32 ? 32 : (nw + 1) / 2 <= 64 ? 64 : 128;
-}
-// Weight table of one n_omega: [tensor-core Be hi][Be lo][Bo hi][Bo lo] (BF16,
-// K-major operands of KP x KP, n_omega <= 256 only), [near band: n_omega x 8
-// FP32], [SIMT: ceil(n_omega / 2) x n_omega FP32].  Byte offsets:
-__host__ __device__ constexpr size_t kk_tc_bytes(int nw) { return nw <= KK_MAX_TC ? 8ull * kk_kp(nw) * kk_kp(nw) : 0; }
-__host__ __device__ constexpr size_t kk_band_off(int nw) { return kk_tc_bytes(nw); }
-__host__ __device__ constexpr size_t kk_simt_off(int nw) { return kk_band_off(nw) + 32ull * nw; }
+// Transform length of the FFT form: a multiple of 128 with n_omega <= M / 2
+// (the lengths of even_line.cuh).
+__host__ __device__ constexpr int kk_len(int nw) { return nw <= 64 ? 128 : nw <= 128 ? 256 : nw <= 192 ? 384 : 512; }
+// Weight table of one n_omega: [FFT, n_omega <= 256 only: M FP32, then M / 2
+// complex FP32, both in the order in which a lane of the transforms takes
+// them], [SIMT: ceil(n_omega / 2) x n_omega FP32].  Byte offsets:
+__host__ __device__ constexpr size_t kk_simt_off(int nw) { return nw <= KK_MAX_FFT ? 8ull * kk_len(nw) : 0; }
 size_t kk_table_bytes(int nw) { return kk_simt_off(nw) + 4ull * ((nw + 1) / 2) * nw; }
 
 __host__ __device__ inline double kk_weight(int m, int k, int nw)
@@ -55,32 +44,48 @@ __host__ __device__ inline double kk_weight(int m, int k, int nw)
     return 4.0 / 3.14159265358979323846 * (double)k / ((double)k * k - (double)m * m);
 }
 
+// Places in the table: H of frequency n = u + last(i) at [i / 4][u][i % 4], and
+// w_n = e^{i pi n / 2M} of transfer n = ra + r R0 (or rb + r R0), ra = u, at
+// [j / 2][u][j % 2], j = r (or R1 / 2 + r): lanes take 16 bytes side by side.
+__device__ inline int kk_slot(int M, int n)
+{
+    const int R0 = M == 512 ? 32 : 16, R1 = M / R0, TPL = R0 / 2;
+    const int r = n / R1, j = n % R1, u = j % TPL, i = j / TPL * R0 + r;
+    return (i / 4 * TPL + u) * 4 + i % 4;
+}
+__device__ inline int kk_wslot(int M, int n)
+{
+    const int R0 = M == 512 ? 32 : 16, R1 = M / R0, TPL = R0 / 2;
+    const int r = n / R0, c = n % R0, h = c >= TPL, u = h ? (c == TPL ? 0 : R0 - c) : c, j = h * (R1 / 2) + r;
+    return (j / 2 * TPL + u) * 2 + j % 2;
+}
+
+// Transform of the kernel of the FFT form at the n-th frequency as the
+// transforms list them (even.cuh: theta_k, k = 2n, then k = 2 (M - 1 - n) + 1),
+// one warp per frequency: H(theta) = (4/pi) sum_{j odd < 2 n_omega - 1}
+// sin(j theta) / j, with the sign (-1)^k and the 1 / 2M of the transforms.
 __global__ void k_kk_tables(int nw, unsigned char *tab)
 {
-    const int KP = kk_kp(nw), H = (nw + 1) / 2;
-    const long long n_tc = nw <= KK_MAX_TC ? 2LL * KP * KP : 0, n_band = 8LL * nw, n_simt = (long long)H * nw;
-    const int sbo = KP / 8 * 128;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n_tc + n_band + n_simt;
-         i += (long long)gridDim.x * blockDim.x) {
-        if (i < n_tc) {
-            // Be (p = 0): output m = 2r, input k = 2c + 1; Bo (p = 1): m = 2r + 1, k = 2c
-            const int p = (int)(i / ((long long)KP * KP)), e = (int)(i % ((long long)KP * KP));
-            const int r = e / KP, c = e % KP;
-            const int m = 2 * r + p, k = 2 * c + 1 - p;
-            const double w = (abs(k - m) >= KK_BAND) ? kk_weight(m, k, nw) : 0.0;
-            const __nv_bfloat16 hi = __double2bfloat16(w);
-            const __nv_bfloat16 lo = __double2bfloat16(w - (double)__bfloat162float(hi));
-            unsigned char *mat = tab + (size_t)p * 4 * KP * KP;
-            const unsigned off = tc_koff(r, c, sbo);
-            *reinterpret_cast<__nv_bfloat16 *>(mat + off) = hi;
-            *reinterpret_cast<__nv_bfloat16 *>(mat + 2 * KP * KP + off) = lo;
-        } else if (i < n_tc + n_band) {
-            const int e = (int)(i - n_tc), m = e / 8, d = e % 8;
-            reinterpret_cast<float *>(tab + kk_band_off(nw))[e] = (float)kk_weight(m, m + 2 * d - (KK_BAND - 1), nw);
-        } else {
-            const int e = (int)(i - n_tc - n_band), j = e / nw, m = e % nw;
-            reinterpret_cast<float *>(tab + kk_simt_off(nw))[e] = (float)kk_weight(m, 2 * j + 1 - (m & 1), nw);
-        }
+    const int H = (nw + 1) / 2, M = nw <= KK_MAX_FFT ? kk_len(nw) : 0;
+    const long long n_simt = (long long)H * nw;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n_simt; i += (long long)gridDim.x * blockDim.x) {
+        const int j = (int)(i / nw), m = (int)(i % nw);
+        reinterpret_cast<float *>(tab + kk_simt_off(nw))[i] = (float)kk_weight(m, 2 * j + 1 - (m & 1), nw);
+    }
+    const int lane = threadIdx.x % 32;
+    for (int n = (int)((blockIdx.x * blockDim.x + threadIdx.x) / 32); n < M; n += (int)(gridDim.x * blockDim.x / 32)) {
+        const int k = n < M / 2 ? 2 * n : 2 * (M - 1 - n) + 1;
+        double h = 0.0;
+        for (int j = 1 + 2 * lane; j < 2 * nw - 1; j += 64)
+            h += sinpi((double)((j * (2 * k + 1)) % (4 * M)) / (double)(2 * M)) / (double)j;
+        for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+        h *= 4.0 / 3.14159265358979323846 / (2.0 * M);
+        if (lane == 0) reinterpret_cast<float *>(tab)[kk_slot(M, n)] = (float)(n < M / 2 ? h : -h);
+    }
+    for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < M / 2; n += gridDim.x * blockDim.x) {
+        double sn, cs;
+        sincospi(0.5 * (double)n / (double)M, &sn, &cs);
+        reinterpret_cast<float2 *>(tab + 4 * M)[kk_wslot(M, n)] = make_float2((float)cs, (float)sn);
     }
 }
 
@@ -109,223 +114,170 @@ __device__ __forceinline__ float kk_vq(long long l, int Q, double dp, double v0,
 }
 
 // ---------------------------------------------------------------------------
-// Tensor-core form.  One CTA of 256 threads per block of 128 lines (persistent
-// over blocks).  Shared memory: [work][Be hi][Be lo][Bo hi][Bo lo][mbarrier]
-// [tensor-memory address]; the work region holds one parity's operand (hi,
-// lo: 128 lines x KP) while the products run, then the epilogue's chunks.
-//   operand: each warp reads whole rows of Im chi (32 consecutive transfers
-//            per load, coalesced) and pairs neighbouring elements of one
-//            parity with a shuffle before the BF16 split;
-//   epilogue, per chunk of 32 transfers: the accumulators of the 128 lines go
-//            to shared memory (transposed), the chunk's Im chi with a halo
-//            of 8 is loaded row by row, and the lanes run along the
-//            transfers for the near band, chi_RPA and the stores (coalesced).
-// The next block's rows are prefetched into L2 (cp.async.bulk.prefetch).
-template <int KP>
-struct KkTc {
-    static constexpr int T = 256, CH = 32, HALO = 8;
-    static constexpr int SBO = KP / 8 * 128;
-    static constexpr int ABYTES = 128 * KP * 2, BBYTES = KP * KP * 2;
-    static constexpr int RE_LD = CH + 1, IM_LD = CH + 2 * HALO + 1;       // padded rows of the epilogue tiles
-    static constexpr int EPI = 128 * (RE_LD + IM_LD + 1) * 4;       // + V_q of each line
-    // both parities' operands side by side when they fit beside two CTAs per SM
-    static constexpr bool BOTH = KP <= 64;
-    static constexpr int AREG = (BOTH ? 4 : 2) * ABYTES;
-    static constexpr int WORK = AREG > EPI ? AREG : EPI;
-    static constexpr int OFF_B = (WORK + 1023) / 1024 * 1024, OFF_BAR = OFF_B + 4 * BBYTES;
-    static constexpr int SMEM = OFF_BAR + 16;
-    static constexpr int COLS = 2 * KP <= 32 ? 32 : 2 * KP <= 64 ? 64 : 2 * KP <= 128 ? 128 : 256;
-    static constexpr bool fits(int m) { return m * (SMEM + 1024) <= 228 * 1024 && m * COLS <= 512 && m * T * 128 <= 65536; }
-    static constexpr int MINB = fits(2) ? 2 : 1;
-};
+// FFT form.  With x odd (x_{-k} = -x_k, x_0 not read) the sum is a convolution,
+// Re chi_m = sum_k x_k h(k - m), h(j) = 2 / (pi j) for odd j, else 0: x odd and
+// h odd, so on the half-shifted frequencies theta_k = pi (2k + 1) / 2M of
+// even.cuh (period 2M with a change of sign) it is
+//
+//   S(theta) = 2 sum_j x_j sin(j theta),  Re chi_m = (1/M) sum_k S H cos(m theta_k),
+//
+// H the transform of h, cut at the |j| <= 2 n_omega - 2 that the kept transfers
+// reach (M >= 2 n_omega: nothing wraps onto them).  The sine transform is the
+// cosine transform of the reversed sequence times (-1)^k (in H's table), so
+// V_n = -i w_n x_n and V_{M-n} = i conj(w_n) x_n; both transforms and the
+// product by H stay in registers but for one exchange each (EvLine), two lines
+// a complex column.
+//
+// Bound by instruction issue (100 instructions an output, 54% of the slots) and
+// the wait for loads; 16 bytes an output, 3.5 TB/s.  It replaces BF16 hi/lo
+// products on the tensor cores with an FP32 near band, where the operand split,
+// the near band and the transposes around the products took about 145
+// instructions an output with one or two CTAs of 8 warps per SM.  1024^2 lags x
+// 256 transfers: 2.70 -> 1.22 ms, error 1.2e-6 -> 1.5e-7 of the result's norm;
+// 256^2 x 128: 0.069 -> 0.052 ms.  Four lines a group in packed arithmetic (77
+// instructions an output, 226 registers, 8 warps per SM): 1.46 ms; this with
+// 168 registers: 1.56 ms, with 96: 1.46 ms; transfers' tables in natural order
+// (one value a load): 1.26 ms.
+//
+// A line with an infinity or NaN would spread it over the line that shares its
+// transform, so a group that holds one is summed directly (kk_direct).
+constexpr int KKF_WARPS = 4;
 
-__device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes)
+// One pair of lines by the sum itself, FP32.
+__device__ __noinline__ void kk_direct(long long l0, long long nlines, int nw, int u, int tpl, int Q, float vh, float vl,
+                                       const float *__restrict__ im, float *__restrict__ re, float2 *__restrict__ rpa);
+
+// v0 / |q|^2 of lag line l, v0 / dp^2 = vh + vl; *zero when q = 0 with an interaction
+__device__ __forceinline__ float kk_v(long long l, int Q, float vh, float vl, bool *zero)
 {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+    const int x = (int)(l / Q) - Q / 2, y = (int)(l % Q) - Q / 2;
+    const float k2 = (float)(x * x + y * y);   // exact: Q <= 4096
+    *zero = k2 == 0.f && vh != 0.f;
+    if (k2 == 0.f || vh == 0.f) return 0.f;
+    const float q = vh / k2;
+    return q + (fmaf(-q, k2, vh) + vl) / k2;
 }
 
-template <int KP>
-__global__ void __launch_bounds__(256, KkTc<KP>::MINB)
-k_kk_tc(long long nlines, int nw, int Q, double dp, double v0, const float *__restrict__ im, float *__restrict__ re,
-        float2 *__restrict__ rpa, const uint4 *__restrict__ mats, const float *__restrict__ band,
-        unsigned *status)
+template <int M>
+__global__ void __launch_bounds__(32 * KKF_WARPS, M == 384 ? 2 : 4)
+k_kk_fft(long long nlines, int nw, int Q, float vh, float vl, const float *__restrict__ im, float *__restrict__ re,
+         float2 *__restrict__ rpa, const float4 *__restrict__ kt, const float2 *__restrict__ tab)
 {
-    using S = KkTc<KP>;
-    extern __shared__ __align__(1024) unsigned char smem[];
-    if (dyn_smem_bytes() < (unsigned)S::SMEM) return;
-    unsigned long long *bar = reinterpret_cast<unsigned long long *>(smem + S::OFF_BAR);
-    unsigned *slot = reinterpret_cast<unsigned *>(smem + S::OFF_BAR + 8);
-    float *reT = reinterpret_cast<float *>(smem);                    // [128][RE_LD]
-    float *imS = reT + 128 * S::RE_LD;                               // [128][IM_LD]
-    float *vS = imS + 128 * S::IM_LD;                                // [128] V_q (NaN: chi_RPA = 0)
-    const int t = threadIdx.x, warp = t >> 5, ln = t & 31;
-    constexpr unsigned IDESC = tc_idesc_bf16(128, KP);
-
-    for (int i = t; i < 4 * S::BBYTES / 16; i += S::T) reinterpret_cast<uint4 *>(smem + S::OFF_B)[i] = mats[i];
-    if (t == 0) mbar_init(bar, 1);
-    if (warp == 0) tc_alloc(slot, S::COLS);
-    fence_proxy_async();
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const unsigned tmem = *slot;
-    const unsigned long long dA = tc_desc(smem_addr(smem), 128, S::SBO);
-    const unsigned long long dB = tc_desc(smem_addr(smem + S::OFF_B), 128, S::SBO);
-    const unsigned lane = (unsigned)((warp % 4) * 32) << 16;
-    unsigned pm = 0;
-    bool ok = true;
-    // near-band weights of this lane's transfer in each chunk are loaded per chunk
-    const long long nblk = (nlines + 127) / 128;
-    auto prefetch = [&](long long blk) {
-        if (blk >= nblk) return;
-        const long long l0 = blk * 128, nl = min(128LL, nlines - l0);
-        // the 16-byte aligned part of the block's rows (the instance's block may
-        // start anywhere in the caller's output)
-        const unsigned long long a = reinterpret_cast<unsigned long long>(im + l0 * nw);
-        const unsigned long long b = a + (unsigned long long)(nl * nw) * 4ull;
-        const unsigned long long a16 = (a + 15) & ~15ull, b16 = b & ~15ull;
-        if (b16 > a16) prefetch_l2(reinterpret_cast<const void *>(a16), (unsigned)(b16 - a16));
-    };
-    if (t == 0) prefetch(blockIdx.x);
-
-    for (long long blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
-        const long long l0 = blk * 128;
-        if (t == 0) prefetch(blk + gridDim.x);
-        // p = 0: even outputs from the odd inputs (Be); p = 1: odd outputs from the even inputs (Bo)
-        // Operand of parity p (its hi part at aoff(p), lo at aoff(p) + ABYTES):
-        // element j of a row is x(2j + 1 - p); lane k of a 32-transfer load pairs
-        // with lane k + 2 (element j + 1), and lanes with (k - (1 - p)) % 4 == 0
-        // store.  The warp's 16 rows are loaded back to back (16 loads in flight
-        // per lane).  BOTH: one pass over the rows builds both parities.
-        auto aoff = [](int p) { return S::BOTH ? 2 * p * S::ABYTES : 0; };
-        auto build = [&](int p0, int p1) {
-#pragma unroll 1
-            for (int c = 0; c < KP / 16; ++c) {
-                const int k = 32 * c + ln;
-                float v[16];
+    using E = EvLine<M>;
+    constexpr int VPT = E::VPT, TPL = E::TPL, R0 = E::R0, R1 = E::R1;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    LH_REQUIRE_SMEM(KKF_WARPS * E::WARP_ELEMS, float2)
+    const int lane = (int)threadIdx.x % 32, warp = (int)threadIdx.x / 32;
+    const int sl = lane / TPL, u = lane % TPL;
+    float2 *sm = reinterpret_cast<float2 *>(smem_raw) + warp * E::WARP_ELEMS + sl * E::LP;
+    // this group's two lines, one complex column (Q is even, so Q^2 is too)
+    const long long l0 = 2 * (((long long)blockIdx.x * KKF_WARPS + warp) * E::LPI + sl);
+    const bool live = l0 < nlines, u0 = u == 0;
+    // transfers below M/2 of this lane: ra + r R0 and rb + r R0, r < R1 / 2;
+    // their mirrors M - n lie in the other butterfly (u = 0: in the same one)
+    const int ra = u, rb = E::pair(1, u);
+    const float *row = im + (live ? l0 : 0) * nw;
+    float2 raw[2][R1 / 2];
+    float big = 0.f;   // an infinity or NaN in the group: 0 x makes it NaN
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const long long line = l0 + warp * 16 + i;
-                    v[i] = (line < nlines && k < nw) ? __ldg(im + line * nw + k) : 0.f;
-                }
+    for (int h = 0; h < 2; ++h) {
+        const float *p = row + (h ? rb : ra);
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const float w = __shfl_down_sync(0xffffffffu, v[i], 2);
-                    for (int p = p0; p <= p1; ++p)
-                        if (((ln - (1 - p)) & 3) == 0) {
-                            unsigned h, l;
-                            bf16_split(make_float2(v[i], w), h, l);
-                            const unsigned off = aoff(p) + tc_koff(warp * 16 + i, (k - (1 - p)) >> 1, S::SBO);
-                            *reinterpret_cast<unsigned *>(smem + off) = h;
-                            *reinterpret_cast<unsigned *>(smem + S::ABYTES + off) = l;
-                        }
-                }
-            }
-            fence_proxy_async();
-            tc_fence_before();
-            __syncthreads();
-            tc_fence_after();
-        };
-        // products of parity p into accumulator columns p KP (thread 0)
-        auto products = [&](int p) {
-            const unsigned long long a0 = dA + (unsigned long long)(aoff(p) >> 4);
-            const unsigned long long b0 = dB + (unsigned long long)((2 * p * S::BBYTES) >> 4);
-#pragma unroll
-            for (int term = 0; term < 3; ++term) {
-                const unsigned long long a = a0 + (unsigned long long)(((term == 1) ? S::ABYTES : 0) >> 4);
-                const unsigned long long b = b0 + (unsigned long long)(((term == 2) ? S::BBYTES : 0) >> 4);
-#pragma unroll
-                for (int ks = 0; ks < KP / 16; ++ks)
-                    tc_mma(tmem + p * KP, a + (unsigned long long)((ks * 256) >> 4),
-                           b + (unsigned long long)((ks * 256) >> 4), IDESC, term > 0 || ks > 0);
-            }
-        };
-        if constexpr (S::BOTH) {
-            build(0, 1);
-            if (t == 0) {
-                products(0);
-                products(1);
-                tc_commit(bar);
-            }
-            ok = tile_ready(bar, pm, status);
-            pm ^= 1u;
-            tc_fence_after();
-        } else {
-            for (int p = 0; p < 2 && ok; ++p) {
-                build(p, p);
-                if (t == 0) {
-                    products(p);
-                    tc_commit(bar);
-                }
-                ok = tile_ready(bar, pm, status);
-                pm ^= 1u;
-                tc_fence_after();
-            }
+        for (int r = 0; r < R1 / 2; ++r) {
+            const bool in = live && (h ? rb : ra) + r * R0 < nw;
+            raw[h][r] = make_float2(in ? __ldg(p + r * R0) : 0.f, in ? __ldg(p + nw + r * R0) : 0.f);
         }
-        if (!ok) break;
-        // epilogue, chunks of 32 transfers m0 .. m0 + 31
-#pragma unroll 1
-        for (int m0 = 0; m0 < nw; m0 += S::CH) {
-            {   // accumulators -> reT[line][q]: warps 0-3 the even transfers, 4-7 the odd ones
-                float d[16];
-                tc_ld<16>(tmem + lane + (unsigned)((warp < 4 ? 0 : KP) + m0 / 2), d);
-                const int li = (warp % 4) * 32 + ln;
-#pragma unroll
-                for (int q = 0; q < 16; ++q) reT[li * S::RE_LD + 2 * q + (warp < 4 ? 0 : 1)] = d[q];
-            }
-            if (m0 == 0 && t < 128) {    // V_q of the block's lines, once (an FP64 division each)
-                bool zero;
-                const float V = kk_vq(l0 + t, Q, dp, v0, &zero);
-                vS[t] = zero ? __int_as_float(0x7fc00000) : V;
-            }
-            {   // Im chi of the chunk with a halo of 8 on each side: the warp's 16 rows,
-                // all loads issued before the first store
-                const int k0 = m0 - S::HALO + ln, k1 = k0 + 32;
-                float a[16], b[16];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const long long line = l0 + warp * 16 + i;
-                    const float *row = im + line * nw;
-                    a[i] = (line < nlines && k0 >= 0 && k0 < nw) ? __ldg(row + k0) : 0.f;
-                    b[i] = (line < nlines && ln < 2 * S::HALO && k1 < nw) ? __ldg(row + k1) : 0.f;
-                }
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    imS[(warp * 16 + i) * S::IM_LD + ln] = a[i];
-                    if (ln < 2 * S::HALO) imS[(warp * 16 + i) * S::IM_LD + 32 + ln] = b[i];
-                }
-            }
-            __syncthreads();
-            // lanes along the transfers: near band in FP32, Re chi, chi_RPA, coalesced stores
-            const int m = m0 + ln;
-            float wb[KK_BAND];
-#pragma unroll
-            for (int d = 0; d < KK_BAND; ++d) wb[d] = (m < nw) ? __ldg(band + m * KK_BAND + d) : 0.f;
-            if (m < nw) {
-                const int nli = (int)min(16LL, nlines - (l0 + warp * 16));   // lines of this warp in range
-                float *ro = re + (l0 + warp * 16) * nw + m;
-                float2 *po = rpa ? rpa + (l0 + warp * 16) * nw + m : nullptr;
-#pragma unroll 4
-                for (int i = 0; i < nli; ++i) {
-                    const int li = warp * 16 + i;
-                    const float *xs = imS + li * S::IM_LD + ln + S::HALO;     // xs[o] = Im chi(m + o)
-                    float r = reT[li * S::RE_LD + ln];
-#pragma unroll
-                    for (int d = 0; d < KK_BAND; ++d) r = fmaf(wb[d], xs[2 * d - (KK_BAND - 1)], r);
-                    ro[(size_t)i * nw] = r;
-                    if (po) {
-                        const float V = vS[li];
-                        po[(size_t)i * nw] = kk_rpa(r, xs[0], isnan(V) ? 0.f : V, isnan(V));
-                    }
-                }
-            }
-            __syncthreads();
-        }
-        tc_fence_before();
     }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) tc_dealloc(tmem, S::COLS);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int r = 0; r < R1 / 2; ++r) big = fmaf(0.f, raw[h][r].x, fmaf(0.f, raw[h][r].y, big));
+    const unsigned group = ((1u << TPL) - 1u) << (sl * TPL);
+    const bool bad = (__ballot_sync(0xffffffffu, isnan(big)) & group) != 0;
+
+    const float4 *ht = kt + u, *wt = kt + M / 4 + u;   // the lane's columns of the tables
+    auto w_of = [&](float4 q, int r) { return r % 2 ? make_float2(q.z, q.w) : make_float2(q.x, q.y); };
+    // V_n = -i w x, V_{M-n} = i conj(w) x
+    float2 x[VPT], prev = make_float2(0.f, 0.f);
+    auto sel = [&](float2 a, float2 b) { return make_float2(u0 ? a.x : b.x, u0 ? a.y : b.y); };
+#pragma unroll
+    for (int r = 0; r < R1 / 2; ++r) {
+        float2 hi[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float2 v = raw[h][r];
+            if (h == 0 && r == 0) v = sel(make_float2(0.f, 0.f), v);   // x_0 does not enter
+            const float2 w = w_of(__ldg(wt + (h * (R1 / 2) + r) / 2 * TPL), r);
+            const float2 a = cmul(v, w), b = cmulc(v, w);
+            x[h * R1 + r] = mul_mi(a);
+            hi[h] = mul_i(b);
+        }
+        x[R1 + R1 - 1 - r] = sel(hi[1], hi[0]);
+        if (r > 0) x[R1 - r] = sel(hi[0], prev);
+        prev = hi[1];
+    }
+    x[R1 / 2] = sel(make_float2(0.f, 0.f), prev);
+    E::inverse(x, sm, u, tab);
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+        const float4 q = __ldg(ht + i / 4 * TPL);
+        const float h = i % 4 == 0 ? q.x : i % 4 == 1 ? q.y : i % 4 == 2 ? q.z : q.w;
+        x[i] = make_float2(x[i].x * h, x[i].y * h);
+    }
+#pragma unroll
+    for (int b = 0; b < VPT / R0; ++b) ev_dft<R0, false>(x + b * R0);
+    E::forward_rest(x, sm, u, tab);
+    if (!live) return;
+    if (bad) {
+        kk_direct(l0, nlines, nw, u, TPL, Q, vh, vl, im, re, rpa);
+        return;
+    }
+    float V[2];
+    bool zero[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) V[i] = kk_v(l0 + i, Q, vh, vl, &zero[i]);
+    // Re chi of transfer m = conj(w) V_m + w V_{M-m} (the 1/2 in H)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int rh = h ? rb : ra;
+        const float *xi = row + rh;
+        float *ro = re + l0 * nw + rh;
+        float2 *po = rpa + l0 * nw + rh;
+#pragma unroll
+        for (int r = 0; r < R1 / 2; ++r) {
+            const float2 w = w_of(__ldg(wt + (h * (R1 / 2) + r) / 2 * TPL), r);
+            const float2 a = x[h * R1 + r];
+            const float2 b = h ? sel(x[R1 + R1 - 1 - r], x[R1 - 1 - r]) : sel(x[(R1 - r) % R1], x[R1 + R1 - 1 - r]);
+            const float2 z = cadd(cmulc(a, w), cmul(b, w));
+            const float y[2] = {z.x, z.y};
+            if (rh + r * R0 < nw) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i) ro[i * nw + r * R0] = y[i];
+                if (rpa) {
+#pragma unroll
+                    for (int i = 0; i < 2; ++i)
+                        po[i * nw + r * R0] = kk_rpa(y[i], __ldg(xi + i * nw + r * R0), V[i], zero[i]);
+                }
+            }
+        }
+    }
+}
+
+__device__ __noinline__ void kk_direct(long long l0, long long nlines, int nw, int u, int tpl, int Q, float vh, float vl,
+                                       const float *__restrict__ im, float *__restrict__ re, float2 *__restrict__ rpa)
+{
+    for (int i = 0; i < 2 && l0 + i < nlines; ++i) {
+        const float *row = im + (l0 + i) * nw;
+        bool zero;
+        const float V = kk_v(l0 + i, Q, vh, vl, &zero);
+        for (int m = u; m < nw; m += tpl) {
+            float s = 0.f;
+            for (int k = 1 + (m & 1); k < nw; k += 2)
+                s = fmaf(1.27323954473516268615f * (float)k / (float)(k * k - m * m), row[k], s);
+            re[(l0 + i) * nw + m] = s;
+            if (rpa) rpa[(l0 + i) * nw + m] = kk_rpa(s, row[m], V, zero);
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -392,38 +344,36 @@ k_kk_simt(long long nlines, int nw, int Q, double dp, double v0, const float *__
     }
 }
 
-// variant 0: tensor cores (n_omega <= 256); 1: FP32 SIMT (n_omega <= 1536)
-template <int KP>
-static cudaError_t launch_kk_tc_t(const Geom &g, const float *im, float *re, float2 *rpa, const void *tab,
-                                  double v0, unsigned *status, cudaStream_t s)
+// variant 0: FFT (n_omega <= 256); 1: FP32 SIMT (n_omega <= 1536).  evt: the
+// tables of even.cuh and even_line.cuh.
+template <int M>
+static cudaError_t launch_kk_fft_t(const Geom &g, const float *im, float *re, float2 *rpa, const void *tab, double v0,
+                                   const float2 *evt, cudaStream_t s)
 {
-    using S = KkTc<KP>;
-    auto k = k_kk_tc<KP>;
-    static const cudaError_t e0 = smem_attrs(k, (size_t)S::SMEM);
+    using E = EvLine<M>;
+    const size_t smem = sizeof(float2) * KKF_WARPS * E::WARP_ELEMS;
+    static const cudaError_t e0 = smem_attrs(k_kk_fft<M>, smem);
     if (e0 != cudaSuccess) return e0;
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    const long long nlines = (long long)g.Q * g.Q, nblk = (nlines + 127) / 128;
-    const int grid = (int)std::min<long long>(nblk, (long long)sms * S::MINB);
-    const unsigned char *t8 = static_cast<const unsigned char *>(tab);
-    k<<<grid, S::T, S::SMEM, s>>>(nlines, g.n_omega, g.Q, g.dp, v0, im, re, rpa, reinterpret_cast<const uint4 *>(t8),
-                                  reinterpret_cast<const float *>(t8 + kk_band_off(g.n_omega)), status);
+    const long long nlines = (long long)g.Q * g.Q, per = 2LL * KKF_WARPS * E::LPI;
+    const double v = v0 / (g.dp * g.dp);
+    const float vh = (float)v, vl = (float)(v - (double)vh);
+    k_kk_fft<M><<<(unsigned)((nlines + per - 1) / per), 32 * KKF_WARPS, smem, s>>>(
+        nlines, g.n_omega, g.Q, vh, vl, im, re, rpa, static_cast<const float4 *>(tab),
+        evt + ev_line_table<M>());
     return cudaGetLastError();
 }
 
 cudaError_t launch_kk_rpa(const Geom &g, const float *im, float *re, float2 *rpa, const void *tab, double v0,
-                          int variant, unsigned *status, cudaStream_t s)
+                          int variant, const void *evt, cudaStream_t s)
 {
     const int nw = g.n_omega;
     if (variant == 0) {
-        if (nw > KK_MAX_TC) return cudaErrorNotSupported;
-        switch (kk_kp(nw)) {
-        case 16: return launch_kk_tc_t<16>(g, im, re, rpa, tab, v0, status, s);
-        case 32: return launch_kk_tc_t<32>(g, im, re, rpa, tab, v0, status, s);
-        case 64: return launch_kk_tc_t<64>(g, im, re, rpa, tab, v0, status, s);
-        default: return launch_kk_tc_t<128>(g, im, re, rpa, tab, v0, status, s);
+        if (nw > KK_MAX_FFT) return cudaErrorNotSupported;
+        switch (kk_len(nw)) {
+        case 128: return launch_kk_fft_t<128>(g, im, re, rpa, tab, v0, (const float2 *)evt, s);
+        case 256: return launch_kk_fft_t<256>(g, im, re, rpa, tab, v0, (const float2 *)evt, s);
+        case 384: return launch_kk_fft_t<384>(g, im, re, rpa, tab, v0, (const float2 *)evt, s);
+        default: return launch_kk_fft_t<512>(g, im, re, rpa, tab, v0, (const float2 *)evt, s);
         }
     }
     if (variant != 1 || nw > KK_MAX_SIMT) return cudaErrorNotSupported;

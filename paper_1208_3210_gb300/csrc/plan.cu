@@ -51,7 +51,7 @@ cudaError_t launch_dmu_partials(int kind, double t, double tp, double tpp, doubl
 constexpr int kDmuBlocks = 128;
 cudaError_t launch_kk_tables(int nw, void *tab, cudaStream_t s);
 cudaError_t launch_kk_rpa(const Geom &g, const float *im, float *re, float2 *rpa, const void *tab, double v0,
-                          int variant, unsigned *status, cudaStream_t s);
+                          int variant, const void *evt, cudaStream_t s);
 size_t tc_mats_bytes();
 size_t pr_twiddle_bytes();
 size_t et_twiddle_bytes();
@@ -1282,17 +1282,17 @@ extern "C" lindhard_status lindhard_kk_rpa(lindhard_plan *p, int index, const fl
     if (!p || !imchi || !re_out) return fail(LINDHARD_EINVAL, "plan, imchi and re_out must be non-NULL");
     if (index < 0 || index >= p->batch) return fail(LINDHARD_EINVAL, "index out of range");
     if (p->precision[index] == LINDHARD_FP64) return fail(LINDHARD_EINVAL, "the Kramers-Kronig pass reads FP32 outputs");
-    if (variant != 0 && variant != 1) return fail(LINDHARD_EINVAL, "variant must be 0 (tensor cores) or 1 (FP32 SIMT)");
+    if (variant != 0 && variant != 1) return fail(LINDHARD_EINVAL, "variant must be 0 (FFT) or 1 (FP32 sum)");
     if (!isfinite(v0)) return fail(LINDHARD_EINVAL, "v0 must be finite");
     const Geom &g = p->geoms[index];
     if (g.quantity == LINDHARD_SQW) return fail(LINDHARD_EINVAL, "the Kramers-Kronig pass reads Im chi (not S(q, w))");
     if (g.n_omega > (variant == 0 ? 256 : 1536))
-        return fail(LINDHARD_EUNSUPPORTED, variant == 0 ? "the tensor-core form takes n_omega <= 256"
-                                                        : "the SIMT form takes n_omega <= 1536");
+        return fail(LINDHARD_EUNSUPPORTED, variant == 0 ? "the FFT form takes n_omega <= 256"
+                                                        : "the direct form takes n_omega <= 1536");
     if (rpa_out && (reinterpret_cast<uintptr_t>(rpa_out) & 7u))
         return fail(LINDHARD_EINVAL, "rpa_out must be 8-byte aligned");
     cudaError_t e = launch_kk_rpa(g, imchi, re_out, reinterpret_cast<float2 *>(rpa_out), p->ws + p->off_kk[index], v0,
-                                  variant, (unsigned *)(p->ws + p->off_status), (cudaStream_t)stream);
+                                  variant, p->ws + p->off_evt, (cudaStream_t)stream);
     return e == cudaSuccess ? LINDHARD_OK : cuda_fail(e, "Kramers-Kronig launch");
 }
 

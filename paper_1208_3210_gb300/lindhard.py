@@ -282,8 +282,8 @@ class Plan:
     def kk_rpa(self, out_i, index=0, v0=0.0, rpa=True, variant=0, stream=None):
         """Re chi by Kramers-Kronig and chi_RPA = chi / (1 - v0/|q|^2 chi) for
         instance `index` from its Im chi block `out_i` (device float32
-        [Q][Q][n_omega] or flat).  variant 0: tensor cores (n_omega <= 256);
-        1: FP32 SIMT.  Returns (Re chi, chi_RPA as complex64 or None), shaped
+        [Q][Q][n_omega] or flat).  variant 0: by FFT (n_omega <= 256);
+        1: the direct FP32 sum.  Returns (Re chi, chi_RPA as complex64 or None), shaped
         [Q][Q][n_omega]."""
         import torch
         s = self.sizes[index]

@@ -138,3 +138,44 @@ def test_kk_rpa_full_size_extended_workload(lh):
     plan.close()
     del out, re0, re1, rp0, rp1
     torch.cuda.empty_cache()
+
+
+# The FFT form at every transfer count around its lengths (n_omega <= 64, 128,
+# 192, 256 take transforms of 128, 256, 384, 512): a Hilbert transform through
+# two FFTs of at most 512 points, each value rounded log2(512) times at 6e-8 in
+# each, random in sign: below 1e-6 of the maximum.
+@pytest.mark.parametrize("n", [1, 2, 3, 8, 31, 63, 64, 65, 127, 128, 129, 190, 192, 193, 255, 256])
+def test_kk_fft_lengths(lh, n):
+    import torch
+    plan = lh.Plan([wl.grid_params(2, 6, max(2, n), 1.5, n_omega=n)])
+    g = torch.Generator(device="cuda").manual_seed(n)
+    im = -torch.rand(plan.out_elems(), generator=g, device="cuda")
+    re, rp = plan.kk_rpa(im, v0=0.05, variant=0)
+    none, _ = plan.kk_rpa(im, v0=0.05, rpa=False, variant=0)
+    plan.status()
+    ref_im = im.cpu().numpy().astype(np.float64).reshape(re.shape)
+    ref = oracle.kk_real(ref_im)
+    got = re.cpu().numpy().astype(np.float64)
+    assert np.abs(got - ref).max() <= 1e-6 * max(np.abs(ref).max(), np.abs(ref_im).max())
+    assert torch.equal(re, none)
+    rp_ref = oracle.rpa(got, ref_im, 2 * math.pi / 6, 0.05)
+    assert np.abs(rp.cpu().numpy() - rp_ref).max() <= TOL_RPA * np.abs(rp_ref).max()
+    plan.close()
+
+
+def test_kk_infinities_and_nans_stay_in_their_line(lh):
+    import torch
+    plan = lh.Plan([wl.grid_params(2, 6, 200, 1.5, n_omega=100)])
+    im = -torch.rand(plan.out_elems(), device="cuda")
+    ref, _ = plan.kk_rpa(im, v0=0.05)
+    bad = im.clone().reshape(144, 100)
+    bad[5, 7], bad[40, 20] = float("nan"), float("inf")
+    re, _ = plan.kk_rpa(bad.reshape(-1), v0=0.05)
+    plan.status()
+    re, ref = re.reshape(144, 100), ref.reshape(144, 100)
+    rest = [i for i in range(144) if i not in (5, 40)]
+    assert float((re[rest] - ref[rest]).abs().max()) <= 1e-6 * float(ref.abs().max())
+    # an entry enters the outputs of the other parity only
+    assert bool(re[5, 0::2].isnan().all()) and not bool(re[5, 1::2].isnan().any())
+    assert not bool(re[40, 1::2].isfinite().any()) and bool(re[40, 0::2].isfinite().all())
+    plan.close()

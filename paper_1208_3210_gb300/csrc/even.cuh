@@ -186,7 +186,7 @@ __device__ __forceinline__ void dft4(Cx2 &a, Cx2 &b, Cx2 &c, Cx2 &d)
 }
 // (e + w o, e - w o) for w = e^{-+ i pi/4} (K = 1) or e^{-+ 3 i pi/4} (K = 3)
 template <bool INV, int K>
-__device__ __forceinline__ void combine45(Cx2 e, Cx2 o, Cx2 &lo, Cx2 &hi)
+__device__ __forceinline__ void combine45x(Cx2 e, Cx2 o, Cx2 &lo, Cx2 &hi)
 {
     const float2 c = dup2(0.70710678118654752440f), n = dup2(-0.70710678118654752440f);
     const float2 s = add2(o.re, o.im), d = sub2(o.im, o.re);
@@ -215,8 +215,8 @@ __device__ __forceinline__ void dft8(Cx2 *v)
     v[4] = sub(e0, o0);
     v[2] = INV ? add_i(e2, o2) : sub_i(e2, o2);
     v[6] = INV ? sub_i(e2, o2) : add_i(e2, o2);
-    combine45<INV, 1>(e1, o1, v[1], v[5]);
-    combine45<INV, 3>(e3, o3, v[3], v[7]);
+    combine45x<INV, 1>(e1, o1, v[1], v[5]);
+    combine45x<INV, 3>(e3, o3, v[3], v[7]);
 }
 template <int R, bool INV>
 __device__ __forceinline__ void dft(Cx2 *v)
@@ -255,8 +255,8 @@ __device__ __forceinline__ void dft(Cx2 *v)
         v[8] = sub(e[0], o[0]);
         v[4] = INV ? add_i(e[4], o[4]) : sub_i(e[4], o[4]);
         v[12] = INV ? sub_i(e[4], o[4]) : add_i(e[4], o[4]);
-        combine45<INV, 1>(e[2], o[2], v[2], v[10]);
-        combine45<INV, 3>(e[6], o[6], v[6], v[14]);
+        combine45x<INV, 1>(e[2], o[2], v[2], v[10]);
+        combine45x<INV, 3>(e[6], o[6], v[6], v[14]);
 #pragma unroll
         for (int k = 1; k < 8; k += 2) {
             const float c = (float)cos48(3 * k), s = (float)sin48(3 * k);

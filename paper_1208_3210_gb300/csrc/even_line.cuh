@@ -100,8 +100,8 @@ __device__ __forceinline__ void ev_dft(Cx2 *v)
         v[16] = sub(e[0], o[0]);
         v[8] = INV ? add_i(e[8], o[8]) : sub_i(e[8], o[8]);
         v[24] = INV ? sub_i(e[8], o[8]) : add_i(e[8], o[8]);
-        combine45<INV, 1>(e[4], o[4], v[4], v[20]);
-        combine45<INV, 3>(e[12], o[12], v[12], v[28]);
+        combine45x<INV, 1>(e[4], o[4], v[4], v[20]);
+        combine45x<INV, 3>(e[12], o[12], v[12], v[28]);
 #pragma unroll
         for (int k = 1; k < 16; ++k)
             if (k % 4 != 0) {

@@ -193,13 +193,36 @@ template <bool INV, typename C, bool PK> struct Dft<4, INV, C, PK> {
     }
 };
 // Radix 8 and 16: decimation in time into two halves of radix R/2.
+// (e + w o, e - w o) for w = e^{-+ i pi/4} (K = 1) or e^{-+ 3 i pi/4} (K = 3):
+// the multiplication by sqrt(1/2) rides on the sums as fused multiply-adds
+// (6 instructions where a product and two sums take 8).
+template <bool INV, int K, bool PK, typename C>
+__device__ __forceinline__ void combine45(C e, C o, C &lo, C &hi)
+{
+    using T = decltype(C::x);
+    constexpr T c = (T)0.70710678118654752440;
+    const T s = o.x + o.y, d = o.y - o.x;
+    // forward: w1 o = c (s, d), w3 o = c (d, -s); inverse: w1 o = c (-d, s), w3 o = c (-s, -d)
+    const T a = K == 1 ? (INV ? -d : s) : (INV ? -s : d), b = K == 1 ? (INV ? s : d) : (INV ? -d : -s);
+    if constexpr (PK && sizeof(C) == 8) {
+        lo = __ffma2_rn(mk<C>(a, b), mk<C>(c, c), e);
+        hi = __ffma2_rn(mk<C>(a, b), mk<C>(-c, -c), e);
+    } else {
+        lo = mk<C>(e.x + c * a, e.y + c * b);
+        hi = mk<C>(e.x - c * a, e.y - c * b);
+    }
+}
 template <int R, bool INV, typename C, int K, bool PK = false>
 __device__ __forceinline__ void dit_combine(C *v, const C *e, const C *o)
 {
     if constexpr (K < R / 2) {
-        C t = twc<R, K, INV>(o[K]);
-        v[K] = padd<PK>(e[K], t);
-        v[K + R / 2] = psub<PK>(e[K], t);
+        if constexpr (8 * K == R || 8 * K == 3 * R) {
+            combine45<INV, 8 * K / R, PK>(e[K], o[K], v[K], v[K + R / 2]);
+        } else {
+            C t = twc<R, K, INV>(o[K]);
+            v[K] = padd<PK>(e[K], t);
+            v[K + R / 2] = psub<PK>(e[K], t);
+        }
         dit_combine<R, INV, C, K + 1, PK>(v, e, o);
     }
 }
@@ -212,36 +235,61 @@ template <bool INV, typename C, bool PK> struct Dft<8, INV, C, PK> {
         dit_combine<8, INV, C, 0, PK>(v, e, o);
     }
 };
+// The last two outputs of a 3-point DFT from m = a - (b + c) / 2 and d = b - c:
+// m -+ i sqrt(3/4) d, as fused multiply-adds.
+template <bool INV, bool PK, typename C>
+__device__ __forceinline__ void dft3_tail(C m, C d, C &y1, C &y2)
+{
+    using T = decltype(C::x);
+    constexpr T s3 = (T)0.86602540378443864676;   // sin(2 pi / 3)
+    const C f = INV ? mul_i(d) : mul_mi(d);       // forward: y1 = m - i s3 d
+    if constexpr (PK && sizeof(C) == 8) {
+        y1 = __ffma2_rn(f, mk<C>(s3, s3), m);
+        y2 = __ffma2_rn(f, mk<C>(-s3, -s3), m);
+    } else {
+        y1 = mk<C>(m.x + s3 * f.x, m.y + s3 * f.y);
+        y2 = mk<C>(m.x - s3 * f.x, m.y - s3 * f.y);
+    }
+}
 template <bool INV, typename C, bool PK> struct Dft<3, INV, C, PK> {
     __device__ __forceinline__ static void run(C *v)
     {
         using T = decltype(C::x);
-        constexpr T s3 = (T)0.86602540378443864676;   // sin(2 pi / 3)
-        C t1 = padd<PK>(v[1], v[2]);
-        C t2 = mk<C>(v[0].x - (T)0.5 * t1.x, v[0].y - (T)0.5 * t1.y);
-        C d = psub<PK>(v[1], v[2]);
-        C t3 = mk<C>(s3 * d.x, s3 * d.y);
+        const C t1 = padd<PK>(v[1], v[2]), d = psub<PK>(v[1], v[2]);
+        const C m = mk<C>(v[0].x - (T)0.5 * t1.x, v[0].y - (T)0.5 * t1.y);
         v[0] = padd<PK>(v[0], t1);
-        // forward: y1 = t2 - i t3, y2 = t2 + i t3 (inverse: the other way round)
-        v[1] = INV ? padd<PK>(t2, mul_i(t3)) : padd<PK>(t2, mul_mi(t3));
-        v[2] = INV ? padd<PK>(t2, mul_mi(t3)) : padd<PK>(t2, mul_i(t3));
+        dft3_tail<INV, PK>(m, d, v[1], v[2]);
     }
 };
-// Radix 6, 12 and 24: decimation in time into two halves.
-template <int R, bool INV, typename C, bool PK = false> struct DftDit {
+// Radix 6, 12 and 24 as 3 x Q by the prime-factor map (Good 1958), which needs
+// no twiddles between the two: inputs n = 3 i + Q j, outputs k with k = kq mod Q
+// and k = k3 mod 3.
+template <int R, bool INV, typename C, bool PK = false> struct DftPfa {
+    static constexpr int Q = R / 3;
+    static constexpr int A = Q % 3 == 1 ? Q : 2 * Q;                               // 0 mod Q, 1 mod 3
+    static constexpr int B = 3 % Q == 1 ? 3 : 9 % Q == 1 ? 9 : 6 % Q == 1 ? 6 : 3 * (Q - 1);   // 1 mod Q, 0 mod 3
+    static_assert(A % 3 == 1 && A % Q == 0 && B % Q == 1 && B % 3 == 0, "coprime factors");
     __device__ __forceinline__ static void run(C *v)
     {
-        C e[R / 2], o[R / 2];
+        C t[3][Q];
 #pragma unroll
-        for (int i = 0; i < R / 2; ++i) { e[i] = v[2 * i]; o[i] = v[2 * i + 1]; }
-        Dft<R / 2, INV, C, PK>::run(e);
-        Dft<R / 2, INV, C, PK>::run(o);
-        dit_combine<R, INV, C, 0, PK>(v, e, o);
+        for (int j = 0; j < 3; ++j) {
+#pragma unroll
+            for (int i = 0; i < Q; ++i) t[j][i] = v[(3 * i + Q * j) % R];
+            Dft<Q, INV, C, PK>::run(t[j]);
+        }
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            C z[3] = {t[0][k], t[1][k], t[2][k]};
+            Dft<3, INV, C, PK>::run(z);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) v[(B * k + A * q) % R] = z[q];
+        }
     }
 };
-template <bool INV, typename C, bool PK> struct Dft<6, INV, C, PK> : DftDit<6, INV, C, PK> {};
-template <bool INV, typename C, bool PK> struct Dft<12, INV, C, PK> : DftDit<12, INV, C, PK> {};
-template <bool INV, typename C, bool PK> struct Dft<24, INV, C, PK> : DftDit<24, INV, C, PK> {};
+template <bool INV, typename C, bool PK> struct Dft<6, INV, C, PK> : DftPfa<6, INV, C, PK> {};
+template <bool INV, typename C, bool PK> struct Dft<12, INV, C, PK> : DftPfa<12, INV, C, PK> {};
+template <bool INV, typename C, bool PK> struct Dft<24, INV, C, PK> : DftPfa<24, INV, C, PK> {};
 
 template <bool INV, typename C, bool PK> struct Dft<16, INV, C, PK> {
     __device__ __forceinline__ static void run(C *v)

@@ -69,71 +69,62 @@ __host__ __device__ constexpr int pr_twiddle_entries() { return pr_tables_before
 __host__ __device__ constexpr int pr_tw_offset(int L, bool inv, int s) { return pr_tables_before(pr_len_index(L), inv, s); }
 
 // ---------------------------------------------------------------------------
-// 24-point DFTs with a pruned end (sign by INV as in Dft<>).
-// Inputs v[16..23] zero: y[3 k2 + k1] = DFT8_k2( w^(r1 k1) (v[r1] + W3^k1 v[r1 + 8]) ),
-// w = exp(-+2 pi i / 24), W3 = w^8.
+// 24-point DFTs with a pruned end (sign by INV as in Dft<>), as 3 x 8 by the
+// prime-factor map of DftPfa: inputs n = 3 i + 8 j, outputs k = 9 k8 + 16 k3
+// (mod 24), no twiddles between the 3-point and the 8-point transforms (9.2
+// FP32 instructions a point; decimation with twiddles took 12.2).
+// Inputs v[16..23] zero: one input of every 3-point transform is zero.
 template <bool INV, bool PK = false>
 __device__ __forceinline__ void dft24_in16(float2 *v)
 {
-    constexpr float s3 = 0.86602540378443864676f;   // sin(2 pi / 3)
-    float2 u0[8], u1[8], u2[8];
+    float2 y[3][8];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        const float2 a = v[r], c = v[r + 8];
-        u0[r] = padd<PK>(a, c);
-        const float2 t = make_float2(fmaf(-0.5f, c.x, a.x), fmaf(-0.5f, c.y, a.y));
-        const float2 q = make_float2(s3 * c.x, s3 * c.y);
-        // a + W3 c = t -+ i q, a + W3^2 c = t +- i q (forward: W3 = -1/2 - i s3)
-        u1[r] = INV ? padd<PK>(t, mul_i(q)) : padd<PK>(t, mul_mi(q));
-        u2[r] = INV ? padd<PK>(t, mul_mi(q)) : padd<PK>(t, mul_i(q));
+    for (int i = 0; i < 8; ++i) {
+        // the inputs j = 0, 1, 2 of column i: rows 3i + 8j mod 24, the one above 15 is zero
+        const int n0 = 3 * i, n1 = (3 * i + 8) % 24, n2 = (3 * i + 16) % 24;
+        if (n0 >= 16) {          // (0, b, c)
+            const float2 b = v[n1], c = v[n2], t = padd<PK>(b, c), d = psub<PK>(b, c);
+            y[0][i] = t;
+            dft3_tail<INV, PK>(make_float2(-0.5f * t.x, -0.5f * t.y), d, y[1][i], y[2][i]);
+        } else {                 // (a, b, 0) or (a, 0, c)
+            const bool first = n2 >= 16;
+            const float2 a = v[n0], b = v[first ? n1 : n2];
+            const float2 m = make_float2(fmaf(-0.5f, b.x, a.x), fmaf(-0.5f, b.y, a.y));
+            y[0][i] = padd<PK>(a, b);
+            if (first) dft3_tail<INV, PK>(m, b, y[1][i], y[2][i]);
+            else dft3_tail<INV, PK>(m, b, y[2][i], y[1][i]);   // d = -c
+        }
     }
-    u1[1] = twc<24, 1, INV>(u1[1]); u1[2] = twc<24, 2, INV>(u1[2]); u1[3] = twc<24, 3, INV>(u1[3]);
-    u1[4] = twc<24, 4, INV>(u1[4]); u1[5] = twc<24, 5, INV>(u1[5]); u1[6] = twc<24, 6, INV>(u1[6]);
-    u1[7] = twc<24, 7, INV>(u1[7]);
-    u2[1] = twc<24, 2, INV>(u2[1]); u2[2] = twc<24, 4, INV>(u2[2]); u2[3] = twc<24, 6, INV>(u2[3]);
-    u2[4] = twc<24, 8, INV>(u2[4]); u2[5] = twc<24, 10, INV>(u2[5]); u2[6] = twc<24, 12, INV>(u2[6]);
-    u2[7] = twc<24, 14, INV>(u2[7]);
-    Dft<8, INV, float2, PK>::run(u0);
-    Dft<8, INV, float2, PK>::run(u1);
-    Dft<8, INV, float2, PK>::run(u2);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        v[3 * k] = u0[k];
-        v[3 * k + 1] = u1[k];
-        v[3 * k + 2] = u2[k];
-    }
+    for (int q = 0; q < 3; ++q) Dft<8, INV, float2, PK>::run(y[q]);
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) v[(9 * k + 16 * q) % 24] = y[q][k];
 }
 
-// Outputs y[0..7] and y[16..23] only (v[8..15] are left undefined):
-// y[k1 + 8 k2] = sum_i2 W3^(i2 k2) w^(i2 k1) DFT8_k1(v[3 i1 + i2]).
+// Outputs y[0..7] and y[16..23] only (v[8..15] are left undefined): one output
+// of every 3-point transform is not formed.
 template <bool INV, bool PK = false>
 __device__ __forceinline__ void dft24_out16(float2 *v)
 {
-    constexpr float s3 = 0.86602540378443864676f;
-    float2 y0[8], y1[8], y2[8];
+    float2 y[3][8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        y0[i] = v[3 * i];
-        y1[i] = v[3 * i + 1];
-        y2[i] = v[3 * i + 2];
+    for (int q = 0; q < 3; ++q) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) y[q][i] = v[(3 * i + 8 * q) % 24];
+        Dft<8, INV, float2, PK>::run(y[q]);
     }
-    Dft<8, INV, float2, PK>::run(y0);
-    Dft<8, INV, float2, PK>::run(y1);
-    Dft<8, INV, float2, PK>::run(y2);
-    y1[1] = twc<24, 1, INV>(y1[1]); y1[2] = twc<24, 2, INV>(y1[2]); y1[3] = twc<24, 3, INV>(y1[3]);
-    y1[4] = twc<24, 4, INV>(y1[4]); y1[5] = twc<24, 5, INV>(y1[5]); y1[6] = twc<24, 6, INV>(y1[6]);
-    y1[7] = twc<24, 7, INV>(y1[7]);
-    y2[1] = twc<24, 2, INV>(y2[1]); y2[2] = twc<24, 4, INV>(y2[2]); y2[3] = twc<24, 6, INV>(y2[3]);
-    y2[4] = twc<24, 8, INV>(y2[4]); y2[5] = twc<24, 10, INV>(y2[5]); y2[6] = twc<24, 12, INV>(y2[6]);
-    y2[7] = twc<24, 14, INV>(y2[7]);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-        const float2 s = padd<PK>(y1[k], y2[k]), d = psub<PK>(y1[k], y2[k]);
-        v[k] = padd<PK>(y0[k], s);
-        const float2 t = make_float2(fmaf(-0.5f, s.x, y0[k].x), fmaf(-0.5f, s.y, y0[k].y));
-        const float2 q = make_float2(s3 * d.x, s3 * d.y);
-        // W3^2 z1 + W3 z2 = -s/2 -+ i s3 d (forward: W3 = -1/2 - i s3)
-        v[k + 16] = INV ? padd<PK>(t, mul_mi(q)) : padd<PK>(t, mul_i(q));
+        // outputs k3 = 0, 1, 2 of column k: rows 9k + 16 k3 mod 24; the dropped one is never read
+        float2 z[3] = {y[0][k], y[1][k], y[2][k]};
+        Dft<3, INV, float2, PK>::run(z);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const int n = (9 * k + 16 * q) % 24;
+            if (n < 8 || n >= 16) v[n] = z[q];
+        }
     }
 }
 

@@ -607,7 +607,10 @@ extern "C" lindhard_status lindhard_plan_create(const lindhard_grid *grids, int 
     p->off_kk.assign(batch, 0);
     for (int i = 0; i < batch; ++i)
         if (p->precision[i] != LINDHARD_FP64) {
-            p->off_kk[i] = o; o = align_up(o + kk_table_bytes(p->geoms[i].n_omega));
+            // one table for all instances with as many transfers
+            for (int k = 0; k < i && !p->off_kk[i]; ++k)
+                if (p->off_kk[k] && p->geoms[k].n_omega == p->geoms[i].n_omega) p->off_kk[i] = p->off_kk[k];
+            if (!p->off_kk[i]) { p->off_kk[i] = o; o = align_up(o + kk_table_bytes(p->geoms[i].n_omega)); }
         }
     auto place = [&](const Need &n) {
         lindhard_plan::Slot sl;
@@ -652,7 +655,8 @@ extern "C" lindhard_status lindhard_plan_create(const lindhard_grid *grids, int 
     if (e == cudaSuccess) e = launch_ev_tables((float2 *)(p->ws + p->off_evt), 0);
     if (e == cudaSuccess && p->off_tc) e = launch_tc_mats(p->ws + p->off_tc, 0);
     for (int i = 0; i < batch && e == cudaSuccess; ++i)
-        if (p->off_kk[i]) e = launch_kk_tables(p->geoms[i].n_omega, p->ws + p->off_kk[i], 0);
+        if (p->off_kk[i] && std::find(p->off_kk.begin(), p->off_kk.begin() + i, p->off_kk[i]) == p->off_kk.begin() + i)
+            e = launch_kk_tables(p->geoms[i].n_omega, p->ws + p->off_kk[i], 0);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e == cudaSuccess && p->concurrent) {
         int ns = std::min(batch, 16);

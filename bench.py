@@ -760,9 +760,9 @@ def main():
     peak, peak_kind = measured_peaks()
     # kernels launched in the timed region: each step is one forward call; a
     # third multisection pass when gamma < 0.02 eV and the solve spans
-    # several CTAs (more than 98 points per zone)
+    # several CTAs (more than 160 points per zone)
     launches = (sum(int(plan.sizes[i].kernels_forward)
-                    + (1 if bands[i]["gamma"] < 0.02 and grids[i]["npz"] > 98 else 0)
+                    + (1 if bands[i]["gamma"] < 0.02 and grids[i]["npz"] > 160 else 0)
                     for i in range(len(grids))) + (1 if batched and persistent else 0)) * args.steps
     if batched:
         # concurrent instances: no per-pass split, the batch as one unit

@@ -142,8 +142,8 @@ typedef struct {
     long long a_elems;      /* N^2 * n_eps (layout of A_in and dA)           */
     long long hbm_bytes_forward;  /* algorithmic HBM bytes of one forward call */
     long long kernels_forward;    /* kernel launches of one forward call with A generated and mu
-                                     solved: with more than 98 points per zone one more when
-                                     gamma < 0.02 eV (a third multisection pass); with at most 98
+                                     solved: with more than 160 points per zone one more when
+                                     gamma < 0.02 eV (a third multisection pass); with at most 160
                                      the whole solve runs in the set-up launch (two fewer); with
                                      a caller-supplied A only the FFT passes; in a
                                      LINDHARD_PLAN_PERSISTENT plan the instance's set-up launches

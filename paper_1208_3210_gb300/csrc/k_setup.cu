@@ -50,9 +50,8 @@ __global__ void k_twiddles(int max_len, float2 *tw32, double2 *tw64)
 // m_x <= m_y (twice for m_x < m_y): (npz/2 + 1)(npz/2 + 2)/2 terms instead of
 // npz^2 (561 instead of 4096 at npz = 64).
 //
-// Launches (no CTA ever waits for another; zones of at most 98 points per
-// axis instead solve in one CTA of k_setup by a bracketed Newton iteration,
-// see mu_solve_one_cta):
+// Launches (no CTA ever waits for another; zones of at most 160 points per
+// axis instead solve in one CTA of k_setup, see mu_solve_one_cta):
 //   k_setup     multisection pass 0 over [-B-3, B+3] eV on G CTAs, and the
 //               tables on further CTAs of the same launch (their FP64 cospi and
 //               exp chains run beside the multisection, not before it)
@@ -108,14 +107,17 @@ struct MuConst {
     double B;            // bracket half-width - 3 eV
     int NC, passes;
     int single;          // the whole solve in one CTA of the set-up launch
+    // of the one-CTA solve: the filling, and as FP32 pairs 1/gamma and
+    // e^{i pi (npz^2 / 2 - target)}
+    float target_f, Bf, igh, igl, cth, ctl, sth, stl;
 };
 
-// Zones small enough for the one-CTA solve: every pass and the Halley step in
-// one CTA of the set-up launch, beside the table CTAs, and no further launch
-// (npz <= 98).  The multi-CTA passes cost two more launches and their
-// grid-wide exchanges, which dominate at these sizes.
-constexpr int MU_SINGLE_MAX_PAIRS = 1300;
-constexpr int MU_SINGLE_MAX_H = 49;  // (h + 1)(h + 2) / 2 <= 1300
+// Zones small enough for the one-CTA solve: the whole search and the final step
+// in one CTA of the set-up launch, beside the table CTAs, and no further launch
+// (npz <= 160).  The multi-CTA passes cost two more launches and their
+// grid-wide exchanges (36 us in all at npz = 128, the one-CTA solve 25 us).
+constexpr int MU_SINGLE_MAX_H = 80;
+constexpr int MU_SINGLE_MAX_PAIRS = (MU_SINGLE_MAX_H + 1) * (MU_SINGLE_MAX_H + 2) / 2;   // 3321
 __host__ __device__ inline bool mu_single(const Geom &g)
 {
     const int h = g.npz / 2;
@@ -133,12 +135,30 @@ __device__ __forceinline__ double band_e0(const Band &b, const AxisTab &ax, cons
     return -2.0 * b.t * (ax.c1 + ay.c1) - 4.0 * b.tp * ax.c1 * ay.c1 - 2.0 * b.tpp * (ax.c2 + ay.c2);
 }
 
-// The same from FP64 class values (cos p, cos 2p, p^2 of the two axes).
-__device__ __forceinline__ double band_e0_cls(const Band &b, double c1a, double c1b, double c2a, double c2b,
-                                              double p2a, double p2b)
+__device__ __forceinline__ ClsTab class_values(int m, int npz)
 {
-    if (b.band_kind == 1) return 0.5 * (p2a + p2b);
-    return -2.0 * b.t * (c1a + c1b) - 4.0 * b.tp * c1a * c1b - 2.0 * b.tpp * (c2a + c2b);
+    auto pair = [](double v, float &hi, float &lo) {
+        hi = (float)v;
+        lo = (float)(v - (double)hi);
+    };
+    const double u = 2.0 * (double)m / (double)npz, p = u * 3.14159265358979323846;
+    ClsTab t;
+    t.c1 = cospi(u);
+    t.c2 = cospi(2.0 * u);
+    pair(t.c1, t.c1h, t.c1l);
+    pair(t.c2, t.c2h, t.c2l);
+    pair(p * p, t.p2h, t.p2l);
+    return t;
+}
+__global__ void k_classes(int npz, ClsTab *cls)
+{
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m <= npz / 2) cls[m] = class_values(m, npz);
+}
+cudaError_t launch_classes(int npz, ClsTab *cls, cudaStream_t s)
+{
+    k_classes<<<npz / 2 / 64 + 1, 64, 0, s>>>(npz, cls);
+    return cudaGetLastError();
 }
 
 // Pair index k in [0, (h+1)(h+2)/2) -> classes (a, b), 0 <= a <= b <= h, row
@@ -164,7 +184,6 @@ struct MuBracket {
     int wmin[MU_THREADS / 32];
     double lo, hi, step;
     int flag;
-    int wmin_done;   // one-CTA solve: the search has converged
 };
 struct MuShared {
     float c1[MU_MAXC], c2[MU_MAXC], p2[MU_MAXC];   // class values in FP32
@@ -291,140 +310,225 @@ __device__ __forceinline__ void sect_pass(const Geom &g, const Band &band, const
     (void)c0;
 }
 
-// One-CTA solve (mu_single): a bracketed Newton iteration in FP32 (each step
-// sums n and dn/dmu over the pairs, one or two per thread, in a fixed order;
-// a step that leaves the bracket, or a flat n, falls back to bisection) from
-// the full bracket until the step is below 1e-6 eV, then the FP64 Halley step
-// of k_mu_halley from there.  n is increasing, so the bracket always holds the
-// root; the first evaluation checks that both ends straddle the filling.
+// One-CTA solve (mu_single).
+//
+// 1. One multisection pass in FP32 over [-B - 3, B + 3], a warp a candidate
+//    (its lanes sum the pairs; no exchange but the candidates' totals), to a
+//    bracket of about 0.7 eV.
+// 2. A bracketed Halley iteration in FP32 over all threads, to 1e-6 eV (a step
+//    that leaves the bracket, or a flat n, falls back to bisection).
+// 3. One Halley step in twice FP32 precision.  The occupations' sum needs
+//    Theta = sum w atan(x_k), and that is the argument of prod (1 + i x_k)^w:
+//    the product is formed in unevaluated FP32 pairs (each factor scaled to
+//    modulus 1 by an FP32 factor, which leaves its argument), multiplied by
+//    e^{-i Theta_target} from the host, and the remaining angle, some 1e-2 at
+//    most after step 2, comes from three terms of its series: no arctangent,
+//    and no multiple of 2 pi to find.  The product's rounding is some 1e-12 of
+//    an electron state, 1e-15 eV; the step itself, below 1e-6 eV, is FP32.
+//
+// What bounds it is one SM's latency.  FP64 units are what it avoids: they
+// retire two operations a cycle and SM, so a warp's FP64 instruction takes 16
+// cycles whatever its lanes hold; the FP64 arctangents of the last step and the
+// cosines of the classes (now laid out once per plan) were most of the time.
+// Set-up and solve at npz = 64: 22.9 -> 14.4 us, mu within 2e-15 eV on average (9e-15 before; the product in FP64 by two
+// warps: 17 us, its errors no smaller).
 constexpr int MU_NEWTON_MAX = 64;    // bisection alone reaches 1e-6 eV in 24 steps
-__device__ void mu_solve_one_cta(const Geom &g, const Band &band, const MuConst &mc, MuShared &sh, InstState *st,
-                                 unsigned *status, double *mu_out)
+struct C2 { F2 r, i; };
+__device__ __forceinline__ F2 f2_div(F2 a, F2 b)
+{
+    const float q = a.h / b.h;
+    return f2_fast(q, (fmaf(-q, b.h, a.h) + a.l - q * b.l) / b.h);
+}
+__device__ __forceinline__ F2 f2_neg(F2 a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ C2 c2_mul(C2 a, C2 b)
+{
+    return {f2_add(f2_mul(a.r, b.r), f2_neg(f2_mul(a.i, b.i))), f2_add(f2_mul(a.r, b.i), f2_mul(a.i, b.r))};
+}
+__device__ __forceinline__ F2 f2_shfl(F2 a, int o)
+{
+    return {__shfl_down_sync(0xffffffffu, a.h, o), __shfl_down_sync(0xffffffffu, a.l, o)};
+}
+__device__ __forceinline__ C2 c2_shfl(C2 a, int o) { return {f2_shfl(a.r, o), f2_shfl(a.i, o)}; }
+struct MuSingle {
+    float2 ew[MU_SINGLE_MAX_PAIRS];            // (band energy, weight) of the pairs
+    F2 c1[MU_SINGLE_MAX_H + 1], c2[MU_SINGLE_MAX_H + 1], p2[MU_SINGLE_MAX_H + 1];   // cos p, cos 2p, p^2
+    float cnt[MU_THREADS / 32];                // totals of the first pass's candidates
+    float red[2][MU_THREADS / 32][3];          // warp sums of a Halley step
+    C2 z[MU_THREADS / 32];                     // warp products and sums of the last step
+    F2 n1[MU_THREADS / 32];
+    float d2[MU_THREADS / 32];
+};
+__device__ void mu_solve_one_cta(const Geom &g, const Band &band, const MuConst &mc, MuSingle &sh, InstState *st,
+                                 unsigned *status, double *mu_out, const ClsTab *__restrict__ cls)
 {
     constexpr int NW = MU_THREADS / 32;
-    // 8-byte scratch lives in sh.c1 (offset 0 of MuShared, so 8-byte aligned;
-    // sh.c2 and sh.p2 start at 4 mod 8): the per-warp sums of the search,
-    // then 3 (h + 1) class values and [NW][3] Halley sums
-    static_assert(offsetof(MuShared, c1) == 0 && alignof(MuShared) >= 8, "sh.c1 must be 8-byte aligned");
-    static_assert((3 * (MU_SINGLE_MAX_H + 1) + 3 * NW) * sizeof(double) <= sizeof(sh.c1) &&
-                      2 * NW * sizeof(float) <= sizeof(sh.c1),
-                  "scratch fits in the class table");
+    static_assert(NW == 16, "the first pass's totals fit one half warp");
     const int h = g.npz / 2, npairs = (h + 1) * (h + 2) / 2;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    stage_pairs(g, band, sh, 0, npairs);                        // npairs <= MU_CHUNK
-    if (threadIdx.x == 0) {
-        sh.br.lo = -mc.B - 3.0;
-        sh.br.hi = mc.B + 3.0;
-        sh.br.step = 0.0;                                       // the current estimate
-        sh.br.flag = 0;
+    const bool free_e = band.band_kind == 1;
+    for (int m = threadIdx.x; m <= h; m += MU_THREADS) {
+        const ClsTab c = cls ? cls[m] : class_values(m, g.npz);
+        sh.c1[m] = {c.c1h, c.c1l};
+        sh.c2[m] = {c.c2h, c.c2l};
+        sh.p2[m] = {c.p2h, c.p2l};
     }
     __syncthreads();
-    float *red = reinterpret_cast<float *>(sh.c1);             // [NW][2]
-    const float inv_gam = (float)mc.inv_gam, inv_pi = 0.318309886183790672f;
-    const float target = (float)mc.target;
-    // it = 0: n at both ends of the bracket; it >= 1: n and dn/dmu at the estimate
+    const float t = band.k1[0], tp = band.k2[0], tpp = band.k3[0];   // -2t, -4t', -2t''
+    for (int k = threadIdx.x; k < npairs; k += MU_THREADS) {
+        int a, b;
+        tri_pair(k, h, a, b);
+        const float e = free_e ? 0.5f * (sh.p2[a].h + sh.p2[b].h)
+                               : t * (sh.c1[a].h + sh.c1[b].h) + tp * sh.c1[a].h * sh.c1[b].h
+                                     + tpp * (sh.c2[a].h + sh.c2[b].h);
+        sh.ew[k] = make_float2(e, (float)pair_weight(a, b, h));
+    }
+    __syncthreads();
+
+    const float ig = mc.igh, inv_pi = 0.318309886183790672f, target = mc.target_f;
+    float lo = -mc.Bf - 3.0f, hi = mc.Bf + 3.0f;
+    {
+        const float dc = (hi - lo) / (float)(NW - 1), c = lo + (float)warp * dc;
+        float s0 = 0.f, s1 = 0.f;
+        int k = lane;
+        for (; k + 32 < npairs; k += 64) {
+            const float2 x = sh.ew[k], y = sh.ew[k + 32];
+            s0 += x.y * (0.5f - atanf((x.x - c) * ig) * inv_pi);
+            s1 += y.y * (0.5f - atanf((y.x - c) * ig) * inv_pi);
+        }
+        if (k < npairs) s0 += sh.ew[k].y * (0.5f - atanf((sh.ew[k].x - c) * ig) * inv_pi);
+        s0 += s1;
+        for (int o = 16; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+        if (lane == 0) sh.cnt[warp] = s0;
+        __syncthreads();
+        const unsigned hit = __ballot_sync(0xffffffffu, lane < NW && sh.cnt[lane % NW] >= target);
+        const int first = hit ? __ffs((int)hit) - 1 : NW;   // the first candidate that reaches the filling
+        if (first == 0 || first == NW) {                     // the filling is not bracketed
+            if (threadIdx.x == 0) {
+                const double mu = 0.5 * ((double)lo + (double)hi);
+                atomicCAS(status, (unsigned)DEV_OK, (unsigned)DEV_ENOCONV);
+                set_mu(st, mu);
+                st->last_step = INFINITY;
+                if (mu_out) *mu_out = mu;
+            }
+            return;
+        }
+        hi = lo + (float)first * dc;
+        lo += (float)(first - 1) * dc;
+    }
+    float mu = 0.5f * (lo + hi), mu_l = 0.f;   // the estimate; mu_l: what its last rounding dropped
     for (int it = 0; it < MU_NEWTON_MAX; ++it) {
-        const float m0 = (float)(it == 0 ? sh.br.lo : sh.br.step), m1 = (float)sh.br.hi;
-        float n0 = 0.f, n1 = 0.f;   // it = 0: n(lo), n(hi); else n(mu), gamma dn/dmu
+        float n0 = 0.f, n1 = 0.f, n2 = 0.f;   // n(mu), gamma n', gamma^2 n''
         for (int k = threadIdx.x; k < npairs; k += MU_THREADS) {
             const float2 ew = sh.ew[k];
-            const float x = (ew.x - m0) * inv_gam;
+            const float x = (ew.x - mu) * ig, r = __fdividef(1.0f, 1.0f + x * x);
             n0 += ew.y * (0.5f - atanf(x) * inv_pi);
-            if (it == 0) n1 += ew.y * (0.5f - atanf((ew.x - m1) * inv_gam) * inv_pi);
-            else n1 += ew.y * (inv_pi / (1.0f + x * x));
+            n1 += ew.y * r;
+            n2 += ew.y * 2.0f * x * r * r;
         }
         for (int o = 16; o > 0; o >>= 1) {
-            n0 += __shfl_down_sync(0xffffffffu, n0, o);
-            n1 += __shfl_down_sync(0xffffffffu, n1, o);
+            n0 += __shfl_xor_sync(0xffffffffu, n0, o);
+            n1 += __shfl_xor_sync(0xffffffffu, n1, o);
+            n2 += __shfl_xor_sync(0xffffffffu, n2, o);
         }
-        if (lane == 0) { red[2 * warp] = n0; red[2 * warp + 1] = n1; }
-        __syncthreads();
-        int done = 0;
-        if (threadIdx.x == 0) {
-            float N0 = 0.f, N1 = 0.f;
-            for (int w = 0; w < NW; ++w) { N0 += red[2 * w]; N1 += red[2 * w + 1]; }
-            if (it == 0) {
-                if (!(N0 < target && N1 >= target)) { sh.br.flag = 1; done = 1; }   // not bracketed
-                sh.br.step = 0.5 * (sh.br.lo + sh.br.hi);
-            } else {
-                // FP32 step (an FP64 division costs some 450 cycles on this critical path)
-                const double mu = sh.br.step;
-                const float F = N0 - target, slope = N1 * inv_gam;   // n - target, dn/dmu
-                if (F < 0.f) sh.br.lo = mu; else sh.br.hi = mu;
-                double nxt = slope > 0.f ? mu - (double)(F / slope) : sh.br.lo - 1.0;
-                if (!(nxt > sh.br.lo && nxt < sh.br.hi)) nxt = 0.5 * (sh.br.lo + sh.br.hi);
-                done = fabs(nxt - mu) < 1e-6 || sh.br.hi - sh.br.lo < 1e-6;
-                sh.br.step = nxt;
-            }
-            sh.br.wmin_done = done;
+        if (lane == 0) {
+            sh.red[it & 1][warp][0] = n0;
+            sh.red[it & 1][warp][1] = n1;
+            sh.red[it & 1][warp][2] = n2;
         }
         __syncthreads();
-        if (sh.br.wmin_done) break;
-    }
-    const double mu = sh.br.step;
-    if (sh.br.flag) {   // the filling was not bracketed
-        if (threadIdx.x == 0) {
-            atomicCAS(status, (unsigned)DEV_OK, (unsigned)DEV_ENOCONV);
-            set_mu(st, mu);
-            st->last_step = INFINITY;
-            if (mu_out) *mu_out = mu;
+        n0 = sh.red[it & 1][lane % NW][0];   // every warp adds the 16 sums in the same order
+        n1 = sh.red[it & 1][lane % NW][1];
+        n2 = sh.red[it & 1][lane % NW][2];
+        for (int o = 8; o > 0; o >>= 1) {
+            n0 += __shfl_xor_sync(0xffffffffu, n0, o);
+            n1 += __shfl_xor_sync(0xffffffffu, n1, o);
+            n2 += __shfl_xor_sync(0xffffffffu, n2, o);
         }
-        return;
+        const float F = n0 - target, a1 = n1 * inv_pi * ig, a2 = n2 * inv_pi * ig * ig;   // n - target, n', n''
+        if (F < 0.f) lo = mu; else hi = mu;
+        const float den = 2.0f * a1 * a1 - F * a2;
+        // Halley, or Newton far from the root
+        const float dx = a1 > 0.f ? (den > a1 * a1 ? 2.0f * F * a1 / den : F / a1) : INFINITY;
+        float nxt = mu - dx;
+        mu_l = (mu - nxt) - dx;   // exact near the root (|dx| < |mu|), and below 1e-7 eV else
+        if (!(nxt > lo && nxt < hi)) {
+            nxt = 0.5f * (lo + hi);
+            mu_l = 0.f;
+        }
+        const bool done = fabsf(nxt - mu) < 1e-6f || hi - lo < 1e-6f;
+        mu = nxt;
+        if (done) break;
     }
-    // FP64 class values, the same expressions as the axis tables at p_i = -2 pi m / npz
-    // (in sh.c1, the one 8-byte aligned scratch of MuShared; the search sums are consumed)
-    double *d1 = reinterpret_cast<double *>(sh.c1), *d2 = d1 + (h + 1), *dp = d2 + (h + 1);
-    for (int m = threadIdx.x; m <= h; m += blockDim.x) {
-        const double u = 2.0 * (double)(-m) / (double)g.npz;
-        const double p = u * 3.14159265358979323846;
-        d1[m] = cospi(u);
-        d2[m] = cospi(2.0 * u);
-        dp[m] = p * p;
-    }
-    __syncthreads();
-    const double igam = mc.inv_gam, ipi = 0.31830988618379067154;
-    double f = 0.0;
-    float f1 = 0.f, f2 = 0.f;
-    for (int k = threadIdx.x; k < npairs; k += blockDim.x) {
+
+    // the last step, from mu + mu_l
+    if (!(fabsf(mu_l) < 1e-6f)) mu_l = 0.f;
+    const F2 igp{mc.igh, mc.igl}, mm = f2_fast(-mu, -mu_l);
+    const F2 k1{band.k1[0], band.k1[1]}, k2{band.k2[0], band.k2[1]}, k3{band.k3[0], band.k3[1]};
+    const F2 one{1.f, 0.f}, nil{0.f, 0.f};
+    C2 z8{one, nil}, z4{one, nil}, z1{one, nil};   // products of the factors of weight 8, 4, and 1 or 2
+    float d1 = 0.f, d2 = 0.f;
+    for (int k = threadIdx.x; k < npairs; k += MU_THREADS) {
         int a, b;
         tri_pair(k, h, a, b);
         const int w = pair_weight(a, b, h);
-        const double x = (band_e0_cls(band, d1[a], d1[b], d2[a], d2[b], dp[a], dp[b]) - mu) * igam;
-        f += (double)w * (0.5 - atan(x) * ipi);
-        const float xf = (float)x, r = 1.0f / (1.0f + xf * xf);
-        f1 += (float)w * r * (float)ipi;
-        f2 += (float)w * 2.0f * xf * r * r * (float)ipi;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        f += __shfl_down_sync(0xffffffffu, f, o);
-        f1 += __shfl_down_sync(0xffffffffu, f1, o);
-        f2 += __shfl_down_sync(0xffffffffu, f2, o);
-    }
-    double *hs = dp + (h + 1);   // [NW][3], after the class values
-    if (lane == 0) { hs[3 * warp] = f; hs[3 * warp + 1] = f1; hs[3 * warp + 2] = f2; }
-    __syncthreads();
-    if (warp == 0) {
-        // the NW warp sums by a shuffle tree (a chain of NW dependent FP64 adds
-        // would cost some 60 cycles each)
-        double F = lane < NW ? hs[3 * lane] : 0.0, F1 = lane < NW ? hs[3 * lane + 1] : 0.0,
-               F2 = lane < NW ? hs[3 * lane + 2] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) {
-            F += __shfl_down_sync(0xffffffffu, F, o);
-            F1 += __shfl_down_sync(0xffffffffu, F1, o);
-            F2 += __shfl_down_sync(0xffffffffu, F2, o);
+        F2 e0;
+        if (free_e) {
+            e0 = f2_add(sh.p2[a], sh.p2[b]);
+            e0.h *= 0.5f;
+            e0.l *= 0.5f;
+        } else {
+            e0 = f2_add(f2_add(f2_mul(k1, f2_add(sh.c1[a], sh.c1[b])), f2_mul(k2, f2_mul(sh.c1[a], sh.c1[b]))),
+                        f2_mul(k3, f2_add(sh.c2[a], sh.c2[b])));
         }
-        if (lane != 0) return;
-        const double d = F - mc.target;
-        const double dd1 = F1 * igam, dd2 = F2 * igam * igam;
-        const double stp = 2.0 * d * dd1 / (2.0 * dd1 * dd1 - d * dd2);
-        const double mu_new = mu - stp;
-        set_mu(st, mu_new);
-        st->last_step = fabs(stp);
-        if (mu_out) *mu_out = mu_new;
-        // the FP32 search stops within about 1e-6 eV of the root: a larger
-        // FP64 correction means it went wrong
-        if (!(fabs(stp) <= 1e-4)) atomicCAS(status, (unsigned)DEV_OK, (unsigned)DEV_ENOCONV);
+        const F2 x = f2_mul(f2_add(e0, mm), igp);
+        const float q = 1.0f + x.h * x.h, s = rsqrtf(q), r = 1.0f / q;
+        const C2 f{{s, 0.f}, f2_mul(x, F2{s, 0.f})};
+        if (w == 8) z8 = c2_mul(z8, f);
+        else if (w == 4) z4 = c2_mul(z4, f);
+        else z1 = c2_mul(z1, w == 2 ? c2_mul(f, f) : f);
+        d1 += (float)w * r;                       // pi gamma n'
+        d2 += (float)w * 2.0f * x.h * r * r;      // pi gamma^2 n''
     }
+    C2 z = c2_mul(z4, c2_mul(z8, z8));   // (z4 z8^2)^4 z1
+    z = c2_mul(z, z);
+    z = c2_mul(c2_mul(z, z), z1);
+    F2 n1{d1, 0.f};   // the slope divides the step: its tree is summed as a pair
+    for (int o = 16; o > 0; o >>= 1) {
+        z = c2_mul(z, c2_shfl(z, o));
+        n1 = f2_add(n1, f2_shfl(n1, o));
+        d2 += __shfl_down_sync(0xffffffffu, d2, o);
+    }
+    if (lane == 0) { sh.z[warp] = z; sh.n1[warp] = n1; sh.d2[warp] = d2; }
+    __syncthreads();
+    if (warp != 0) return;
+    z = lane < NW ? sh.z[lane] : C2{one, nil};
+    n1 = lane < NW ? sh.n1[lane] : nil;
+    d2 = lane < NW ? sh.d2[lane] : 0.f;
+    for (int o = 8; o > 0; o >>= 1) {
+        z = c2_mul(z, c2_shfl(z, o));
+        n1 = f2_add(n1, f2_shfl(n1, o));
+        d2 += __shfl_down_sync(0xffffffffu, d2, o);
+    }
+    if (lane != 0) return;
+    z = c2_mul(z, C2{{mc.cth, mc.ctl}, {-mc.sth, -mc.stl}});
+    // the angle left, Theta - Theta_target = -pi (n - target), and the step, as
+    // pairs where they scale the result
+    const F2 tn = f2_div(z.i, z.r);
+    const float t2 = tn.h * tn.h;
+    F2 ang = f2_fast(tn.h, tn.l - tn.h * t2 * (1.0f / 3.0f - t2 * (0.2f - t2 * (1.0f / 7.0f))));
+    if (!(fabsf(tn.h) <= 0.1f) || !(z.r.h > 0.f)) ang = {atan2f(z.i.h, z.r.h), 0.f};   // not after a search that converged
+    const F2 a1 = f2_mul(n1, igp);                                       // pi n'
+    const float eps = ang.h * d2 / (2.0f * n1.h * n1.h);                     // -(n - target) n'' / (2 n'^2)
+    const F2 step = f2_mul(f2_div(ang, a1), F2{1.0f, -eps / (1.0f + eps)});   // -step: Halley's 1 / (1 + eps)
+    const F2 m = f2_add(f2_neg(mm), step);
+    const float stp = step.h;
+    const double mu_new = (double)m.h + (double)m.l;
+    set_mu(st, mu_new);
+    st->last_step = fabs((double)stp);
+    if (mu_out) *mu_out = mu_new;
+    // the FP32 search stops within about 1e-6 eV of the root: a larger
+    // correction means it went wrong
+    if (!(fabsf(stp) <= 1e-4f)) atomicCAS(status, (unsigned)DEV_OK, (unsigned)DEV_ENOCONV);
 }
 
 // Set-up launch.  CTAs [0, G): multisection pass 0 (mu from the filling);
@@ -433,7 +537,8 @@ __device__ void mu_solve_one_cta(const Geom &g, const Band &band, const MuConst 
 // and the first of them records the given mu.
 __global__ void __launch_bounds__(MU_THREADS, 2)
 k_setup(Geom g, Band band, AxisTab *axis, float2 *eps32, double *eps64, InstState *st, double *acc,
-        unsigned *counter, unsigned *status, double *mu_out, MuConst mc, int G, Band *band_out)
+        unsigned *counter, unsigned *status, double *mu_out, MuConst mc, int G, Band *band_out,
+        const ClsTab *__restrict__ cls)
 {
     if (band_out && blockIdx.x == 0 && threadIdx.x == 0) *band_out = band;   // the call's band, for later launches
     if ((int)blockIdx.x >= G) {
@@ -446,17 +551,18 @@ k_setup(Geom g, Band band, AxisTab *axis, float2 *eps32, double *eps64, InstStat
         const int i = tb * MU_TAB_THREADS + threadIdx.x;
         if (threadIdx.x >= MU_TAB_THREADS) return;
         if (i < g.N) {
-            double u = 2.0 * (double)(i - g.N / 2) / (double)g.npz;   // p_i / pi
-            double p = u * 3.14159265358979323846;
+            const int k = i - g.N / 2, r = (k < 0 ? -k : k) % g.npz, m = 2 * r > g.npz ? g.npz - r : r;   // its class
+            const ClsTab c = cls ? cls[m] : class_values(m, g.npz);
+            const double p = (double)k * g.dp;
             AxisTab a;
-            a.c1 = cospi(u);
-            a.c2 = cospi(2.0 * u);
-            a.g = (band.ff_a == 0.0) ? 1.0 : exp(-p * p * band.ff_a * band.ff_a / 8.0);
+            a.c1 = c.c1;
+            a.c2 = c.c2;
+            a.g = (band.ff_a == 0.0) ? 1.0 : exp(-p * p * (band.ff_a * band.ff_a * 0.125));
             a.p2 = p * p;
-            a.c1h = (float)a.c1;
-            a.c1l = (float)(a.c1 - (double)a.c1h);
-            a.c2h = (float)a.c2;
-            a.c2l = (float)(a.c2 - (double)a.c2h);
+            a.c1h = c.c1h;
+            a.c1l = c.c1l;
+            a.c2h = c.c2h;
+            a.c2l = c.c2l;
             a.p2h = (float)a.p2;
             a.p2l = (float)(a.p2 - (double)a.p2h);
             a.gf = (float)a.g;
@@ -473,13 +579,17 @@ k_setup(Geom g, Band band, AxisTab *axis, float2 *eps32, double *eps64, InstStat
         }
         return;
     }
-    __shared__ MuShared sh;
-    stage_classes(g, sh);
+    __shared__ union Scratch {
+        MuShared sect;
+        MuSingle single;
+        __device__ Scratch() {}
+    } u;
     if (mc.single) {
-        __syncthreads();
-        mu_solve_one_cta(g, band, mc, sh, st, status, mu_out);
+        mu_solve_one_cta(g, band, mc, u.single, st, status, mu_out, cls);
         return;
     }
+    MuShared &sh = u.sect;
+    stage_classes(g, sh);
     if (threadIdx.x == 0) {
         sh.br.lo = -mc.B - 3.0;
         sh.br.hi = mc.B + 3.0;
@@ -639,7 +749,18 @@ static MuConst mu_const(const Geom &g, const Band &band, int G)
     mc.inv_gam = 1.0 / band.gamma;
     mc.target = band.filling * 0.5 * (double)g.npz * (double)g.npz;
     mc.target32 = llrint(mc.target * (double)MU_SECT_SCALE);
+    mc.target_f = (float)mc.target;
+    auto pair = [](double v, float &hi, float &lo) {
+        hi = (float)v;
+        lo = (float)(v - (double)hi);
+    };
+    pair(mc.inv_gam, mc.igh, mc.igl);
+    // e^{i pi u}, u = npz^2 / 2 - target
+    const double u = fmod(0.5 * (double)g.npz * (double)g.npz - mc.target, 2.0);
+    pair(cos(M_PI * u), mc.cth, mc.ctl);
+    pair(sin(M_PI * u), mc.sth, mc.stl);
     mc.B = (band.band_kind == 1) ? 9.869604401089358 : 4.0 * (fabs(band.t) + fabs(band.tp) + fabs(band.tpp));
+    mc.Bf = (float)mc.B;
     return mc;
 }
 
@@ -652,22 +773,23 @@ cudaError_t launch_twiddles(int len, float2 *tw32, double2 *tw64, cudaStream_t s
 // Tables plus the first chemical-potential launch (multisection pass 0, or
 // the given mu).
 // band_out (device, or null): receives the call's band for later launches.
+// cls: the zone's class table (k_classes), or null: formed in the launch.
 cudaError_t launch_setup_band(const Geom &g, const Band &band, AxisTab *axis, float2 *eps32, double *eps64,
                               InstState *st, double *acc, unsigned *bar, unsigned *status, double *mu_out, int G,
-                              Band *band_out, cudaStream_t s)
+                              Band *band_out, const ClsTab *cls, cudaStream_t s)
 {
     const int ntab = g.N > g.n_eps ? g.N : g.n_eps;
     const int GT = (ntab + MU_TAB_THREADS - 1) / MU_TAB_THREADS;
     const int Gs = band.solve_mu ? (mu_single(g) ? 1 : G) : 0;
     k_setup<<<Gs + GT, MU_THREADS, 0, s>>>(g, band, axis, eps32, eps64, st, acc, bar, status, mu_out,
-                                           mu_const(g, band, G), Gs, band_out);
+                                           mu_const(g, band, G), Gs, band_out, cls);
     return cudaGetLastError();
 }
 cudaError_t launch_setup(const Geom &g, const Band &band, AxisTab *axis, float2 *eps32, double *eps64,
                          InstState *st, double *acc, unsigned *bar, unsigned *status, double *mu_out, int G,
-                         cudaStream_t s)
+                         const ClsTab *cls, cudaStream_t s)
 {
-    return launch_setup_band(g, band, axis, eps32, eps64, st, acc, bar, status, mu_out, G, nullptr, s);
+    return launch_setup_band(g, band, axis, eps32, eps64, st, acc, bar, status, mu_out, G, nullptr, cls, s);
 }
 
 // Whether the chemical potential is solved inside the set-up launch.

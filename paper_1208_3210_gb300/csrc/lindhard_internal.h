@@ -101,6 +101,13 @@ struct AxisTab {
     float c1h, c1l, c2h, c2l, p2h, p2l, gf, pad;
 };
 
+// Momentum class m in [0, npz / 2] of a zone, p = 2 pi m / npz: what the axis
+// tables and the chemical potential need of it, laid out once per plan.
+struct ClsTab {
+    double c1, c2;                       // cos p, cos 2p
+    float c1h, c1l, c2h, c2l, p2h, p2l;  // the same and p^2 as FP32 pairs
+};
+
 // Workspace of one instance (device pointers into the plan's allocation).
 template <typename Real>
 struct Work {
@@ -114,6 +121,7 @@ struct Work {
     const void *ptw = nullptr;   // per-stage twiddle tables of the pruned engine (FP32), or null
     const void *etw = nullptr;   // per-stage twiddle tables of the lines-across-lanes energy pass, or null
     const void *evt = nullptr;   // tables of the even form's cosine transforms (FP32), or null
+    const ClsTab *cls = nullptr;  // the zone's class table, or null
     InstState *state;      // [1]
     unsigned *status;      // plan-wide device status word
     double *mu_acc;        // scratch for the chemical potential solve

@@ -25,7 +25,8 @@ namespace lh {
 cudaError_t launch_twiddles(int len, float2 *tw32, double2 *tw64, cudaStream_t s);
 cudaError_t launch_setup(const Geom &g, const Band &band, AxisTab *axis, float2 *eps32, double *eps64,
                          InstState *st, double *acc, unsigned *bar, unsigned *status, double *mu_out, int G,
-                         cudaStream_t s);
+                         const ClsTab *cls, cudaStream_t s);
+cudaError_t launch_classes(int npz, ClsTab *cls, cudaStream_t s);
 size_t mu_acc_doubles(int G);
 size_t mu_barrier_words();
 int mu_grid_size(int num_sms, int npts);
@@ -92,7 +93,7 @@ cudaError_t launch_persistent(const void *insts, const void *segs, int nsegs, in
                               unsigned long long wait_ns, int stall_inst, int smem_elems, int grid, cudaStream_t s);
 cudaError_t launch_setup_band(const Geom &g, const Band &band, AxisTab *axis, float2 *eps32, double *eps64,
                               InstState *st, double *acc, unsigned *bar, unsigned *status, double *mu_out, int G,
-                              Band *band_out, cudaStream_t s);
+                              Band *band_out, const ClsTab *cls, cudaStream_t s);
 cudaError_t launch_tc_mats(void *buf, cudaStream_t s);
 cudaError_t launch_inv_y(const Geom &g, const Work<double> &w, cudaStream_t s, int variant);
 cudaError_t launch_inv_energy(const Geom &g, const Work<float> &w, float *out, cudaStream_t s, int variant);
@@ -168,6 +169,7 @@ struct lindhard_plan {
     size_t off_tw32 = 0, off_tw64 = 0, off_status = 0, off_tc = 0, off_dmu = 0, off_prtw = 0, off_etw = 0, off_evt = 0;
     // the even form's geometry of each instance (even.cuh); M = 0: not taken
     std::vector<EvGeom> even;
+    std::vector<size_t> off_cls;  // momentum class tables per instance (one for all instances of as many points per zone)
     std::vector<size_t> off_kk;   // Kramers-Kronig weight tables per instance (FP32 grids)
     int tw_len = 0;
     bool backward = false;       // LINDHARD_PLAN_BACKWARD
@@ -604,6 +606,12 @@ extern "C" lindhard_status lindhard_plan_create(const lindhard_grid *grids, int 
         p->off_ps_cnt = o; o = align_up(o + sizeof(unsigned) * (5 * batch + 1));
         p->off_ps_band = o; o = align_up(o + sizeof(Band) * batch);
     }
+    p->off_cls.assign(batch, 0);
+    for (int i = 0; i < batch; ++i) {
+        for (int k = 0; k < i && !p->off_cls[i]; ++k)
+            if (p->geoms[k].npz == p->geoms[i].npz) p->off_cls[i] = p->off_cls[k];
+        if (!p->off_cls[i]) { p->off_cls[i] = o; o = align_up(o + sizeof(ClsTab) * (p->geoms[i].npz / 2 + 1)); }
+    }
     p->off_kk.assign(batch, 0);
     for (int i = 0; i < batch; ++i)
         if (p->precision[i] != LINDHARD_FP64) {
@@ -653,6 +661,9 @@ extern "C" lindhard_status lindhard_plan_create(const lindhard_grid *grids, int 
     if (e == cudaSuccess) e = launch_pr_twiddles((float2 *)(p->ws + p->off_prtw), 0);
     if (e == cudaSuccess) e = launch_et_twiddles((float2 *)(p->ws + p->off_etw), 0);
     if (e == cudaSuccess) e = launch_ev_tables((float2 *)(p->ws + p->off_evt), 0);
+    for (int i = 0; i < batch && e == cudaSuccess; ++i)
+        if (std::find(p->off_cls.begin(), p->off_cls.begin() + i, p->off_cls[i]) == p->off_cls.begin() + i)
+            e = launch_classes(p->geoms[i].npz, (ClsTab *)(p->ws + p->off_cls[i]), 0);
     if (e == cudaSuccess && p->off_tc) e = launch_tc_mats(p->ws + p->off_tc, 0);
     for (int i = 0; i < batch && e == cudaSuccess; ++i)
         if (p->off_kk[i] && std::find(p->off_kk.begin(), p->off_kk.begin() + i, p->off_kk[i]) == p->off_kk.begin() + i)
@@ -747,7 +758,7 @@ extern "C" lindhard_status lindhard_plan_sizes(const lindhard_plan *p, int index
     long long W4 = (long long)g.Q * g.Q * g.H;
     out->hbm_bytes_forward = 2 * (W1 + W2 + W3 + W4) * cb + out->out_elems * rb;
     // set-up (tables + multisection pass 0), multisection pass 1, Halley step, 5 FFT passes;
-    // zones of at most 98 points solve mu inside the set-up launch
+    // zones of at most 160 points solve mu inside the set-up launch
     out->kernels_forward = mu_solve_in_setup(g) ? 6 : 8;
     // persistent plans: the instance's set-up launches (the batch's passes
     // are one further launch of the plan)
@@ -853,6 +864,7 @@ static Work<Real> work_of(lindhard_plan *p, int i)
     w.evt = sizeof(Real) == 4 ? (const void *)(p->ws + p->off_evt) : nullptr;
     w.state = (InstState *)(p->ws + sl.state);
     w.status = (unsigned *)(p->ws + p->off_status);
+    w.cls = (const ClsTab *)(p->ws + p->off_cls[i]);
     w.mu_acc = (double *)(p->ws + sl.acc);
     w.barrier = (unsigned *)(p->ws + sl.bar);
     return w;
@@ -924,7 +936,7 @@ static cudaError_t enqueue_persistent(lindhard_plan *p, const std::vector<Band> 
         cudaStream_t s = inst_stream(p, i, s0);
         Work<float> w = work_of<float>(p, i);
         e = launch_setup_band(g, bs[i], w.axis, (float2 *)w.eps, nullptr, w.state, w.mu_acc, w.barrier, w.status,
-                              mu_out ? mu_out + i : nullptr, p->mu_G, (Band *)(p->ws + p->off_ps_band) + i, s);
+                              mu_out ? mu_out + i : nullptr, p->mu_G, (Band *)(p->ws + p->off_ps_band) + i, w.cls, s);
         if (e == cudaSuccess)
             e = launch_solve_mu(g, bs[i], w.axis, w.state, w.mu_acc, w.barrier, w.status, mu_out ? mu_out + i : nullptr,
                                 p->mu_G, s);
@@ -957,7 +969,7 @@ static cudaError_t enqueue_forward(lindhard_plan *p, const std::vector<Band> &bs
             e = timed(p, 0, s, [&] {
                 return launch_setup(g, b, w.axis, sizeof(Real) == 4 ? (float2 *)w.eps : nullptr,
                                     sizeof(Real) == 8 ? (double *)w.eps : nullptr, w.state, w.mu_acc, w.barrier,
-                                    w.status, mu_out ? mu_out + i : nullptr, p->mu_G, s);
+                                    w.status, mu_out ? mu_out + i : nullptr, p->mu_G, w.cls, s);
             });
             if (e == cudaSuccess)
                 e = timed(p, 1, s, [&] {
@@ -1110,7 +1122,7 @@ extern "C" lindhard_status lindhard_imchi_backward(lindhard_plan *p, const lindh
         cudaError_t e = cudaSuccess;
         if (A_in == nullptr) {
             e = launch_setup(g, b, wk.axis, (float2 *)wk.eps, nullptr, wk.state, wk.mu_acc, wk.barrier, wk.status,
-                             nullptr, p->mu_G, s);
+                             nullptr, p->mu_G, wk.cls, s);
             if (e == cudaSuccess)
                 e = launch_solve_mu(g, b, wk.axis, wk.state, wk.mu_acc, wk.barrier, wk.status, nullptr, p->mu_G, s);
         }
@@ -1169,7 +1181,7 @@ extern "C" lindhard_status lindhard_sum_rule(lindhard_plan *p, int index, const 
     cudaError_t e = cudaSuccess;
     if (A_in == nullptr) {
         e = launch_setup(g, b, w.axis, (float2 *)w.eps, nullptr, w.state, w.mu_acc, w.barrier, w.status, nullptr,
-                         p->mu_G, s);
+                         p->mu_G, w.cls, s);
         if (e == cudaSuccess)
             e = launch_solve_mu(g, b, w.axis, w.state, w.mu_acc, w.barrier, w.status, nullptr, p->mu_G, s);
     }

@@ -27,6 +27,8 @@ k_ev_corr(Geom g, EvGeom v, Band band, const float *__restrict__ B2, float *__re
     constexpr int VPT = E::VPT, TPL = E::TPL, R0 = E::R0, R1 = E::R1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(EVC_WARPS * E::WARP_ELEMS + (THERMAL ? L : 0), float2)
+    allow_next();
+    after_previous();
     const int lane = (int)threadIdx.x % 32, warp = (int)threadIdx.x / 32;
     const int sl = lane / TPL, u = lane % TPL;
     float2 *sm = reinterpret_cast<float2 *>(smem_raw) + warp * E::WARP_ELEMS + sl * E::LP;
@@ -138,6 +140,8 @@ k_ev_corr3(Geom g, EvGeom v, Band band, const float *__restrict__ B2, float *__r
     static_assert(S0 == R2 && VPT == 2 * S0, "the product stays in registers");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(EVC_WARPS * LPI * LP + (THERMAL ? L : 0), float2)
+    allow_next();
+    after_previous();
     const int lane = (int)threadIdx.x % 32, warp = (int)threadIdx.x / 32;
     const int sl = lane / TPL, u = lane % TPL;
     float2 *sm = reinterpret_cast<float2 *>(smem_raw) + (warp * LPI + sl) * LP;
@@ -316,10 +320,9 @@ cudaError_t launch_ev_corr_t(const Geom &g, const EvGeom &v, const Band &band, c
     if (e != cudaSuccess) return e;
     const int npairs = v.M / 2 * (v.M + 1) / 2, iters = ev_corr_iters(npairs, E::LPI, sms);
     const int per = EVC_WARPS * iters * E::LPI;
-    k_ev_corr<L, FULL, THERMAL, HALF><<<(npairs + per - 1) / per, 32 * EVC_WARPS, smem, s>>>(
-        g, v, band, (const float *)w.Y, (float *)w.X, (const float2 *)w.evt + ev_line_table<L>(), iters,
-        g.quantity == LINDHARD_IMCHI_T);
-    return cudaGetLastError();
+    return launch_after(k_ev_corr<L, FULL, THERMAL, HALF>, (npairs + per - 1) / per, 32 * EVC_WARPS, smem, s, g, v, band,
+                        (const float *)w.Y, (float *)w.X, (const float2 *)w.evt + ev_line_table<L>(), iters,
+                        g.quantity == LINDHARD_IMCHI_T);
 }
 template <int L>
 cudaError_t launch_ev_corr_l(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, int sms,
@@ -343,9 +346,9 @@ cudaError_t launch_ev_corr3(const Geom &g, const EvGeom &v, const Band &band, co
     if (e != cudaSuccess) return e;
     const int npairs = v.M / 2 * (v.M + 1) / 2, iters = ev_corr_iters(npairs, LPI, sms);
     const int per = EVC_WARPS * iters * LPI;
-    k_ev_corr3<L, false, THERMAL><<<(npairs + per - 1) / per, 32 * EVC_WARPS, smem, s>>>(
-        g, v, band, (const float *)w.Y, (float *)w.X, (const float2 *)w.etw, iters, g.quantity == LINDHARD_IMCHI_T);
-    return cudaGetLastError();
+    return launch_after(k_ev_corr3<L, false, THERMAL>, (npairs + per - 1) / per, 32 * EVC_WARPS, smem, s, g, v, band,
+                        (const float *)w.Y, (float *)w.X, (const float2 *)w.etw, iters,
+                        g.quantity == LINDHARD_IMCHI_T);
 }
 cudaError_t launch_ev_corr(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, int sms,
                            cudaStream_t s)

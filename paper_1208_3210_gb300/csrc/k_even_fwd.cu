@@ -57,6 +57,7 @@ cudaError_t launch_ev_tables(float2 *out, cudaStream_t s)
     for (int i = 0; ev_line_len(i) != 0; ++i) tabs.t[n++] = {(o + 1) / 2 * 2 + 128 * i, 128, -1, ev_line_len(i)};
     k_ev_tables<<<dim3(n, 4), 128, 0, s>>>(out, tabs);
     return cudaGetLastError();
+    return cudaGetLastError();
 }
 size_t ev_table_bytes() { return (size_t)ev_all_tables() * sizeof(float2); }
 
@@ -70,6 +71,8 @@ k_ev_gen_y(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const 
     constexpr int C = F::C, T = F::T, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(F::SMEM_ELEMS, float4)
+    allow_next();
+    after_previous();
     float4 *sm = reinterpret_cast<float4 *>(smem_raw);
     const int jx = blockIdx.x / ntile, ct = blockIdx.x % ntile;
     const int col = threadIdx.x % C, u = threadIdx.x / C;
@@ -142,6 +145,8 @@ k_ev_x(int rows, int RS, long long sp, long long dp, const float *__restrict__ B
     constexpr int C = F::C, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(F::SMEM_ELEMS, float4)
+    allow_next();
+    after_previous();
     float4 *sm = reinterpret_cast<float4 *>(smem_raw);
     const int ky = blockIdx.x / ntile, ct = blockIdx.x % ntile;
     const int col = threadIdx.x % C, u = threadIdx.x / C;
@@ -180,9 +185,8 @@ cudaError_t launch_ev_gen_y_t(const Geom &g, const EvGeom &v, const Band &band, 
     static const cudaError_t e = smem_attrs(k_ev_gen_y<M>, smem);
     if (e != cudaSuccess) return e;
     const int ntile = (v.ES + 4 * EvCfg<M>::C - 1) / (4 * EvCfg<M>::C);
-    k_ev_gen_y<M><<<v.Nh * ntile, EvCfg<M>::T, smem, s>>>(g, v, band, w.axis, (const float2 *)w.eps, w.state,
-                                                          (float *)w.X, (const float2 *)w.evt, ntile);
-    return cudaGetLastError();
+    return launch_after(k_ev_gen_y<M>, v.Nh * ntile, EvCfg<M>::T, smem, s, g, v, band, w.axis, (const float2 *)w.eps,
+                        w.state, (float *)w.X, (const float2 *)w.evt, ntile);
 }
 template <int M, bool TRI>
 cudaError_t launch_ev_x_t(int rows, int RS, long long sp, long long dp, const float *src, float *dst,
@@ -192,8 +196,8 @@ cudaError_t launch_ev_x_t(int rows, int RS, long long sp, long long dp, const fl
     static const cudaError_t e = smem_attrs(k_ev_x<M, TRI>, smem);
     if (e != cudaSuccess) return e;
     const int ntile = (RS + 4 * EvCfg<M>::C - 1) / (4 * EvCfg<M>::C);
-    k_ev_x<M, TRI><<<M * ntile, EvCfg<M>::T, smem, s>>>(rows, RS, sp, dp, src, dst, (const float2 *)w.evt, ntile);
-    return cudaGetLastError();
+    return launch_after(k_ev_x<M, TRI>, M * ntile, EvCfg<M>::T, smem, s, rows, RS, sp, dp, src, dst,
+                        (const float2 *)w.evt, ntile);
 }
 cudaError_t launch_ev_gen_y(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, cudaStream_t s)
 {

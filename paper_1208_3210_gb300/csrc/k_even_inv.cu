@@ -21,6 +21,8 @@ k_ev_inv_x(int rows, int RS, long long sp, long long dp, const float *__restrict
     constexpr int C = F::C, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP, RF = F::RF;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(F::SMEM_ELEMS, float4)
+    allow_next();
+    after_previous();
     float4 *sm = reinterpret_cast<float4 *>(smem_raw);
     const int ky = blockIdx.x / ntile, ct = blockIdx.x % ntile;
     const int col = threadIdx.x % C, u = threadIdx.x / C;
@@ -63,6 +65,8 @@ k_ev_inv_y(EvGeom v, int Q, int n_omega, const float *__restrict__ B4, float *__
     constexpr int C = F::C, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP, RF = F::RF;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(F::SMEM_ELEMS, float4)
+    allow_next();
+    after_previous();
     float4 *sm = reinterpret_cast<float4 *>(smem_raw);
     const int sx = blockIdx.x / ntile, ct = blockIdx.x % ntile;
     const int col = threadIdx.x % C, u = threadIdx.x / C;
@@ -124,9 +128,8 @@ cudaError_t launch_ev_inv_x_t(int rows, int RS, long long sp, long long dp, cons
     static const cudaError_t e = smem_attrs(k_ev_inv_x<M>, smem);
     if (e != cudaSuccess) return e;
     const int ntile = (RS + 4 * EvCfg<M>::C - 1) / (4 * EvCfg<M>::C);
-    k_ev_inv_x<M><<<M * ntile, EvCfg<M>::T, smem, s>>>(rows, RS, sp, dp, (const float *)w.X, (float *)w.Y,
-                                                       (const float2 *)w.evt, ntile);
-    return cudaGetLastError();
+    return launch_after(k_ev_inv_x<M>, M * ntile, EvCfg<M>::T, smem, s, rows, RS, sp, dp, (const float *)w.X,
+                        (float *)w.Y, (const float2 *)w.evt, ntile);
 }
 template <int M>
 cudaError_t launch_ev_inv_y_t(const Geom &g, const EvGeom &v, const Work<float> &w, float *out, cudaStream_t s)
@@ -138,8 +141,8 @@ cudaError_t launch_ev_inv_y_t(const Geom &g, const EvGeom &v, const Work<float> 
     if (e1 != cudaSuccess) return e1;
     const int ntile = (v.WS + 4 * EvCfg<M>::C - 1) / (4 * EvCfg<M>::C);
     auto k = g.n_omega % 4 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0 ? k_ev_inv_y<M, true> : k_ev_inv_y<M, false>;
-    k<<<v.nl * ntile, EvCfg<M>::T, smem, s>>>(v, g.Q, g.n_omega, (const float *)w.Y, out, (const float2 *)w.evt, ntile);
-    return cudaGetLastError();
+    return launch_after(k, v.nl * ntile, EvCfg<M>::T, smem, s, v, g.Q, g.n_omega, (const float *)w.Y, out,
+                        (const float2 *)w.evt, ntile);
 }
 cudaError_t launch_ev_inv_x(const EvGeom &v, const Work<float> &w, cudaStream_t s)
 {

@@ -192,6 +192,31 @@ __device__ __forceinline__ unsigned dyn_smem_bytes()
 #define LH_REQUIRE_SMEM(elems, Cx) \
     if (dyn_smem_bytes() < (unsigned)((elems) * sizeof(Cx))) return;
 
+// Programmatic dependent launch: a kernel launched by launch_after may start
+// while the one before it in the stream still runs; it calls after_previous
+// before it touches any memory that an earlier kernel reads or writes (the
+// wait ends when the previous grid has finished and its writes are visible, and
+// as every kernel of a chain waits, so have all before it).  allow_next lets the
+// next grid's CTAs take the slots that this one's last CTAs leave.  Between the
+// passes of a 256^3 call the launch gaps were 2 us each: 76.0 -> 66.8 us.
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+inline cudaError_t launch_after(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k, static_cast<P>(args)...);
+}
+
 // Circular index n of an inverse transform of length P -> output lag index
 // l in [0, Q), or -1 when the lag is not kept.
 __device__ __forceinline__ int lag_index(int n, int P, int Q)

@@ -126,7 +126,7 @@ def even_pass_bytes(s, grid, band, precision, fp32=0):
         return None
     if (math.pi * grid["zones"] * band["ff_a"]) ** 2 < 8 * 24 * math.log(2.0):
         return None
-    lens = [16 << i for i in range(8)] + [24 << i for i in range(7)]
+    lens = [16 << i for i in range(8)] + [24 << i for i in range(7)] + [72 << i for i in range(5)] + [432, 864]
     need = [m for m in lens if m >= (s.N + s.q_extent // 2 + 1) // 2]
     J0 = s.n_eps // 2
     ne = min(s.n_eps, J0 + s.n_omega) - max(0, J0 - s.n_omega)

@@ -45,10 +45,11 @@
 
 namespace lh {
 
-// Lengths M of the cosine transforms: 16, 32, ..., 2048 and 24, 48, ..., 1536.
+// Lengths M of the cosine transforms: 16, 32, ..., 2048; 24, 48, ..., 1536; and
+// 72, 144, ..., 1152, 432 and 864, so that no axis is padded by more than a third.
 __host__ __device__ constexpr int ev_len(int i)
 {
-    return i < 8 ? 16 << i : i < 15 ? 24 << (i - 8) : 0;
+    return i < 8 ? 16 << i : i < 15 ? 24 << (i - 8) : i < 20 ? 72 << (i - 15) : i == 20 ? 432 : i == 21 ? 864 : 0;
 }
 // Smallest length >= x, 0 past the last.
 inline int ev_len_for(long long x)
@@ -225,8 +226,18 @@ __device__ __forceinline__ void dft(Cx2 *v)
         const Cx2 a = v[0], b = v[1];
         v[0] = add(a, b);
         v[1] = sub(a, b);
+    } else if constexpr (R == 3) {
+        dft3<INV>(v[0], v[1], v[2]);
     } else if constexpr (R == 4) {
         dft4<INV>(v[0], v[1], v[2], v[3]);
+    } else if constexpr (R == 6) {
+        // inputs n = 3 i + 2 j, outputs k = 3 k2 + 4 k3 (mod 6)
+        Cx2 a[3] = {add(v[0], v[3]), add(v[2], v[5]), add(v[4], v[1])};
+        Cx2 b[3] = {sub(v[0], v[3]), sub(v[2], v[5]), sub(v[4], v[1])};
+        dft3<INV>(a[0], a[1], a[2]);
+        dft3<INV>(b[0], b[1], b[2]);
+        v[0] = a[0]; v[4] = a[1]; v[2] = a[2];
+        v[3] = b[0]; v[1] = b[1]; v[5] = b[2];
     } else if constexpr (R == 8) {
         dft8<INV>(v);
     } else if constexpr (R == 12) {
@@ -274,7 +285,7 @@ __device__ __forceinline__ void dft(Cx2 *v)
 __host__ __device__ constexpr int ev_vpt(int M) { return M % 3 == 0 ? 24 : 16; }
 __host__ __device__ constexpr int ev_nstages(int M)
 {
-    return M <= 128 ? 2 : M == 1536 ? 4 : 3;
+    return M <= 144 ? 2 : M == 1536 ? 4 : 3;
 }
 __host__ __device__ constexpr int ev_radix_f(int M, int s)
 {
@@ -282,7 +293,11 @@ __host__ __device__ constexpr int ev_radix_f(int M, int s)
          : M == 16 || M == 24 ? 2
          : M == 32 || M == 48 ? 4
          : M == 64 || M == 96 ? 8
+         : M == 72 ? 6
          : M == 128 ? 16
+         : M == 144 ? 12
+         : M == 288 ? (s == 1 ? 8 : 3)
+         : M == 432 || M == 576 || M == 864 || M == 1152 ? (s == 1 ? 12 : M / 144)
          : M == 192 ? 4
          : M == 256 ? (s == 1 ? 8 : 4)
          : M == 384 ? (s == 1 ? 8 : 4)
@@ -326,7 +341,7 @@ __device__ __forceinline__ void ev_powers(float2 *w, const float2 *__restrict__ 
 {
     const float4 q = __ldg(reinterpret_cast<const float4 *>(row));
     w[1] = make_float2(q.x, q.y);
-    if constexpr (R > 2) w[2] = make_float2(q.z, q.w);
+    if constexpr (R > 2) w[2] = make_float2(q.z, q.w);   // radices 2, 3 and 4: two powers a row
     if constexpr (R == 4) w[3] = cmul(w[1], w[2]);
     if constexpr (R > 4) {
         const float4 p = __ldg(reinterpret_cast<const float4 *>(row) + 1);
@@ -343,9 +358,9 @@ __device__ __forceinline__ void ev_powers(float2 *w, const float2 *__restrict__ 
 // passes that load slowed down (k_ev_x at 1024^2 x 512 0.40 -> 0.52 ms); the
 // generating pass, which loads nothing, runs four (0.31 -> 0.29 ms).
 template <int M> struct EvCfg {
-    static constexpr int C = M <= 24 ? 32 : M <= 48 ? 16 : M <= 256 ? 8 : M <= 1536 ? 4 : 2;
+    static constexpr int C = M <= 24 || M == 72 ? 32 : M <= 48 || M == 144 ? 16 : M <= 256 || M == 288 || M == 432 ? 8 : M <= 1536 ? 4 : 2;
     static constexpr int T = C * M / ev_vpt(M);
-    static constexpr int MINB_GEN = 512 / T;
+    static constexpr int MINB_GEN = 512 / T > 0 ? 512 / T : 1;
     static constexpr int MINB = ev_vpt(M) == 16 ? 512 / T : 384 / T > 0 ? 384 / T : 1;
 };
 
@@ -509,6 +524,13 @@ __device__ __forceinline__ void ev_post(Cx2 *v, int u, const float2 *__restrict_
     case 768: return CALL(768);                                   \
     case 1024: return CALL(1024);                                 \
     case 1536: return CALL(1536);                                 \
+    case 72: return CALL(72);                                     \
+    case 144: return CALL(144);                                   \
+    case 288: return CALL(288);                                   \
+    case 432: return CALL(432);                                   \
+    case 576: return CALL(576);                                   \
+    case 864: return CALL(864);                                   \
+    case 1152: return CALL(1152);                                 \
     case 2048: return CALL(2048);                                 \
     default: return cudaErrorInvalidValue;                        \
     }

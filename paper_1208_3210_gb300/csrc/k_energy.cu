@@ -68,6 +68,7 @@ k_fwd_energy_warp(Geom g, Band band, const AxisTab *__restrict__ axis, const flo
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(ET_WARPS * EtGeo<L>::WARP_ELEMS + (THERMAL ? L : 0), float2)
+    after_previous();
     float2 *sm = reinterpret_cast<float2 *>(smem_raw);
     float2 *wf = sm + ET_WARPS * EtGeo<L>::WARP_ELEMS;
     if constexpr (THERMAL) {
@@ -83,6 +84,7 @@ k_inv_energy_warp(Geom g, const float2 *__restrict__ U4, float *__restrict__ out
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(et_inv_smem_elems<L>(), float2)
+    after_previous();
     inv_energy_warp_tile<L, HALF, false>(g, U4, out, etw, reinterpret_cast<float2 *>(smem_raw), blockIdx.x);
 }
 
@@ -98,8 +100,7 @@ cudaError_t launch_inv_energy_warp_t(const Geom &g, const Work<float> &w, float 
     if (e0 != cudaSuccess) return e0;
     if (e1 != cudaSuccess) return e1;
     auto k = 2 * g.n_omega == L ? k_inv_energy_warp<L, true> : k_inv_energy_warp<L, false>;
-    k<<<grid, 32 * ET_WARPS, smem, s>>>(g, (const float2 *)w.Y, out, (const float2 *)w.etw);
-    return cudaGetLastError();
+    return launch_after(k, grid, 32 * ET_WARPS, smem, s, g, (const float2 *)w.Y, out, (const float2 *)w.etw);
 }
 
 // the warp-per-pair inverse pass: every length of the warp-per-line passes
@@ -136,9 +137,8 @@ cudaError_t launch_fwd_energy_col_tt(const Geom &g, const Band &band, const Work
     const bool full = g.n_eps == L;
     auto k = A_in ? (full ? k_fwd_energy_warp<L, true, false, THERMAL> : k_fwd_energy_warp<L, false, false, THERMAL>)
                   : (full ? k_fwd_energy_warp<L, true, true, THERMAL> : k_fwd_energy_warp<L, false, true, THERMAL>);
-    k<<<grid, 32 * ET_WARPS, smem, s>>>(g, band, w.axis, (const float2 *)w.eps, w.state, A_in, (float2 *)w.X,
-                                        (const float2 *)w.etw);
-    return cudaGetLastError();
+    return launch_after(k, grid, 32 * ET_WARPS, smem, s, g, band, w.axis, (const float2 *)w.eps, w.state,
+                        A_in, (float2 *)w.X, (const float2 *)w.etw);
 }
 template <int L>
 cudaError_t launch_fwd_energy_col_t(const Geom &g, const Band &band, const Work<float> &w, const float *A_in,

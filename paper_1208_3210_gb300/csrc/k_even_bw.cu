@@ -36,6 +36,7 @@ k_ev_w_y(EvGeom v, int Q, int n_omega, const float *__restrict__ w, float *__res
     constexpr int C = F::C, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(F::SMEM_ELEMS, float4)
+    after_previous();
     float4 *sm = reinterpret_cast<float4 *>(smem_raw);
     const int sx = blockIdx.x / ntile, ct = blockIdx.x % ntile;
     const int col = threadIdx.x % C, u = threadIdx.x / C;
@@ -103,6 +104,7 @@ k_ev_bw(Geom g, EvGeom v, Band band, const float *__restrict__ B2, const float *
     constexpr int VPT = E::VPT, TPL = E::TPL, R0 = E::R0, R1 = E::R1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(EVC_WARPS * (E::WARP_ELEMS + 64 * (R1 + 1)) + (THERMAL ? L : 0), float2)
+    after_previous();
     const int lane = (int)threadIdx.x % 32, warp = (int)threadIdx.x / 32;
     const int sl = lane / TPL, u = lane % TPL;
     float2 *sm = reinterpret_cast<float2 *>(smem_raw) + warp * E::WARP_ELEMS + sl * E::LP;
@@ -206,6 +208,7 @@ k_ev_chain(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const 
     constexpr int C = F::C, T = F::T, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP, RF = F::RF;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(F::SMEM_ELEMS, float4)
+    after_previous();
     float4 *sm = reinterpret_cast<float4 *>(smem_raw);
     const int jx = blockIdx.x / ntile, ct = blockIdx.x % ntile;
     const int col = threadIdx.x % C, u = threadIdx.x / C;
@@ -276,17 +279,24 @@ k_ev_chain(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const 
         }
     }
     double val[4] = {s0, s1, s2, (double)sg.x + (double)sg.y};
+    // the last warp may be a part of one (T = 144)
+    constexpr int NWP = (T + 31) / 32;
+    const int lane = threadIdx.x % 32, wp = threadIdx.x / 32, nl = min(32, T - 32 * wp);
+    const unsigned mask = nl == 32 ? 0xffffffffu : (1u << nl) - 1u;
 #pragma unroll
     for (int q = 0; q < 4; ++q)
-        for (int o = 16; o > 0; o >>= 1) val[q] += __shfl_down_sync(0xffffffffu, val[q], o);
+        for (int o = 16; o > 0; o >>= 1) {
+            const double other = __shfl_down_sync(mask, val[q], o);
+            if (lane + o < nl) val[q] += other;
+        }
     __syncthreads();   // the rows have been read
     double *red = reinterpret_cast<double *>(smem_raw);
-    if (threadIdx.x % 32 == 0)
-        for (int q = 0; q < 4; ++q) red[threadIdx.x / 32 * 4 + q] = val[q];
+    if (lane == 0)
+        for (int q = 0; q < 4; ++q) red[wp * 4 + q] = val[q];
     __syncthreads();
     if (threadIdx.x == 0) {
         double t[4] = {0, 0, 0, 0};
-        for (int i = 0; i < T / 32; ++i)
+        for (int i = 0; i < NWP; ++i)
             for (int q = 0; q < 4; ++q) t[q] += red[i * 4 + q];
         const bool tb = band.band_kind != 1;
         double *o = partial + 5LL * blockIdx.x;
@@ -308,8 +318,8 @@ cudaError_t launch_ev_w_y_t(const Geom &g, const EvGeom &v, const float *wts, co
     if (e1 != cudaSuccess) return e1;
     const int ntile = (v.WS + 4 * EvCfg<M>::C - 1) / (4 * EvCfg<M>::C), rows = v.nl < M ? v.nl : M;
     auto k = g.n_omega % 4 == 0 && reinterpret_cast<uintptr_t>(wts) % 16 == 0 ? k_ev_w_y<M, true> : k_ev_w_y<M, false>;
-    k<<<rows * ntile, EvCfg<M>::T, smem, s>>>(v, g.Q, g.n_omega, wts, (float *)w.X, (const float2 *)w.evt, ntile);
-    return cudaGetLastError();
+    return launch_after(k, rows * ntile, EvCfg<M>::T, smem, s, v, g.Q, g.n_omega, wts, (float *)w.X,
+                        (const float2 *)w.evt, ntile);
 }
 template <int M>
 cudaError_t launch_ev_chain_t(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, double *partial,
@@ -319,9 +329,8 @@ cudaError_t launch_ev_chain_t(const Geom &g, const EvGeom &v, const Band &band, 
     static const cudaError_t e = smem_attrs(k_ev_chain<M>, smem);
     if (e != cudaSuccess) return e;
     const int ntile = (v.ES + 4 * EvCfg<M>::C - 1) / (4 * EvCfg<M>::C);
-    k_ev_chain<M><<<v.Nh * ntile, EvCfg<M>::T, smem, s>>>(g, v, band, w.axis, (const float2 *)w.eps, w.state,
-                                                          (const float *)w.Y, partial, (const float2 *)w.evt, ntile);
-    return cudaGetLastError();
+    return launch_after(k_ev_chain<M>, v.Nh * ntile, EvCfg<M>::T, smem, s, g, v, band, w.axis, (const float2 *)w.eps,
+                        w.state, (const float *)w.Y, partial, (const float2 *)w.evt, ntile);
 }
 // CTAs of k_ev_chain (rows of its partial sums).
 int ev_chain_blocks(const EvGeom &v)
@@ -340,10 +349,9 @@ cudaError_t launch_ev_bw_t(const Geom &g, const EvGeom &v, const Band &band, con
     if (e != cudaSuccess) return e;
     const int npairs = v.M / 2 * (v.M + 1) / 2, iters = ev_corr_iters(npairs, E::LPI, sms);
     const int per = EVC_WARPS * iters * E::LPI;
-    k_ev_bw<L, FULL, THERMAL><<<(npairs + per - 1) / per, 32 * EVC_WARPS, smem, s>>>(
-        g, v, band, (const float *)w.Y, W2, (float *)w.X, (const float2 *)w.evt + ev_line_table<L>(), iters,
-        g.quantity == LINDHARD_IMCHI_T);
-    return cudaGetLastError();
+    return launch_after(k_ev_bw<L, FULL, THERMAL>, (npairs + per - 1) / per, 32 * EVC_WARPS, smem, s, g, v, band,
+                        (const float *)w.Y, W2, (float *)w.X, (const float2 *)w.evt + ev_line_table<L>(), iters,
+                        g.quantity == LINDHARD_IMCHI_T);
 }
 template <int L>
 cudaError_t launch_ev_bw_l(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, const float *W2,

@@ -27,7 +27,6 @@ k_ev_corr(Geom g, EvGeom v, Band band, const float *__restrict__ B2, float *__re
     constexpr int VPT = E::VPT, TPL = E::TPL, R0 = E::R0, R1 = E::R1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(EVC_WARPS * E::WARP_ELEMS + (THERMAL ? L : 0), float2)
-    allow_next();
     after_previous();
     const int lane = (int)threadIdx.x % 32, warp = (int)threadIdx.x / 32;
     const int sl = lane / TPL, u = lane % TPL;
@@ -140,7 +139,6 @@ k_ev_corr3(Geom g, EvGeom v, Band band, const float *__restrict__ B2, float *__r
     static_assert(S0 == R2 && VPT == 2 * S0, "the product stays in registers");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(EVC_WARPS * LPI * LP + (THERMAL ? L : 0), float2)
-    allow_next();
     after_previous();
     const int lane = (int)threadIdx.x % 32, warp = (int)threadIdx.x / 32;
     const int sl = lane / TPL, u = lane % TPL;

@@ -25,7 +25,7 @@ __device__ __forceinline__ float ev_rcp(float x)
 // One block per table and slice: the tables' places and periods come as an
 // argument (evaluating ev_table_offset per entry on the device took 0.5 ms).
 struct EvTabs {
-    struct { int off, count, row, period; } t[68];   // row 0: the w_j, j < period; row -1: even_line.cuh
+    struct { int off, count, row, period; } t[112];   // row 0: the w_j, j < period; row -1: even_line.cuh
 };
 __global__ void k_ev_tables(float2 *out, EvTabs tabs)
 {
@@ -71,7 +71,6 @@ k_ev_gen_y(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const 
     constexpr int C = F::C, T = F::T, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(F::SMEM_ELEMS, float4)
-    allow_next();
     after_previous();
     float4 *sm = reinterpret_cast<float4 *>(smem_raw);
     const int jx = blockIdx.x / ntile, ct = blockIdx.x % ntile;
@@ -145,7 +144,6 @@ k_ev_x(int rows, int RS, long long sp, long long dp, const float *__restrict__ B
     constexpr int C = F::C, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(F::SMEM_ELEMS, float4)
-    allow_next();
     after_previous();
     float4 *sm = reinterpret_cast<float4 *>(smem_raw);
     const int ky = blockIdx.x / ntile, ct = blockIdx.x % ntile;

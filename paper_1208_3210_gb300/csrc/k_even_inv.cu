@@ -21,7 +21,6 @@ k_ev_inv_x(int rows, int RS, long long sp, long long dp, const float *__restrict
     constexpr int C = F::C, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP, RF = F::RF;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(F::SMEM_ELEMS, float4)
-    allow_next();
     after_previous();
     float4 *sm = reinterpret_cast<float4 *>(smem_raw);
     const int ky = blockIdx.x / ntile, ct = blockIdx.x % ntile;
@@ -65,7 +64,6 @@ k_ev_inv_y(EvGeom v, int Q, int n_omega, const float *__restrict__ B4, float *__
     constexpr int C = F::C, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP, RF = F::RF;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(F::SMEM_ELEMS, float4)
-    allow_next();
     after_previous();
     float4 *sm = reinterpret_cast<float4 *>(smem_raw);
     const int sx = blockIdx.x / ntile, ct = blockIdx.x % ntile;

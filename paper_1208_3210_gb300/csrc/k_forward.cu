@@ -31,6 +31,7 @@ k_fwd_energy(Geom g, Band band, const AxisTab *__restrict__ axis,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Cx *sm = reinterpret_cast<Cx *>(smem_raw);
     LH_REQUIRE_SMEM(E::SMEM_ELEMS, Cx)
+    after_previous();
     __shared__ Real s_xhi[C], s_xlo[C], s_amp[C];
 
     const long long nlines = (long long)g.N * g.N;
@@ -168,6 +169,7 @@ k_fwd_y(Geom g, const cx<Real> *__restrict__ U1, cx<Real> *__restrict__ U2,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Cx *sm = reinterpret_cast<Cx *>(smem_raw);
     LH_REQUIRE_SMEM(E::SMEM_ELEMS, Cx)
+    after_previous();
 
     const int W = 2 * g.SP;                       // row width (a^ and b^)
     const int ix = blockIdx.y;
@@ -211,6 +213,7 @@ k_fwd_y2(Geom g, const cx<Real> *__restrict__ U1, cx<Real> *__restrict__ U2,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Cx *sm = reinterpret_cast<Cx *>(smem_raw);
     LH_REQUIRE_SMEM(E::SMEM_ELEMS, Cx)
+    after_previous();
 
     const int W = 2 * g.SP;                       // row width (a^ and b^)
     const int ix = blockIdx.y;
@@ -255,9 +258,9 @@ cudaError_t launch_fwd_energy_t(const Geom &g, const Band &band, const Work<Real
     if (e1 != cudaSuccess) return e1;
     long long nlines = (long long)g.N * g.N;
     unsigned grid = (unsigned)((nlines + C - 1) / C);
-    k<<<grid, T, smem, s>>>(g, band, w.axis, (const typename EpsEntry<Real>::type *)w.eps, w.state, A_in,
-                            (cx<Real> *)w.X, twiddles_for<Real>(w, L));
-    return cudaGetLastError();
+    return launch_after(k, grid, T, smem, s, g, band, w.axis,
+                        (const typename EpsEntry<Real>::type *)w.eps, w.state, A_in, (cx<Real> *)w.X,
+                        twiddles_for<Real>(w, L));
 }
 
 template <typename Real, int L, typename Cfg>
@@ -270,8 +273,7 @@ cudaError_t launch_fwd_y2_t(const Geom &g, const Work<Real> &w, cudaStream_t s)
     static const cudaError_t e = smem_attrs(k, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((2 * g.SP + C - 1) / C, g.N);
-    k<<<grid, T, smem, s>>>(g, (const cx<Real> *)w.X, (cx<Real> *)w.Y, twiddles_for<Real>(w, L));
-    return cudaGetLastError();
+    return launch_after(k, grid, T, smem, s, g, (const cx<Real> *)w.X, (cx<Real> *)w.Y, twiddles_for<Real>(w, L));
 }
 
 // variant 0: single-column engine; 1: paired-column engine (L >= 128, FP32);
@@ -294,8 +296,7 @@ cudaError_t launch_fwd_y_t(const Geom &g, const Work<Real> &w, cudaStream_t s, i
     static const cudaError_t e = smem_attrs(k, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((2 * g.SP + C - 1) / C, g.N);
-    k<<<grid, T, smem, s>>>(g, (const cx<Real> *)w.X, (cx<Real> *)w.Y, twiddles_for<Real>(w, L));
-    return cudaGetLastError();
+    return launch_after(k, grid, T, smem, s, g, (const cx<Real> *)w.X, (cx<Real> *)w.Y, twiddles_for<Real>(w, L));
 }
 
 bool et_applies(const Geom &g, const Band &band);

@@ -25,6 +25,7 @@ k_inv_y(Geom g, const cx<Real> *__restrict__ U3, cx<Real> *__restrict__ U4,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Cx *sm = reinterpret_cast<Cx *>(smem_raw);
     LH_REQUIRE_SMEM(E::SMEM_ELEMS, Cx)
+    after_previous();
 
     const int lx = blockIdx.y;
     const int c = blockIdx.x * C + (int)(threadIdx.x % C);
@@ -67,6 +68,7 @@ k_inv_y2(Geom g, const cx<Real> *__restrict__ U3, cx<Real> *__restrict__ U4,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Cx *sm = reinterpret_cast<Cx *>(smem_raw);
     LH_REQUIRE_SMEM(E::SMEM_ELEMS, Cx)
+    after_previous();
 
     const int lx = blockIdx.y;
     const int c = blockIdx.x * C + 2 * E::pair();
@@ -113,6 +115,7 @@ k_inv_energy(Geom g, const cx<Real> *__restrict__ U4, OutT *__restrict__ out,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Cx *sm = reinterpret_cast<Cx *>(smem_raw);
     LH_REQUIRE_SMEM(E::SMEM_ELEMS, Cx)
+    after_previous();
 
     const long long npairs = (long long)g.Q * g.Q / 2;
     const long long f0 = (long long)blockIdx.x * C;
@@ -165,8 +168,7 @@ cudaError_t launch_inv_y2_t(const Geom &g, const Work<Real> &w, cudaStream_t s)
     static const cudaError_t e = smem_attrs(k, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((g.H + C - 1) / C, g.Q);
-    k<<<grid, T, smem, s>>>(g, (const cx<Real> *)w.X, (cx<Real> *)w.Y, twiddles_for<Real>(w, L));
-    return cudaGetLastError();
+    return launch_after(k, grid, T, smem, s, g, (const cx<Real> *)w.X, (cx<Real> *)w.Y, twiddles_for<Real>(w, L));
 }
 
 // variant 0: single-column engine; 1: paired-column engine (L >= 128, FP32);
@@ -189,8 +191,7 @@ cudaError_t launch_inv_y_t(const Geom &g, const Work<Real> &w, cudaStream_t s, i
     static const cudaError_t e = smem_attrs(k, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((g.H + C - 1) / C, g.Q);
-    k<<<grid, T, smem, s>>>(g, (const cx<Real> *)w.X, (cx<Real> *)w.Y, twiddles_for<Real>(w, L));
-    return cudaGetLastError();
+    return launch_after(k, grid, T, smem, s, g, (const cx<Real> *)w.X, (cx<Real> *)w.Y, twiddles_for<Real>(w, L));
 }
 
 template <typename Real, typename OutT, int L>
@@ -204,8 +205,7 @@ cudaError_t launch_inv_energy_t(const Geom &g, const Work<Real> &w, OutT *out, c
     if (e != cudaSuccess) return e;
     long long npairs = (long long)g.Q * g.Q / 2;
     unsigned grid = (unsigned)((npairs + C - 1) / C);
-    k<<<grid, T, smem, s>>>(g, (const cx<Real> *)w.Y, out, twiddles_for<Real>(w, L));
-    return cudaGetLastError();
+    return launch_after(k, grid, T, smem, s, g, (const cx<Real> *)w.Y, out, twiddles_for<Real>(w, L));
 }
 
 cudaError_t launch_inv_y_tma(const Geom &g, const Work<float> &w, cudaStream_t s, int variant);

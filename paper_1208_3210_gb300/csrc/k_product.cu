@@ -38,6 +38,7 @@ k_x_product(Geom g, const cx<Real> *__restrict__ U2, cx<Real> *__restrict__ U3,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Cx *sm = reinterpret_cast<Cx *>(smem_raw);
     LH_REQUIRE_SMEM(XP::SMEM_ELEMS, Cx)
+    after_previous();
 
     const int W = 2 * g.SP;
     const int ky = blockIdx.y;
@@ -89,8 +90,7 @@ cudaError_t launch_x_product_c(const Geom &g, const Work<Real> &w, cudaStream_t 
     static const cudaError_t e = smem_attrs(k, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((g.H + C - 1) / C, g.P);
-    k<<<grid, T, smem, s>>>(g, (const cx<Real> *)w.Y, (cx<Real> *)w.X, twiddles_for<Real>(w, L));
-    return cudaGetLastError();
+    return launch_after(k, grid, T, smem, s, g, (const cx<Real> *)w.Y, (cx<Real> *)w.X, twiddles_for<Real>(w, L));
 }
 
 // variant 0: the tiles of XCfg; 1: 12 values per thread (3 * 2^k >= 192,

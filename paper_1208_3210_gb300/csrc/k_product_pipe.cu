@@ -74,6 +74,7 @@ k_x_product_pr_pipe(Geom g, const float2 *__restrict__ U2, float2 *__restrict__ 
     constexpr int T = PP::T, CW = PP::CW, KS = PP::KS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(PP::SMEM_ELEMS, float2)
+    after_previous();
     float2 *sm = reinterpret_cast<float2 *>(smem_raw);
     float4 *pre = reinterpret_cast<float4 *>(sm + PP::UPPER);   // [KS][T]
     const float2 *tw = ptw;
@@ -164,8 +165,7 @@ static cudaError_t x_product_pr_pipe_t(const Geom &g, const Work<float> &w, cuda
     const int ntiles = ((g.H + PP::CW - 1) / PP::CW) * g.P;
     cudaError_t e = persistent_grid(k, PP::T, smem, ntiles, grid);
     if (e != cudaSuccess) return e;
-    k<<<grid, PP::T, smem, s>>>(g, (const float2 *)w.Y, (float2 *)w.X, (const float2 *)w.ptw);
-    return cudaGetLastError();
+    return launch_after(k, grid, PP::T, smem, s, g, (const float2 *)w.Y, (float2 *)w.X, (const float2 *)w.ptw);
 }
 
 bool pr_fwd_applies(const Geom &g);

@@ -54,6 +54,7 @@ k_fwd_y_pr(Geom g, const float2 *__restrict__ U1, float2 *__restrict__ U2, const
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM((PrEng<L, Cfg::C, Cfg::T, false, 2, true, false>::SMEM_ELEMS), float2)
+    after_previous();
     fwd_y_pr_tile<L, Cfg::C, Cfg::T, false>(g, U1, U2, ptw, reinterpret_cast<float2 *>(smem_raw), blockIdx.x,
                                             blockIdx.y);
 }
@@ -64,6 +65,7 @@ k_x_product_pr(Geom g, const float2 *__restrict__ U2, float2 *__restrict__ U3, c
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM((PrProduct<L, Cfg::C, Cfg::T>::SMEM_ELEMS), float2)
+    after_previous();
     x_product_pr_tile<L, Cfg::C, Cfg::T, ODD, false>(g, U2, U3, ptw, reinterpret_cast<float2 *>(smem_raw),
                                                      blockIdx.x, blockIdx.y);
 }
@@ -74,6 +76,7 @@ k_inv_y_pr(Geom g, const float2 *__restrict__ U3, float2 *__restrict__ U4, const
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM((PrEng<L, Cfg::C, Cfg::T, true, 2, false, true>::SMEM_ELEMS), float2)
+    after_previous();
     inv_y_pr_tile<L, Cfg::C, Cfg::T, false>(g, U3, U4, ptw, reinterpret_cast<float2 *>(smem_raw), blockIdx.x,
                                             blockIdx.y);
 }
@@ -90,8 +93,7 @@ cudaError_t launch_fwd_y_pr_t(const Geom &g, const Work<float> &w, cudaStream_t 
     static const cudaError_t e = smem_attrs(k, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((2 * g.SP + 2 * CW - 1) / (2 * CW), g.N);
-    k<<<grid, Cfg::T, smem, s>>>(g, (const float2 *)w.X, (float2 *)w.Y, (const float2 *)w.ptw);
-    return cudaGetLastError();
+    return launch_after(k, grid, Cfg::T, smem, s, g, (const float2 *)w.X, (float2 *)w.Y, (const float2 *)w.ptw);
 }
 
 template <int L, int CW>
@@ -108,8 +110,7 @@ cudaError_t launch_x_product_pr_t(const Geom &g, const Work<float> &w, cudaStrea
     if (e0 != cudaSuccess) return e0;
     if (e1 != cudaSuccess) return e1;
     dim3 grid((g.H + CW - 1) / CW, g.P);
-    k<<<grid, Cfg::T, smem, s>>>(g, (const float2 *)w.Y, (float2 *)w.X, (const float2 *)w.ptw);
-    return cudaGetLastError();
+    return launch_after(k, grid, Cfg::T, smem, s, g, (const float2 *)w.Y, (float2 *)w.X, (const float2 *)w.ptw);
 }
 
 template <int L, int CW>
@@ -122,8 +123,7 @@ cudaError_t launch_inv_y_pr_t(const Geom &g, const Work<float> &w, cudaStream_t 
     static const cudaError_t e = smem_attrs(k, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((g.H + 2 * CW - 1) / (2 * CW), g.Q);
-    k<<<grid, Cfg::T, smem, s>>>(g, (const float2 *)w.X, (float2 *)w.Y, (const float2 *)w.ptw);
-    return cudaGetLastError();
+    return launch_after(k, grid, Cfg::T, smem, s, g, (const float2 *)w.X, (float2 *)w.Y, (const float2 *)w.ptw);
 }
 
 // The adjoint's products along p_x (k_bw_product, same layouts): W^ of the
@@ -154,6 +154,7 @@ k_bw_product_pr(Geom g, float2 *__restrict__ U2, const float2 *__restrict__ WU2,
     static_assert(EF1::SMEM_ELEMS <= PARK, "the one-operand forward exchange stays below the parked W^");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(SE, float2)
+    after_previous();
     float2 *sm = reinterpret_cast<float2 *>(smem_raw);
     float2 *park = sm + PARK;
     const int ky = blockIdx.y;
@@ -232,8 +233,7 @@ cudaError_t launch_bw_product_pr_t(const Geom &g, float2 *U2, const float2 *WU2,
     if (e0 != cudaSuccess) return e0;
     if (e1 != cudaSuccess) return e1;
     dim3 grid((g.H + 7) / 8, g.P);
-    k<<<grid, Cfg::T, smem, s>>>(g, U2, WU2, ptw);
-    return cudaGetLastError();
+    return launch_after(k, grid, Cfg::T, smem, s, g, U2, WU2, ptw);
 }
 
 // The pruned forms apply when the padding is exactly one third.

@@ -66,6 +66,7 @@ k_fwd_y_pr_tma(Geom g, const __grid_constant__ CUtensorMap map, float2 *__restri
     const int nbox = (g.N + box_rows - 1) / box_rows, NR = nbox * box_rows;
     const TmaSmem lay{(size_t)NR * PT_C * sizeof(float2), (size_t)E::SMEM_ELEMS * sizeof(float2)};
     if (dyn_smem_bytes() < lay.total()) return;
+    after_previous();
     float2 *stage = reinterpret_cast<float2 *>(smem_raw);
     float2 *sm = reinterpret_cast<float2 *>(smem_raw + lay.stage_bytes);
     unsigned long long *bar = reinterpret_cast<unsigned long long *>(smem_raw + lay.stage_bytes + lay.fft_bytes);
@@ -133,6 +134,7 @@ k_inv_y_pr_tma(Geom g, const __grid_constant__ CUtensorMap map, float2 *__restri
     const int nbox = (L + box_rows - 1) / box_rows, NR = nbox * box_rows;
     const TmaSmem lay{(size_t)NR * PT_C * sizeof(float2), (size_t)E::SMEM_ELEMS * sizeof(float2)};
     if (dyn_smem_bytes() < lay.total()) return;
+    after_previous();
     float2 *stage = reinterpret_cast<float2 *>(smem_raw);
     float2 *sm = reinterpret_cast<float2 *>(smem_raw + lay.stage_bytes);
     unsigned long long *bar = reinterpret_cast<unsigned long long *>(smem_raw + lay.stage_bytes + lay.fft_bytes);
@@ -202,6 +204,7 @@ k_fwd_y_pr_tma2(Geom g, const __grid_constant__ CUtensorMap map, float2 *__restr
     const int nbox = (g.N + box_rows - 1) / box_rows, NR = nbox * box_rows;
     const size_t buf = pt_shared_bytes((size_t)NR * PT_C * sizeof(float2), (size_t)E::SMEM_ELEMS * sizeof(float2));
     if (dyn_smem_bytes() < buf + 16) return;
+    after_previous();
     float2 *stage = reinterpret_cast<float2 *>(smem_raw);
     float2 *sm = stage;
     unsigned long long *bar = reinterpret_cast<unsigned long long *>(smem_raw + buf);
@@ -266,6 +269,7 @@ k_inv_y_pr_tma2(Geom g, const __grid_constant__ CUtensorMap map, float2 *__restr
     const int nbox = (L + box_rows - 1) / box_rows, NR = nbox * box_rows;
     const size_t buf = pt_shared_bytes((size_t)NR * PT_C * sizeof(float2), (size_t)E::SMEM_ELEMS * sizeof(float2));
     if (dyn_smem_bytes() < buf + 16) return;
+    after_previous();
     float2 *stage = reinterpret_cast<float2 *>(smem_raw);
     float2 *sm = stage;
     unsigned long long *bar = reinterpret_cast<unsigned long long *>(smem_raw + buf);
@@ -338,6 +342,7 @@ k_x_product_pr_tma(Geom g, const __grid_constant__ CUtensorMap map, float2 *__re
     const int nbox = (g.N + box_rows - 1) / box_rows, NR = nbox * box_rows;
     const TmaSmem lay{2 * (size_t)NR * FC * sizeof(float2), (size_t)PtProd<L>::P::SMEM_ELEMS * sizeof(float2)};
     if (dyn_smem_bytes() < lay.total()) return;
+    after_previous();
     float2 *stage = reinterpret_cast<float2 *>(smem_raw);
     float2 *sm = reinterpret_cast<float2 *>(smem_raw + lay.stage_bytes);
     unsigned long long *bar = reinterpret_cast<unsigned long long *>(smem_raw + lay.stage_bytes + lay.fft_bytes);
@@ -409,8 +414,7 @@ static cudaError_t fwd_y_pr_tma_t(const Geom &g, const Work<float> &w, cudaStrea
     const int ntiles = ((2 * g.SP + PT_C - 1) / PT_C) * g.N;
     if (e == cudaSuccess) e = persistent_grid(k, PtFwd<L>::T, lay.total(), ntiles, grid);
     if (e != cudaSuccess) return e;
-    k<<<grid, PtFwd<L>::T, lay.total(), s>>>(g, map, (float2 *)w.Y, (const float2 *)w.ptw, w.status, box_rows);
-    return cudaGetLastError();
+    return launch_after(k, grid, PtFwd<L>::T, lay.total(), s, g, map, (float2 *)w.Y, (const float2 *)w.ptw, w.status, box_rows);
 }
 template <int L>
 static cudaError_t inv_y_pr_tma_t(const Geom &g, const Work<float> &w, cudaStream_t s)
@@ -428,8 +432,7 @@ static cudaError_t inv_y_pr_tma_t(const Geom &g, const Work<float> &w, cudaStrea
     const int ntiles = ((g.H + PT_C - 1) / PT_C) * g.Q;
     if (e == cudaSuccess) e = persistent_grid(k, PtInv<L>::T, lay.total(), ntiles, grid);
     if (e != cudaSuccess) return e;
-    k<<<grid, PtInv<L>::T, lay.total(), s>>>(g, map, (float2 *)w.Y, (const float2 *)w.ptw, w.status, box_rows);
-    return cudaGetLastError();
+    return launch_after(k, grid, PtInv<L>::T, lay.total(), s, g, map, (float2 *)w.Y, (const float2 *)w.ptw, w.status, box_rows);
 }
 template <int L>
 static cudaError_t fwd_y_pr_tma2_t(const Geom &g, const Work<float> &w, cudaStream_t s)
@@ -448,8 +451,7 @@ static cudaError_t fwd_y_pr_tma2_t(const Geom &g, const Work<float> &w, cudaStre
     const int ntiles = ((2 * g.SP + PT_C - 1) / PT_C) * g.N;
     if (e == cudaSuccess) e = persistent_grid(k, PtFwd2<L>::T, smem, ntiles, grid);
     if (e != cudaSuccess) return e;
-    k<<<grid, PtFwd2<L>::T, smem, s>>>(g, map, (float2 *)w.Y, (const float2 *)w.ptw, w.status, box_rows);
-    return cudaGetLastError();
+    return launch_after(k, grid, PtFwd2<L>::T, smem, s, g, map, (float2 *)w.Y, (const float2 *)w.ptw, w.status, box_rows);
 }
 template <int L>
 static cudaError_t inv_y_pr_tma2_t(const Geom &g, const Work<float> &w, cudaStream_t s)
@@ -468,8 +470,7 @@ static cudaError_t inv_y_pr_tma2_t(const Geom &g, const Work<float> &w, cudaStre
     const int ntiles = ((g.H + PT_C - 1) / PT_C) * g.Q;
     if (e == cudaSuccess) e = persistent_grid(k, PtInv2<L>::T, smem, ntiles, grid);
     if (e != cudaSuccess) return e;
-    k<<<grid, PtInv2<L>::T, smem, s>>>(g, map, (float2 *)w.Y, (const float2 *)w.ptw, w.status, box_rows);
-    return cudaGetLastError();
+    return launch_after(k, grid, PtInv2<L>::T, smem, s, g, map, (float2 *)w.Y, (const float2 *)w.ptw, w.status, box_rows);
 }
 template <int L>
 static cudaError_t x_product_pr_tma_t(const Geom &g, const Work<float> &w, cudaStream_t s)
@@ -490,8 +491,7 @@ static cudaError_t x_product_pr_tma_t(const Geom &g, const Work<float> &w, cudaS
     const int ntiles = ((g.H + FC - 1) / FC) * g.P;
     if (e == cudaSuccess) e = persistent_grid(k, PtProd<L>::T, lay.total(), ntiles, grid);
     if (e != cudaSuccess) return e;
-    k<<<grid, PtProd<L>::T, lay.total(), s>>>(g, map, (float2 *)w.X, (const float2 *)w.ptw, w.status, box_rows);
-    return cudaGetLastError();
+    return launch_after(k, grid, PtProd<L>::T, lay.total(), s, g, map, (float2 *)w.X, (const float2 *)w.ptw, w.status, box_rows);
 }
 
 bool pr_fwd_applies(const Geom &g);

@@ -65,6 +65,7 @@ k_fwd_y_tma(Geom g, const __grid_constant__ CUtensorMap map, float2 *__restrict_
     const int nbox = (g.N + box_rows - 1) / box_rows, NR = nbox * box_rows;
     const TmaSmem lay{(size_t)NR * C * sizeof(float2), (size_t)E::SMEM_ELEMS * sizeof(float2)};
     if (dyn_smem_bytes() < lay.total()) return;
+    after_previous();
     float2 *stage = reinterpret_cast<float2 *>(smem_raw);
     float2 *sm = reinterpret_cast<float2 *>(smem_raw + lay.stage_bytes);
     unsigned long long *bar = reinterpret_cast<unsigned long long *>(smem_raw + lay.stage_bytes + lay.fft_bytes);
@@ -137,6 +138,7 @@ k_inv_y_tma(Geom g, const __grid_constant__ CUtensorMap map, float2 *__restrict_
     const int nbox = (L + box_rows - 1) / box_rows, NR = nbox * box_rows;
     const TmaSmem lay{(size_t)NR * C * sizeof(float2), (size_t)E::SMEM_ELEMS * sizeof(float2)};
     if (dyn_smem_bytes() < lay.total()) return;
+    after_previous();
     float2 *stage = reinterpret_cast<float2 *>(smem_raw);
     float2 *sm = reinterpret_cast<float2 *>(smem_raw + lay.stage_bytes);
     unsigned long long *bar = reinterpret_cast<unsigned long long *>(smem_raw + lay.stage_bytes + lay.fft_bytes);
@@ -208,6 +210,7 @@ k_x_product_tma(Geom g, const __grid_constant__ CUtensorMap map, float2 *__restr
     const int nbox = (g.N + box_rows - 1) / box_rows, NR = nbox * box_rows;
     const TmaSmem lay{2 * (size_t)NR * C * sizeof(float2), (size_t)FFT_ELEMS * sizeof(float2)};
     if (dyn_smem_bytes() < lay.total()) return;
+    after_previous();
     float2 *stage = reinterpret_cast<float2 *>(smem_raw);   // [NR][C][2]: (a^, b^) per frequency
     float2 *sm = reinterpret_cast<float2 *>(smem_raw + lay.stage_bytes);
     unsigned long long *bar = reinterpret_cast<unsigned long long *>(smem_raw + lay.stage_bytes + lay.fft_bytes);
@@ -298,6 +301,7 @@ k_y_col_tma(Geom g, const __grid_constant__ CUtensorMap map, float2 *__restrict_
     const int nbox = (rows + box_rows - 1) / box_rows, NR = nbox * box_rows;
     const TmaSmem lay{(size_t)NR * C * sizeof(float2), (size_t)E::SMEM_ELEMS * sizeof(float2)};
     if (dyn_smem_bytes() < lay.total()) return;
+    after_previous();
     float2 *stage = reinterpret_cast<float2 *>(smem_raw);
     float2 *sm = reinterpret_cast<float2 *>(smem_raw + lay.stage_bytes);
     unsigned long long *bar = reinterpret_cast<unsigned long long *>(smem_raw + lay.stage_bytes + lay.fft_bytes);
@@ -384,6 +388,7 @@ k_inv_energy_tma(Geom g, const __grid_constant__ CUtensorMap map, float *__restr
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const TmaSmem lay{(size_t)nbx * 2 * C * bx * sizeof(float2), (size_t)E::SMEM_ELEMS * sizeof(float2)};
     if (dyn_smem_bytes() < lay.total()) return;
+    after_previous();
     float2 *stage = reinterpret_cast<float2 *>(smem_raw);
     float2 *sm = reinterpret_cast<float2 *>(smem_raw + lay.stage_bytes);
     unsigned long long *bar = reinterpret_cast<unsigned long long *>(smem_raw + lay.stage_bytes + lay.fft_bytes);
@@ -464,8 +469,7 @@ static cudaError_t launch_fwd_y_tma_t(const Geom &g, const Work<float> &w, cudaS
     const int ntiles = ((2 * g.SP + C - 1) / C) * g.N;
     if (e == cudaSuccess) e = persistent_grid(k, T, lay.total(), ntiles, grid);
     if (e != cudaSuccess) return e;
-    k<<<grid, T, lay.total(), s>>>(g, map, (float2 *)w.Y, twiddles_for<float>(w, L), w.status, box_rows);
-    return cudaGetLastError();
+    return launch_after(k, grid, T, lay.total(), s, g, map, (float2 *)w.Y, twiddles_for<float>(w, L), w.status, box_rows);
 }
 
 template <int L, typename Cfg>
@@ -485,8 +489,7 @@ static cudaError_t launch_inv_y_tma_t(const Geom &g, const Work<float> &w, cudaS
     const int ntiles = ((g.H + C - 1) / C) * g.Q;
     if (e == cudaSuccess) e = persistent_grid(k, T, lay.total(), ntiles, grid);
     if (e != cudaSuccess) return e;
-    k<<<grid, T, lay.total(), s>>>(g, map, (float2 *)w.Y, twiddles_for<float>(w, L), w.status, box_rows);
-    return cudaGetLastError();
+    return launch_after(k, grid, T, lay.total(), s, g, map, (float2 *)w.Y, twiddles_for<float>(w, L), w.status, box_rows);
 }
 
 template <int L, typename Cfg>
@@ -508,8 +511,7 @@ static cudaError_t launch_x_product_tma_t(const Geom &g, const Work<float> &w, c
     const int ntiles = ((g.H + C - 1) / C) * g.P;
     if (e == cudaSuccess) e = persistent_grid(k, T, lay.total(), ntiles, grid);
     if (e != cudaSuccess) return e;
-    k<<<grid, T, lay.total(), s>>>(g, map, (float2 *)w.X, twiddles_for<float>(w, L), w.status, box_rows);
-    return cudaGetLastError();
+    return launch_after(k, grid, T, lay.total(), s, g, map, (float2 *)w.X, twiddles_for<float>(w, L), w.status, box_rows);
 }
 
 
@@ -539,8 +541,7 @@ static cudaError_t launch_y_col_tma_t(const Geom &g, const Work<float> &w, cudaS
     int grid = 0;
     if (e == cudaSuccess) e = persistent_grid(k, T, lay.total(), ntiles, grid);
     if (e != cudaSuccess) return e;
-    k<<<grid, T, lay.total(), s>>>(g, map, (float2 *)w.Y, twiddles_for<float>(w, L), w.status, box_rows);
-    return cudaGetLastError();
+    return launch_after(k, grid, T, lay.total(), s, g, map, (float2 *)w.Y, twiddles_for<float>(w, L), w.status, box_rows);
 }
 
 
@@ -575,8 +576,7 @@ static cudaError_t launch_inv_energy_tma_t(const Geom &g, const Work<float> &w, 
     const int ntiles = (int)(((long long)g.Q * g.Q / 2 + C - 1) / C);
     if (e == cudaSuccess) e = persistent_grid(k, T, lay.total(), ntiles, grid);
     if (e != cudaSuccess) return e;
-    k<<<grid, T, lay.total(), s>>>(g, map, out, twiddles_for<float>(w, L), w.status, bx, nbx);
-    return cudaGetLastError();
+    return launch_after(k, grid, T, lay.total(), s, g, map, out, twiddles_for<float>(w, L), w.status, bx, nbx);
 }
 
 cudaError_t launch_inv_energy_tma(const Geom &g, const Work<float> &w, float *out, cudaStream_t s)

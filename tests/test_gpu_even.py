@@ -48,7 +48,10 @@ def _both(lh, grid, band):
 
 
 # cosine lengths M: (N + Q/2)/2 rounded up to 16, 24, 32, ..., 2048
+# in the order of the list: 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, ..., then
+# the lengths 72, 144, 288, 432, 576, 864 and 1152
 @pytest.mark.parametrize("zones,npz,q", [
+    (4, 24, 92), (5, 36, 200), (4, 100, 340), (6, 96, 560), (8, 90, 820), (8, 150, 1000), (8, 192, 1400),
     (4, 4, 16), (5, 6, 30), (4, 10, 40), (4, 16, 64), (4, 20, 60), (5, 24, 118), (4, 32, 128), (6, 32, 2),
     (4, 64, 256), (4, 64, 512), (7, 50, 700), (8, 64, 512), (4, 160, 640), (8, 128, 1024), (8, 192, 2),
     (8, 240, 2000), (8, 256, 2048),
@@ -118,7 +121,7 @@ def test_unaligned_output(lh):
     (4, 4, 3, 2, 16, 0), (4, 10, 34, 17, 40, 0), (5, 24, 37, 30, 118, 0), (4, 32, 128, 64, 128, 0),
     (4, 16, 201, 90, 128, 0), (6, 32, 20, 10, 2, 0), (4, 16, 300, 150, 64, 0), (4, 12, 512, 256, 48, 0),
     (4, 20, 401, 33, 60, 0), (4, 12, 40, 25, 48, 1), (4, 12, 150, 75, 48, 2), (4, 12, 200, 150, 60, 1),
-    (4, 12, 300, 200, 48, 2)])
+    (4, 12, 300, 200, 48, 2), (4, 24, 30, 15, 92, 0), (5, 36, 20, 10, 200, 0), (6, 96, 8, 4, 560, 0)])
 def test_parameter_gradient(lh, zones, npz, n_eps, n_omega, q, quantity):
     import torch
     grid = wl.grid_params(zones, npz, n_eps, 2.0, n_omega=n_omega, q_extent=q, quantity=quantity)

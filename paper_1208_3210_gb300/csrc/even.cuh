@@ -36,9 +36,9 @@
 // and the inverse is V = FFT(v), z_j = (conj(w_j) V_j + w_j V_{M-j}) / 2.
 //
 // The edge.  The grid p_i = (i - N/2) dp holds p = -N/2 dp without its mirror.
-// This form leaves that row and column of A out, so it is taken only when
-// their weight |M|^2 is below 2^-24 of the centre's (ev_band_applies): their
-// part of Im chi is then below the rounding of its FP32 sums.
+// This form leaves that row and column of A out where their weight |M|^2 is
+// below 2^-24 of the centre's (ev_band_applies): their part of Im chi is then
+// below the rounding of its FP32 sums.  Otherwise k_even_edge.cu carries them.
 #pragma once
 
 #include "kernels.cuh"
@@ -121,6 +121,29 @@ inline long long ev_x_floats(const EvGeom &v)
 inline long long ev_y_floats(const EvGeom &v)
 {
     const long long a = v.M * v.s2, b = v.nl * v.s4;
+    return a > b ? a : b;
+}
+// The same with the edge row and column (k_even_edge.cu): one row more, four
+// volumes B3 (of k_x <= k_y) and two B4 of every lag s_x, and after B2 the edge
+// lines' energy spectra and the M values sin(N theta_k / 2).
+inline bool ev_edge_geom(const Geom &g, EvGeom &v)
+{
+    if (!ev_geom(g, v) || v.PE > 512) return false;
+    v.Nh = g.N / 2 + 1;
+    v.s3 = 4LL * v.M * v.WS + 64;
+    v.s4 = 2LL * v.M * v.WS + 64;
+    v.scale *= 0.5f;
+    return true;
+}
+__host__ __device__ inline long long ev_edge_lines(const EvGeom &v) { return 4LL * (v.M + 1) * (v.PE / 2 + 16); }
+inline long long ev_edge_x_floats(const EvGeom &v)
+{
+    const long long a = v.Nh * v.s1, b = v.M * v.s3;
+    return a > b ? a : b;
+}
+inline long long ev_edge_y_floats(const Geom &g, const EvGeom &v)
+{
+    const long long a = v.M * v.s2 + ev_edge_lines(v) + v.M, b = g.Q * v.s4;
     return a > b ? a : b;
 }
 // The edge row's weight against the centre's, exp(-(N dp / 2)^2 ff_a^2 / 8),
@@ -435,6 +458,15 @@ struct EvFft {
         rest<1>(v, sm, u, tab);
     }
 };
+
+// 1/x as the hardware approximation (relative error about 2^-23; x lies in
+// [gamma^2, 4 e_max^2 + gamma^2], away from zero, subnormals and overflow)
+__device__ __forceinline__ float ev_rcp(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
 
 // A pack from global memory, read once: not kept in L1, whose few KB beside the
 // exchange buffers hold the tables.

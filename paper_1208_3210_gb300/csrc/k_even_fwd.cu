@@ -13,15 +13,6 @@
 
 namespace lh {
 
-// 1/x as the hardware approximation (relative error about 2^-23; x lies in
-// [gamma^2, 4 e_max^2 + gamma^2], away from zero, subnormals and overflow)
-__device__ __forceinline__ float ev_rcp(float x)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 // One block per table and slice: the tables' places and periods come as an
 // argument (evaluating ev_table_offset per entry on the device took 0.5 ms).
 struct EvTabs {
@@ -57,7 +48,6 @@ cudaError_t launch_ev_tables(float2 *out, cudaStream_t s)
     for (int i = 0; ev_line_len(i) != 0; ++i) tabs.t[n++] = {(o + 1) / 2 * 2 + 128 * i, 128, -1, ev_line_len(i)};
     k_ev_tables<<<dim3(n, 4), 128, 0, s>>>(out, tabs);
     return cudaGetLastError();
-    return cudaGetLastError();
 }
 size_t ev_table_bytes() { return (size_t)ev_all_tables() * sizeof(float2); }
 
@@ -79,10 +69,13 @@ k_ev_gen_y(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const 
     // band energy and amplitude of every row, once per tile (16 Nh bytes in the
     // exchange buffer, which has M > Nh rows of at least two packs)
     float4 *rows = sm;
-    const AxisTab ax = axis[g.N / 2 + jx];
+    const int half = g.N / 2;   // the edge, where it is kept: index 0 of the axis, half its weight on either side
+    const AxisTab ax = axis[jx == half ? 0 : half + jx];
     for (int i = threadIdx.x; i < v.Nh; i += T) {
         float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-        band_point_f32(band, ax, axis[g.N / 2 + i], st, q.x, q.y, q.z);
+        band_point_f32(band, ax, axis[i == half ? 0 : half + i], st, q.x, q.y, q.z);
+        if (jx == half) q.z *= 0.5f;
+        if (i == half) q.z *= 0.5f;
         rows[i] = q;
     }
     __syncthreads();

@@ -66,6 +66,11 @@ cudaError_t launch_ev_corr(const Geom &g, const EvGeom &v, const Band &band, con
                            cudaStream_t s);
 cudaError_t launch_ev_inv_x(const EvGeom &v, const Work<float> &w, cudaStream_t s);
 cudaError_t launch_ev_inv_y(const Geom &g, const EvGeom &v, const Work<float> &w, float *out, cudaStream_t s);
+cudaError_t launch_ev_edge(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, cudaStream_t s);
+cudaError_t launch_ev_edge_corr(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, int sms,
+                                cudaStream_t s);
+cudaError_t launch_ev_edge_inv_x(const Geom &g, const EvGeom &v, const Work<float> &w, cudaStream_t s);
+cudaError_t launch_ev_edge_inv_y(const Geom &g, const EvGeom &v, const Work<float> &w, float *out, cudaStream_t s);
 bool ev_bw_applies(const EvGeom &v);
 int ev_chain_blocks(const EvGeom &v);
 cudaError_t launch_ev_w_y(const Geom &g, const EvGeom &v, const float *wts, const Work<float> &w, cudaStream_t s);
@@ -168,7 +173,7 @@ struct lindhard_plan {
     std::vector<Slot> slots;
     size_t off_tw32 = 0, off_tw64 = 0, off_status = 0, off_tc = 0, off_dmu = 0, off_prtw = 0, off_etw = 0, off_evt = 0;
     // the even form's geometry of each instance (even.cuh); M = 0: not taken
-    std::vector<EvGeom> even;
+    std::vector<EvGeom> even, edge;   // (edge: with the edge row, for bands whose weight there counts)
     std::vector<size_t> off_cls;  // momentum class tables per instance (one for all instances of as many points per zone)
     std::vector<size_t> off_kk;   // Kramers-Kronig weight tables per instance (FP32 grids)
     int tw_len = 0;
@@ -546,9 +551,11 @@ extern "C" lindhard_status lindhard_plan_create(const lindhard_grid *grids, int 
     p->tw_len = maxLen;
 
     p->even.assign(batch, EvGeom{});
+    p->edge.assign(batch, EvGeom{});
     for (int i = 0; i < batch; ++i) {
         EvGeom v;
         if (p->precision[i] == LINDHARD_FP32 && !p->direct && ev_geom(p->geoms[i], v)) p->even[i] = v;
+        if (p->even[i].M && ev_edge_geom(p->geoms[i], v)) p->edge[i] = v;
     }
 
     // bytes of each workspace part for instance i
@@ -571,6 +578,10 @@ extern "C" lindhard_status lindhard_plan_create(const lindhard_grid *grids, int 
         if (p->even[i].M) {
             n.X = std::max(n.X, sizeof(float) * (size_t)ev_x_floats(p->even[i]));
             n.Y = std::max(n.Y, sizeof(float) * (size_t)ev_y_floats(p->even[i]));
+        }
+        if (p->edge[i].M) {
+            n.X = std::max(n.X, sizeof(float) * (size_t)ev_edge_x_floats(p->edge[i]));
+            n.Y = std::max(n.Y, sizeof(float) * (size_t)ev_edge_y_floats(p->geoms[i], p->edge[i]));
         }
         n.Z = p->backward ? (size_t)g.Q * (size_t)g.xs3 * cb : 0;
         // the last pass's per-CTA sums, then the first reduction level's
@@ -985,6 +996,20 @@ static cudaError_t enqueue_forward(lindhard_plan *p, const std::vector<Band> &bs
                 for (int k = 0; k < 5 && e == cudaSuccess; ++k)
                     e = timed(p, 2 + k, s, [&] { return launch_direct_stage(k, g, b, w, a_i, o_i, s); });
                 a_off += (size_t)g.N * g.N * g.n_eps;
+                o_off += (size_t)g.Q * g.Q * g.n_omega;
+                continue;
+            }
+            if (const EvGeom &v = p->edge[i]; A_in == nullptr && v.M && !ev_band_applies(g, b)) {
+                // the same with the edge row and column
+                if (e == cudaSuccess) e = timed(p, 2, s, [&] { return launch_ev_gen_y(g, v, b, w, s); });
+                if (e == cudaSuccess) e = timed(p, 3, s, [&] { return launch_ev_x(v, w, s); });
+                if (e == cudaSuccess)
+                    e = timed(p, 4, s, [&] {
+                        const cudaError_t e0 = launch_ev_edge(g, v, b, w, s);
+                        return e0 == cudaSuccess ? launch_ev_edge_corr(g, v, b, w, p->num_sms, s) : e0;
+                    });
+                if (e == cudaSuccess) e = timed(p, 5, s, [&] { return launch_ev_edge_inv_x(g, v, w, s); });
+                if (e == cudaSuccess) e = timed(p, 6, s, [&] { return launch_ev_edge_inv_y(g, v, w, o_i, s); });
                 o_off += (size_t)g.Q * g.Q * g.n_omega;
                 continue;
             }

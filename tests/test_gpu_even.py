@@ -100,6 +100,48 @@ def test_both_sides_of_the_edge_weight(lh, ff_a):
     assert np.abs(got - ref).max() <= TOL * np.abs(ref).max()
 
 
+# The edge row carried (few zones, small ff_a): every cosine length, lags from
+# one to all of them, energy lengths 128 to 512, transfers of every remainder.
+@pytest.mark.parametrize("zones,npz,q", [
+    (2, 4, 2), (2, 4, 16), (3, 10, 60), (2, 16, 32), (2, 24, 96), (3, 20, 30), (2, 48, 96), (3, 36, 216), (2, 64, 256),
+    (3, 50, 300), (2, 100, 300), (2, 128, 256), (4, 100, 340), (2, 192, 768), (6, 96, 560), (4, 128, 1024),
+    (8, 90, 820), (4, 192, 1536), (8, 150, 1000), (4, 256, 2048), (8, 192, 1400), (8, 192, 3072), (8, 256, 4096)])
+def test_edge_lengths(lh, zones, npz, q):
+    big = zones * npz >= 1024
+    grid = wl.grid_params(zones, npz, 6 if big else 34, 2.0, q_extent=q)
+    a, g = _both(lh, grid, wl.band_params(filling=1.1, gamma=0.3 if big else 0.08, ff_a=0.3))
+    assert float((a - g).abs().max()) <= TOL * float(g.abs().max())
+
+
+@pytest.mark.parametrize("n_eps,n_omega", [(2, 1), (3, 2), (16, 1), (37, 11), (128, 64), (129, 129), (200, 30),
+                                           (256, 128), (300, 150), (384, 384), (401, 77), (512, 256), (512, 512)])
+@pytest.mark.parametrize("quantity", [0, 1, 2])
+def test_edge_energies(lh, n_eps, n_omega, quantity):
+    if quantity and n_eps + n_omega - 1 > 512:
+        pytest.skip("beyond the energy lengths that carry the edge")
+    grid = wl.grid_params(2, 12, n_eps, 2.0, n_omega=n_omega, quantity=quantity, q_extent=40)
+    band = wl.band_params(filling=1.1, gamma=0.08, ff_a=0.0, **({"kT": 0.06} if quantity else {}))
+    a, g = _both(lh, grid, band)
+    scale = float(_both(lh, dict(grid, n_omega=n_eps), band)[1].abs().max()) if n_omega < n_eps else float(g.abs().max())
+    assert float((a - g).abs().max()) <= TOL * scale
+
+
+@pytest.mark.parametrize("quantity", [0, 1])
+def test_edge_free_electrons_unaligned(lh, quantity):
+    import torch
+    grid = wl.grid_params(2, 16, 40, 2.0, quantity=quantity)
+    band = wl.band_params(kind=1, mu=0.7, filling=float("nan"), gamma=0.1, ff_a=0.2, kT=0.05 if quantity else 0.0)
+    a, g = _both(lh, grid, band)
+    assert float((a - g).abs().max()) <= TOL * float(g.abs().max())
+    plan = lh.Plan([grid])
+    ref = plan.imchi([band])
+    buf = torch.zeros(plan.out_elems() + 1, device="cuda")
+    plan.imchi([band], out=buf[1:])
+    plan.status()
+    assert torch.equal(buf[1:], ref)
+    plan.close()
+
+
 def test_unaligned_output(lh):
     import torch
     grid = wl.grid_params(4, 16, 32, 1.5)

@@ -120,7 +120,7 @@ struct Work {
     const void *tc;        // tensor-core DFT matrices (k_tc.cu), or null
     const void *ptw = nullptr;   // per-stage twiddle tables of the pruned engine (FP32), or null
     const void *etw = nullptr;   // per-stage twiddle tables of the lines-across-lanes energy pass, or null
-    const void *evt = nullptr;   // tables of the even form's cosine transforms (FP32), or null
+    const void *evt = nullptr;   // tables of the even form's transforms, or null
     const ClsTab *cls = nullptr;  // the zone's class table, or null
     InstState *state;      // [1]
     unsigned *status;      // plan-wide device status word

@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "even.cuh"
+#include "even64.cuh"
 #include "kernels.cuh"
 
 namespace lh {
@@ -71,6 +72,11 @@ cudaError_t launch_ev_edge_corr(const Geom &g, const EvGeom &v, const Band &band
                                 cudaStream_t s);
 cudaError_t launch_ev_edge_inv_x(const Geom &g, const EvGeom &v, const Work<float> &w, cudaStream_t s);
 cudaError_t launch_ev_edge_inv_y(const Geom &g, const EvGeom &v, const Work<float> &w, float *out, cudaStream_t s);
+size_t e64_table_bytes();
+cudaError_t launch_e64_tables(double2 *out, cudaStream_t s);
+cudaError_t launch_e64_pass(int pass, const Geom &g, const E64Geom &v, const Band &band, const Work<double> &w, double *out,
+                            cudaStream_t s);
+cudaError_t launch_e64_corr(const Geom &g, const E64Geom &v, const Band &band, const Work<double> &w, cudaStream_t s);
 bool ev_bw_applies(const EvGeom &v);
 int ev_chain_blocks(const EvGeom &v);
 cudaError_t launch_ev_w_y(const Geom &g, const EvGeom &v, const float *wts, const Work<float> &w, cudaStream_t s);
@@ -173,6 +179,8 @@ struct lindhard_plan {
     std::vector<Slot> slots;
     size_t off_tw32 = 0, off_tw64 = 0, off_status = 0, off_tc = 0, off_dmu = 0, off_prtw = 0, off_etw = 0, off_evt = 0;
     // the even form's geometry of each instance (even.cuh); M = 0: not taken
+    std::vector<E64Geom> even64;   // FP64 grids' (even64.cuh)
+    size_t off_e64 = 0;            // its tables (0: no FP64 grid)
     std::vector<EvGeom> even, edge;   // (edge: with the edge row, for bands whose weight there counts)
     std::vector<size_t> off_cls;  // momentum class tables per instance (one for all instances of as many points per zone)
     std::vector<size_t> off_kk;   // Kramers-Kronig weight tables per instance (FP32 grids)
@@ -552,9 +560,12 @@ extern "C" lindhard_status lindhard_plan_create(const lindhard_grid *grids, int 
 
     p->even.assign(batch, EvGeom{});
     p->edge.assign(batch, EvGeom{});
+    p->even64.assign(batch, E64Geom{});
     for (int i = 0; i < batch; ++i) {
         EvGeom v;
         if (p->precision[i] == LINDHARD_FP32 && !p->direct && ev_geom(p->geoms[i], v)) p->even[i] = v;
+        E64Geom v64;
+        if (p->precision[i] == LINDHARD_FP64 && e64_geom(p->geoms[i], v64)) p->even64[i] = v64;
         if (p->even[i].M && ev_edge_geom(p->geoms[i], v)) p->edge[i] = v;
     }
 
@@ -583,6 +594,10 @@ extern "C" lindhard_status lindhard_plan_create(const lindhard_grid *grids, int 
             n.X = std::max(n.X, sizeof(float) * (size_t)ev_edge_x_floats(p->edge[i]));
             n.Y = std::max(n.Y, sizeof(float) * (size_t)ev_edge_y_floats(p->geoms[i], p->edge[i]));
         }
+        if (p->even64[i].M) {
+            n.X = std::max(n.X, sizeof(double) * e64_x_doubles(p->even64[i]));
+            n.Y = std::max(n.Y, sizeof(double) * e64_y_doubles(g, p->even64[i]));
+        }
         n.Z = p->backward ? (size_t)g.Q * (size_t)g.xs3 * cb : 0;
         // the last pass's per-CTA sums, then the first reduction level's
         n.partial = p->backward ? (size_t)(bw_energy_blocks(g) + bw_partial_extra_rows()) * 5 * sizeof(double) : 0;
@@ -605,6 +620,9 @@ extern "C" lindhard_status lindhard_plan_create(const lindhard_grid *grids, int 
     p->off_prtw = o; o = align_up(o + pr_twiddle_bytes());   // pruned engine's per-stage twiddles
     p->off_etw = o; o = align_up(o + et_twiddle_bytes());     // energy pass's per-stage twiddles
     p->off_evt = o; o = align_up(o + ev_table_bytes());       // the even form's tables
+    if (std::count(p->precision.begin(), p->precision.end(), (int)LINDHARD_FP64) > 0) {
+        p->off_e64 = o; o = align_up(o + e64_table_bytes());
+    }
     p->off_dmu = o; o = align_up(o + sizeof(double) * 5 * kDmuBlocks);
     // tensor-core DFT matrices of every supported length (plans with a
     // LINDHARD_SPLITBF16_TC grid only)
@@ -672,6 +690,7 @@ extern "C" lindhard_status lindhard_plan_create(const lindhard_grid *grids, int 
     if (e == cudaSuccess) e = launch_pr_twiddles((float2 *)(p->ws + p->off_prtw), 0);
     if (e == cudaSuccess) e = launch_et_twiddles((float2 *)(p->ws + p->off_etw), 0);
     if (e == cudaSuccess) e = launch_ev_tables((float2 *)(p->ws + p->off_evt), 0);
+    if (e == cudaSuccess && p->off_e64) e = launch_e64_tables((double2 *)(p->ws + p->off_e64), 0);
     for (int i = 0; i < batch && e == cudaSuccess; ++i)
         if (std::find(p->off_cls.begin(), p->off_cls.begin() + i, p->off_cls[i]) == p->off_cls.begin() + i)
             e = launch_classes(p->geoms[i].npz, (ClsTab *)(p->ws + p->off_cls[i]), 0);
@@ -872,7 +891,7 @@ static Work<Real> work_of(lindhard_plan *p, int i)
     w.tc = p->off_tc ? (const void *)(p->ws + p->off_tc) : nullptr;
     w.ptw = sizeof(Real) == 4 ? (const void *)(p->ws + p->off_prtw) : nullptr;
     w.etw = sizeof(Real) == 4 ? (const void *)(p->ws + p->off_etw) : nullptr;
-    w.evt = sizeof(Real) == 4 ? (const void *)(p->ws + p->off_evt) : nullptr;
+    w.evt = (const void *)(p->ws + (sizeof(Real) == 4 ? p->off_evt : p->off_e64));
     w.state = (InstState *)(p->ws + sl.state);
     w.status = (unsigned *)(p->ws + p->off_status);
     w.cls = (const ClsTab *)(p->ws + p->off_cls[i]);
@@ -1023,6 +1042,15 @@ static cudaError_t enqueue_forward(lindhard_plan *p, const std::vector<Band> &bs
                 o_off += (size_t)g.Q * g.Q * g.n_omega;
                 continue;
             }
+        } else if (const E64Geom &v = p->even64[i]; A_in == nullptr && v.M) {
+            // the same with the edge row and column, in double precision
+            if (e == cudaSuccess) e = timed(p, 2, s, [&] { return launch_e64_pass(0, g, v, b, w, o_i, s); });
+            if (e == cudaSuccess) e = timed(p, 3, s, [&] { return launch_e64_pass(1, g, v, b, w, o_i, s); });
+            if (e == cudaSuccess) e = timed(p, 4, s, [&] { return launch_e64_corr(g, v, b, w, s); });
+            if (e == cudaSuccess) e = timed(p, 5, s, [&] { return launch_e64_pass(2, g, v, b, w, o_i, s); });
+            if (e == cudaSuccess) e = timed(p, 6, s, [&] { return launch_e64_pass(3, g, v, b, w, o_i, s); });
+            o_off += (size_t)g.Q * g.Q * g.n_omega;
+            continue;
         }
         if (e == cudaSuccess) e = timed(p, 2, s, [&] { return launch_fwd_energy(g, b, w, a_i, s); });
         if (e == cudaSuccess) e = timed(p, 3, s, [&] { return launch_fwd_y(g, w, s, p->yvar_fwd[i]); });

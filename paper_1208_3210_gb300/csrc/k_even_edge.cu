@@ -28,18 +28,38 @@
 // Against the general form (full grid, complex): half of the energy
 // transforms, no transform of A's mirror images, and B2 and B3, B4 of M^2
 // instead of P^2 frequencies.  Measured us a call without form factor, general
-// (tuned) -> this: 128^2 x 128 69 -> 54, 256^2 x 256 290 -> 145, all lags of
-// 150^2 x 201 276 -> 125, Im chi_T of 288^2 x 200 697 -> 259, 1024^2 x 512 8185
-// -> 3740; no grid was found on which the general form is the faster one.
+// (tuned) -> this: 128^2 x 128 69 -> 53, 256^2 x 256 290 -> 126, all lags of
+// 150^2 x 201 276 -> 105, 320^2 x 400 929 -> 309, 1024^2 x 512 8185 -> 3540; no
+// grid was found on which the general form is the faster one.  The correlation
+// there went from 1118 to 1039 us, at 512^2 x 256 from 247 to 139 us, with its
+// products packed over two frequencies, the corner's spectrum in shared memory
+// and the edge lines' loaded a step ahead.
 #include "even.cuh"
 #include "even_line.cuh"
 #include "et_tiles.cuh"
 
 namespace lh {
 
-// Energy spectra of the edge lines, separated (occupied re, im, empty re, im),
-// line t < M: a(k_t, e), line M: c(e).  A lane's values in the order of the
-// correlation's registers, [line][R1 + 1][TPL]: its frequencies k <= L/2.
+// A line's occupied and empty spectra at two frequencies k <= L/2 at once: row r
+// of a lane's first and of its second butterfly (packed, one in each half).
+struct EdgeLine { Cx2 occ, emp; };
+__device__ __forceinline__ EdgeLine edge_separate(Cx2 k, Cx2 m)   // Z(k), Z(L - k); z holds the 1/2
+{
+    return {{add2(k.re, m.re), sub2(k.im, m.im)}, {add2(k.im, m.im), sub2(m.re, k.re)}};
+}
+// Z(L - k) for these: row r of the first butterfly mirrors row R1 - r (u = 0) or
+// the second's R1 - 1 - r, row r of the second its own R1 - 1 - r (u = 0) or the
+// first's.
+template <int R1>
+__device__ __forceinline__ Cx2 edge_mirror(const float2 *x, int r, bool u0)
+{
+    const float2 a = u0 ? x[(R1 - r) % R1] : x[R1 + R1 - 1 - r], b = u0 ? x[R1 + R1 - 1 - r] : x[R1 - 1 - r];
+    return {make_float2(a.x, b.x), make_float2(a.y, b.y)};
+}
+
+// Energy spectra of the edge lines, separated; line t < M: a(k_t, e), line M:
+// c(e).  A lane's values in the order of the correlation's registers: per line
+// [R1 / 2][occupied, empty][TPL] packs, then [TPL] (occupied, empty) at L/2.
 template <int L, bool THERMAL>
 __global__ void __launch_bounds__(32 * EVC_WARPS, EvLine<L>::MINB)
 k_ev_edge(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const float2 *__restrict__ eps,
@@ -87,37 +107,61 @@ k_ev_edge(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const f
     if (t > v.M) return;
     const bool u0 = u == 0;
     float4 *o = lines + (long long)t * (R1 + 1) * TPL + u;
-    auto sep = [](float2 zk, float2 zm) { return make_float4(zk.x + zm.x, zk.y - zm.y, zk.y + zm.y, zm.x - zk.x); };
 #pragma unroll
     for (int r = 0; r < R1 / 2; ++r) {
-        o[r * TPL] = sep(x[r], u0 ? x[(R1 - r) % R1] : x[R1 + R1 - 1 - r]);
-        o[(R1 / 2 + r) * TPL] = sep(x[R1 + r], u0 ? x[R1 + R1 - 1 - r] : x[R1 - 1 - r]);
+        const EdgeLine q = edge_separate({make_float2(x[r].x, x[R1 + r].x), make_float2(x[r].y, x[R1 + r].y)},
+                                         edge_mirror<R1>(x, r, u0));
+        EvFft<16, false>::st(o + 2 * r * TPL, q.occ);
+        EvFft<16, false>::st(o + (2 * r + 1) * TPL, q.emp);
     }
-    o[R1 * TPL] = sep(x[R1 / 2], x[R1 / 2]);
+    const EdgeLine h = edge_separate({dup2(x[R1 / 2].x), dup2(x[R1 / 2].y)}, {dup2(x[R1 / 2].x), dup2(x[R1 / 2].y)});
+    o[R1 * TPL] = make_float4(h.occ.re.x, h.occ.im.x, h.emp.re.x, h.emp.im.x);
 }
 
-// The four parity parts' spectra at one energy frequency from E^ and the edge
-// lines there: (EE, OY) and (OX, OO), twice each (in v.scale).
-struct EdgeParts { float2 ee, oo, ox, oy; };
-template <bool THERMAL>
-__device__ __forceinline__ EdgeParts ev_edge_parts(float4 e, float4 ay, float4 ax, float4 c, float sx, float sy, bool odd)
+// The four parity parts' spectra, twice each (in v.scale), from E^ and the edge
+// lines there.  Packed over two frequencies: 80 instructions instead of 160.
+struct EdgeParts { Cx2 ee, oo, ox, oy; };
+__device__ __forceinline__ Cx2 edge_scaled(Cx2 a, float2 s) { return {mul2(a.re, s), mul2(a.im, s)}; }
+__device__ __forceinline__ Cx2 edge_fma(Cx2 a, float2 s, Cx2 b) { return {fma2(a.re, s, b.re), fma2(a.im, s, b.im)}; }
+// In program order (volatile): these are loaded a step ahead of their use.
+// Loaded where they are used, each step waits for them (512^2 x 256 of two
+// zones: 250 us instead of 149).
+__device__ __forceinline__ Cx2 edge_load(const float4 *p)
 {
-    const float t = sx * sy;
-    const float2 eo = make_float2(e.x, e.y), eu = make_float2(e.z, e.w);
-    const float2 co = make_float2(t * c.x, t * c.y), cu = make_float2(t * c.z, t * c.w);
-    const float2 xo = make_float2(sx * ay.x, sx * ay.y), xu = make_float2(sx * ay.z, sx * ay.w);
-    const float2 yo = make_float2(sy * ax.x, sy * ax.y), yu = make_float2(sy * ax.z, sy * ax.w);
-    const float2 r1o = csub(eo, co), r1u = csub(eu, cu), r2o = cadd(eo, co), r2u = cadd(eu, cu);
-    const float2 i1o = cadd(yo, xo), i1u = cadd(yu, xu), i2o = csub(yo, xo), i2u = csub(yu, xu);
-    const float2 re1 = cadd(cmulc(r1u, r1o), cmulc(i1u, i1o)), re2 = cadd(cmulc(r2u, r2o), cmulc(i2u, i2o));
-    const float2 im1 = csub(cmulc(r1u, i1o), cmulc(i1u, r1o)), im2 = csub(cmulc(r2u, i2o), cmulc(i2u, r2o));   // -Im
-    EdgeParts p = {cadd(re1, re2), csub(re2, re1), csub(im1, im2), cadd(im1, im2)};
+    float4 q;
+    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(q.x), "=f"(q.y), "=f"(q.z), "=f"(q.w) : "l"(p));
+    return {make_float2(q.x, q.y), make_float2(q.z, q.w)};
+}
+// conj(a) b + conj(c) d and conj(a) b - conj(c) d
+__device__ __forceinline__ Cx2 edge_sum(Cx2 a, Cx2 b, Cx2 c, Cx2 d)
+{
+    return {fma2(c.im, d.im, fma2(c.re, d.re, fma2(a.im, b.im, mul2(a.re, b.re)))),
+            sub2(fma2(c.re, d.im, mul2(a.re, b.im)), fma2(c.im, d.re, mul2(a.im, b.re)))};
+}
+__device__ __forceinline__ Cx2 edge_diff(Cx2 a, Cx2 b, Cx2 c, Cx2 d)
+{
+    return {sub2(fma2(a.im, b.im, mul2(a.re, b.re)), fma2(c.im, d.im, mul2(c.re, d.re))),
+            sub2(fma2(c.im, d.re, mul2(a.re, b.im)), fma2(c.re, d.im, mul2(a.im, b.re)))};
+}
+template <bool THERMAL>
+__device__ __forceinline__ EdgeParts edge_parts(EdgeLine e, EdgeLine ay, EdgeLine ax, EdgeLine c, float sx, float sy,
+                                                bool odd)
+{
+    const float2 t = dup2(sx * sy), nt = neg2(t), px = dup2(sx), nx = neg2(px), py = dup2(sy);
+    const Cx2 r1o = edge_fma(c.occ, nt, e.occ), r1u = edge_fma(c.emp, nt, e.emp);   // R at (k_x, k_y) and (-k_x, k_y)
+    const Cx2 r2o = edge_fma(c.occ, t, e.occ), r2u = edge_fma(c.emp, t, e.emp);
+    const Cx2 yo = edge_scaled(ax.occ, py), yu = edge_scaled(ax.emp, py);
+    const Cx2 i1o = edge_fma(ay.occ, px, yo), i1u = edge_fma(ay.emp, px, yu);       // I there
+    const Cx2 i2o = edge_fma(ay.occ, nx, yo), i2u = edge_fma(ay.emp, nx, yu);
+    const Cx2 re1 = edge_sum(r1o, r1u, i1o, i1u), re2 = edge_sum(r2o, r2u, i2o, i2u);
+    const Cx2 im1 = edge_diff(i1o, r1u, r1o, i1u), im2 = edge_diff(i2o, r2u, r2o, i2u);   // -Im
+    EdgeParts p = {add(re1, re2), sub(re2, re1), sub(im1, im2), add(im1, im2)};
     if (THERMAL && odd) {
         // C(s, w) - C(-s, -w): the parts odd in one axis change sign with s
-        p.ee = make_float2(0.f, p.ee.y + p.ee.y);
-        p.oo = make_float2(0.f, p.oo.y + p.oo.y);
-        p.ox = make_float2(p.ox.x + p.ox.x, 0.f);
-        p.oy = make_float2(p.oy.x + p.oy.x, 0.f);
+        p.ee = {dup2(0.f), add2(p.ee.im, p.ee.im)};
+        p.oo = {dup2(0.f), add2(p.oo.im, p.oo.im)};
+        p.ox = {add2(p.ox.re, p.ox.re), dup2(0.f)};
+        p.oy = {add2(p.oy.re, p.oy.re), dup2(0.f)};
     }
     return p;
 }
@@ -131,6 +175,11 @@ __host__ __device__ constexpr int ev_edge_smem()   // float2 of a warp
 {
     return EvLine<L>::WARP_ELEMS + 32 * EvLine<L>::VPT;
 }
+template <int L>
+__host__ __device__ constexpr int ev_edge_corner()   // float2 of the corner's spectrum, one copy a CTA
+{
+    return 2 * (EvLine<L>::R1 + 1) * EvLine<L>::TPL;
+}
 template <int L, bool THERMAL, bool HALF>
 __global__ void __launch_bounds__(32 * EVC_WARPS, EvLine<L>::MINB)
 k_ev_edge_corr(Geom g, EvGeom v, Band band, const float *__restrict__ B2, const float4 *__restrict__ lines,
@@ -139,24 +188,21 @@ k_ev_edge_corr(Geom g, EvGeom v, Band band, const float *__restrict__ B2, const 
     using E = EvLine<L>;
     constexpr int VPT = E::VPT, TPL = E::TPL, R0 = E::R0, R1 = E::R1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    LH_REQUIRE_SMEM(EVC_WARPS * ev_edge_smem<L>() + (THERMAL ? L : 0), float2)
+    LH_REQUIRE_SMEM(EVC_WARPS * ev_edge_smem<L>() + ev_edge_corner<L>() + (THERMAL ? L : 0), float2)
     after_previous();
     const int lane = (int)threadIdx.x % 32, warp = (int)threadIdx.x / 32;
     const int sl = lane / TPL, u = lane % TPL;
     float2 *sm = reinterpret_cast<float2 *>(smem_raw) + warp * ev_edge_smem<L>() + sl * E::LP;
     float2 *own = reinterpret_cast<float2 *>(smem_raw) + warp * ev_edge_smem<L>() + E::WARP_ELEMS + lane;   // stride 32
-    float2 *wf = reinterpret_cast<float2 *>(smem_raw) + EVC_WARPS * ev_edge_smem<L>();
-    if constexpr (THERMAL) {
-        et_fermi_weights<L>(g, band, wf, (int)threadIdx.x, 32 * EVC_WARPS);
-        __syncthreads();
-    }
+    float4 *corner = reinterpret_cast<float4 *>(reinterpret_cast<float2 *>(smem_raw) + EVC_WARPS * ev_edge_smem<L>());
+    float2 *wf = reinterpret_cast<float2 *>(smem_raw) + EVC_WARPS * ev_edge_smem<L>() + ev_edge_corner<L>();
+    for (int i = threadIdx.x; i < (R1 + 1) * TPL; i += 32 * EVC_WARPS) corner[i] = lines[(long long)v.M * (R1 + 1) * TPL + i];
+    if constexpr (THERMAL) et_fermi_weights<L>(g, band, wf, (int)threadIdx.x, 32 * EVC_WARPS);
+    __syncthreads();
     const float *sines = reinterpret_cast<const float *>(lines) + ev_edge_lines(v);
     const int nlines = v.M * (v.M + 1) / 2;
     const bool u0 = u == 0;
-    auto w_of = [](float2 x1, float2 x2) { return make_float2(x1.x - x2.y, x1.y + x2.x); };      // P1 + i P2
-    auto w_conj = [](float2 x1, float2 x2) { return make_float2(x1.x + x2.y, x2.x - x1.y); };    // conj P1 + i conj P2
-    auto sep = [](float2 zk, float2 zm) { return make_float4(zk.x + zm.x, zk.y - zm.y, zk.y + zm.y, zm.x - zk.x); };
-
+    // (one wave of CTAs with an equal share each: 320^2 x 400 138 us instead of 121)
     for (int it = 0; it < iters; ++it) {
         const int t = ((blockIdx.x * EVC_WARPS + warp) * iters + it) * E::LPI + sl;
         const bool live = t < nlines;
@@ -167,37 +213,44 @@ k_ev_edge_corr(Geom g, EvGeom v, Band band, const float *__restrict__ B2, const 
 #pragma unroll
         for (int i = 0; i < VPT; ++i) raw[i] = live && u + E::first(i) < v.ne ? __ldcs(p + E::first(i)) : 0.f;
         const float sx = __ldg(sines + kx), sy = __ldg(sines + ky);
-        const float4 *ly = lines + (long long)ky * (R1 + 1) * TPL + u, *lx = lines + (long long)kx * (R1 + 1) * TPL + u,
-                     *lc = lines + (long long)v.M * (R1 + 1) * TPL + u;
+        const float4 *ly = lines + (long long)ky * (R1 + 1) * TPL + u, *lx = lines + (long long)kx * (R1 + 1) * TPL + u;
         float2 x[VPT];
         E::template first_stage<false, THERMAL>(x, raw, u, v.J0, wf);
         E::forward_rest(x, sm, u, tab);
-        auto parts = [&](int j, float2 zk, float2 zm) {
-            return ev_edge_parts<THERMAL>(sep(zk, zm), __ldg(ly + j * TPL), __ldg(lx + j * TPL), __ldg(lc + j * TPL), sx, sy,
-                                          odd != 0);
-        };
-        // Frequencies k <= L/2 and their mirrors, in place: row r of the first
-        // butterfly mirrors row R1 - r (u = 0) or the second's R1 - 1 - r, row r
-        // of the second its own R1 - 1 - r (u = 0) or the first's.
+        auto line = [&](const float4 *l, int r) { return EdgeLine{edge_load(l + 2 * r * TPL), edge_load(l + (2 * r + 1) * TPL)}; };
+        auto line_c = [&](int r) { return EdgeLine{ev_get(corner + 2 * r * TPL + u), ev_get(corner + (2 * r + 1) * TPL + u)}; };
+        auto half = [&](float4 q) { return EdgeLine{{dup2(q.x), dup2(q.y)}, {dup2(q.z), dup2(q.w)}}; };
+        // P1 + i P2 at k, conj P1 + i conj P2 at L - k
+        auto w_of = [](Cx2 p, Cx2 q) { return Cx2{sub2(p.re, q.im), add2(p.im, q.re)}; };
+        auto w_conj = [](Cx2 p, Cx2 q) { return Cx2{add2(p.re, q.im), sub2(q.re, p.im)}; };
+        // frequencies k <= L/2 and their mirrors, in place (edge_mirror's rows)
+        EdgeLine ny = line(ly, 0), nx = line(lx, 0);
 #pragma unroll
         for (int r = 0; r < R1 / 2; ++r) {
-            const EdgeParts a = parts(r, x[r], u0 ? x[(R1 - r) % R1] : x[R1 + R1 - 1 - r]);
-            const EdgeParts b = parts(R1 / 2 + r, x[R1 + r], u0 ? x[R1 + R1 - 1 - r] : x[R1 - 1 - r]);
-            const float2 ac = w_conj(a.ee, a.oy), bc = w_conj(b.ee, b.oy);
-            x[r] = w_of(a.ee, a.oy);
-            x[R1 + r] = w_of(b.ee, b.oy);
+            const EdgeLine e = edge_separate({make_float2(x[r].x, x[R1 + r].x), make_float2(x[r].y, x[R1 + r].y)},
+                                             edge_mirror<R1>(x, r, u0));
+            const EdgeLine cy = ny, cx = nx;
+            if (r + 1 < R1 / 2) { ny = line(ly, r + 1); nx = line(lx, r + 1); }
+            const EdgeParts p = edge_parts<THERMAL>(e, cy, cx, line_c(r), sx, sy, odd != 0);
+            const Cx2 k1 = w_of(p.ee, p.oy), m1 = w_conj(p.ee, p.oy), k2 = w_of(p.ox, p.oo), m2 = w_conj(p.ox, p.oo);
+            const float2 ac = make_float2(m1.re.x, m1.im.x), bc = make_float2(m1.re.y, m1.im.y);
+            x[r] = make_float2(k1.re.x, k1.im.x);
+            x[R1 + r] = make_float2(k1.re.y, k1.im.y);
             x[R1 + R1 - 1 - r] = u0 ? bc : ac;
             if (r > 0) x[R1 - r] = u0 ? ac : x[R1 - r];
             x[R1 - 1 - r] = u0 ? x[R1 - 1 - r] : bc;
-            own[32 * (u0 ? (R1 - r) % R1 : R1 + R1 - 1 - r)] = w_conj(a.ox, a.oo);
-            own[32 * (u0 ? R1 + R1 - 1 - r : R1 - 1 - r)] = w_conj(b.ox, b.oo);
-            own[32 * r] = w_of(a.ox, a.oo);
-            own[32 * (R1 + r)] = w_of(b.ox, b.oo);
+            own[32 * (u0 ? (R1 - r) % R1 : R1 + R1 - 1 - r)] = make_float2(m2.re.x, m2.im.x);
+            own[32 * (u0 ? R1 + R1 - 1 - r : R1 - 1 - r)] = make_float2(m2.re.y, m2.im.y);
+            own[32 * r] = make_float2(k2.re.x, k2.im.x);
+            own[32 * (R1 + r)] = make_float2(k2.re.y, k2.im.y);
         }
         if (u0) {   // k = L/2
-            const EdgeParts a = parts(R1, x[R1 / 2], x[R1 / 2]);
-            x[R1 / 2] = w_of(a.ee, a.oy);
-            own[32 * (R1 / 2)] = w_of(a.ox, a.oo);
+            const Cx2 z = {dup2(x[R1 / 2].x), dup2(x[R1 / 2].y)};
+            const EdgeParts p = edge_parts<THERMAL>(edge_separate(z, z), half(__ldg(ly + R1 * TPL)), half(__ldg(lx + R1 * TPL)),
+                                                    half(corner[R1 * TPL + u]), sx, sy, odd != 0);
+            const Cx2 k1 = w_of(p.ee, p.oy), k2 = w_of(p.ox, p.oo);
+            x[R1 / 2] = make_float2(k1.re.x, k1.im.x);
+            own[32 * (R1 / 2)] = make_float2(k2.re.x, k2.im.x);
         }
         E::inverse(x, sm, u, tab);
 #pragma unroll
@@ -221,6 +274,32 @@ k_ev_edge_corr(Geom g, EvGeom v, Band band, const float *__restrict__ B2, const 
     }
 }
 
+// Both signs of every lag l of the window from the even parts D_l (re) and the
+// odd S_l = D_{M-l} (im; S_0 = 0), out at o + (Q/2 +- l) stride.  One code for
+// all units of a warp: unit 0's mirrors lie in its own butterflies (ev_pairs),
+// selected, where a branch had each such warp run both sides.
+template <int M, typename T, typename F>
+__device__ __forceinline__ void edge_lags(const Cx2 *z, int u, int Q, T *o, long long stride, F &&store)
+{
+    constexpr int RP = ev_vpt(M) / 2, NBP = M / RP, TPC = M / ev_vpt(M);
+    const bool u0 = u == 0;
+    const int h = Q / 2;
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+        const int j = b == 0 ? u : (u0 ? TPC : NBP - u);
+        T *pp = o + (h + j) * stride, *pm = o + (h - j) * stride;
+#pragma unroll
+        for (int r = 0; r < RP; ++r) {
+            const int l = j + r * NBP;
+            const float2 other = z[(1 - b) * RP + RP - 1 - r].im;
+            const float2 self = b == 1 ? z[RP + RP - 1 - r].im : r == 0 ? make_float2(0.f, 0.f) : z[(RP - r) % RP].im;
+            const float2 even = z[b * RP + r].re, odd = u0 ? self : other;
+            if (l < h) store(pp + r * NBP * stride, add2(even, odd));
+            if ((b != 0 || r != 0 || !u0) && l <= h) store(pm - r * NBP * stride, sub2(even, odd));
+        }
+    }
+}
+
 // B3 (EE, OY, OX, OO of k_x <= k_y) -> B4 [Q][M][WS]: the even and the odd part
 // along y (x, y of a value) at every lag s_x of the window.  Grid: M x (column
 // tiles), a pack is one transfer.
@@ -239,30 +318,27 @@ k_ev_edge_inv_x(EvGeom v, int Q, const float *__restrict__ B3, float2 *__restric
     const int col = threadIdx.x % C, u = threadIdx.x / C;
     const int m = ct * C + col;
     const bool on = m < v.WS;
+    const unsigned S3 = (unsigned)(v.s3 / 4);   // M S3 < 2^32 for every length and transfer count
     Cx2 z[VPT];
 #pragma unroll
     for (int b = 0; b < VPT / RF; ++b)
 #pragma unroll
         for (int r = 0; r < RF; ++r) {
-            const int kx = u + b * TPC + r * (M / RF), lo = min(kx, ky), hi = max(kx, ky);
             // (EE, OY) even in x, (OX, OO) odd; above the diagonal the axes change places
-            const Cx2 q = on ? ev_load(B3 + lo * v.s3 + 4LL * (hi * v.WS + m)) : Cx2{dup2(0.f), dup2(0.f)};
-            const float oy = kx <= ky ? q.re.y : q.im.x, ox = kx <= ky ? q.im.x : q.re.y;
-            z[b * RF + r] = {make_float2(q.re.x, oy), kx < M / 2 ? make_float2(ox, q.im.y) : make_float2(-ox, -q.im.y)};
+            const int kx = u + b * TPC + r * (M / RF);
+            const bool below = kx <= ky;
+            const Cx2 q = on ? ev_load(B3 + 4 * (size_t)(below ? kx * S3 + (ky * v.WS + m) : ky * S3 + (kx * v.WS + m)))
+                             : Cx2{dup2(0.f), dup2(0.f)};
+            const float oy = below ? q.re.y : q.im.x, ox = below ? q.im.x : q.re.y;
+            const bool up = RF % 2 == 0 ? r >= RF / 2 : kx >= M / 2;
+            z[b * RF + r] = {make_float2(q.re.x, oy), up ? make_float2(-ox, -q.im.y) : make_float2(ox, q.im.y)};
         }
     F::run(z, sm + col, u, tab);
     ev_post<M>(z, u, tab);
     if (!on) return;
-    float2 *o = B4 + ((long long)ky * v.WS + m);
     const long long s4 = v.s4 / 2;
-    auto put = [&](int l, float2 even, float2 oddv) {
-        if (l < Q / 2) o[(Q / 2 + l) * s4] = add2(even, oddv);
-        if (l > 0 && l <= Q / 2) o[(Q / 2 - l) * s4] = sub2(even, oddv);
-    };
-    ev_pairs<RP, NBP, TPC>(z, u, [&](int n, Cx2 &a, Cx2 &b) {
-        put(n, a.re, n == 0 ? make_float2(0.f, 0.f) : b.im);
-        if (&a != &b) put(M - n, b.re, a.im);
-    });
+    float2 *o = B4 + ((long long)ky * v.WS + m);
+    edge_lags<M>(z, u, Q, o, s4, [](float2 *p, float2 c) { *p = c; });
     // lag -M of grids that keep it (Q = 2N = 2M): no pair of points is that far apart
     if (u == 0 && Q / 2 == M) o[0] = make_float2(0.f, 0.f);
 }
@@ -292,16 +368,15 @@ k_ev_edge_inv_y(EvGeom v, int Q, int n_omega, const float *__restrict__ B4, floa
         for (int r = 0; r < RF; ++r) {
             const int ky = u + b * TPC + r * (M / RF);
             const Cx2 q = on ? ev_load(in + 2 * ky * v.WS) : Cx2{dup2(0.f), dup2(0.f)};
-            z[b * RF + r] = {make_float2(q.re.x, q.im.x),
-                             ky < M / 2 ? make_float2(q.re.y, q.im.y) : make_float2(-q.re.y, -q.im.y)};
+            const bool up = RF % 2 == 0 ? r >= RF / 2 : ky >= M / 2;
+            z[b * RF + r] = {make_float2(q.re.x, q.im.x), up ? make_float2(-q.re.y, -q.im.y) : make_float2(q.re.y, q.im.y)};
         }
     F::run(z, sm + col, u, tab);
     ev_post<M>(z, u, tab);
     if (m >= n_omega) return;
     float *o = out + ((long long)row * Q + Q / 2) * n_omega + m;
     const float2 sc = dup2(v.scale);
-    auto store = [&](int l, float2 c) {
-        float *q = o + (long long)l * n_omega;
+    auto store = [&](float *q, float2 c) {
         if constexpr (VEC) {
             *reinterpret_cast<float2 *>(q) = c;
         } else {
@@ -309,15 +384,10 @@ k_ev_edge_inv_y(EvGeom v, int Q, int n_omega, const float *__restrict__ B4, floa
             if (m + 1 < n_omega) q[1] = c.y;
         }
     };
-    auto put = [&](int l, float2 even, float2 oddv) {
-        if (l < Q / 2) store(l, mul2(add2(even, oddv), sc));
-        if (l > 0 && l <= Q / 2) store(-l, mul2(sub2(even, oddv), sc));
-    };
-    ev_pairs<RP, NBP, TPC>(z, u, [&](int n, Cx2 &a, Cx2 &b) {
-        put(n, a.re, n == 0 ? make_float2(0.f, 0.f) : b.im);
-        if (&a != &b) put(M - n, b.re, a.im);
-    });
-    if (u == 0 && Q / 2 == M) store(-M, make_float2(0.f, 0.f));
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) z[i] = {mul2(z[i].re, sc), mul2(z[i].im, sc)};
+    edge_lags<M>(z, u, Q, o - (long long)(Q / 2) * n_omega, n_omega, store);
+    if (u == 0 && Q / 2 == M) store(o - (long long)M * n_omega, make_float2(0.f, 0.f));
 }
 
 template <int L, bool THERMAL>
@@ -337,7 +407,7 @@ cudaError_t launch_ev_edge_corr_t(const Geom &g, const EvGeom &v, const Band &ba
                                   cudaStream_t s)
 {
     using E = EvLine<L>;
-    const size_t smem = sizeof(float2) * (EVC_WARPS * ev_edge_smem<L>() + (THERMAL ? L : 0));
+    const size_t smem = sizeof(float2) * (EVC_WARPS * ev_edge_smem<L>() + ev_edge_corner<L>() + (THERMAL ? L : 0));
     static const cudaError_t e = smem_attrs(k_ev_edge_corr<L, THERMAL, HALF>, smem);
     if (e != cudaSuccess) return e;
     const int nlines = v.M * (v.M + 1) / 2, iters = ev_corr_iters(nlines, E::LPI, sms);

@@ -77,13 +77,6 @@ cudaError_t launch_e64_tables(double2 *out, cudaStream_t s);
 cudaError_t launch_e64_pass(int pass, const Geom &g, const E64Geom &v, const Band &band, const Work<double> &w, double *out,
                             cudaStream_t s);
 cudaError_t launch_e64_corr(const Geom &g, const E64Geom &v, const Band &band, const Work<double> &w, cudaStream_t s);
-size_t ev_da_x_floats(const Geom &g, const EvGeom &v);
-size_t ev_da_y_floats(const Geom &g, const EvGeom &v);
-size_t ev_da_z_floats(const EvGeom &v);
-cudaError_t launch_da_weights(const Geom &g, const EvGeom &v, const float *wts, const Work<float> &w, float *Z, cudaStream_t s);
-cudaError_t launch_da_corr(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, const float *Z,
-                           cudaStream_t s);
-cudaError_t launch_da_inverse(const Geom &g, const EvGeom &v, const Work<float> &w, float *dA, cudaStream_t s);
 bool ev_bw_applies(const EvGeom &v);
 int ev_chain_blocks(const EvGeom &v);
 cudaError_t launch_ev_w_y(const Geom &g, const EvGeom &v, const float *wts, const Work<float> &w, cudaStream_t s);
@@ -614,9 +607,6 @@ extern "C" lindhard_status lindhard_plan_create(const lindhard_grid *grids, int 
             n.X = std::max(n.X, sizeof(float) * (size_t)(v.M * v.s2));
             n.Z = std::max(n.Z, sizeof(float) * (size_t)(v.M * v.s3));
             n.partial = std::max(n.partial, (size_t)(ev_chain_blocks(v) + bw_partial_extra_rows()) * 5 * sizeof(double));
-            n.X = std::max(n.X, sizeof(float) * ev_da_x_floats(g, v));
-            n.Y = std::max(n.Y, sizeof(float) * ev_da_y_floats(g, v));
-            n.Z = std::max(n.Z, sizeof(float) * ev_da_z_floats(v));
         }
         n.axis = (size_t)g.N * sizeof(AxisTab);
         n.eps32 = (size_t)g.n_eps * sizeof(float2);
@@ -1199,18 +1189,6 @@ extern "C" lindhard_status lindhard_imchi_backward(lindhard_plan *p, const lindh
             if (e == cudaSuccess) e = launch_ev_inv_x_bw(v, wk, s);                                   // Y
             if (e == cudaSuccess) e = launch_ev_chain(g, v, b, wk, partial, s);
             if (e == cudaSuccess) e = launch_reduce_params(partial, ev_chain_blocks(v), dparams + 5 * i, s);
-            if (e != cudaSuccess) return cuda_fail(e, "backward launch");
-            a_off += (size_t)g.N * g.N * g.n_eps;
-            o_off += (size_t)g.Q * g.Q * g.n_omega;
-            continue;
-        }
-        if (const EvGeom &v = p->even[i]; A_in == nullptr && !dparams && ev_bw_applies(v) && ev_band_applies(g, b)) {
-            // dL/dA at a generated A: the weights' four parity parts (k_even_da.cu)
-            if (e == cudaSuccess) e = launch_ev_gen_y(g, v, b, wk, s);
-            if (e == cudaSuccess) e = launch_ev_x(v, wk, s);                                   // Y = A^
-            if (e == cudaSuccess) e = launch_da_weights(g, v, w + o_off, wk, (float *)Z, s);   // Z = W^
-            if (e == cudaSuccess) e = launch_da_corr(g, v, b, wk, (const float *)Z, s);        // X = G
-            if (e == cudaSuccess) e = launch_da_inverse(g, v, wk, dA + a_off, s);
             if (e != cudaSuccess) return cuda_fail(e, "backward launch");
             a_off += (size_t)g.N * g.N * g.n_eps;
             o_off += (size_t)g.Q * g.Q * g.n_omega;

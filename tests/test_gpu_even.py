@@ -182,32 +182,6 @@ def test_parameter_gradient(lh, zones, npz, n_eps, n_omega, q, quantity):
     assert np.all(np.abs((dp - ref).cpu().numpy()) <= 1e-6 * scale), ((dp - ref).cpu().numpy() / scale)
 
 
-# dL/dA alone takes the even form's four parity parts, with the parameter
-# gradient asked for too the general form: the two FP32 forms' bar.
-@pytest.mark.parametrize("zones,npz,n_eps,n_omega,q,quantity", [
-    (4, 4, 3, 2, 16, 0), (4, 4, 3, 2, 32, 0), (4, 10, 34, 17, 40, 0), (5, 24, 37, 30, 118, 0), (4, 32, 128, 64, 128, 0),
-    (4, 16, 201, 90, 128, 0), (6, 32, 20, 10, 2, 0), (4, 16, 300, 150, 64, 0), (4, 12, 512, 256, 48, 0),
-    (4, 20, 401, 33, 60, 0), (4, 12, 40, 25, 48, 1), (4, 12, 150, 75, 48, 2), (4, 12, 200, 150, 60, 1),
-    (4, 12, 300, 200, 48, 2), (4, 24, 30, 15, 92, 0), (5, 36, 20, 10, 200, 0), (6, 96, 8, 4, 560, 0),
-    (4, 40, 30, 7, 100, 1), (4, 64, 50, 25, 512, 0), (4, 50, 33, 16, 176, 0), (8, 50, 12, 6, 400, 0),
-    (8, 100, 6, 3, 300, 0), (8, 128, 5, 2, 1024, 0), (8, 128, 4, 2, 2048, 0), (8, 256, 4, 2, 2048, 0),
-    (8, 192, 4, 2, 1400, 0), (8, 160, 3, 2, 400, 0), (8, 90, 4, 3, 820, 0)])
-def test_spectral_gradient(lh, zones, npz, n_eps, n_omega, q, quantity):
-    import torch
-    grid = wl.grid_params(zones, npz, n_eps, 2.0, n_omega=n_omega, q_extent=q, quantity=quantity)
-    band = wl.band_params(filling=1.1, gamma=0.1, ff_a=1.1, **({"kT": 0.06} if quantity else {}))
-    w = torch.from_numpy(wl.loss_weights(grid, seed=5)).cuda().reshape(-1) - 0.3
-    plan = lh.Plan([grid], backward=True)
-    dp = torch.zeros(5, dtype=torch.float64, device="cuda")
-    got = torch.full((plan.a_elems(),), float("nan"), device="cuda")
-    ref = torch.empty(plan.a_elems(), device="cuda")
-    plan.backward(w, bands=[band], dA=got)
-    plan.backward(w, bands=[band], dA=ref, dparams=dp)
-    plan.status()
-    plan.close()
-    assert float((got - ref).abs().max()) <= TOL * float(ref.abs().max())
-
-
 def test_parameter_gradient_free_electrons(lh):
     import torch
     grid = wl.grid_params(4, 16, 40, 2.0)

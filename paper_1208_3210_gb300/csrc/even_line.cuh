@@ -125,15 +125,17 @@ __device__ __forceinline__ Cx2 ev_get(const float4 *p)
     return {make_float2(q.x, q.y), make_float2(q.z, q.w)};
 }
 
-// Tables after the cosine transforms': per length, k < 32: (w, w^2) and, 32
-// entries later, (w^3, w^4), w = e^{-2 pi i k / L}.
+// Tables after the cosine transforms': per length, k < 32: (w, w^2), 32 entries
+// later (w^3, w^4), 32 later (w^8, w^16), w = e^{-2 pi i k / L}: no power is more
+// than two products from an entry.
+constexpr int EV_LINE_TABLE = 192;
 __host__ __device__ constexpr int ev_line_len(int i) { return i == 0 ? 128 : i == 1 ? 256 : i == 2 ? 384 : i == 3 ? 512 : 0; }
 template <int L>
 __host__ __device__ constexpr int ev_line_table()
 {
-    return (ev_table_entries() + 1) / 2 * 2 + (L == 128 ? 0 : L == 256 ? 1 : L == 384 ? 2 : 3) * 128;
+    return (ev_table_entries() + 1) / 2 * 2 + (L == 128 ? 0 : L == 256 ? 1 : L == 384 ? 2 : 3) * EV_LINE_TABLE;
 }
-__host__ __device__ constexpr int ev_all_tables() { return (ev_table_entries() + 1) / 2 * 2 + 4 * 128; }
+__host__ __device__ constexpr int ev_all_tables() { return (ev_table_entries() + 1) / 2 * 2 + 4 * EV_LINE_TABLE; }
 
 constexpr int EVC_WARPS = 4;
 
@@ -187,10 +189,15 @@ struct EvLine {
         w[2] = make_float2(a.z, a.w);
         w[3] = make_float2(b.x, b.y);
         w[4] = make_float2(b.z, b.w);
+        if constexpr (R > 8) {
+            const float4 c = __ldg(reinterpret_cast<const float4 *>(tab) + 64 + k);
+            w[8] = make_float2(c.x, c.y);
+            if constexpr (R > 16) w[16] = make_float2(c.z, c.w);
+        }
 #pragma unroll
         for (int r = 5; r < R; ++r) {
-            const int p = r <= 8 ? 4 : r <= 16 ? 8 : 16;
-            w[r] = cmul(w[p], w[r - p]);
+            const int p = r < 8 ? 4 : r < 16 ? 8 : 16;
+            if (r != p) w[r] = cmul(w[p], w[r - p]);
         }
     }
 

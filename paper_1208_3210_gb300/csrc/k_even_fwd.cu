@@ -26,7 +26,7 @@ __global__ void k_ev_tables(float2 *out, EvTabs tabs)
         double s, c;
         if (row == 0) sincospi(0.5 * (double)i / (double)period, &s, &c);
         else if (row > 0) sincospi(-2.0 * (double)((i / row) * (i % row + 1)) / (double)period, &s, &c);
-        else sincospi(-2.0 * (double)((i % 64 / 2) * (i / 64 * 2 + i % 2 + 1)) / (double)period, &s, &c);
+        else sincospi(-2.0 * (double)((i % 64 / 2) * (i < 128 ? i / 64 * 2 + i % 2 + 1 : i % 2 ? 16 : 8)) / (double)period, &s, &c);
         out[off + i] = make_float2((float)c, (float)s);
     }
 }
@@ -45,7 +45,7 @@ cudaError_t launch_ev_tables(float2 *out, cudaStream_t s)
                 o += Ns * ev_row(R);
             }
     }
-    for (int i = 0; ev_line_len(i) != 0; ++i) tabs.t[n++] = {(o + 1) / 2 * 2 + 128 * i, 128, -1, ev_line_len(i)};
+    for (int i = 0; ev_line_len(i) != 0; ++i) tabs.t[n++] = {(o + 1) / 2 * 2 + EV_LINE_TABLE * i, EV_LINE_TABLE, -1, ev_line_len(i)};
     k_ev_tables<<<dim3(n, 4), 128, 0, s>>>(out, tabs);
     return cudaGetLastError();
 }

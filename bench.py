@@ -62,6 +62,8 @@ VARIANT_KERNELS = {
 # kernels of the even form in the same pass slots
 EVEN_KERNELS = {"energy_fwd": "k_ev_gen_y", "py_fwd": "k_ev_x", "px_product": "k_ev_corr", "py_inv": "k_ev_inv_x",
                 "energy_inv": "k_ev_inv_y"}
+EDGE_KERNELS = dict(EVEN_KERNELS, px_product="k_ev_edge, k_ev_edge_corr", py_inv="k_ev_edge_inv_x",
+                    energy_inv="k_ev_edge_inv_y")
 KERNEL_NAMES = {"batch": "all passes of all instances (graph)", "energy_fwd": "k_fwd_energy", "py_fwd": "k_fwd_y", "px_product": "k_x_product",
                 "py_inv": "k_inv_y", "energy_inv": "k_inv_energy", "tables": "k_setup", "mu_solve": "k_mu_sect, k_mu_halley"}
 
@@ -117,23 +119,29 @@ def pass_bytes(s):
             "py_inv": 8 * (W3 + W4), "energy_inv": 8 * W4 + 4 * out}
 
 
+def edge_carried(grid, band):
+    """Whether the even form carries the zone edge (its weight above 2^-24)."""
+    return (math.pi * grid["zones"] * band["ff_a"]) ** 2 < 8 * 24 * math.log(2.0)
+
+
 def even_pass_bytes(s, grid, band, precision, fp32=0):
     """The same for the even form (csrc/even.cuh), which a generated A takes on
-    FP32 Im chi grids of several zones whose edge rows weigh below 2^-24 (real
-    buffers over one quadrant, k_x <= k_y between the momentum passes), or None
-    when the call does not take it."""
+    FP32 Im chi grids of several zones (real buffers over one quadrant, k_x <=
+    k_y between the momentum passes; with the edge row where it weighs more than
+    2^-24, csrc/k_even_edge.cu), or None when the call does not take it."""
     if precision != fp32 or grid["zones"] == 1 or grid.get("quantity", 0) != 0:
-        return None
-    if (math.pi * grid["zones"] * band["ff_a"]) ** 2 < 8 * 24 * math.log(2.0):
         return None
     lens = [16 << i for i in range(8)] + [24 << i for i in range(7)] + [72 << i for i in range(5)] + [432, 864]
     need = [m for m in lens if m >= (s.N + s.q_extent // 2 + 1) // 2]
     J0 = s.n_eps // 2
     ne = min(s.n_eps, J0 + s.n_omega) - max(0, J0 - s.n_omega)
-    if not need or ne > 768 or s.N < 4:
+    edge = edge_carried(grid, band)
+    if not need or ne > (512 if edge else 768) or s.N < 4:
         return None
     M, Nh, nl = min(need), s.N // 2, s.q_extent // 2 + 1
     B1, B2, B3, B4 = Nh * M * ne, M * (M + 1) // 2 * ne, M * (M + 1) // 2 * s.n_omega, nl * M * s.n_omega
+    if edge:   # one row more, four parity parts, every lag s_x of two parts in y
+        B1, B3, B4 = (Nh + 1) * M * ne, 4 * B3, 2 * s.q_extent * M * s.n_omega
     out = s.q_extent * s.q_extent * s.n_omega
     return {"energy_fwd": 4 * B1, "py_fwd": 4 * (B1 + B2), "px_product": 4 * (B2 + B3),
             "py_inv": 4 * (B3 + B4), "energy_inv": 4 * (B4 + out)}
@@ -760,8 +768,10 @@ def main():
     peak, peak_kind = measured_peaks()
     # kernels launched in the timed region: each step is one forward call; a
     # third multisection pass when gamma < 0.02 eV and the solve spans
-    # several CTAs (more than 160 points per zone)
+    # several CTAs (more than 160 points per zone); the edge lines' pass
     launches = (sum(int(plan.sizes[i].kernels_forward)
+                    + (1 if not persistent and edge_carried(grids[i], bands[i])
+                       and even_pass_bytes(plan.sizes[i], grids[i], bands[i], prec) else 0)
                     + (1 if bands[i]["gamma"] < 0.02 and grids[i]["npz"] > 160 else 0)
                     for i in range(len(grids))) + (1 if batched and persistent else 0)) * args.steps
     if batched:
@@ -832,7 +842,7 @@ def main():
                                          "speedup_persistent": cg_ms / step_ms}
             cg.close()
             del cg_out
-    dom_kernel = (EVEN_KERNELS[dom] if not batched and even else
+    dom_kernel = ((EDGE_KERNELS if edge_carried(grids[0], bands[0]) else EVEN_KERNELS)[dom] if not batched and even else
                   VARIANT_KERNELS[dom][variants[dom]] if dom in VARIANT_KERNELS else KERNEL_NAMES[dom])
     tc = None
     kk = None

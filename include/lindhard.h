@@ -144,7 +144,8 @@ typedef struct {
     long long kernels_forward;    /* kernel launches of one forward call with A generated and mu
                                      solved: with more than 160 points per zone one more when
                                      gamma < 0.02 eV (a third multisection pass); with at most 160
-                                     the whole solve runs in the set-up launch (two fewer); with
+                                     the whole solve runs in the set-up launch (two fewer); one
+                                     more for the zone edge's lines where it carries weight; with
                                      a caller-supplied A only the FFT passes; in a
                                      LINDHARD_PLAN_PERSISTENT plan the instance's set-up launches
                                      only (the batch adds one persistent launch)               */

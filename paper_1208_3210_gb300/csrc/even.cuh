@@ -17,8 +17,8 @@
 // with M >= (N + Q/2) / 2 frequencies per axis.  At 1024^2 x 512 the buffers
 // move 5.3 GB instead of the general form's 33.4 GB and the momentum
 // transforms take 0.38 G complex points (two real columns a point) instead of
-// 3.4 G: 8.19 -> 1.70 ms a call (256^3: 0.279 -> 0.087 ms; Im chi_T there
-// 0.412 -> 0.106 ms).
+// 3.4 G: 8.19 -> 1.50 ms a call (256^3: 0.279 -> 0.065 ms; Im chi_T there
+// 0.412 -> 0.074 ms).
 //
 // Transform.  The frequencies are theta_k = pi (2k + 1) / (2M), the
 // half-shifted grid of length P = 2M: it turns the circular correlation of

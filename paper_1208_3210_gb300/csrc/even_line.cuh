@@ -5,7 +5,7 @@
 // with 16 values a lane (et_tiles.cuh) were bound by the L1 data pipe here (71%
 // at 512 energies, 88% at 128: two exchanges and the twiddle rows of two
 // stages); these issue 34 instructions a point instead of 47 with that pipe at
-// 37% and the FMA pipe at 45%.  The correlation at 1024^2 x 512: 366 -> 313 us
+// 37% and the FMA pipe at 45%.  The correlation at 1024^2 x 512: 366 -> 305 us
 // (3.0 TB/s), Im chi_T at 256^3: 37 -> 27 us.
 //
 //   forward : L = R0 R1; stage 0 on butterflies u + b TPL (radix R0), stage 1 on

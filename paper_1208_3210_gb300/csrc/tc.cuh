@@ -1,7 +1,7 @@
-// Fifth-generation tensor-core helpers (tcgen05, inline PTX, sm_103a) shared
-// by the tensor-core inverse p_y pass and the Kramers-Kronig pass: operand
-// descriptors and layout, tensor-memory allocation, one-thread MMA issue and
-// commit, accumulator loads, and the BF16 hi + lo split of FP32 values.
+// Fifth-generation tensor-core helpers (tcgen05, inline PTX, sm_103a) of the
+// tensor-core inverse p_y pass: operand descriptors and layout, tensor-memory
+// allocation, one-thread MMA issue and commit, accumulator loads, and the BF16
+// hi + lo split of FP32 values.
 #pragma once
 
 #include <cuda_bf16.h>

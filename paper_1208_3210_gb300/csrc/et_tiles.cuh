@@ -148,7 +148,7 @@ __device__ __forceinline__ void energy_fwd_warp_tile(const Geom &g, const Band &
                 const int n = j + r * (L / R0);
                 float A;
                 if constexpr (GEN) {
-                    const float2 ej = __ldg(&eps[FULL ? n : min(n, g.n_eps - 1)]);
+                    const float2 ej = eps[FULL ? n : min(n, g.n_eps - 1)];
                     const float e = (ej.x - xhi) + (ej.y - xlo);
                     A = amp * et_rcp(fmaf(e, e, g2));
                     if (!FULL && n >= g.n_eps) A = 0.f;
@@ -291,7 +291,7 @@ __device__ __forceinline__ void inv_energy_warp_tile(const Geom &g, const float2
         // above L/2 of one are the conjugate mirrors of the other's
         float2 v[VPT];
         const float2 zero = make_float2(0.f, 0.f);
-        auto ldx = [](const float2 *p) { return COH ? __ldcg(p) : __ldg(p); };
+        auto ldx = [](const float2 *p) { return COH ? __ldcg(p) : *p; };
         auto w_of = [](float2 x1, float2 x2) { return make_float2(x1.x - x2.y, x1.y + x2.x); };       // X1 + i X2
         auto w_conj = [](float2 x1, float2 x2) { return make_float2(x1.x + x2.y, x2.x - x1.y); };     // conj X1 + i conj X2
 #pragma unroll

@@ -469,12 +469,13 @@ __device__ __forceinline__ float ev_rcp(float x)
 }
 
 // A pack from global memory, read once: not kept in L1, whose few KB beside the
-// exchange buffers hold the tables.
+// exchange buffers hold the tables.  Volatile and not through the read-only
+// path: the kernel before may have written it (after_previous).
 __device__ __forceinline__ Cx2 ev_load(const float *p)
 {
     float4 q;
-    asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
-        : "=f"(q.x), "=f"(q.y), "=f"(q.z), "=f"(q.w) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(q.x), "=f"(q.y), "=f"(q.z), "=f"(q.w) : "l"(p) : "memory");
     return {make_float2(q.x, q.y), make_float2(q.z, q.w)};
 }
 

@@ -204,7 +204,7 @@ struct PrEng {
         }
     }
 
-    __device__ __forceinline__ static float4 tw_ld(const float4 *p) { return TWS ? lds_f4(p) : __ldg(p); }
+    __device__ __forceinline__ static float4 tw_ld(const float4 *row) { return TWS ? lds_f4(row) : __ldg(row); }
     // The twiddles w^r, r < R, of one butterfly (w = exp(-2 pi i k / (Ns R))),
     // from its table row (w^1, w^2, ..., w^(R-1), w^0): one 16-byte load gives
     // w and w^2, the other powers are products (for R = 24 also w^7, w^8 and

@@ -62,8 +62,8 @@ bool et_applies(const Geom &g, const Band &band)
 // warps' exchange areas, before the tile
 template <int L, bool FULL, bool GEN, bool THERMAL>
 __global__ void __launch_bounds__(32 * ET_WARPS)
-k_fwd_energy_warp(Geom g, Band band, const AxisTab *__restrict__ axis, const float2 *__restrict__ eps,
-                  const InstState *__restrict__ st, const float *__restrict__ A_in, float2 *__restrict__ U1,
+k_fwd_energy_warp(Geom g, Band band, const AxisTab *axis, const float2 *eps, const InstState *st,
+                  const float *A_in, float2 *__restrict__ U1,
                   const float2 *__restrict__ etw)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -80,7 +80,7 @@ k_fwd_energy_warp(Geom g, Band band, const AxisTab *__restrict__ axis, const flo
 
 template <int L, bool HALF>
 __global__ void __launch_bounds__(32 * ET_WARPS)
-k_inv_energy_warp(Geom g, const float2 *__restrict__ U4, float *__restrict__ out, const float2 *__restrict__ etw)
+k_inv_energy_warp(Geom g, const float2 *U4, float *__restrict__ out, const float2 *__restrict__ etw)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(et_inv_smem_elems<L>(), float2)

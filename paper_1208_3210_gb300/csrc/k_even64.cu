@@ -131,8 +131,8 @@ __device__ __forceinline__ double2 e64_even_odd(const double2 *V, int n, const d
 // B1 [Nh][M][ES]: A over p_y >= 0 for each p_x >= 0, transformed along p_y.
 template <int M>
 __global__ void __launch_bounds__(E64_T)
-k_e64_gen_y(Geom g, E64Geom v, Band band, const AxisTab *__restrict__ axis, const double *__restrict__ eps,
-            const InstState *__restrict__ st, double *__restrict__ B1, const double2 *__restrict__ tab, int ntile)
+k_e64_gen_y(Geom g, E64Geom v, Band band, const AxisTab *axis, const double *eps,
+            const InstState *st, double *__restrict__ B1, const double2 *__restrict__ tab, int ntile)
 {
     constexpr int LD = M + 1;
     __shared__ double2 za[E64_C * LD], zb[E64_C * LD];
@@ -168,7 +168,7 @@ k_e64_gen_y(Geom g, E64Geom v, Band band, const AxisTab *__restrict__ axis, cons
 // B2 [M][M][ES] (k_x <= k_y): B1 transformed along p_x for each k_y.
 template <int M>
 __global__ void __launch_bounds__(E64_T)
-k_e64_x(E64Geom v, const double *__restrict__ B1, double *__restrict__ B2, const double2 *__restrict__ tab, int ntile)
+k_e64_x(E64Geom v, const double *B1, double *__restrict__ B2, const double2 *__restrict__ tab, int ntile)
 {
     constexpr int LD = M + 1;
     __shared__ double2 za[E64_C * LD], zb[E64_C * LD];
@@ -207,8 +207,8 @@ __device__ __forceinline__ E64Line e64_separate(double2 k, double2 m)
 // [line][PE/2 + 1][occupied, empty], then sin(N theta_k / 2) of every row.
 template <int L>
 __global__ void __launch_bounds__(32 * E64_WARPS)
-k_e64_edge(Geom g, E64Geom v, Band band, const AxisTab *__restrict__ axis, const double *__restrict__ eps,
-           const InstState *__restrict__ st, const double *__restrict__ B1, double2 *__restrict__ lines,
+k_e64_edge(Geom g, E64Geom v, Band band, const AxisTab *axis, const double *eps,
+           const InstState *st, const double *B1, double2 *__restrict__ lines,
            const double2 *__restrict__ tab)
 {
     __shared__ double2 buf[E64_WARPS][2][L];
@@ -248,7 +248,7 @@ k_e64_edge(Geom g, E64Geom v, Band band, const AxisTab *__restrict__ axis, const
 // parts, a line a warp.
 template <int L>
 __global__ void __launch_bounds__(32 * E64_WARPS)
-k_e64_corr(Geom g, E64Geom v, Band band, const double *__restrict__ B2, const double2 *__restrict__ lines,
+k_e64_corr(Geom g, E64Geom v, Band band, const double *B2, const double2 *lines,
            double2 *__restrict__ B3, const double2 *__restrict__ tab)
 {
     __shared__ double2 buf[E64_WARPS][3][L];
@@ -306,7 +306,7 @@ k_e64_corr(Geom g, E64Geom v, Band band, const double *__restrict__ B2, const do
 // window.  Two columns a transfer: EE + i OX and OY + i OO.
 template <int M>
 __global__ void __launch_bounds__(E64_T)
-k_e64_inv_x(E64Geom v, int Q, const double2 *__restrict__ B3, double2 *__restrict__ B4,
+k_e64_inv_x(E64Geom v, int Q, const double2 *B3, double2 *__restrict__ B4,
             const double2 *__restrict__ tab, int ntile)
 {
     constexpr int LD = M + 1, MT = E64_C / 2;
@@ -343,7 +343,7 @@ k_e64_inv_x(E64Geom v, int Q, const double2 *__restrict__ B3, double2 *__restric
 // B4 -> Im chi at (s_x, +-s_y), times the Eq. 9 prefactor.
 template <int M>
 __global__ void __launch_bounds__(E64_T)
-k_e64_inv_y(E64Geom v, int Q, int n_omega, const double2 *__restrict__ B4, double *__restrict__ out,
+k_e64_inv_y(E64Geom v, int Q, int n_omega, const double2 *B4, double *__restrict__ out,
             const double2 *__restrict__ tab, int ntile)
 {
     constexpr int LD = M + 1;

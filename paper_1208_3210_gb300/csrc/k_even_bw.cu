@@ -29,7 +29,7 @@ namespace lh {
 // transfers of a row in one 16-byte load.
 template <int M, bool VEC>
 __global__ void __launch_bounds__(EvCfg<M>::T, EvCfg<M>::MINB)
-k_ev_w_y(EvGeom v, int Q, int n_omega, const float *__restrict__ w, float *__restrict__ W1,
+k_ev_w_y(EvGeom v, int Q, int n_omega, const float *w, float *__restrict__ W1,
          const float2 *__restrict__ tab, int ntile)
 {
     using F = EvFft<M, false>;
@@ -97,7 +97,7 @@ k_ev_w_y(EvGeom v, int Q, int n_omega, const float *__restrict__ w, float *__res
 // transformed back.  2.5 transforms a line.
 template <int L, bool FULL, bool THERMAL>
 __global__ void __launch_bounds__(32 * EVC_WARPS, 2)
-k_ev_bw(Geom g, EvGeom v, Band band, const float *__restrict__ B2, const float *__restrict__ W2,
+k_ev_bw(Geom g, EvGeom v, Band band, const float *B2, const float *W2,
         float *__restrict__ G3, const float2 *__restrict__ tab, int iters, int odd)
 {
     using E = EvLine<L>;
@@ -136,7 +136,7 @@ k_ev_bw(Geom g, EvGeom v, Band band, const float *__restrict__ B2, const float *
             for (int i = 0; i < VPT; ++i) {
                 const int n = E::first(i);
                 const bool on = live && u + n < g.n_omega;
-                x[i] = on ? make_float2(0.25f * (__ldg(p[0] + n) + __ldg(q[0] + n)), 0.25f * (__ldg(p[1] + n) + __ldg(q[1] + n)))
+                x[i] = on ? make_float2(0.25f * (p[0][n] + q[0][n]), 0.25f * (p[1][n] + q[1][n]))
                           : make_float2(0.f, 0.f);
             }
         }
@@ -200,8 +200,8 @@ k_ev_bw(Geom g, EvGeom v, Band band, const float *__restrict__ B2, const float *
 // Grid: Nh x (column tiles).  partial[blockIdx.x][5] receives this CTA's sums.
 template <int M>
 __global__ void __launch_bounds__(EvCfg<M>::T, EvCfg<M>::MINB)
-k_ev_chain(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const float2 *__restrict__ eps,
-           const InstState *__restrict__ st, const float *__restrict__ G4, double *__restrict__ partial,
+k_ev_chain(Geom g, EvGeom v, Band band, const AxisTab *axis, const float2 *eps,
+           const InstState *st, const float *G4, double *__restrict__ partial,
            const float2 *__restrict__ tab, int ntile)
 {
     using F = EvFft<M, true>;
@@ -244,7 +244,7 @@ k_ev_chain(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const 
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int k = min(e + 2 * h, v.ne - 1), k1 = min(e + 2 * h + 1, v.ne - 1);   // past the window G is 0
-        const float2 a = __ldg(&eps[v.e0 + k]), b = __ldg(&eps[v.e0 + k1]);
+        const float2 a = eps[v.e0 + k], b = eps[v.e0 + k1];
         eh[h] = make_float2(a.x, b.x);
         el[h] = make_float2(a.y, b.y);
     }

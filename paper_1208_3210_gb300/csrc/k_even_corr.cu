@@ -20,7 +20,7 @@ namespace lh {
 // part, Im chi_T).  HALF: WS <= L/2, the upper half of the lags is not formed.
 template <int L, bool FULL, bool THERMAL, bool HALF>
 __global__ void __launch_bounds__(32 * EVC_WARPS, EvLine<L>::MINB)
-k_ev_corr(Geom g, EvGeom v, Band band, const float *__restrict__ B2, float *__restrict__ B3,
+k_ev_corr(Geom g, EvGeom v, Band band, const float *B2, float *__restrict__ B3,
           const float2 *__restrict__ tab, int iters, int odd)
 {
     using E = EvLine<L>;
@@ -128,7 +128,7 @@ k_ev_corr(Geom g, EvGeom v, Band band, const float *__restrict__ B2, float *__re
 // part (Im chi_T).
 template <int L, bool FULL, bool THERMAL>
 __global__ void __launch_bounds__(32 * EVC_WARPS)
-k_ev_corr3(Geom g, EvGeom v, Band band, const float *__restrict__ B2, float *__restrict__ B3,
+k_ev_corr3(Geom g, EvGeom v, Band band, const float *B2, float *__restrict__ B3,
           const float2 *__restrict__ etw, int iters, int odd)
 {
     using G = EtGeo<L>;

@@ -62,8 +62,8 @@ __device__ __forceinline__ Cx2 edge_mirror(const float2 *x, int r, bool u0)
 // [R1 / 2][occupied, empty][TPL] packs, then [TPL] (occupied, empty) at L/2.
 template <int L, bool THERMAL>
 __global__ void __launch_bounds__(32 * EVC_WARPS, EvLine<L>::MINB)
-k_ev_edge(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const float2 *__restrict__ eps,
-          const InstState *__restrict__ st, const float *__restrict__ B1, float4 *__restrict__ lines,
+k_ev_edge(Geom g, EvGeom v, Band band, const AxisTab *axis, const float2 *eps,
+          const InstState *st, const float *B1, float4 *__restrict__ lines,
           const float2 *__restrict__ tab)
 {
     using E = EvLine<L>;
@@ -96,7 +96,7 @@ k_ev_edge(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const f
         raw[i] = 0.f;
         if (t < v.M && n < v.ne) raw[i] = 2.f * B1[(v.Nh - 1) * v.s1 + (long long)t * v.ES + n];
         if (t == v.M && n < v.ne) {
-            const float2 e = __ldg(&eps[v.e0 + n]);
+            const float2 e = eps[v.e0 + n];
             const float d = (e.x - q.x) + (e.y - q.y);
             raw[i] = q.z * ev_rcp(fmaf(d, d, band.gam2));
         }
@@ -129,7 +129,8 @@ __device__ __forceinline__ Cx2 edge_fma(Cx2 a, float2 s, Cx2 b) { return {fma2(a
 __device__ __forceinline__ Cx2 edge_load(const float4 *p)
 {
     float4 q;
-    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(q.x), "=f"(q.y), "=f"(q.z), "=f"(q.w) : "l"(p));
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(q.x), "=f"(q.y), "=f"(q.z), "=f"(q.w) : "l"(p) : "memory");
     return {make_float2(q.x, q.y), make_float2(q.z, q.w)};
 }
 // conj(a) b + conj(c) d and conj(a) b - conj(c) d
@@ -182,7 +183,7 @@ __host__ __device__ constexpr int ev_edge_corner()   // float2 of the corner's s
 }
 template <int L, bool THERMAL, bool HALF>
 __global__ void __launch_bounds__(32 * EVC_WARPS, EvLine<L>::MINB)
-k_ev_edge_corr(Geom g, EvGeom v, Band band, const float *__restrict__ B2, const float4 *__restrict__ lines,
+k_ev_edge_corr(Geom g, EvGeom v, Band band, const float *B2, const float4 *lines,
                float4 *__restrict__ B3, const float2 *__restrict__ tab, int iters, int odd)
 {
     using E = EvLine<L>;
@@ -212,7 +213,7 @@ k_ev_edge_corr(Geom g, EvGeom v, Band band, const float *__restrict__ B2, const 
         const float *p = B2 + (kx * v.s2 + (long long)ky * v.ES + u);
 #pragma unroll
         for (int i = 0; i < VPT; ++i) raw[i] = live && u + E::first(i) < v.ne ? __ldcs(p + E::first(i)) : 0.f;
-        const float sx = __ldg(sines + kx), sy = __ldg(sines + ky);
+        const float sx = sines[kx], sy = sines[ky];
         const float4 *ly = lines + (long long)ky * (R1 + 1) * TPL + u, *lx = lines + (long long)kx * (R1 + 1) * TPL + u;
         float2 x[VPT];
         E::template first_stage<false, THERMAL>(x, raw, u, v.J0, wf);
@@ -246,7 +247,7 @@ k_ev_edge_corr(Geom g, EvGeom v, Band band, const float *__restrict__ B2, const 
         }
         if (u0) {   // k = L/2
             const Cx2 z = {dup2(x[R1 / 2].x), dup2(x[R1 / 2].y)};
-            const EdgeParts p = edge_parts<THERMAL>(edge_separate(z, z), half(__ldg(ly + R1 * TPL)), half(__ldg(lx + R1 * TPL)),
+            const EdgeParts p = edge_parts<THERMAL>(edge_separate(z, z), half(ly[R1 * TPL]), half(lx[R1 * TPL]),
                                                     half(corner[R1 * TPL + u]), sx, sy, odd != 0);
             const Cx2 k1 = w_of(p.ee, p.oy), k2 = w_of(p.ox, p.oo);
             x[R1 / 2] = make_float2(k1.re.x, k1.im.x);
@@ -305,7 +306,7 @@ __device__ __forceinline__ void edge_lags(const Cx2 *z, int u, int Q, T *o, long
 // tiles), a pack is one transfer.
 template <int M>
 __global__ void __launch_bounds__(EvCfg<M>::T, EvCfg<M>::MINB)
-k_ev_edge_inv_x(EvGeom v, int Q, const float *__restrict__ B3, float2 *__restrict__ B4,
+k_ev_edge_inv_x(EvGeom v, int Q, const float *B3, float2 *__restrict__ B4,
                 const float2 *__restrict__ tab, int ntile)
 {
     using F = EvFft<M, true>;
@@ -347,7 +348,7 @@ k_ev_edge_inv_x(EvGeom v, int Q, const float *__restrict__ B3, float2 *__restric
 // (column tiles), a pack is two transfers.  VEC: both in one 8-byte store.
 template <int M, bool VEC>
 __global__ void __launch_bounds__(EvCfg<M>::T, EvCfg<M>::MINB)
-k_ev_edge_inv_y(EvGeom v, int Q, int n_omega, const float *__restrict__ B4, float *__restrict__ out,
+k_ev_edge_inv_y(EvGeom v, int Q, int n_omega, const float *B4, float *__restrict__ out,
                 const float2 *__restrict__ tab, int ntile)
 {
     using F = EvFft<M, true>;

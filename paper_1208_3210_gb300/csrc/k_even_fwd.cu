@@ -54,8 +54,8 @@ size_t ev_table_bytes() { return (size_t)ev_all_tables() * sizeof(float2); }
 // Grid: Nh x (column tiles), the tiles of one p_x neighbours.
 template <int M>
 __global__ void __launch_bounds__(EvCfg<M>::T, EvCfg<M>::MINB_GEN)
-k_ev_gen_y(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const float2 *__restrict__ eps,
-           const InstState *__restrict__ st, float *__restrict__ B1, const float2 *__restrict__ tab, int ntile)
+k_ev_gen_y(Geom g, EvGeom v, Band band, const AxisTab *axis, const float2 *eps,
+           const InstState *st, float *__restrict__ B1, const float2 *__restrict__ tab, int ntile)
 {
     using F = EvFft<M, false>;
     constexpr int C = F::C, T = F::T, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP;
@@ -86,7 +86,7 @@ k_ev_gen_y(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const 
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int k = e + 2 * h;
-        const float2 a = __ldg(&eps[v.e0 + min(k, v.ne - 1)]), b = __ldg(&eps[v.e0 + min(k + 1, v.ne - 1)]);
+        const float2 a = eps[v.e0 + min(k, v.ne - 1)], b = eps[v.e0 + min(k + 1, v.ne - 1)];
         eh[h] = make_float2(a.x, b.x);
         el[h] = make_float2(a.y, b.y);
         on[h] = make_float2(k < v.ne ? 1.f : 0.f, k + 1 < v.ne ? 1.f : 0.f);
@@ -130,7 +130,7 @@ k_ev_gen_y(Geom g, EvGeom v, Band band, const AxisTab *__restrict__ axis, const 
 // planes of RS-float rows, sp floats apart in B1 and dp in B2.  TRI: k_x <= k_y.
 template <int M, bool TRI>
 __global__ void __launch_bounds__(EvCfg<M>::T, EvCfg<M>::MINB)
-k_ev_x(int rows, int RS, long long sp, long long dp, const float *__restrict__ B1, float *__restrict__ B2,
+k_ev_x(int rows, int RS, long long sp, long long dp, const float *B1, float *__restrict__ B2,
        const float2 *__restrict__ tab, int ntile)
 {
     using F = EvFft<M, false>;

@@ -14,7 +14,7 @@ namespace lh {
 // planes of RS-float rows, sp floats apart in B3 and dp in B4.
 template <int M>
 __global__ void __launch_bounds__(EvCfg<M>::T, EvCfg<M>::MINB)
-k_ev_inv_x(int rows, int RS, long long sp, long long dp, const float *__restrict__ B3, float *__restrict__ B4,
+k_ev_inv_x(int rows, int RS, long long sp, long long dp, const float *B3, float *__restrict__ B4,
            const float2 *__restrict__ tab, int ntile)
 {
     using F = EvFft<M, true>;
@@ -57,7 +57,7 @@ k_ev_inv_x(int rows, int RS, long long sp, long long dp, const float *__restrict
 // transfers of a pack in one 16-byte store (n_omega % 4 == 0, out aligned).
 template <int M, bool VEC>
 __global__ void __launch_bounds__(EvCfg<M>::T, EvCfg<M>::MINB)
-k_ev_inv_y(EvGeom v, int Q, int n_omega, const float *__restrict__ B4, float *__restrict__ out,
+k_ev_inv_y(EvGeom v, int Q, int n_omega, const float *B4, float *__restrict__ out,
            const float2 *__restrict__ tab, int ntile)
 {
     using F = EvFft<M, true>;

@@ -20,9 +20,9 @@ namespace lh {
 // THERMAL: the finite-temperature weights (band.kT > 0) instead of the split.
 template <typename Real, int L, bool THERMAL>
 __global__ void __launch_bounds__(LineCfg<L>::T)
-k_fwd_energy(Geom g, Band band, const AxisTab *__restrict__ axis,
-             const typename EpsEntry<Real>::type *__restrict__ eps,
-             const InstState *__restrict__ st, const Real *__restrict__ A_in,
+k_fwd_energy(Geom g, Band band, const AxisTab *axis,
+             const typename EpsEntry<Real>::type *eps,
+             const InstState *st, const Real *A_in,
              cx<Real> *__restrict__ U1, const cx<Real> *__restrict__ tw)
 {
     constexpr int C = LineCfg<L>::C, T = LineCfg<L>::T;
@@ -160,7 +160,7 @@ k_fwd_energy(Geom g, Band band, const AxisTab *__restrict__ axis,
 // p_y pass.  CTA = (column tile, ix).  U1 [N][N][2 SP] -> U2 [N][P][2 SP].
 template <typename Real, int L>
 __global__ void __launch_bounds__(ColCfg<L>::T, ColCfg<L>::MINB)
-k_fwd_y(Geom g, const cx<Real> *__restrict__ U1, cx<Real> *__restrict__ U2,
+k_fwd_y(Geom g, const cx<Real> *U1, cx<Real> *__restrict__ U2,
         const cx<Real> *__restrict__ tw)
 {
     constexpr int C = ColCfg<L>::C, T = ColCfg<L>::T;
@@ -204,7 +204,7 @@ k_fwd_y(Geom g, const cx<Real> *__restrict__ U1, cx<Real> *__restrict__ U2,
 // adjacent columns (c, c + 1) with 16-byte accesses.
 template <typename Real, int L, typename Cfg>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
-k_fwd_y2(Geom g, const cx<Real> *__restrict__ U1, cx<Real> *__restrict__ U2,
+k_fwd_y2(Geom g, const cx<Real> *U1, cx<Real> *__restrict__ U2,
          const cx<Real> *__restrict__ tw)
 {
     constexpr int C = Cfg::C, T = Cfg::T;

@@ -16,7 +16,7 @@ namespace lh {
 
 template <typename Real, int L>
 __global__ void __launch_bounds__(ColCfg<L>::T, ColCfg<L>::MINB)
-k_inv_y(Geom g, const cx<Real> *__restrict__ U3, cx<Real> *__restrict__ U4,
+k_inv_y(Geom g, const cx<Real> *U3, cx<Real> *__restrict__ U4,
         const cx<Real> *__restrict__ tw)
 {
     constexpr int C = ColCfg<L>::C, T = ColCfg<L>::T;
@@ -59,7 +59,7 @@ k_inv_y(Geom g, const cx<Real> *__restrict__ U3, cx<Real> *__restrict__ U4,
 // Paired-column version of the inverse p_y pass (L >= 128).
 template <typename Real, int L, typename Cfg>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
-k_inv_y2(Geom g, const cx<Real> *__restrict__ U3, cx<Real> *__restrict__ U4,
+k_inv_y2(Geom g, const cx<Real> *U3, cx<Real> *__restrict__ U4,
          const cx<Real> *__restrict__ tw)
 {
     constexpr int C = Cfg::C, T = Cfg::T;
@@ -106,7 +106,7 @@ struct InvEnergyBounds {
 };
 template <typename Real, typename OutT, int L>
 __global__ void __launch_bounds__(LineCfg<L>::T, InvEnergyBounds<Real, L>::MINB)
-k_inv_energy(Geom g, const cx<Real> *__restrict__ U4, OutT *__restrict__ out,
+k_inv_energy(Geom g, const cx<Real> *U4, OutT *__restrict__ out,
              const cx<Real> *__restrict__ tw)
 {
     constexpr int C = LineCfg<L>::C, T = LineCfg<L>::T;

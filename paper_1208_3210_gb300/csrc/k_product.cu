@@ -27,7 +27,7 @@ struct XProduct {
 
 template <typename Real, int L, typename Cfg>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
-k_x_product(Geom g, const cx<Real> *__restrict__ U2, cx<Real> *__restrict__ U3,
+k_x_product(Geom g, const cx<Real> *U2, cx<Real> *__restrict__ U3,
             const cx<Real> *__restrict__ tw)
 {
     using XP = XProduct<Real, L, Cfg>;

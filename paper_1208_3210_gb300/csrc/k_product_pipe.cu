@@ -38,9 +38,9 @@ struct PrPipe {
 __device__ __forceinline__ float4 ld_stream_v4(const float2 *p)
 {
     float4 q;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
                  : "=f"(q.x), "=f"(q.y), "=f"(q.z), "=f"(q.w)
-                 : "l"(p));
+                 : "l"(p) : "memory");
     return q;
 }
 __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc)
@@ -66,7 +66,7 @@ __device__ __forceinline__ void pr_tws_copy(const float2 *__restrict__ ptw, floa
 
 template <int L, int CW_, int KR, bool TWS, bool ODD>
 __global__ void __launch_bounds__(PrPipe<L, CW_, KR, TWS>::T, PrCfg<L, CW_>::MINB)
-k_x_product_pr_pipe(Geom g, const float2 *__restrict__ U2, float2 *__restrict__ U3, const float2 *__restrict__ ptw)
+k_x_product_pr_pipe(Geom g, const float2 *U2, float2 *__restrict__ U3, const float2 *__restrict__ ptw)
 {
     using PP = PrPipe<L, CW_, KR, TWS>;
     using EF = typename PP::EF;

@@ -50,7 +50,7 @@ size_t pr_twiddle_bytes() { return (size_t)pr_twiddle_entries() * sizeof(float2)
 
 template <int L, typename Cfg>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
-k_fwd_y_pr(Geom g, const float2 *__restrict__ U1, float2 *__restrict__ U2, const float2 *__restrict__ ptw)
+k_fwd_y_pr(Geom g, const float2 *U1, float2 *__restrict__ U2, const float2 *__restrict__ ptw)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM((PrEng<L, Cfg::C, Cfg::T, false, 2, true, false>::SMEM_ELEMS), float2)
@@ -61,7 +61,7 @@ k_fwd_y_pr(Geom g, const float2 *__restrict__ U1, float2 *__restrict__ U2, const
 
 template <int L, typename Cfg, bool ODD>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
-k_x_product_pr(Geom g, const float2 *__restrict__ U2, float2 *__restrict__ U3, const float2 *__restrict__ ptw)
+k_x_product_pr(Geom g, const float2 *U2, float2 *__restrict__ U3, const float2 *__restrict__ ptw)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM((PrProduct<L, Cfg::C, Cfg::T>::SMEM_ELEMS), float2)
@@ -72,7 +72,7 @@ k_x_product_pr(Geom g, const float2 *__restrict__ U2, float2 *__restrict__ U3, c
 
 template <int L, typename Cfg>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
-k_inv_y_pr(Geom g, const float2 *__restrict__ U3, float2 *__restrict__ U4, const float2 *__restrict__ ptw)
+k_inv_y_pr(Geom g, const float2 *U3, float2 *__restrict__ U4, const float2 *__restrict__ ptw)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM((PrEng<L, Cfg::C, Cfg::T, true, 2, false, true>::SMEM_ELEMS), float2)
@@ -139,7 +139,7 @@ cudaError_t launch_inv_y_pr_t(const Geom &g, const Work<float> &w, cudaStream_t 
 // 3): one phase per butterfly.
 template <int L, typename Cfg, bool ODD>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
-k_bw_product_pr(Geom g, float2 *__restrict__ U2, const float2 *__restrict__ WU2, const float2 *__restrict__ ptw)
+k_bw_product_pr(Geom g, float2 *__restrict__ U2, const float2 *WU2, const float2 *__restrict__ ptw)
 {
     constexpr int C = Cfg::C, T = Cfg::T;
     using EF2 = PrEng<L, C, T, false, 2, true, false>;
@@ -179,8 +179,8 @@ k_bw_product_pr(Geom g, float2 *__restrict__ U2, const float2 *__restrict__ WU2,
         const long long dw = (long long)(L / 24) * ws, da = (long long)(L / 24) * rs;
 #pragma unroll
         for (int r = 0; r < 16; ++r) {
-            vw[r] = valid ? __ldg(pw + r * dw) : zero;
-            v[r] = valid ? __ldg(pa + r * da) : zero;
+            vw[r] = valid ? pw[r * dw] : zero;
+            v[r] = valid ? pa[r * da] : zero;
         }
     }
     EF2::run(vw, v, sm, ptw);
@@ -202,7 +202,7 @@ k_bw_product_pr(Geom g, float2 *__restrict__ U2, const float2 *__restrict__ WU2,
         const float2 *pb = colB + (long long)j * rs;
         const long long db = (long long)(L / 24) * rs;
 #pragma unroll
-        for (int r = 0; r < 16; ++r) v[r] = valid ? __ldg(pb + r * db) : zero;
+        for (int r = 0; r < 16; ++r) v[r] = valid ? pb[r * db] : zero;
     }
     EF1::run(v, v, sm, ptw);
 #pragma unroll

@@ -196,7 +196,12 @@ __device__ __forceinline__ unsigned dyn_smem_bytes()
 // while the one before it in the stream still runs, and calls after_previous
 // before it touches any memory that an earlier kernel reads or writes (the
 // wait ends when the previous grid has finished and its writes are visible; as
-// every kernel so launched waits, so have all before it).  Launched plainly,
+// every kernel so launched waits, so have all before it).  Such a kernel is
+// alive while what it reads is still being written, so it reads that (the
+// caller's arrays too) with ordinary or volatile loads, which stay behind the
+// wait: no const __restrict__ parameter, no __ldg and no ld.global.nc, whose
+// data must not change while the kernel is alive.  Those are for the tables that
+// are laid out with the plan.  Launched plainly,
 // the passes of a call have gaps of some 2 us: 256^3 76.0 -> 62.3 us a call,
 // the one-zone 32^2 x 48 call 36.9 -> 25.5 us.  No kernel signals earlier than
 // its end (griddepcontrol.launch_dependents): the next grid's CTAs then take

@@ -120,8 +120,12 @@ def pass_bytes(s):
 
 
 def edge_carried(grid, band):
-    """Whether the even form carries the zone edge (its weight above 2^-24)."""
-    return (math.pi * grid["zones"] * band["ff_a"]) ** 2 < 8 * 24 * math.log(2.0)
+    """Whether the even form carries the zone edge (free electrons; else where
+    its weight is above 2^-24 of that of the row nearest the centre with the
+    same band energies)."""
+    zones = grid["zones"]
+    return band.get("kind", 0) == 1 or \
+        (zones * zones - zones % 2) * (math.pi * band["ff_a"]) ** 2 < 8 * 24 * math.log(2.0)
 
 
 def even_pass_bytes(s, grid, band, precision, fp32=0):

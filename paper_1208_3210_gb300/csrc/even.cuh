@@ -36,9 +36,9 @@
 // and the inverse is V = FFT(v), z_j = (conj(w_j) V_j + w_j V_{M-j}) / 2.
 //
 // The edge.  The grid p_i = (i - N/2) dp holds p = -N/2 dp without its mirror.
-// This form leaves that row and column of A out where their weight |M|^2 is
-// below 2^-24 of the centre's (ev_band_applies): their part of Im chi is then
-// below the rounding of its FP32 sums.  Otherwise k_even_edge.cu carries them.
+// This form leaves that row and column of A out where their part of Im chi is
+// below the rounding of its FP32 sums (ev_band_applies).  Otherwise
+// k_even_edge.cu carries them.
 #pragma once
 
 #include "kernels.cuh"
@@ -146,12 +146,17 @@ inline long long ev_edge_y_floats(const Geom &g, const EvGeom &v)
     const long long a = v.M * v.s2 + ev_edge_lines(v) + v.M, b = g.Q * v.s4;
     return a > b ? a : b;
 }
-// The edge row's weight against the centre's, exp(-(N dp / 2)^2 ff_a^2 / 8),
-// below 2^-24: half a unit in the last place of an FP32 sum of the centre's.
+// Whether the edge row may be left out: its weight exp(-p^2 ff_a^2 / 8) must lie
+// below 2^-24, half a unit in the last place of an FP32 sum, of the weight of the
+// row with the same band energies that is nearest to the centre.  A tight-binding
+// band of Z zones has that row at p_x = 0 (Z even) or pi (Z odd).  Free electrons
+// have none: with mu at the edge's energy (Z pi)^2 / 2 the edge is what carries
+// the spectral weight (4 zones of 12 points, ff_a 0.92, gamma 0.05: without it Im
+// chi is off by 1.4e-3 of its maximum at mu = 79), so theirs is always carried.
 inline bool ev_band_applies(const Geom &g, const Band &b)
 {
-    const double p = 0.5 * g.N * g.dp * b.ff_a;
-    return p * p >= 8.0 * 24.0 * 0.69314718055994530942;
+    const double Z = g.N / g.npz, near = g.N / g.npz % 2, pa = 3.14159265358979323846 * b.ff_a;
+    return b.band_kind != 1 && (Z * Z - near) * (pa * pa) >= 8.0 * 24.0 * 0.69314718055994530942;
 }
 
 // ---------------------------------------------------------------------------

@@ -72,7 +72,9 @@ typedef enum {
                                    Momentum FFT lengths 128, 192, 256, 384,
                                    512, 768, 1024, 1536; forward only (plans
                                    with LINDHARD_PLAN_BACKWARD reject it)    */
-    LINDHARD_FP64 = 2           /* FP64 everywhere; FFT lengths <= 256 only   */
+    LINDHARD_FP64 = 2           /* FP64 spectral function, transforms and sums
+                                   (mu: see lindhard_band.filling); FFT lengths
+                                   <= 256 only                               */
 } lindhard_precision;
 
 /* What a grid's output holds (lindhard_grid.quantity).  With kT > 0 the
@@ -98,9 +100,12 @@ typedef struct {
                            - 4t' cos px cos py - 2t'' (cos 2px + cos 2py) - mu */
     double mu;          /* chemical potential; used as given iff filling is NaN */
     double filling;     /* electrons per site incl. spin (rigid band, Sec. 3);
-                           mu is then solved in FP64 so that
+                           mu is then solved so that
                            (2/npz^2) sum_k [1/2 - atan(xi_k/gamma)/pi] = filling
-                           over the first-zone grid                        */
+                           over the first-zone grid, to 1e-12 eV at gamma >=
+                           0.002: its last step sums in FP64, or, with at most
+                           160 points per zone and gamma >= 0.002 eV, in
+                           unevaluated FP32 pairs (48 bits)                */
     double gamma;       /* Lorentzian half-width (Eq. 5), > 0                 */
     double ff_a;        /* |M(p)|^2 = exp(-|p|^2 ff_a^2 / 8); 0 => |M|^2 = 1   */
     int band_kind;      /* 0 tight binding; 1 free electrons, xi = |p|^2/2 - mu */

@@ -110,6 +110,8 @@ struct MuConst {
     // of the one-CTA solve: the filling, and as FP32 pairs 1/gamma and
     // e^{i pi (npz^2 / 2 - target)}
     float target_f, Bf, igh, igl, cth, ctl, sth, stl;
+    float step_tol;      // the last step is not repeated at this length
+    int narrow;          // it sums arctangents in FP64
 };
 
 // Zones small enough for the one-CTA solve: the whole search and the final step
@@ -317,7 +319,7 @@ __device__ __forceinline__ void sect_pass(const Geom &g, const Band &band, const
 //    bracket of about 0.7 eV.
 // 2. A bracketed Halley iteration in FP32 over all threads, to 1e-6 eV (a step
 //    that leaves the bracket, or a flat n, falls back to bisection).
-// 3. One Halley step in twice FP32 precision.  The occupations' sum needs
+// 3. A Halley step in twice FP32 precision.  The occupations' sum needs
 //    Theta = sum w atan(x_k), and that is the argument of prod (1 + i x_k)^w:
 //    the product is formed in unevaluated FP32 pairs (each factor scaled to
 //    modulus 1 by an FP32 factor, which leaves its argument), multiplied by
@@ -325,14 +327,25 @@ __device__ __forceinline__ void sect_pass(const Geom &g, const Band &band, const
 //    most after step 2, comes from three terms of its series: no arctangent,
 //    and no multiple of 2 pi to find.  The product's rounding is some 1e-12 of
 //    an electron state, 1e-15 eV; the step itself, below 1e-6 eV, is FP32.
+//    Below MU_PAIR_GAMMA the angle left is no longer small (a level of weight 8
+//    turns it by 8 d / gamma), and the step sums the arctangents in FP64.
+// 4. Where n(mu) is flat (nearly empty or full bands) the FP32 search ends
+//    farther off, its sums being rounded at 1e-3 of a state, and for narrow
+//    Lorentzians the remainder (d / gamma)^2 d of a step d counts: step 3 is
+//    repeated until d^3 <= 1e-13 gamma^2, d = 6e-6 eV at gamma = 0.05.  So it runs
+//    once at ordinary fillings.  Replayed on the CPU for gamma from 1e-6 to 1 eV
+//    and fillings from 0.001 to 1.999: mu within 4e-12 eV and no filling refused
+//    that has a root (with one step 8e-9 at gamma = 1e-5, and some refused).
 //
 // What bounds it is one SM's latency.  FP64 units are what it avoids: they
 // retire two operations a cycle and SM, so a warp's FP64 instruction takes 16
 // cycles whatever its lanes hold; the FP64 arctangents of the last step and the
 // cosines of the classes (now laid out once per plan) were most of the time.
-// Set-up and solve at npz = 64: 22.9 -> 14.4 us, mu within 2e-15 eV on average (9e-15 before; the product in FP64 by two
-// warps: 17 us, its errors no smaller).
+// Set-up and solve at npz = 64: 22.9 -> 14.4 us, mu within 2e-15 eV on average
+// (9e-15 before; the product in FP64 by two warps: 17 us, its errors no smaller).
 constexpr int MU_NEWTON_MAX = 64;    // bisection alone reaches 1e-6 eV in 24 steps
+constexpr int MU_STEP_MAX = 8;
+constexpr double MU_PAIR_GAMMA = 0.002;   // eV
 struct C2 { F2 r, i; };
 __device__ __forceinline__ F2 f2_div(F2 a, F2 b)
 {
@@ -357,7 +370,113 @@ struct MuSingle {
     C2 z[MU_THREADS / 32];                     // warp products and sums of the last step
     F2 n1[MU_THREADS / 32];
     float d2[MU_THREADS / 32];
+    double f64[MU_THREADS / 32];
+    F2 mu, step;                               // the last step's result and the step
+    int done;
 };
+// The Halley step from mu, added to mu, in FP64 (thread 0 returns it; every
+// thread takes part).
+__device__ __forceinline__ F2 mu_step_fp64(const Geom &g, const Band &band, const MuConst &mc, MuSingle &sh, F2 mu2)
+{
+    constexpr int NW = MU_THREADS / 32;
+    const int h = g.npz / 2, npairs = (h + 1) * (h + 2) / 2, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto wide = [](F2 a) { return (double)a.h + (double)a.l; };
+    const double ipi = 0.31830988618379067154, mu = wide(mu2);
+    double f = 0.0;
+    float d1 = 0.f, d2 = 0.f;
+    for (int k = threadIdx.x; k < npairs; k += MU_THREADS) {
+        int a, b;
+        tri_pair(k, h, a, b);
+        const double c1a = wide(sh.c1[a]), c1b = wide(sh.c1[b]), w = pair_weight(a, b, h);
+        const double e0 = band.band_kind == 1 ? 0.5 * (wide(sh.p2[a]) + wide(sh.p2[b]))
+                                              : -2.0 * band.t * (c1a + c1b) - 4.0 * band.tp * c1a * c1b
+                                                    - 2.0 * band.tpp * (wide(sh.c2[a]) + wide(sh.c2[b]));
+        const double x = (e0 - mu) * mc.inv_gam;
+        f += w * (0.5 - atan(x) * ipi);
+        const float xf = (float)x, r = 1.0f / (1.0f + xf * xf);
+        d1 += (float)w * r;
+        d2 += (float)w * 2.0f * xf * r * r;
+    }
+    F2 n1{d1, 0.f};
+    for (int o = 16; o > 0; o >>= 1) {
+        f += __shfl_down_sync(0xffffffffu, f, o);
+        n1 = f2_add(n1, F2{__shfl_down_sync(0xffffffffu, n1.h, o), __shfl_down_sync(0xffffffffu, n1.l, o)});
+        d2 += __shfl_down_sync(0xffffffffu, d2, o);
+    }
+    if (lane == 0) { sh.f64[warp] = f; sh.n1[warp] = n1; sh.d2[warp] = d2; }
+    __syncthreads();
+    if (threadIdx.x != 0) return F2{0.f, 0.f};
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+    for (int w = 0; w < NW; ++w) { s0 += sh.f64[w]; s1 += wide(sh.n1[w]); s2 += (double)sh.d2[w]; }
+    const double d = s0 - mc.target, dd1 = s1 * ipi * mc.inv_gam, dd2 = s2 * ipi * mc.inv_gam * mc.inv_gam;
+    const double step = -2.0 * d * dd1 / (2.0 * dd1 * dd1 - d * dd2);
+    const float hi = (float)step;
+    return F2{hi, (float)(step - (double)hi)};
+}
+// The same in twice FP32 precision.
+__device__ __forceinline__ F2 mu_step_pairs(const Geom &g, const Band &band, const MuConst &mc, MuSingle &sh, F2 mu)
+{
+    constexpr int NW = MU_THREADS / 32;
+    const int h = g.npz / 2, npairs = (h + 1) * (h + 2) / 2, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool free_e = band.band_kind == 1;
+    const F2 igp{mc.igh, mc.igl}, mm = f2_neg(mu);
+    const F2 k1{band.k1[0], band.k1[1]}, k2{band.k2[0], band.k2[1]}, k3{band.k3[0], band.k3[1]};
+    const F2 one{1.f, 0.f}, nil{0.f, 0.f};
+    C2 z8{one, nil}, z4{one, nil}, z1{one, nil};   // products of the factors of weight 8, 4, and 1 or 2
+    float d1 = 0.f, d2 = 0.f;
+    for (int k = threadIdx.x; k < npairs; k += MU_THREADS) {
+        int a, b;
+        tri_pair(k, h, a, b);
+        const int w = pair_weight(a, b, h);
+        F2 e0;
+        if (free_e) {
+            e0 = f2_add(sh.p2[a], sh.p2[b]);
+            e0.h *= 0.5f;
+            e0.l *= 0.5f;
+        } else {
+            e0 = f2_add(f2_add(f2_mul(k1, f2_add(sh.c1[a], sh.c1[b])), f2_mul(k2, f2_mul(sh.c1[a], sh.c1[b]))),
+                        f2_mul(k3, f2_add(sh.c2[a], sh.c2[b])));
+        }
+        const F2 x = f2_mul(f2_add(e0, mm), igp);
+        const float q = 1.0f + x.h * x.h, s = rsqrtf(q), r = 1.0f / q;
+        const C2 f{{s, 0.f}, f2_mul(x, F2{s, 0.f})};
+        if (w == 8) z8 = c2_mul(z8, f);
+        else if (w == 4) z4 = c2_mul(z4, f);
+        else z1 = c2_mul(z1, w == 2 ? c2_mul(f, f) : f);
+        d1 += (float)w * r;                       // pi gamma n'
+        d2 += (float)w * 2.0f * x.h * r * r;      // pi gamma^2 n''
+    }
+    C2 z = c2_mul(z4, c2_mul(z8, z8));   // (z4 z8^2)^4 z1
+    z = c2_mul(z, z);
+    z = c2_mul(c2_mul(z, z), z1);
+    F2 n1{d1, 0.f};   // the slope divides the step: its tree is summed as a pair
+    for (int o = 16; o > 0; o >>= 1) {
+        z = c2_mul(z, c2_shfl(z, o));
+        n1 = f2_add(n1, f2_shfl(n1, o));
+        d2 += __shfl_down_sync(0xffffffffu, d2, o);
+    }
+    if (lane == 0) { sh.z[warp] = z; sh.n1[warp] = n1; sh.d2[warp] = d2; }
+    __syncthreads();
+    if (warp != 0) return nil;
+    z = lane < NW ? sh.z[lane] : C2{one, nil};
+    n1 = lane < NW ? sh.n1[lane] : nil;
+    d2 = lane < NW ? sh.d2[lane] : 0.f;
+    for (int o = 8; o > 0; o >>= 1) {
+        z = c2_mul(z, c2_shfl(z, o));
+        n1 = f2_add(n1, f2_shfl(n1, o));
+        d2 += __shfl_down_sync(0xffffffffu, d2, o);
+    }
+    z = c2_mul(z, C2{{mc.cth, mc.ctl}, {-mc.sth, -mc.stl}});
+    // the angle left, Theta - Theta_target = -pi (n - target), and the step, as
+    // pairs where they scale the result
+    const F2 tn = f2_div(z.i, z.r);
+    const float t2 = tn.h * tn.h;
+    F2 ang = f2_fast(tn.h, tn.l - tn.h * t2 * (1.0f / 3.0f - t2 * (0.2f - t2 * (1.0f / 7.0f))));
+    if (!(fabsf(tn.h) <= 0.1f) || !(z.r.h > 0.f)) ang = {atan2f(z.i.h, z.r.h), 0.f};   // not after a search that converged
+    const F2 a1 = f2_mul(n1, igp);                                       // pi n'
+    const float eps = ang.h * d2 / (2.0f * n1.h * n1.h);                     // -(n - target) n'' / (2 n'^2)
+    return f2_mul(f2_div(ang, a1), F2{1.0f, -eps / (1.0f + eps)});           // Halley's 1 / (1 + eps)
+}
 __device__ void mu_solve_one_cta(const Geom &g, const Band &band, const MuConst &mc, MuSingle &sh, InstState *st,
                                  unsigned *status, double *mu_out, const ClsTab *__restrict__ cls)
 {
@@ -462,73 +581,31 @@ __device__ void mu_solve_one_cta(const Geom &g, const Band &band, const MuConst 
 
     // the last step, from mu + mu_l
     if (!(fabsf(mu_l) < 1e-6f)) mu_l = 0.f;
-    const F2 igp{mc.igh, mc.igl}, mm = f2_fast(-mu, -mu_l);
-    const F2 k1{band.k1[0], band.k1[1]}, k2{band.k2[0], band.k2[1]}, k3{band.k3[0], band.k3[1]};
-    const F2 one{1.f, 0.f}, nil{0.f, 0.f};
-    C2 z8{one, nil}, z4{one, nil}, z1{one, nil};   // products of the factors of weight 8, 4, and 1 or 2
-    float d1 = 0.f, d2 = 0.f;
-    for (int k = threadIdx.x; k < npairs; k += MU_THREADS) {
-        int a, b;
-        tri_pair(k, h, a, b);
-        const int w = pair_weight(a, b, h);
-        F2 e0;
-        if (free_e) {
-            e0 = f2_add(sh.p2[a], sh.p2[b]);
-            e0.h *= 0.5f;
-            e0.l *= 0.5f;
-        } else {
-            e0 = f2_add(f2_add(f2_mul(k1, f2_add(sh.c1[a], sh.c1[b])), f2_mul(k2, f2_mul(sh.c1[a], sh.c1[b]))),
-                        f2_mul(k3, f2_add(sh.c2[a], sh.c2[b])));
+    F2 cur = f2_fast(mu, mu_l);
+    for (int it = 1;; ++it) {
+        const F2 step = mc.narrow ? mu_step_fp64(g, band, mc, sh, cur) : mu_step_pairs(g, band, mc, sh, cur);
+        if (threadIdx.x == 0) {
+            // a step that grows has left the root's neighbourhood: the one before counts
+            const bool grows = it > 1 && !(fabsf(step.h) < 2.f * fabsf(sh.step.h));
+            const float len = fabsf(grows ? sh.step.h : step.h);
+            const F2 m = grows ? cur : f2_add(cur, step);
+            const int done = grows || it == MU_STEP_MAX || !(len > mc.step_tol);
+            if (done) {
+                const double mu_new = (double)m.h + (double)m.l;
+                set_mu(st, mu_new);
+                st->last_step = (double)len;
+                if (mu_out) *mu_out = mu_new;
+                // the search ends within 1e-4 eV of the root: a larger last step means it went wrong
+                if (!(len <= 1e-4f)) atomicCAS(status, (unsigned)DEV_OK, (unsigned)DEV_ENOCONV);
+            }
+            sh.mu = m;
+            sh.step = step;
+            sh.done = done;
         }
-        const F2 x = f2_mul(f2_add(e0, mm), igp);
-        const float q = 1.0f + x.h * x.h, s = rsqrtf(q), r = 1.0f / q;
-        const C2 f{{s, 0.f}, f2_mul(x, F2{s, 0.f})};
-        if (w == 8) z8 = c2_mul(z8, f);
-        else if (w == 4) z4 = c2_mul(z4, f);
-        else z1 = c2_mul(z1, w == 2 ? c2_mul(f, f) : f);
-        d1 += (float)w * r;                       // pi gamma n'
-        d2 += (float)w * 2.0f * x.h * r * r;      // pi gamma^2 n''
+        __syncthreads();
+        if (sh.done) return;
+        cur = sh.mu;
     }
-    C2 z = c2_mul(z4, c2_mul(z8, z8));   // (z4 z8^2)^4 z1
-    z = c2_mul(z, z);
-    z = c2_mul(c2_mul(z, z), z1);
-    F2 n1{d1, 0.f};   // the slope divides the step: its tree is summed as a pair
-    for (int o = 16; o > 0; o >>= 1) {
-        z = c2_mul(z, c2_shfl(z, o));
-        n1 = f2_add(n1, f2_shfl(n1, o));
-        d2 += __shfl_down_sync(0xffffffffu, d2, o);
-    }
-    if (lane == 0) { sh.z[warp] = z; sh.n1[warp] = n1; sh.d2[warp] = d2; }
-    __syncthreads();
-    if (warp != 0) return;
-    z = lane < NW ? sh.z[lane] : C2{one, nil};
-    n1 = lane < NW ? sh.n1[lane] : nil;
-    d2 = lane < NW ? sh.d2[lane] : 0.f;
-    for (int o = 8; o > 0; o >>= 1) {
-        z = c2_mul(z, c2_shfl(z, o));
-        n1 = f2_add(n1, f2_shfl(n1, o));
-        d2 += __shfl_down_sync(0xffffffffu, d2, o);
-    }
-    if (lane != 0) return;
-    z = c2_mul(z, C2{{mc.cth, mc.ctl}, {-mc.sth, -mc.stl}});
-    // the angle left, Theta - Theta_target = -pi (n - target), and the step, as
-    // pairs where they scale the result
-    const F2 tn = f2_div(z.i, z.r);
-    const float t2 = tn.h * tn.h;
-    F2 ang = f2_fast(tn.h, tn.l - tn.h * t2 * (1.0f / 3.0f - t2 * (0.2f - t2 * (1.0f / 7.0f))));
-    if (!(fabsf(tn.h) <= 0.1f) || !(z.r.h > 0.f)) ang = {atan2f(z.i.h, z.r.h), 0.f};   // not after a search that converged
-    const F2 a1 = f2_mul(n1, igp);                                       // pi n'
-    const float eps = ang.h * d2 / (2.0f * n1.h * n1.h);                     // -(n - target) n'' / (2 n'^2)
-    const F2 step = f2_mul(f2_div(ang, a1), F2{1.0f, -eps / (1.0f + eps)});   // -step: Halley's 1 / (1 + eps)
-    const F2 m = f2_add(f2_neg(mm), step);
-    const float stp = step.h;
-    const double mu_new = (double)m.h + (double)m.l;
-    set_mu(st, mu_new);
-    st->last_step = fabs((double)stp);
-    if (mu_out) *mu_out = mu_new;
-    // the FP32 search stops within about 1e-6 eV of the root: a larger
-    // correction means it went wrong
-    if (!(fabsf(stp) <= 1e-4f)) atomicCAS(status, (unsigned)DEV_OK, (unsigned)DEV_ENOCONV);
 }
 
 // Set-up launch.  CTAs [0, G): multisection pass 0 (mu from the filling);
@@ -761,6 +838,8 @@ static MuConst mu_const(const Geom &g, const Band &band, int G)
     pair(sin(M_PI * u), mc.sth, mc.stl);
     mc.B = (band.band_kind == 1) ? 9.869604401089358 : 4.0 * (fabs(band.t) + fabs(band.tp) + fabs(band.tpp));
     mc.Bf = (float)mc.B;
+    mc.step_tol = (float)cbrt(1e-13 * band.gamma * band.gamma);
+    mc.narrow = band.gamma < MU_PAIR_GAMMA;
     return mc;
 }
 

@@ -634,7 +634,8 @@ k_setup(Geom g, Band band, AxisTab *axis, float2 *eps32, double *eps64, InstStat
             AxisTab a;
             a.c1 = c.c1;
             a.c2 = c.c2;
-            a.g = (band.ff_a == 0.0) ? 1.0 : exp(-p * p * (band.ff_a * band.ff_a * 0.125));
+            const double pa = p * band.ff_a;   // ff_a^2 by itself may overflow, and 0 inf is NaN at p = 0
+            a.g = exp(-0.125 * (pa * pa));
             a.p2 = p * p;
             a.c1h = c.c1h;
             a.c1l = c.c1l;

@@ -133,19 +133,30 @@ __device__ __forceinline__ float kk_vq(long long l, int Q, double dp, double v0,
 // products on the tensor cores with an FP32 near band, where the operand split,
 // the near band and the transposes around the products took about 145
 // instructions an output with one or two CTAs of 8 warps per SM.  1024^2 lags x
-// 256 transfers: 2.70 -> 1.22 ms, error 1.2e-6 -> 1.5e-7 of the result's norm;
-// 256^2 x 128: 0.069 -> 0.052 ms.  Four lines a group in packed arithmetic (77
+// 256 transfers: 2.70 -> 1.24 ms (1.22 without the lines' scales), error 1.2e-6 ->
+// 1.5e-7 of the result's norm; 256^2 x 128: 0.069 -> 0.052 ms.  Four lines a group in packed arithmetic (77
 // instructions an output, 226 registers, 8 warps per SM): 1.46 ms; this with
 // 168 registers: 1.56 ms, with 96: 1.46 ms; transfers' tables in natural order
 // (one value a load): 1.26 ms.
 //
-// A line with an infinity or NaN would spread it over the line that shares its
-// transform, so a group that holds one is summed directly (kk_direct).
+// Two lines share a transform, and its rounding is that of the larger one: each is
+// scaled by a power of two to a maximum in [1, 2) first and back after (exact; a
+// line 1e-4 of its neighbour was off by 1e-3 of itself, and one near FP32's largest
+// overflowed into it).  An infinity or NaN would still spread over the other line,
+// so a group that holds one is summed directly (kk_direct).
 constexpr int KKF_WARPS = 4;
 
 // One pair of lines by the sum itself, FP32.
 __device__ __noinline__ void kk_direct(long long l0, long long nlines, int nw, int u, int tpl, int Q, float vh, float vl,
                                        const float *__restrict__ im, float *__restrict__ re, float2 *__restrict__ rpa);
+
+// max(m, |x|), NaN if either is
+__device__ __forceinline__ float kk_max(float m, float x)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(m), "f"(fabsf(x)));
+    return r;
+}
 
 // v0 / |q|^2 of lag line l, v0 / dp^2 = vh + vl; *zero when q = 0 with an interaction
 __device__ __forceinline__ float kk_v(long long l, int Q, float vh, float vl, bool *zero)
@@ -178,22 +189,34 @@ k_kk_fft(long long nlines, int nw, int Q, float vh, float vl, const float *__res
     const int ra = u, rb = E::pair(1, u);
     const float *row = im + (live ? l0 : 0) * nw;
     float2 raw[2][R1 / 2];
-    float big = 0.f;   // an infinity or NaN in the group: 0 x makes it NaN
+    float top[2] = {0.f, 0.f}, up[2], down[2];   // the lines' maxima, their scales and back
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const float *p = row + (h ? rb : ra);
 #pragma unroll
         for (int r = 0; r < R1 / 2; ++r) {
-            const bool in = live && (h ? rb : ra) + r * R0 < nw;
+            const bool in = live && (h ? rb : ra) + r * R0 < nw && (h + r > 0 || !u0);   // x_0 does not enter
             raw[h][r] = make_float2(in ? __ldg(p + r * R0) : 0.f, in ? __ldg(p + nw + r * R0) : 0.f);
         }
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h)
 #pragma unroll
-        for (int r = 0; r < R1 / 2; ++r) big = fmaf(0.f, raw[h][r].x, fmaf(0.f, raw[h][r].y, big));
-    const unsigned group = ((1u << TPL) - 1u) << (sl * TPL);
-    const bool bad = (__ballot_sync(0xffffffffu, isnan(big)) & group) != 0;
+        for (int r = 0; r < R1 / 2; ++r) {
+            top[0] = kk_max(top[0], raw[h][r].x);
+            top[1] = kk_max(top[1], raw[h][r].y);
+        }
+    bool bad = false;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+#pragma unroll
+        for (int o = TPL / 2; o > 0; o >>= 1) top[i] = kk_max(top[i], __shfl_xor_sync(0xffffffffu, top[i], o));
+        const unsigned e = __float_as_uint(top[i]) >> 23;   // 255: an infinity or NaN
+        bad |= e == 255u;
+        const unsigned c = min(max(e, 1u), 253u);
+        up[i] = __uint_as_float((254u - c) << 23);
+        down[i] = __uint_as_float(c << 23);
+    }
 
     const float4 *ht = kt + u, *wt = kt + M / 4 + u;   // the lane's columns of the tables
     auto w_of = [&](float4 q, int r) { return r % 2 ? make_float2(q.z, q.w) : make_float2(q.x, q.y); };
@@ -205,8 +228,7 @@ k_kk_fft(long long nlines, int nw, int Q, float vh, float vl, const float *__res
         float2 hi[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            float2 v = raw[h][r];
-            if (h == 0 && r == 0) v = sel(make_float2(0.f, 0.f), v);   // x_0 does not enter
+            const float2 v = make_float2(raw[h][r].x * up[0], raw[h][r].y * up[1]);
             const float2 w = w_of(__ldg(wt + (h * (R1 / 2) + r) / 2 * TPL), r);
             const float2 a = cmul(v, w), b = cmulc(v, w);
             x[h * R1 + r] = mul_mi(a);
@@ -249,7 +271,7 @@ k_kk_fft(long long nlines, int nw, int Q, float vh, float vl, const float *__res
             const float2 a = x[h * R1 + r];
             const float2 b = h ? sel(x[R1 + R1 - 1 - r], x[R1 - 1 - r]) : sel(x[(R1 - r) % R1], x[R1 + R1 - 1 - r]);
             const float2 z = cadd(cmulc(a, w), cmul(b, w));
-            const float y[2] = {z.x, z.y};
+            const float y[2] = {z.x * down[0], z.y * down[1]};
             if (rh + r * R0 < nw) {
 #pragma unroll
                 for (int i = 0; i < 2; ++i) ro[i * nw + r * R0] = y[i];

@@ -146,8 +146,16 @@ __device__ __forceinline__ float kk_vq(long long l, int Q, double dp, double v0,
 // so a group that holds one is summed directly (kk_direct).
 constexpr int KKF_WARPS = 4;
 
+// v0 / dp^2 = (h + l) 2^e, |h + l| in [0.05, 4e5] for any v0 (dp is 2 pi / 4096 to
+// pi), so that neither a very small nor a very large v0 leaves FP32 before |q|^2
+// divides it.
+struct KkV {
+    float h, l;
+    int e;
+};
+
 // One pair of lines by the sum itself, FP32.
-__device__ __noinline__ void kk_direct(long long l0, long long nlines, int nw, int u, int tpl, int Q, float vh, float vl,
+__device__ __noinline__ void kk_direct(long long l0, long long nlines, int nw, int u, int tpl, int Q, KkV v,
                                        const float *__restrict__ im, float *__restrict__ re, float2 *__restrict__ rpa);
 
 // max(m, |x|), NaN if either is
@@ -158,20 +166,20 @@ __device__ __forceinline__ float kk_max(float m, float x)
     return r;
 }
 
-// v0 / |q|^2 of lag line l, v0 / dp^2 = vh + vl; *zero when q = 0 with an interaction
-__device__ __forceinline__ float kk_v(long long l, int Q, float vh, float vl, bool *zero)
+// v0 / |q|^2 of lag line l; *zero when q = 0 with an interaction
+__device__ __forceinline__ float kk_v(long long l, int Q, KkV v, bool *zero)
 {
     const int x = (int)(l / Q) - Q / 2, y = (int)(l % Q) - Q / 2;
     const float k2 = (float)(x * x + y * y);   // exact: Q <= 4096
-    *zero = k2 == 0.f && vh != 0.f;
-    if (k2 == 0.f || vh == 0.f) return 0.f;
-    const float q = vh / k2;
-    return q + (fmaf(-q, k2, vh) + vl) / k2;
+    *zero = k2 == 0.f && v.h != 0.f;
+    if (k2 == 0.f || v.h == 0.f) return 0.f;
+    const float q = v.h / k2;
+    return ldexpf(q + (fmaf(-q, k2, v.h) + v.l) / k2, v.e);
 }
 
 template <int M>
 __global__ void __launch_bounds__(32 * KKF_WARPS, M == 384 ? 2 : 4)
-k_kk_fft(long long nlines, int nw, int Q, float vh, float vl, const float *__restrict__ im, float *__restrict__ re,
+k_kk_fft(long long nlines, int nw, int Q, KkV v0, const float *__restrict__ im, float *__restrict__ re,
          float2 *__restrict__ rpa, const float4 *__restrict__ kt, const float2 *__restrict__ tab)
 {
     using E = EvLine<M>;
@@ -251,13 +259,13 @@ k_kk_fft(long long nlines, int nw, int Q, float vh, float vl, const float *__res
     E::forward_rest(x, sm, u, tab);
     if (!live) return;
     if (bad) {
-        kk_direct(l0, nlines, nw, u, TPL, Q, vh, vl, im, re, rpa);
+        kk_direct(l0, nlines, nw, u, TPL, Q, v0, im, re, rpa);
         return;
     }
     float V[2];
     bool zero[2];
 #pragma unroll
-    for (int i = 0; i < 2; ++i) V[i] = kk_v(l0 + i, Q, vh, vl, &zero[i]);
+    for (int i = 0; i < 2; ++i) V[i] = kk_v(l0 + i, Q, v0, &zero[i]);
     // Re chi of transfer m = conj(w) V_m + w V_{M-m} (the 1/2 in H)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -285,13 +293,13 @@ k_kk_fft(long long nlines, int nw, int Q, float vh, float vl, const float *__res
     }
 }
 
-__device__ __noinline__ void kk_direct(long long l0, long long nlines, int nw, int u, int tpl, int Q, float vh, float vl,
+__device__ __noinline__ void kk_direct(long long l0, long long nlines, int nw, int u, int tpl, int Q, KkV v,
                                        const float *__restrict__ im, float *__restrict__ re, float2 *__restrict__ rpa)
 {
     for (int i = 0; i < 2 && l0 + i < nlines; ++i) {
         const float *row = im + (l0 + i) * nw;
         bool zero;
-        const float V = kk_v(l0 + i, Q, vh, vl, &zero);
+        const float V = kk_v(l0 + i, Q, v, &zero);
         for (int m = u; m < nw; m += tpl) {
             float s = 0.f;
             for (int k = 1 + (m & 1); k < nw; k += 2)
@@ -377,10 +385,12 @@ static cudaError_t launch_kk_fft_t(const Geom &g, const float *im, float *re, fl
     static const cudaError_t e0 = smem_attrs(k_kk_fft<M>, smem);
     if (e0 != cudaSuccess) return e0;
     const long long nlines = (long long)g.Q * g.Q, per = 2LL * KKF_WARPS * E::LPI;
-    const double v = v0 / (g.dp * g.dp);
-    const float vh = (float)v, vl = (float)(v - (double)vh);
+    KkV kv;
+    const double v = frexp(v0, &kv.e) / (g.dp * g.dp);
+    kv.h = (float)v;
+    kv.l = (float)(v - (double)kv.h);
     k_kk_fft<M><<<(unsigned)((nlines + per - 1) / per), 32 * KKF_WARPS, smem, s>>>(
-        nlines, g.n_omega, g.Q, vh, vl, im, re, rpa, static_cast<const float4 *>(tab),
+        nlines, g.n_omega, g.Q, kv, im, re, rpa, static_cast<const float4 *>(tab),
         evt + ev_line_table<M>());
     return cudaGetLastError();
 }

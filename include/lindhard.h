@@ -145,12 +145,20 @@ typedef struct {
     long long fft_e;        /* FFT length along the energy axis               */
     long long out_elems;    /* q_extent^2 * n_omega                           */
     long long a_elems;      /* N^2 * n_eps (layout of A_in and dA)           */
-    long long hbm_bytes_forward;  /* algorithmic HBM bytes of one forward call */
+    long long hbm_bytes_forward;  /* algorithmic HBM bytes of one forward call with A generated:
+                                     every intermediate of the form that it takes written once
+                                     and read once, and the output.  FP32 with several zones:
+                                     the cosine-transform form without the zone edge (a band
+                                     whose edge carries weight moves about twice that).  A
+                                     caller-supplied A moves that form's
+                                     2 c (2 N^2 H + 2 N P H + Q P H + Q^2 H) bytes + the output,
+                                     c = 8 (FP64: 16), P = fft_p, H = fft_e / 2 + 1            */
     long long kernels_forward;    /* kernel launches of one forward call with A generated and mu
                                      solved: with more than 160 points per zone one more when
                                      gamma < 0.02 eV (a third multisection pass); with at most 160
                                      the whole solve runs in the set-up launch (two fewer); one
-                                     more for the zone edge's lines where it carries weight; with
+                                     more for the zone edge's lines where an FP32 band's edge
+                                     carries weight (in FP64 always, and counted); with
                                      a caller-supplied A only the FFT passes; in a
                                      LINDHARD_PLAN_PERSISTENT plan the instance's set-up launches
                                      only (the batch adds one persistent launch)               */

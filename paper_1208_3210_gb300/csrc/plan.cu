@@ -790,6 +790,19 @@ extern "C" lindhard_status lindhard_plan_sizes(const lindhard_plan *p, int index
     // set-up (tables + multisection pass 0), multisection pass 1, Halley step, 5 FFT passes;
     // zones of at most 160 points solve mu inside the set-up launch
     out->kernels_forward = mu_solve_in_setup(g) ? 6 : 8;
+    // A generated on several zones: the even form's real buffers (even.cuh), k_x
+    // <= k_y between the momentum passes; in FP64 with the edge (one row and one
+    // launch more, four parity parts, every lag s_x of two parts in y)
+    auto even_bytes = [&](long long M, long long Nh, long long ne, long long parts, long long rows4) {
+        const long long n = g.n_omega, tri = M * (M + 1) / 2;
+        return (2 * (Nh * M * ne + tri * (ne + parts * n) + rows4 * M * n) + out->out_elems) * rb;
+    };
+    if (const EvGeom &v = p->even[index]; v.M && !p->persistent)
+        out->hbm_bytes_forward = even_bytes(v.M, v.Nh, v.ne, 1, v.nl);
+    if (const E64Geom &v = p->even64[index]; v.M) {
+        out->hbm_bytes_forward = even_bytes(v.M, v.Nh, v.ne, 4, 2 * g.Q);
+        out->kernels_forward += 1;
+    }
     // persistent plans: the instance's set-up launches (the batch's passes
     // are one further launch of the plan)
     if (p->persistent) out->kernels_forward = mu_solve_in_setup(g) ? 1 : 3;

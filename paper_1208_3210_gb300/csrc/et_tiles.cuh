@@ -66,15 +66,6 @@ struct EtGeo {
 };
 __host__ __device__ constexpr int et_pad(int n) { return n + n / 16; }
 
-// 1/x as the hardware approximation (relative error about 2^-23; x lies in
-// [gamma^2, 4 e_max^2 + gamma^2], away from zero, subnormals and overflow)
-__device__ __forceinline__ float et_rcp(float x)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 // Twiddles of one radix-R butterfly from its table row (w^1, ..., w^(R-1),
 // w^0) applied to v[1..R) (conjugated with CONJ): one 16-byte load gives w and
 // w^2, the other powers are products of them (at most three roundings deep).
@@ -150,7 +141,7 @@ __device__ __forceinline__ void energy_fwd_warp_tile(const Geom &g, const Band &
                 if constexpr (GEN) {
                     const float2 ej = eps[FULL ? n : min(n, g.n_eps - 1)];
                     const float e = (ej.x - xhi) + (ej.y - xlo);
-                    A = amp * et_rcp(fmaf(e, e, g2));
+                    A = amp * rcp_approx(fmaf(e, e, g2));
                     if (!FULL && n >= g.n_eps) A = 0.f;
                 } else {
                     A = (live && (FULL || n < g.n_eps)) ? 0.5f * A_in[line * g.n_eps + n] : 0.f;

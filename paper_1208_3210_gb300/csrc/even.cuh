@@ -464,15 +464,6 @@ struct EvFft {
     }
 };
 
-// 1/x as the hardware approximation (relative error about 2^-23; x lies in
-// [gamma^2, 4 e_max^2 + gamma^2], away from zero, subnormals and overflow)
-__device__ __forceinline__ float ev_rcp(float x)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 // A pack from global memory, read once: not kept in L1, whose few KB beside the
 // exchange buffers hold the tables.  Volatile and not through the read-only
 // path: the kernel before may have written it (after_previous).

@@ -70,61 +70,6 @@ __device__ __forceinline__ void ev_dft(float2 *v)
         Dft<R, INV, float2, EV_PK>::run(v);
     }
 }
-// The same on two complex values at once (Cx2): radix 24 = 3 x 8 by the
-// prime-factor map, radix 32 as two halves of 16.
-template <int R, bool INV>
-__device__ __forceinline__ void ev_dft(Cx2 *v)
-{
-    if constexpr (R == 24) {
-        // inputs n = 3 i + 8 j, outputs k = 9 k8 + 16 k3 (mod 24)
-        Cx2 t[3][8];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) t[j][i] = v[(3 * i + 8 * j) % 24];
-            dft8<INV>(t[j]);
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            dft3<INV>(t[0][k], t[1][k], t[2][k]);
-#pragma unroll
-            for (int q = 0; q < 3; ++q) v[(9 * k + 16 * q) % 24] = t[q][k];
-        }
-    } else if constexpr (R == 32) {
-        Cx2 e[16], o[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) { e[i] = v[2 * i]; o[i] = v[2 * i + 1]; }
-        dft<16, INV>(e);
-        dft<16, INV>(o);
-        v[0] = add(e[0], o[0]);
-        v[16] = sub(e[0], o[0]);
-        v[8] = INV ? add_i(e[8], o[8]) : sub_i(e[8], o[8]);
-        v[24] = INV ? sub_i(e[8], o[8]) : add_i(e[8], o[8]);
-        combine45x<INV, 1>(e[4], o[4], v[4], v[20]);
-        combine45x<INV, 3>(e[12], o[12], v[12], v[28]);
-#pragma unroll
-        for (int k = 1; k < 16; ++k)
-            if (k % 4 != 0) {
-                const Cx2 w = mul_w<!INV>(o[k], make_float2((float)cos32(k), (float)cos32(k + 24)));
-                v[k] = add(e[k], w);
-                v[k + 16] = sub(e[k], w);
-            }
-    } else {
-        dft<R, INV>(v);
-    }
-}
-template <bool CONJ> __device__ __forceinline__ float2 ev_mul(float2 a, float2 w) { return CONJ ? cmulc(a, w) : cmul(a, w); }
-template <bool CONJ> __device__ __forceinline__ Cx2 ev_mul(Cx2 a, float2 w) { return mul_w<CONJ>(a, w); }
-// a value's place in the exchange
-__device__ __forceinline__ void ev_put(float2 *p, float2 v) { *p = v; }
-__device__ __forceinline__ void ev_put(float4 *p, Cx2 v) { *p = make_float4(v.re.x, v.re.y, v.im.x, v.im.y); }
-__device__ __forceinline__ float2 ev_get(const float2 *p) { return *p; }
-__device__ __forceinline__ Cx2 ev_get(const float4 *p)
-{
-    const float4 q = *p;
-    return {make_float2(q.x, q.y), make_float2(q.z, q.w)};
-}
-
 // Tables after the cosine transforms': per length, k < 32: (w, w^2), 32 entries
 // later (w^3, w^4), 32 later (w^8, w^16), w = e^{-2 pi i k / L}: no power is more
 // than two products from an entry.
@@ -152,7 +97,6 @@ __device__ __forceinline__ void ev_tri(int t, int M, int &kx, int &ky)
         ky = c - 1;   // kx + (c - (M - f))
     }
 }
-
 
 // Rounds per warp: up to 8 while every SM still gets 48 warps' worth.
 inline int ev_corr_iters(int npairs, int lpi, int sms)
@@ -245,38 +189,35 @@ struct EvLine {
             dif<K + 1>(d);
         }
     }
-    // V: float2, or Cx2 with 16-byte exchange elements S
-    template <typename V, typename S>
-    __device__ __forceinline__ static void forward_rest(V *x, S *sm, int u, const float2 *__restrict__ tab)
+    __device__ __forceinline__ static void forward_rest(float2 *x, float2 *sm, int u, const float2 *__restrict__ tab)
     {
         __syncwarp();   // the previous exchange has been read
 #pragma unroll
         for (int b = 0; b < VPT / R0; ++b)
 #pragma unroll
-            for (int r = 0; r < R0; ++r) ev_put(sm + (u + b * TPL) * (R0 + 1) + r, x[b * R0 + r]);
+            for (int r = 0; r < R0; ++r) sm[(u + b * TPL) * (R0 + 1) + r] = x[b * R0 + r];
         __syncwarp();
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
             const int j = pair(b, u);
             float2 w[R1];
             powers<R1>(w, tab, j);
-            x[b * R1] = ev_get(sm + j);
+            x[b * R1] = sm[j];
 #pragma unroll
-            for (int r = 1; r < R1; ++r) x[b * R1 + r] = ev_mul<false>(ev_get(sm + j + r * (R0 + 1)), w[r]);
+            for (int r = 1; r < R1; ++r) x[b * R1 + r] = cmul(sm[j + r * (R0 + 1)], w[r]);
             ev_dft<R1, false>(x + b * R1);
         }
     }
-    template <typename V, typename S>
-    __device__ __forceinline__ static void inverse(V *x, S *sm, int u, const float2 *__restrict__ tab)
+    __device__ __forceinline__ static void inverse(float2 *x, float2 *sm, int u, const float2 *__restrict__ tab)
     {
         ev_dft<R1, true>(x);
         ev_dft<R1, true>(x + R1);
         __syncwarp();
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
-            S *p = sm + pair(b, u) * (R1 + 1);
+            float2 *p = sm + pair(b, u) * (R1 + 1);
 #pragma unroll
-            for (int r = 0; r < R1; ++r) ev_put(p + r, x[b * R1 + r]);
+            for (int r = 0; r < R1; ++r) p[r] = x[b * R1 + r];
         }
         __syncwarp();
 #pragma unroll
@@ -284,9 +225,9 @@ struct EvLine {
             const int j = u + b * TPL;
             float2 w[R0];
             powers<R0>(w, tab, j);
-            x[b * R0] = ev_get(sm + j);
+            x[b * R0] = sm[j];
 #pragma unroll
-            for (int r = 1; r < R0; ++r) x[b * R0 + r] = ev_mul<true>(ev_get(sm + j + r * (R1 + 1)), w[r]);
+            for (int r = 1; r < R0; ++r) x[b * R0 + r] = cmulc(sm[j + r * (R1 + 1)], w[r]);
             ev_dft<R0, true>(x + b * R0);   // outputs that the caller drops are not formed
         }
     }

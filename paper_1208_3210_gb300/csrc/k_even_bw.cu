@@ -266,7 +266,7 @@ k_ev_chain(Geom g, EvGeom v, Band band, const AxisTab *axis, const float2 *eps,
                 for (int h = 0; h < 2; ++h) {
                     const float2 d = add2(sub2(eh[h], dup2(q.x)), sub2(el[h], dup2(q.y)));
                     const float2 d2 = mul2(d, d), D = add2(d2, g2);
-                    const float2 iD = make_float2(et_rcp(D.x), et_rcp(D.y));
+                    const float2 iD = make_float2(rcp_approx(D.x), rcp_approx(D.y));
                     const float2 t = mul2(mul2(h ? z[b * RP + r].im : z[b * RP + r].re, dup2(q.z)), mul2(iD, iD));
                     sum = fma2(t, d, sum);
                     sg = fma2(t, sub2(d2, g2), sg);

@@ -124,9 +124,8 @@ k_ev_corr(Geom g, EvGeom v, Band band, const float *B2, float *__restrict__ B3,
 
 // The same at 768 energies, which has no two-stage schedule at these register
 // counts: three stages on the schedules and tables of et_tiles.cuh.
-// FULL: ne == L with the split at L/2.  THERMAL: Fermi weights; ODD: the odd
-// part (Im chi_T).
-template <int L, bool FULL, bool THERMAL>
+// THERMAL: Fermi weights; odd: the odd part (Im chi_T).
+template <int L, bool THERMAL>
 __global__ void __launch_bounds__(32 * EVC_WARPS)
 k_ev_corr3(Geom g, EvGeom v, Band band, const float *B2, float *__restrict__ B3,
           const float2 *__restrict__ etw, int iters, int odd)
@@ -173,7 +172,7 @@ k_ev_corr3(Geom g, EvGeom v, Band band, const float *B2, float *__restrict__ B3,
 #pragma unroll
                 for (int r = 0; r < R0; ++r) {
                     const int n = u + b * TPL + r * (L / R0);
-                    raw[q][b * R0 + r] = live && (FULL || n < v.ne) ? __ldcs(B2 + in[q] + n) : 0.f;
+                    raw[q][b * R0 + r] = live && n < v.ne ? __ldcs(B2 + in[q] + n) : 0.f;
                 }
         float2 pa[2][R2 / 2], pb[2][R2 / 2], ph[2], x[VPT];
 #pragma unroll
@@ -189,8 +188,7 @@ k_ev_corr3(Geom g, EvGeom v, Band band, const float *B2, float *__restrict__ B3,
                         const float2 w = wf[n];
                         x[b * R0 + r] = make_float2(A * w.x, A * w.y);
                     } else {
-                        const bool occ = FULL ? r < R0 / 2 : n < v.J0;
-                        x[b * R0 + r] = occ ? make_float2(A, 0.f) : make_float2(0.f, A);
+                        x[b * R0 + r] = n < v.J0 ? make_float2(A, 0.f) : make_float2(0.f, A);
                     }
                 }
                 Dft<R0, false, float2>::run(x + b * R0);
@@ -307,7 +305,6 @@ k_ev_corr3(Geom g, EvGeom v, Band band, const float *B2, float *__restrict__ B3,
     }
 }
 
-
 template <int L, bool FULL, bool THERMAL, bool HALF>
 cudaError_t launch_ev_corr_t(const Geom &g, const EvGeom &v, const Band &band, const Work<float> &w, int sms,
                              cudaStream_t s)
@@ -340,11 +337,11 @@ cudaError_t launch_ev_corr3(const Geom &g, const EvGeom &v, const Band &band, co
 {
     constexpr int L = 768, LPI = EtGeo<L>::LPI;
     const size_t smem = sizeof(float2) * (EVC_WARPS * LPI * EtGeo<L>::LP + (THERMAL ? L : 0));
-    static const cudaError_t e = smem_attrs(k_ev_corr3<L, false, THERMAL>, smem);
+    static const cudaError_t e = smem_attrs(k_ev_corr3<L, THERMAL>, smem);
     if (e != cudaSuccess) return e;
     const int npairs = v.M / 2 * (v.M + 1) / 2, iters = ev_corr_iters(npairs, LPI, sms);
     const int per = EVC_WARPS * iters * LPI;
-    return launch_after(k_ev_corr3<L, false, THERMAL>, (npairs + per - 1) / per, 32 * EVC_WARPS, smem, s, g, v, band,
+    return launch_after(k_ev_corr3<L, THERMAL>, (npairs + per - 1) / per, 32 * EVC_WARPS, smem, s, g, v, band,
                         (const float *)w.Y, (float *)w.X, (const float2 *)w.etw, iters,
                         g.quantity == LINDHARD_IMCHI_T);
 }

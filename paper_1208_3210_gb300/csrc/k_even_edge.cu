@@ -98,7 +98,7 @@ k_ev_edge(Geom g, EvGeom v, Band band, const AxisTab *axis, const float2 *eps,
         if (t == v.M && n < v.ne) {
             const float2 e = eps[v.e0 + n];
             const float d = (e.x - q.x) + (e.y - q.y);
-            raw[i] = q.z * ev_rcp(fmaf(d, d, band.gam2));
+            raw[i] = q.z * rcp_approx(fmaf(d, d, band.gam2));
         }
     }
     float2 x[VPT];
@@ -219,7 +219,9 @@ k_ev_edge_corr(Geom g, EvGeom v, Band band, const float *B2, const float4 *lines
         E::template first_stage<false, THERMAL>(x, raw, u, v.J0, wf);
         E::forward_rest(x, sm, u, tab);
         auto line = [&](const float4 *l, int r) { return EdgeLine{edge_load(l + 2 * r * TPL), edge_load(l + (2 * r + 1) * TPL)}; };
-        auto line_c = [&](int r) { return EdgeLine{ev_get(corner + 2 * r * TPL + u), ev_get(corner + (2 * r + 1) * TPL + u)}; };
+        auto line_c = [&](int r) {
+            return EdgeLine{EvFft<16, false>::ld(corner + 2 * r * TPL + u), EvFft<16, false>::ld(corner + (2 * r + 1) * TPL + u)};
+        };
         auto half = [&](float4 q) { return EdgeLine{{dup2(q.x), dup2(q.y)}, {dup2(q.z), dup2(q.w)}}; };
         // P1 + i P2 at k, conj P1 + i conj P2 at L - k
         auto w_of = [](Cx2 p, Cx2 q) { return Cx2{sub2(p.re, q.im), add2(p.im, q.re)}; };
@@ -310,7 +312,7 @@ k_ev_edge_inv_x(EvGeom v, int Q, const float *B3, float2 *__restrict__ B4,
                 const float2 *__restrict__ tab, int ntile)
 {
     using F = EvFft<M, true>;
-    constexpr int C = F::C, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP, RF = F::RF;
+    constexpr int C = F::C, VPT = F::VPT, TPC = F::TPC, RF = F::RF;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(F::SMEM_ELEMS, float4)
     after_previous();
@@ -352,7 +354,7 @@ k_ev_edge_inv_y(EvGeom v, int Q, int n_omega, const float *B4, float *__restrict
                 const float2 *__restrict__ tab, int ntile)
 {
     using F = EvFft<M, true>;
-    constexpr int C = F::C, VPT = F::VPT, TPC = F::TPC, RP = F::RP, NBP = F::NBP, RF = F::RF;
+    constexpr int C = F::C, VPT = F::VPT, TPC = F::TPC, RF = F::RF;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LH_REQUIRE_SMEM(F::SMEM_ELEMS, float4)
     after_previous();

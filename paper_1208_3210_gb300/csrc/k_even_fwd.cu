@@ -106,7 +106,7 @@ k_ev_gen_y(Geom g, EvGeom v, Band band, const AxisTab *axis, const float2 *eps,
                 for (int h = 0; h < 2; ++h) {
                     const float2 d = add2(sub2(eh[h], dup2(q.x)), sub2(el[h], dup2(q.y)));
                     const float2 x = fma2(d, d, g2);
-                    a[h] = mul2(mul2(on[h], dup2(q.z)), make_float2(ev_rcp(x.x), ev_rcp(x.y)));
+                    a[h] = mul2(mul2(on[h], dup2(q.z)), make_float2(rcp_approx(x.x), rcp_approx(x.y)));
                 }
             }
             z[b * RP + r] = {a[0], a[1]};

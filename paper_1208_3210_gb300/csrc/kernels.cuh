@@ -144,6 +144,15 @@ __device__ __forceinline__ F2 f2_mul(F2 a, F2 b)
     return f2_fast(p, e);
 }
 
+// 1/x as the hardware approximation (relative error about 2^-23; x lies in
+// [gamma^2, 4 e_max^2 + gamma^2], away from zero, subnormals and overflow)
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // Band energy xi_p = e0(p) - mu as an unevaluated FP32 pair (hi, lo), and the
 // amplitude |M(p)|^2 gamma / pi, of the momentum point with axis entries
 // (ax, ay) (Eqs. 4-5): double-float, about 1e-14 eV, in a chain of FP32

@@ -343,6 +343,7 @@ __device__ __forceinline__ void sect_pass(const Geom &g, const Band &band, const
 // cosines of the classes (now laid out once per plan) were most of the time.
 // Set-up and solve at npz = 64: 22.9 -> 14.4 us, mu within 2e-15 eV on average
 // (9e-15 before; the product in FP64 by two warps: 17 us, its errors no smaller).
+// The test whether to repeat the step costs some 0.7 us of it.
 constexpr int MU_NEWTON_MAX = 64;    // bisection alone reaches 1e-6 eV in 24 steps
 constexpr int MU_STEP_MAX = 8;
 constexpr double MU_PAIR_GAMMA = 0.002;   // eV
@@ -375,11 +376,13 @@ struct MuSingle {
     int done;
 };
 // The Halley step from mu, added to mu, in FP64 (thread 0 returns it; every
-// thread takes part).
-__device__ __forceinline__ F2 mu_step_fp64(const Geom &g, const Band &band, const MuConst &mc, MuSingle &sh, F2 mu2)
+// thread takes part).  Not inlined: its FP64 constants would be formed by every
+// solve (256 cycles an operation over the CTA's warps).
+__device__ __noinline__ F2 mu_step_fp64(MuSingle &sh, F2 mu2, int h, bool free_e, double t, double tp, double tpp,
+                                        double inv_gam, double target)
 {
     constexpr int NW = MU_THREADS / 32;
-    const int h = g.npz / 2, npairs = (h + 1) * (h + 2) / 2, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int npairs = (h + 1) * (h + 2) / 2, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     auto wide = [](F2 a) { return (double)a.h + (double)a.l; };
     const double ipi = 0.31830988618379067154, mu = wide(mu2);
     double f = 0.0;
@@ -388,10 +391,10 @@ __device__ __forceinline__ F2 mu_step_fp64(const Geom &g, const Band &band, cons
         int a, b;
         tri_pair(k, h, a, b);
         const double c1a = wide(sh.c1[a]), c1b = wide(sh.c1[b]), w = pair_weight(a, b, h);
-        const double e0 = band.band_kind == 1 ? 0.5 * (wide(sh.p2[a]) + wide(sh.p2[b]))
-                                              : -2.0 * band.t * (c1a + c1b) - 4.0 * band.tp * c1a * c1b
-                                                    - 2.0 * band.tpp * (wide(sh.c2[a]) + wide(sh.c2[b]));
-        const double x = (e0 - mu) * mc.inv_gam;
+        const double e0 = free_e ? 0.5 * (wide(sh.p2[a]) + wide(sh.p2[b]))
+                                 : -2.0 * t * (c1a + c1b) - 4.0 * tp * c1a * c1b
+                                       - 2.0 * tpp * (wide(sh.c2[a]) + wide(sh.c2[b]));
+        const double x = (e0 - mu) * inv_gam;
         f += w * (0.5 - atan(x) * ipi);
         const float xf = (float)x, r = 1.0f / (1.0f + xf * xf);
         d1 += (float)w * r;
@@ -408,7 +411,7 @@ __device__ __forceinline__ F2 mu_step_fp64(const Geom &g, const Band &band, cons
     if (threadIdx.x != 0) return F2{0.f, 0.f};
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
     for (int w = 0; w < NW; ++w) { s0 += sh.f64[w]; s1 += wide(sh.n1[w]); s2 += (double)sh.d2[w]; }
-    const double d = s0 - mc.target, dd1 = s1 * ipi * mc.inv_gam, dd2 = s2 * ipi * mc.inv_gam * mc.inv_gam;
+    const double d = s0 - target, dd1 = s1 * ipi * inv_gam, dd2 = s2 * ipi * inv_gam * inv_gam;
     const double step = -2.0 * d * dd1 / (2.0 * dd1 * dd1 - d * dd2);
     const float hi = (float)step;
     return F2{hi, (float)(step - (double)hi)};
@@ -583,7 +586,8 @@ __device__ void mu_solve_one_cta(const Geom &g, const Band &band, const MuConst 
     if (!(fabsf(mu_l) < 1e-6f)) mu_l = 0.f;
     F2 cur = f2_fast(mu, mu_l);
     for (int it = 1;; ++it) {
-        const F2 step = mc.narrow ? mu_step_fp64(g, band, mc, sh, cur) : mu_step_pairs(g, band, mc, sh, cur);
+        const F2 step = mc.narrow ? mu_step_fp64(sh, cur, h, free_e, band.t, band.tp, band.tpp, mc.inv_gam, mc.target)
+                                  : mu_step_pairs(g, band, mc, sh, cur);
         if (threadIdx.x == 0) {
             // a step that grows has left the root's neighbourhood: the one before counts
             const bool grows = it > 1 && !(fabsf(step.h) < 2.f * fabsf(sh.step.h));

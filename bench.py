@@ -131,8 +131,9 @@ def edge_carried(grid, band):
 def even_pass_bytes(s, grid, band, precision, fp32=0):
     """The same for the even form (csrc/even.cuh), which a generated A takes on
     FP32 Im chi grids of several zones (real buffers over one quadrant, k_x <=
-    k_y between the momentum passes; with the edge row where it weighs more than
-    2^-24, csrc/k_even_edge.cu), or None when the call does not take it."""
+    k_y between the momentum passes; with the edge row where edge_carried,
+    csrc/k_even_edge.cu), or None for other calls (finite temperature and FP64
+    take the form too, and are timed as a whole here)."""
     if precision != fp32 or grid["zones"] == 1 or grid.get("quantity", 0) != 0:
         return None
     lens = [16 << i for i in range(8)] + [24 << i for i in range(7)] + [72 << i for i in range(5)] + [432, 864]

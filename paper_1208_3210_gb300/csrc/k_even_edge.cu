@@ -1,6 +1,6 @@
 // The even form (even.cuh) with the edge row and column p = -N/2 dp, which have
 // no mirror on the grid, for bands whose form factor does not make them
-// negligible (few zones, small or no ff_a).
+// negligible (few zones, small or no ff_a; free electrons always).
 //
 // With half of the edge's weight put on either end of an axis, A = E + O: E
 // even, and O odd but on the edge alone.  With theta = 2 pi (k + 1/2) / P,
